@@ -29,19 +29,19 @@ void note_launches(int n) {
 
 namespace {
 
-constexpr int NC_MAX = 255;  // cells per axis (the exclusive scan covers <= 2^24 entries)
+constexpr int NC_MAX = 255;  // cells per axis (24 bits of a key)
+
+// room of one kind of marks (8 bytes of marks are read at a time)
+long long mark_stride(long long n_max) { return (std::max<long long>(n_max, 1) + 7) / 8 * 8; }
 
 struct Buffers {
   // sort
   unsigned long long *keys[2] = {nullptr, nullptr};
   unsigned int *vals[2] = {nullptr, nullptr};
-  unsigned int *hist = nullptr;
-  unsigned int *scan_tmp = nullptr;
-  int n_hist_max = 0;
-  void *scratch = nullptr;  // 8 bytes per particle, permutation staging
-  int32_t *perm = nullptr;  // composed permutation since the first build
-  int32_t *perm_tmp = nullptr;
-  int32_t *pcell = nullptr;
+  unsigned int *build_work = nullptr;  // the sort's and the compactions' counters
+  char *scratch = nullptr;   // the permuted particle arrays, BUILD_SCRATCH bytes per particle
+  uint8_t *marks = nullptr;  // leaf, chunk and group marks
+  int32_t *perm = nullptr;   // composed permutation since the first build
   // leaves (at most one per particle)
   int32_t *leaf_start = nullptr, *leaf_cell = nullptr;
   uint32_t *leaf_k = nullptr;
@@ -61,7 +61,6 @@ struct Buffers {
   int32_t *cell_start = nullptr, *cell_leaf_start = nullptr, *cell_chunk_start = nullptr;
   unsigned int *cell_stamp = nullptr, *cell_rel_stamp = nullptr;
   int32_t *q_act_cells = nullptr;
-  unsigned int *leaf_counts = nullptr, *leaf_offsets = nullptr;
   // neighbour lists of the density loop: list_cap entries per lane of every
   // warp of a persistent density launch
   float2 *nbr = nullptr;
@@ -69,9 +68,7 @@ struct Buffers {
   int32_t *wake_bin = nullptr, *q_wake = nullptr;  // limiter: wake requests and their queue
   // state
   DevState *ds = nullptr;
-  float *d_hmax = nullptr;
   double *diag = nullptr;  // diagnostics: block partials, then the result
-  unsigned int *d_bad = nullptr;  // invalid-input count of the last cell build
   DevState *h_ds = nullptr;  // pinned host mirror
 };
 
@@ -124,7 +121,6 @@ struct sph_ctx {
   long long graph_version = -1;
   bool graph_profiled = false;
   bool uniform_mass = false;   // every particle has the same mass (last cell build)
-  float m_uniform = 0.0f;      // that mass (0: the masses differ)
   bool graph_uniform = false;  // uniform_mass when the graph was captured
   int graph_kernels = 0;       // kernel nodes in the captured step
   sph_particles graph_p;
@@ -239,7 +235,6 @@ View make_view(const sph_ctx *ctx, const sph_particles *p) {
   v.leaf_hi = b.leaf_hi;
   v.leaf_min_bin = b.leaf_min_bin;
   v.leaf_bin_mask = b.leaf_bin_mask;
-  v.pcell = b.pcell;
   v.rec_xm = b.rec_xm;
   v.rec_xH = b.rec_xH;
   v.rec_v = b.rec_v;
@@ -298,8 +293,6 @@ int ensure_cells(sph_ctx *ctx, long long n_cells) {
   dfree(b.cell_stamp);
   dfree(b.cell_rel_stamp);
   dfree(b.q_act_cells);
-  dfree(b.leaf_counts);
-  dfree(b.leaf_offsets);
   long long cap = std::max<long long>(n_cells, b.cell_cap * 2);
   cap = std::min<long long>(cap, (long long)NC_MAX * NC_MAX * NC_MAX);
   cap = std::max(cap, n_cells);
@@ -309,8 +302,6 @@ int ensure_cells(sph_ctx *ctx, long long n_cells) {
   SPH_TRY(dalloc(&b.cell_stamp, cap));
   SPH_TRY(dalloc(&b.cell_rel_stamp, cap));
   SPH_TRY(dalloc(&b.q_act_cells, cap));
-  SPH_TRY(dalloc(&b.leaf_counts, cap + 1));
-  SPH_TRY(dalloc(&b.leaf_offsets, cap + 1));
   SPH_CUDA(cudaMemset(b.cell_stamp, 0, sizeof(unsigned int) * cap));
   SPH_CUDA(cudaMemset(b.cell_rel_stamp, 0, sizeof(unsigned int) * cap));
   b.cell_cap = cap;
@@ -360,33 +351,19 @@ void prof_collect(sph_ctx *ctx) {
   }
 }
 
-int permute_array(sph_ctx *ctx, void *arr, int elem, long long n, const unsigned int *perm,
-                  cudaStream_t st) {
-  if (!arr) return SPH_OK;
-  SPH_CUDA(launch_gather(ctx->b.scratch, arr, perm, n, elem, st, ctx->b.ds));
-  SPH_CUDA(cudaMemcpyAsync(arr, ctx->b.scratch, (size_t)n * elem, cudaMemcpyDeviceToDevice, st));
-  return SPH_OK;
-}
-
 int build_cells(sph_ctx *ctx, sph_particles *p, cudaStream_t st) {
   if (!valid_particles(ctx, p)) return SPH_ERR_ARG;
   Buffers &b = ctx->b;
   const long long n = p->n;
-  if (!ctx->built && n > 0) {
-    // the composed permutation starts as the identity
-    std::vector<int32_t> id((size_t)n);
-    for (long long k = 0; k < n; k++) id[(size_t)k] = (int32_t)k;
-    SPH_CUDA(cudaMemcpyAsync(b.perm, id.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, st));
-    SPH_CUDA(cudaStreamSynchronize(st));
-  }
+  if (n > BUILD_MAX) return SPH_ERR_CUDA;
   View v = make_view(ctx, p);
   // cells per axis from the largest support
   int nc = ctx->prm.n_cells_override;
   if (nc <= 0) {
-    SPH_CUDA(launch_reduce_hmax(v, b.d_hmax, st));
-    float hmax = 0.0f;
-    SPH_CUDA(cudaMemcpyAsync(&hmax, b.d_hmax, sizeof(float), cudaMemcpyDeviceToHost, st));
-    SPH_CUDA(cudaStreamSynchronize(st));
+    SPH_CUDA(launch_reduce_hmax(v, st));
+    SPH_TRY(read_state(ctx, st));
+    float hmax;
+    std::memcpy(&hmax, &b.h_ds->build_hmax_bits, sizeof(float));
     if (n > 0 && !(hmax > 0.0f && std::isfinite(hmax))) return SPH_ERR_ARG;
     hmax = std::max(hmax, ctx->h_floor);
     double Hmax = GAMMA_K_D * (double)hmax;
@@ -397,114 +374,28 @@ int build_cells(sph_ctx *ctx, sph_particles *p, cudaStream_t st) {
   SPH_TRY(ensure_cells(ctx, n_cells));
   v = make_view(ctx, p);
   const double w = ctx->prm.box / (double)nc;
-  // keys, stable radix sort, permutation of every particle array
-  SPH_CUDA(cudaMemsetAsync(b.d_bad, 0, sizeof(unsigned int), st));
-  SPH_CUDA(launch_cell_keys(v, nc, w, b.keys[0], b.vals[0], b.d_bad, st));
-  if (n > 0) {
-    // non-finite positions or h: rejected before anything is reordered
-    unsigned int bad = 0;
-    SPH_CUDA(cudaMemcpyAsync(&bad, b.d_bad, sizeof(unsigned int), cudaMemcpyDeviceToHost, st));
-    SPH_CUDA(cudaStreamSynchronize(st));
-    if (bad) return SPH_ERR_ARG;
-  }
-  int cell_bits = 1;
-  while ((1LL << cell_bits) < n_cells) cell_bits++;
-  bool alt = false;
-  SPH_CUDA(radix_sort_pairs(b.keys[0], b.vals[0], b.keys[1], b.vals[1], (int)n,
-                            KEY_MORTON_BITS + cell_bits, b.hist, b.scan_tmp, b.n_hist_max, &alt,
-                            st, b.ds));
-  unsigned long long *skeys = alt ? b.keys[1] : b.keys[0];
-  unsigned int *perm = alt ? b.vals[1] : b.vals[0];
-  SPH_TRY(permute_array(ctx, p->x, 8, n, perm, st));
-  SPH_TRY(permute_array(ctx, p->y, 8, n, perm, st));
-  SPH_TRY(permute_array(ctx, p->z, 8, n, perm, st));
-  float *f32[] = {p->vx, p->vy, p->vz, p->ax, p->ay, p->az, p->A, p->Adot, p->h,
-                  p->rho, p->f, p->P, p->c, p->vsig, p->m};
-  for (float *a : f32) SPH_TRY(permute_array(ctx, a, 4, n, perm, st));
-  SPH_TRY(permute_array(ctx, p->bin, 1, n, perm, st));
-  SPH_TRY(permute_array(ctx, p->ti_begin, 8, n, perm, st));
-  SPH_TRY(permute_array(ctx, p->ti_end, 8, n, perm, st));
-  SPH_TRY(permute_array(ctx, p->ti_drift, 8, n, perm, st));
-  SPH_TRY(permute_array(ctx, p->ngb_density, 4, n, perm, st));
-  SPH_TRY(permute_array(ctx, p->ngb_force, 4, n, perm, st));
-  SPH_TRY(permute_array(ctx, p->div_v, 4, n, perm, st));
-  SPH_TRY(permute_array(ctx, p->curl_v, 4, n, perm, st));
-  if (n > 0) {
-    SPH_CUDA(launch_gather(b.perm_tmp, b.perm, perm, n, 4, st, b.ds));
-    SPH_CUDA(cudaMemcpyAsync(b.perm, b.perm_tmp, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, st));
-    SPH_CUDA(cudaMemsetAsync(p->active, 0, (size_t)n, st));
-  }
-  // cells and leaves
-  SPH_CUDA(launch_cell_start(skeys, n, (int)n_cells, b.cell_start, b.pcell, st));
-  // (scratch: the marks in b.scratch, the node lists in the sort's spare key
-  // buffer, the counters in the histogram)
-  const unsigned int *d_n_leaves = nullptr;
-  SPH_CUDA(launch_leaves(skeys, b.cell_start, (int)n_cells, n, ctx->prm.leaf_max,
-                         (uint8_t *)b.scratch, (int2 *)(alt ? b.keys[0] : b.keys[1]), b.hist,
-                         b.scan_tmp, b.leaf_start, b.leaf_cell, b.leaf_k, b.cell_leaf_start,
-                         2 * ctx->grid_util, &d_n_leaves, st));
-  SPH_CUDA(cudaMemcpyAsync(SPH_DS_FIELD(b.ds, n_leaves), d_n_leaves, sizeof(int),
-                           cudaMemcpyDeviceToDevice, st));
-  int n_leaves_h = 0;
-  SPH_CUDA(cudaMemcpyAsync(&n_leaves_h, d_n_leaves, sizeof(int), cudaMemcpyDeviceToHost, st));
-  SPH_CUDA(cudaStreamSynchronize(st));
-  // work groups and the leaf of each particle
-  SPH_CUDA(launch_groups(b.cell_leaf_start, b.leaf_start, (int)n_cells, (int)n, b.leaf_counts,
-                         b.leaf_offsets, b.scan_tmp, b.group_leaf0, b.group_cell, b.pleaf, n_leaves_h,
-                         st));
-  SPH_CUDA(cudaMemcpyAsync(SPH_DS_FIELD(b.ds, n_groups), b.leaf_offsets + n_cells, sizeof(int),
-                           cudaMemcpyDeviceToDevice, st));
-  // chunks: octree nodes of at most CHUNK leaves (scratch free again by now:
-  // the leaves' first keys in the spare key buffer, the node lists in the
-  // sorted keys' buffer, the marks in b.scratch, the counters in the
-  // histogram, the unused corners in b.vals[0])
-  const unsigned int *d_n_chunks = nullptr;
-  SPH_CUDA(launch_chunks(skeys, b.leaf_start, b.cell_leaf_start, (int)n_cells, n_leaves_h,
-                         alt ? b.keys[0] : b.keys[1], (uint8_t *)b.scratch,
-                         reinterpret_cast<int2 *>(skeys), b.hist, b.scan_tmp,
-                         reinterpret_cast<uint32_t *>(b.vals[0]), b.chunk_leaf_start, b.chunk_cell,
-                         b.cell_chunk_start, b.leaf_chunk, 2 * ctx->grid_util, &d_n_chunks, st));
-  SPH_CUDA(cudaMemcpyAsync(SPH_DS_FIELD(b.ds, n_chunks), d_n_chunks, sizeof(int),
-                           cudaMemcpyDeviceToDevice, st));
-  // device state of the new structure
-  int ncs[2] = {nc, (int)n_cells};
-  SPH_CUDA(cudaMemcpyAsync(SPH_DS_FIELD(b.ds, nc), &ncs[0], sizeof(int), cudaMemcpyHostToDevice, st));
-  SPH_CUDA(cudaMemcpyAsync(SPH_DS_FIELD(b.ds, n_cells), &ncs[1], sizeof(int), cudaMemcpyHostToDevice, st));
-  SPH_CUDA(cudaMemcpyAsync(SPH_DS_FIELD(b.ds, w), &w, sizeof(double), cudaMemcpyHostToDevice, st));
-  SPH_CUDA(cudaMemsetAsync(SPH_DS_FIELD(b.ds, n_active_leaves), 0, sizeof(int), st));
-  SPH_CUDA(cudaMemsetAsync(SPH_DS_FIELD(b.ds, n_active_groups), 0, sizeof(int), st));
-  SPH_CUDA(cudaMemsetAsync(SPH_DS_FIELD(b.ds, excursion_bits), 0, sizeof(unsigned int), st));
-  SPH_CUDA(cudaMemsetAsync(SPH_DS_FIELD(b.ds, Hmax_bits), 0, sizeof(unsigned int), st));
-  SPH_CUDA(cudaMemsetAsync(SPH_DS_FIELD(b.ds, want_h_bits), 0, sizeof(unsigned int), st));
-  SPH_CUDA(launch_bin_histogram(v, st));
+  const BuildArrays ba = {{b.keys[0], b.keys[1]}, {b.vals[0], b.vals[1]}, b.build_work, b.scratch,
+                          b.marks, b.perm, mark_stride(ctx->n_max)};
+  SPH_CUDA(launch_build(v, ba, nc, w, (int)n_cells, !ctx->built, st));
   SPH_CUDA(launch_refresh_all(v, st));
   // cost estimate of every work group (only heavy-group scheduling uses it)
   if (ctx->prm.heavy_factor > 0.0) SPH_CUDA(launch_group_cost(v, ctx->grid_dens, st));
-  // equal masses: the density loop sums the kernel alone (rho = m sum w)
-  SPH_CUDA(launch_mass_range(v, st));
-  int nl = 0;
-  unsigned int mr[2] = {0u, 0u};
-  SPH_CUDA(cudaMemcpyAsync(&nl, SPH_DS_FIELD(b.ds, n_leaves), sizeof(int), cudaMemcpyDeviceToHost, st));
-  SPH_CUDA(cudaMemcpyAsync(mr, SPH_DS_FIELD(b.ds, m_lo_bits), 2 * sizeof(unsigned int),
-                           cudaMemcpyDeviceToHost, st));
-  SPH_CUDA(cudaStreamSynchronize(st));
-  ctx->n_leaves = nl;
-  {
-    float lo, hi;
-    std::memcpy(&lo, &mr[0], sizeof(float));
-    std::memcpy(&hi, &mr[1], sizeof(float));
-    ctx->m_uniform = (n > 0 && mr[0] == mr[1] && lo > 0.0f && std::isfinite(lo)) ? lo : 0.0f;
-    (void)hi;
+  // no wake request survives a reordering (a halted step may have left some)
+  if (ctx->prm.limiter)
+    SPH_CUDA(cudaMemsetAsync(b.wake_bin, 0x7f, sizeof(int32_t) * (size_t)ctx->n_max, st));
+  SPH_TRY(read_state(ctx, st));
+  const DevState &h = *b.h_ds;
+  // non-finite positions or h: rejected before anything was reordered
+  if (h.build_bad) return SPH_ERR_ARG;
+  if (h.build_fail) {
+    ctx->built = false;
+    return (int)h.build_fail;
   }
-  ctx->uniform_mass = ctx->m_uniform > 0.0f;
-  SPH_CUDA(cudaMemcpyAsync(SPH_DS_FIELD(b.ds, m_uniform), &ctx->m_uniform, sizeof(float),
-                           cudaMemcpyHostToDevice, st));
-  SPH_CUDA(cudaStreamSynchronize(st));  // (the build is complete on return, as before)
+  ctx->n_leaves = h.n_leaves;
+  ctx->uniform_mass = h.m_uniform > 0.0f;
   ctx->h_floor = 0.0f;
   ctx->nc = nc;
   ctx->w = w;
-  // no wake request survives a reordering (a halted step may have left some)
-  SPH_CUDA(cudaMemsetAsync(b.wake_bin, 0x7f, sizeof(int32_t) * (size_t)ctx->n_max, st));
   ctx->built = true;
   ctx->rebuilds++;
   return SPH_OK;
@@ -787,12 +678,10 @@ int sph_create(const sph_params *params, int64_t n_max, sph_ctx **out) {
     }
     Buffers &b = ctx->b;
     const long long n = std::max<long long>(n_max, 1);
-    const long long n_tiles = (n + 4095) / 4096;
-    b.n_hist_max = (int)(256 * n_tiles);
     if ((r = dalloc(&b.keys[0], n)) || (r = dalloc(&b.keys[1], n)) || (r = dalloc(&b.vals[0], n)) ||
-        (r = dalloc(&b.vals[1], n)) || (r = dalloc(&b.hist, b.n_hist_max)) ||
-        (r = dalloc(&b.scan_tmp, 4096)) || (r = dalloc((char **)&b.scratch, 8 * n)) ||
-        (r = dalloc(&b.perm, n)) || (r = dalloc(&b.perm_tmp, n)) || (r = dalloc(&b.pcell, n)) ||
+        (r = dalloc(&b.vals[1], n)) || (r = dalloc(&b.build_work, build_work_words(n))) ||
+        (r = dalloc(&b.scratch, BUILD_SCRATCH * n)) || (r = dalloc(&b.marks, 3 * mark_stride(n))) ||
+        (r = dalloc(&b.perm, n)) ||
         (r = dalloc(&b.leaf_start, n + 1)) || (r = dalloc(&b.leaf_cell, n)) || (r = dalloc(&b.leaf_k, n)) ||
         (r = dalloc(&b.chunk_cell, n)) || (r = dalloc(&b.chunk_leaf_start, n + 1)) ||
         (r = dalloc(&b.leaf_chunk, n)) || (r = dalloc(&b.chunk_lo, n)) || (r = dalloc(&b.chunk_hi, n)) ||
@@ -802,9 +691,8 @@ int sph_create(const sph_params *params, int64_t n_max, sph_ctx **out) {
         (r = dalloc(&b.q_group, n)) || (r = dalloc(&b.pleaf, n)) || (r = dalloc(&b.group_leaf0, n + 1)) ||
         (r = dalloc(&b.group_cell, n)) || (r = dalloc(&b.group_cost, n)) ||
         (r = dalloc(&b.rec_xm, n)) || (r = dalloc(&b.rec_xH, n)) || (r = dalloc(&b.rec_v, n)) ||
-        (r = dalloc(&b.rec_h, n)) || (r = dalloc(&b.ds, 1)) || (r = dalloc(&b.d_hmax, 1)) ||
-        (r = dalloc(&b.diag, (long long)(DIAG_BLOCKS + 1) * DIAG_FIELDS)) ||
-        (r = dalloc(&b.d_bad, 1)))
+        (r = dalloc(&b.rec_h, n)) || (r = dalloc(&b.ds, 1)) ||
+        (r = dalloc(&b.diag, (long long)(DIAG_BLOCKS + 1) * DIAG_FIELDS)))
       break;
     if (cudaMallocHost((void **)&b.h_ds, sizeof(DevState)) != cudaSuccess) {
       r = SPH_ERR_NOMEM;
@@ -861,9 +749,8 @@ int sph_destroy(sph_ctx *ctx) {
         if (ev) cudaEventDestroy(ev);
   Buffers &b = ctx->b;
   dfree(b.keys[0]); dfree(b.keys[1]); dfree(b.vals[0]); dfree(b.vals[1]);
-  dfree(b.hist); dfree(b.scan_tmp);
-  if (b.scratch) cudaFree(b.scratch);
-  dfree(b.perm); dfree(b.perm_tmp); dfree(b.pcell);
+  dfree(b.build_work); dfree(b.scratch); dfree(b.marks);
+  dfree(b.perm);
   dfree(b.leaf_start); dfree(b.leaf_cell); dfree(b.leaf_k);
   dfree(b.chunk_cell); dfree(b.chunk_leaf_start); dfree(b.leaf_chunk); dfree(b.chunk_lo); dfree(b.chunk_hi); dfree(b.leaf_lo); dfree(b.leaf_hi);
   dfree(b.leaf_min_bin); dfree(b.leaf_bin_mask);
@@ -871,8 +758,8 @@ int sph_destroy(sph_ctx *ctx) {
   dfree(b.pleaf); dfree(b.group_leaf0); dfree(b.group_cell); dfree(b.group_cost);
   dfree(b.rec_xm); dfree(b.rec_xH); dfree(b.rec_v); dfree(b.rec_h);
   dfree(b.cell_start); dfree(b.cell_leaf_start); dfree(b.cell_stamp); dfree(b.cell_rel_stamp);
-  dfree(b.q_act_cells); dfree(b.leaf_counts); dfree(b.leaf_offsets);
-  dfree(b.ds); dfree(b.d_hmax); dfree(b.diag); dfree(b.d_bad);
+  dfree(b.cell_chunk_start); dfree(b.q_act_cells);
+  dfree(b.ds); dfree(b.diag);
   dfree(b.nbr); dfree(b.ngb_bin); dfree(b.wake_bin); dfree(b.q_wake);
   if (b.h_ds) cudaFreeHost(b.h_ds);
   delete ctx;

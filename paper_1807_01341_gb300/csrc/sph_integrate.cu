@@ -366,6 +366,7 @@ __device__ void chunk_update(const View &v, int g, bool do_drift, bool do_bins) 
 }
 
 __global__ void __launch_bounds__(UT) k_refresh(View v) {
+  if (v.ds->build_bad | v.ds->build_fail) return;  // (a build that was stopped)
   const int ng = v.ds->n_chunks;
   for (int g = blockIdx.x; g < ng; g += gridDim.x) chunk_update(v, g, false, true);
 }

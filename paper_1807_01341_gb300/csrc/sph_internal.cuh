@@ -83,8 +83,11 @@ struct DevState {
   unsigned long long wakes;   // limiter: inactive particles whose steps were cut
   // time-bin occupancy
   int bin_count[MAX_BINS];
-  // smallest and largest particle mass (float bits), found at each cell build
-  unsigned int m_lo_bits, m_hi_bits;
+  // the cell build in progress: invalid particles, the SPH_ERR_* that stopped
+  // it, the particles' mass range (largest inverted and plain float bits) --
+  // these four are cleared together -- and the largest smoothing length
+  unsigned int build_bad, build_fail, m_nlo_bits, m_hi_bits;
+  unsigned int build_hmax_bits;
 };
 
 // Pointers and constants handed to every kernel (by value).
@@ -121,7 +124,6 @@ struct View {
   float4 *leaf_hi;           // bbox max (cell-relative)
   uint8_t *leaf_min_bin;     // smallest bin in the leaf
   unsigned long long *leaf_bin_mask;  // bins present in the leaf
-  int32_t *pcell;            // [n] cell of each particle
   int32_t *pleaf;            // [n] leaf of each particle
   int32_t *group_leaf0;      // [n_groups + 1] first leaf of each work group
   int32_t *group_cell;       // [n_groups] cell of each work group
@@ -267,44 +269,34 @@ void note_launches(int n);
 // launchers implemented in the .cu files (all asynchronous on `st`)
 // ---------------------------------------------------------------------------
 // sph_cells.cu
-cudaError_t launch_reduce_hmax(const View &v, float *out_max, cudaStream_t st);
-cudaError_t launch_mass_range(const View &v, cudaStream_t st);
-// (bad: a device counter, incremented per particle with a non-finite position
-// or an h that is not a positive finite number)
-cudaError_t launch_cell_keys(const View &v, int nc, double w, unsigned long long *keys,
-                             unsigned int *vals, unsigned int *bad, cudaStream_t st);
-cudaError_t radix_sort_pairs(unsigned long long *keys, unsigned int *vals,
-                             unsigned long long *keys_alt, unsigned int *vals_alt, int n,
-                             int nbits, unsigned int *hist, unsigned int *scan_tmp,
-                             int n_hist_max, bool *result_in_alt, cudaStream_t st,
-                             DevState *ds);  // ds: where a failed bounds check is recorded (may be null)
-cudaError_t exclusive_scan_u32(const unsigned int *in, unsigned int *out, int n,
-                               unsigned int *tmp, cudaStream_t st);
-cudaError_t launch_gather(void *dst, const void *src, const unsigned int *idx, long long n,
-                          int elem_bytes, cudaStream_t st, DevState *ds);
-cudaError_t launch_cell_start(const unsigned long long *sorted_keys, long long n, int n_cells,
-                              int32_t *cell_start, int32_t *pcell, cudaStream_t st);
-// Leaves of every cell in particle order (leaf_start[n_leaves] = n), their
-// cells and corners, and the first leaf of every cell (cell_leaf_start[n_cells]
-// = n_leaves).  Scratch: lead (n bytes), nodes (n int2), work (n/4096 + 12
-// words); *n_leaves points at the device count.
-cudaError_t launch_leaves(const unsigned long long *sorted_keys, const int32_t *cell_start,
-                          int n_cells, long long n, int leaf_max, uint8_t *lead, int2 *nodes,
-                          unsigned int *work, unsigned int *scan_tmp, int32_t *leaf_start,
-                          int32_t *leaf_cell, uint32_t *leaf_k, int32_t *cell_leaf_start,
-                          int grid, const unsigned int **n_leaves, cudaStream_t st);
-cudaError_t launch_bin_histogram(const View &v, cudaStream_t st);
-cudaError_t launch_groups(const int32_t *cell_leaf_start, const int32_t *leaf_start, int n_cells,
-                          int n_leaves_max, unsigned int *counts, unsigned int *offsets,
-                          unsigned int *scan_tmp, int32_t *group_leaf0, int32_t *group_cell,
-                          int32_t *pleaf, int n_leaves_host, cudaStream_t st);
-cudaError_t launch_chunks(const unsigned long long *sorted_keys, const int32_t *leaf_start,
-                          const int32_t *cell_leaf_start, int n_cells, int n_leaves,
-                          unsigned long long *leaf_keys, uint8_t *lead, int2 *nodes,
-                          unsigned int *work, unsigned int *scan_tmp, uint32_t *corner_tmp,
-                          int32_t *chunk_leaf_start, int32_t *chunk_cell,
-                          int32_t *cell_chunk_start, int32_t *leaf_chunk, int grid,
-                          const unsigned int **n_chunks, cudaStream_t st);
+// Largest h of the particles into ds->build_hmax_bits.
+cudaError_t launch_reduce_hmax(const View &v, cudaStream_t st);
+// Scratch words of radix_sort_indices and of a build over n items.
+size_t sort_work_words(long long n);
+size_t build_work_words(long long n);
+// Sorts keys stably by their low nbits (at most 56), vals = the keys' indices in that order;
+// the result is in (keys, vals) or the alternates.
+cudaError_t radix_sort_indices(unsigned long long *keys, unsigned int *vals,
+                               unsigned long long *keys_alt, unsigned int *vals_alt, int n,
+                               int nbits, unsigned int *work, bool *result_in_alt, cudaStream_t st);
+// The buffers of a cell build (one context's, sized for n_max particles).
+constexpr long long BUILD_MAX = 1ll << 24;  // most particles of a build
+constexpr size_t BUILD_SCRATCH = 128;       // scratch bytes per particle (its permuted arrays)
+struct BuildArrays {
+  unsigned long long *keys[2];
+  unsigned int *vals[2];
+  unsigned int *work;           // build_work_words(n_max)
+  char *scratch;                // BUILD_SCRATCH * n_max bytes, 32-byte aligned
+  uint8_t *marks;               // 3 * n_max, n_max a multiple of 8
+  int32_t *perm;
+  long long n_max;
+};
+// Everything of a cell build after its grid is chosen: keys, sort, permutation of the
+// particle arrays, leaves, chunks, work groups, the device state of the structure.  Invalid
+// input (ds->build_bad) or a failed wait (ds->build_fail) stops the remaining
+// kernels.  first: the composed permutation starts here.
+cudaError_t launch_build(const View &v, const BuildArrays &b, int nc, double w, int n_cells,
+                         bool first, cudaStream_t st);
 // sph_integrate.cu
 cudaError_t launch_refresh_all(const View &v, cudaStream_t st);
 cudaError_t launch_mark(const View &v, long long ti_or_neg, cudaStream_t st);

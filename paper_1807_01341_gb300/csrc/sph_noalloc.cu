@@ -15,15 +15,14 @@ namespace sph {
 namespace {
 
 constexpr int NOALLOC_MAX = 1 << 16;                       // particles per call
-constexpr int NOALLOC_TILES = (NOALLOC_MAX + 4095) / 4096;  // radix-sort tiles of 4096 keys
 // byte offsets inside the scratch array (each a multiple of 256)
 constexpr size_t OFF_KEYS0 = 0;
 constexpr size_t OFF_KEYS1 = OFF_KEYS0 + sizeof(unsigned long long) * NOALLOC_MAX;
 constexpr size_t OFF_VALS0 = OFF_KEYS1 + sizeof(unsigned long long) * NOALLOC_MAX;
 constexpr size_t OFF_VALS1 = OFF_VALS0 + sizeof(unsigned int) * NOALLOC_MAX;
-constexpr size_t OFF_HIST = OFF_VALS1 + sizeof(unsigned int) * NOALLOC_MAX;
-constexpr size_t OFF_SCAN = OFF_HIST + sizeof(unsigned int) * 256 * NOALLOC_TILES;
-constexpr size_t SCRATCH_BYTES = OFF_SCAN + sizeof(unsigned int) * 4096;  // 1.6 MB
+constexpr size_t OFF_WORK = OFF_VALS1 + sizeof(unsigned int) * NOALLOC_MAX;
+constexpr size_t WORK_WORDS = 10240;                        // sort_work_words(NOALLOC_MAX)
+constexpr size_t SCRATCH_BYTES = OFF_WORK + sizeof(unsigned int) * WORK_WORDS;  // 1.6 MB
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[SCRATCH_BYTES];
 
@@ -81,8 +80,7 @@ __device__ __forceinline__ unsigned long long spread3_ro(unsigned long long v) {
 
 __global__ void k_cell_keys_ro(const double *__restrict__ xs, const double *__restrict__ ys,
                                const double *__restrict__ zs, int n, double box, int nc, double w,
-                               unsigned long long *__restrict__ keys,
-                               unsigned int *__restrict__ vals) {
+                               unsigned long long *__restrict__ keys) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const double x = wrap_box_ro(xs[i], box), y = wrap_box_ro(ys[i], box), z = wrap_box_ro(zs[i], box);
@@ -92,7 +90,6 @@ __global__ void k_cell_keys_ro(const double *__restrict__ xs, const double *__re
                                   (spread3_ro(axis_morton_ro(y, cy, w)) << 1) |
                                   spread3_ro(axis_morton_ro(z, cz, w));
   keys[i] = (cid << KEY_MORTON_BITS) | mort;
-  vals[i] = (unsigned int)i;
 }
 
 }  // namespace
@@ -114,20 +111,20 @@ extern "C" int sph_cell_order_noalloc(const double *x, const double *y, const do
   auto *keys1 = reinterpret_cast<unsigned long long *>(s + OFF_KEYS1);
   auto *vals0 = reinterpret_cast<unsigned int *>(s + OFF_VALS0);
   auto *vals1 = reinterpret_cast<unsigned int *>(s + OFF_VALS1);
-  auto *hist = reinterpret_cast<unsigned int *>(s + OFF_HIST);
-  auto *scan = reinterpret_cast<unsigned int *>(s + OFF_SCAN);
+  auto *work = reinterpret_cast<unsigned int *>(s + OFF_WORK);
+  if (sort_work_words(n) > WORK_WORDS) return SPH_ERR_CUDA;
   const int nc = n_cells_per_axis;
   const double w = box / (double)nc;
   const long long n_cells = (long long)nc * nc * nc;
   note_launches(1);
-  k_cell_keys_ro<<<(int)((n + 255) / 256), 256, 0, st>>>(x, y, z, (int)n, box, nc, w, keys0, vals0);
+  k_cell_keys_ro<<<(int)((n + 255) / 256), 256, 0, st>>>(x, y, z, (int)n, box, nc, w, keys0);
   if (cudaGetLastError() != cudaSuccess) return SPH_ERR_CUDA;
   int cell_bits = 1;
   while ((1LL << cell_bits) < n_cells) cell_bits++;
-  // every buffer the sort reads is written first in each call: nothing to clear
+  // (each call clears or writes every part of the array it reads)
   bool alt = false;
-  if (radix_sort_pairs(keys0, vals0, keys1, vals1, (int)n, KEY_MORTON_BITS + cell_bits, hist, scan,
-                       256 * NOALLOC_TILES, &alt, st, nullptr) != cudaSuccess)
+  if (radix_sort_indices(keys0, vals0, keys1, vals1, (int)n, KEY_MORTON_BITS + cell_bits, work, &alt,
+                         st) != cudaSuccess)
     return SPH_ERR_CUDA;
   if (cudaMemcpyAsync(perm, alt ? vals1 : vals0, sizeof(int32_t) * (size_t)n,
                       cudaMemcpyDeviceToDevice, st) != cudaSuccess)

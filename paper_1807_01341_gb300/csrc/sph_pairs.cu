@@ -1216,6 +1216,7 @@ __global__ void __launch_bounds__(PT, 2) k_gradient(View v) {
 // mean).
 __global__ void __launch_bounds__(PT, 2) k_group_cost(View v) {
   DevState *ds = v.ds;
+  if (ds->build_bad | ds->build_fail) return;  // (a build that was stopped)
   StageD st;
   stage_init(st);
   const int lane = lane_id();
@@ -1397,8 +1398,6 @@ cudaError_t launch_group_cost(const View &v, int grid, cudaStream_t st) {
   note_launches(1);
   cudaError_t e = cudaFuncSetAttribute(k_group_cost, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)DENS_SMEM);
-  if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(SPH_DS_FIELD(v.ds, group_cost_sum), 0, sizeof(unsigned long long), st);
   if (e != cudaSuccess) return e;
   k_group_cost<<<grid, PT, DENS_SMEM, st>>>(v);
   return cudaGetLastError();
