@@ -1089,7 +1089,7 @@ int sph_grid_density(sph_ctx *ctx, const sph_particles *p, int n_grid, int64_t t
   const size_t ng3 = (size_t)n_grid * n_grid * n_grid;
   SPH_CUDA(cudaMemsetAsync(rho_grid, 0, ng3 * sizeof(double), S(stream)));
   SPH_CUDA(launch_grid_density(*p, n_grid, ti, ctx->prm.dt_min, ctx->prm.box, rho_grid, nullptr,
-                               nullptr, S(stream)));
+                               nullptr, ctx->num_sms, S(stream)));
   return SPH_OK;
 }
 
@@ -1099,7 +1099,7 @@ int sph_grid_density_bwd(sph_ctx *ctx, const sph_particles *p, int n_grid, int64
       ti < 0 || !valid_adjoint(adj, p->n))
     return SPH_ERR_ARG;
   SPH_CUDA(launch_grid_density(*p, n_grid, ti, ctx->prm.dt_min, ctx->prm.box, nullptr,
-                               rho_grid_bar, adj, S(stream)));
+                               rho_grid_bar, adj, ctx->num_sms, S(stream)));
   return SPH_OK;
 }
 

@@ -326,7 +326,7 @@ cudaError_t launch_adj_step(const View &v, const AdjWork &w, const sph_particles
                             int first, int grid_pairs, cudaStream_t st);
 cudaError_t launch_grid_density(const sph_particles &p, int n_grid, long long ti, double dt_min,
                                 double box, double *rho_g, const double *rho_bar,
-                                const sph_adjoint *adj, cudaStream_t st);
+                                const sph_adjoint *adj, int num_sms, cudaStream_t st);
 cudaError_t launch_state_copy(const sph_particles &src, const sph_particles &dst,
                               const int32_t *perm, cudaStream_t st);
 int adj_blocks_per_sm();
