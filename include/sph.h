@@ -111,7 +111,9 @@ typedef struct {
   int list_cap;         /* density loop: entries of each active particle's neighbour list
                            (squared distance and mass of every candidate within
                            search_margin x its support, kept across the h iterations;
-                           a gather that finds more runs in passes of list_cap); 32..4096.
+                           a particle that has more is evaluated without a list, by a
+                           warp of its own, or, with several lanes per particle, in
+                           passes of list_cap); 32..4096.
                            The library holds 8 x list_cap bytes per lane of every warp
                            of the persistent density grid for them (2 blocks of 8 warps
                            per SM: 319 MB at 512 on 152 SMs), whatever the particle count.
@@ -202,7 +204,7 @@ typedef struct {
   int64_t gathers_density; /* density loop: particle gathers (a particle counted once in
                               every staging pass over its candidates) */
   int64_t list_overflows;  /* density loop: gathers whose neighbour list filled up (the
-                              gather then ran further passes over the same leaves) */
+                              particle then goes on without one, see list_cap) */
   int64_t evals_density;   /* density loop: neighbour-list entries evaluated, all h
                               iterations (pair terms computed, in or beyond the support) */
   int64_t wakes;           /* limiter: inactive particles woken (their steps cut short

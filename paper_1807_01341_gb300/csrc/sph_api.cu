@@ -269,6 +269,8 @@ View make_view(const sph_ctx *ctx, const sph_particles *p) {
   v.uniform_mass = ctx->uniform_mass ? 1 : 0;
   v.grid_util = ctx->grid_util;
   v.nbr = b.nbr;
+  static_assert(sizeof(BigItem) <= BUILD_SCRATCH, "the items fit the build's scratch");
+  v.big = reinterpret_cast<BigItem *>(b.scratch);
   v.list_cap = q.list_cap;
   v.list_blocks = ctx->list_blocks;
   v.search_margin = (float)q.search_margin;
@@ -407,6 +409,7 @@ int batched_body(sph_ctx *ctx, const View &v, int flags, cudaStream_t st) {
   SPH_CUDA(launch_drift(v, st));
   prof_begin(ctx, 0, st);
   SPH_CUDA(launch_density(v, flags, -1, true, ctx->grid_dens, st));
+  SPH_CUDA(launch_density_rest(v, flags, ctx->grid_dens, st));
   prof_end(ctx, 0, st);
   if (flags & SPH_DENSITY_INIT_ENTROPY) SPH_CUDA(launch_entropy_from_u(v, st));
   if (v.balsara || v.predict) SPH_CUDA(launch_gradient(v, ctx->grid_force, st));
@@ -439,6 +442,7 @@ int plain_body(sph_ctx *ctx, const View &v, int flags, cudaStream_t st) {
     SPH_CUDA(launch_density(v, flags, bins[k], true, std::min(want, ctx->list_blocks), st));
     prof_end(ctx, 0, st);
   }
+  SPH_CUDA(launch_density_rest(v, flags, ctx->grid_dens, st));
   if (flags & SPH_DENSITY_INIT_ENTROPY) SPH_CUDA(launch_entropy_from_u(v, st));
   if (v.balsara || v.predict) SPH_CUDA(launch_gradient(v, ctx->grid_force, st));
   for (int k = 0; k < nb; k++) {
@@ -806,6 +810,7 @@ int sph_density_active(sph_ctx *ctx, sph_particles *p, int flags, void *stream) 
   if (!ctx->built) return SPH_ERR_NOT_BUILT;
   View v = make_view(ctx, p);
   SPH_CUDA(launch_density(v, flags, -1, true, ctx->grid_dens, S(stream)));
+  SPH_CUDA(launch_density_rest(v, flags, ctx->grid_dens, S(stream)));
   if (flags & SPH_DENSITY_INIT_ENTROPY) SPH_CUDA(launch_entropy_from_u(v, S(stream)));
   if (v.balsara || v.predict) SPH_CUDA(launch_gradient(v, ctx->grid_force, S(stream)));
   return SPH_OK;

@@ -70,6 +70,8 @@ struct DevState {
   unsigned int Hmax_bits;       // max kernel support H (float bits) over all particles
   unsigned int want_h_bits;     // largest h an iteration wanted beyond the cell limit
   int dens_split;               // parts per work group of the last whole-step density launch
+  int n_big;              // density loop: particles left to one warp each (View::big)
+  int head_big;           // work head of those
   // counters of the step in progress (reset when a step starts, added to the
   // totals when it completes, so a halted attempt leaves no trace)
   unsigned long long s_pairs_density, s_pairs_force, s_cand_density, s_cand_force;
@@ -88,6 +90,14 @@ struct DevState {
   // these four are cleared together -- and the largest smoothing length
   unsigned int build_bad, build_fail, m_nlo_bits, m_hi_bits;
   unsigned int build_hmax_bits;
+};
+
+// A particle that the density loop leaves to k_density_big: the state of its
+// h iteration and its work group.
+struct BigItem {
+  double lo, hi;  // bracket
+  float h;
+  int i, it, wg;
 };
 
 // Pointers and constants handed to every kernel (by value).
@@ -150,6 +160,7 @@ struct View {
   // nbr[((b * 8 + w) * list_cap + k) * 32 + s]): the area of a warp is reused
   // by its next work group, so the lists stay in L2.
   float2 *nbr;
+  BigItem *big;              // [n] (the build's scratch, free between builds)
   DevState *ds;
   // parameters
   double box, eta, gamma, alpha, cfl, h_tol, dt_min;
@@ -309,6 +320,10 @@ cudaError_t launch_close_step(const View &v, cudaStream_t st);
 // sph_pairs.cu
 cudaError_t launch_density(const View &v, int flags, int bin_filter, bool persistent,
                            int grid, cudaStream_t st);
+// The particles that the density launches since the step began left to one
+// warp each, then the supports of the leaves whose groups were split or had
+// such particles.
+cudaError_t launch_density_rest(const View &v, int flags, int grid, cudaStream_t st);
 cudaError_t launch_force(const View &v, int bin_filter, bool persistent, int grid,
                          cudaStream_t st);
 cudaError_t launch_entropy_from_u(const View &v, cudaStream_t st);

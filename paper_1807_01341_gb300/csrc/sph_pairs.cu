@@ -93,6 +93,15 @@ __device__ __forceinline__ void fast2sum(float &hi, float &lo, float x) {
   hi = t;
 }
 
+// (hi, lo) += x y, the product fused into the sum and into its error (as the
+// compiler contracts fast2sum(hi, lo, x * y); written out so that every loop
+// that forms these sums rounds them alike)
+__device__ __forceinline__ void fast2sum_prod(float &hi, float &lo, float x, float y) {
+  const float t = __fmaf_rn(x, y, hi);
+  lo += __fmaf_rn(x, y, -(t - hi));
+  hi = t;
+}
+
 struct DSum {
   float n_hi, n_lo, t_hi, t_lo, r_hi, r_lo, rt_hi, rt_lo;
   float p2;
@@ -120,8 +129,8 @@ __device__ __forceinline__ void dens_pair(DSum &s, float r2, float mj, float H2,
   fast2sum(s.n_hi, s.n_lo, wq);
   fast2sum(s.t_hi, s.t_lo, tt);
   if constexpr (!UM) {
-    fast2sum(s.r_hi, s.r_lo, mj * wq);
-    fast2sum(s.rt_hi, s.rt_lo, mj * tt);
+    fast2sum_prod(s.r_hi, s.r_lo, mj, wq);
+    fast2sum_prod(s.rt_hi, s.rt_lo, mj, tt);
   }
   s.cnt++;
 }
@@ -177,6 +186,64 @@ __device__ __forceinline__ void dens_list_r(DSum &s, const float *lst, int ls, i
   }
 }
 
+// The next h of a particle's iteration at h = hd with the sums S_w = sn, S_t =
+// stt and sum q^2 w'' = s2; the bracket [lo, hi] takes hd in.
+__device__ __forceinline__ double next_h(double hd, double sn, double stt, double s2, double Cw,
+                                         double &lo, double &hi) {
+  // Halley step in FP64 (Newton where its denominator is not positive),
+  // kept inside the bracket [lo, hi] (F grows with h).  With
+  // g = S_w - C: a = h g' = 3 S_w - S_t, b = h^2 g'' = sum q^2 w'' - 2 a,
+  // dh / h = -2 g a / (2 a^2 - g b)
+  const double Fr = sn - Cw;              // g, the sign of F(h)
+  const double dFr = 3.0 * sn - stt;      // a
+  if (Fr < 0.0) lo = hd;
+  else hi = hd;
+  double hn;
+  if (Fr == 0.0) {
+    hn = hd;
+  } else if (dFr > 0.0) {
+    const double den = 2.0 * dFr * dFr - Fr * (s2 - 2.0 * dFr);
+    // (Halley, or Newton where its denominator is not positive: one division)
+    // (the quotient in FP32: the conversions and the 2-ulp division move
+    // the new h by about 4e-7 of the step, far inside the FP64
+    // convergence test's tolerance)
+    const bool hal = den > 0.0;
+    hn = hd - hd * (double)__fdividef((float)(hal ? 2.0 * Fr * dFr : Fr),
+                                      (float)(hal ? den : dFr));
+  } else {
+    hn = NAN;
+  }
+  if (!(hn >= lo && hn <= hi)) hn = isinf(hi) ? 2.0 * hd : 0.5 * (lo + hi);
+  hn = fmin(fmax(hn, 0.5 * hd), 2.0 * hd);
+  return hn;
+}
+
+// The results of a particle whose iteration ended at h (H = GAMMA_K h, Hinv =
+// 1 / H) with the mass-weighted sums sr, srt.
+__device__ __forceinline__ void write_density(const View &v, int i, const float4 &xl, float h, float H,
+                                              float Hinv, float sr, float srt, long long ti,
+                                              bool init_entropy) {
+  // density, grad-h factor f = [1 + h/(3 rho) drho/dh]^-1, equation of state
+  const float Hinv3 = Hinv * Hinv * Hinv;
+  const float rho = KERNEL_NORM * sr * Hinv3;
+  const float f = 3.0f * sr / (3.0f * sr - srt);
+  const double dtp =
+      ((double)(ti - v.ti_begin[i]) - 0.5 * (double)(v.ti_end[i] - v.ti_begin[i])) *
+      v.dt_min;
+  float Ap = v.A[i] + v.Adot[i] * (float)dtp;
+  const float g = (float)v.gamma;
+  if (init_entropy) Ap = (g - 1.0f) * v.A[i] / powf(rho, g - 1.0f);  // A holds u
+  const float P = Ap * powf(rho, g);
+  const float c = sqrtf(g * P / rho);
+  v.h[i] = h;
+  v.rho[i] = rho;
+  v.f[i] = f;
+  v.P[i] = P;
+  v.c[i] = c;
+  v.rec_xH[i] = make_float4(xl.x, xl.y, xl.z, H);
+  v.rec_h[i] = make_float4(rho, f * P / (rho * rho), c, Hinv);
+}
+
 // Newton step on F(h) = h^3 n(h) - eta^3 in dimensionless form: with H = GAMMA_K h,
 // h^3 n = (8/pi) S_w / GAMMA_K^3 and h dF/dh = 3 h^3 n + h^4 dn/dh, so
 // dh / h = -(S_w - C) / (3 S_w - S_t), C = eta^3 GAMMA_K^3 / (8/pi),
@@ -188,11 +255,11 @@ __device__ __forceinline__ void dens_list_r(DSum &s, const float *lst, int ls, i
 // with r^2 < R_i^2 goes into the particle's neighbour list (squared distance
 // and mass).  Each h iteration evaluates its sums at its H from the list
 // alone, in record order, as long as H <= R_i; a particle whose h outgrows
-// R_i gathers again.  A list holds list_cap entries per particle (list_cap / G
-// per lane): a gather that accepts more runs in passes over the same leaves,
-// each pass listing (and summing) the next list_cap accepted records, and the
-// particle's list is then not kept (later iterations gather at R_i = H).
-// Whatever the capacity, margin or staging depth, a particle's sums visit the
+// R_i gathers again.  A list holds list_cap entries per lane.  A particle whose
+// gather accepts more is left to k_density_big; with several lanes per particle
+// the gather runs in passes over the same leaves, each pass listing (and
+// summing) the next list_cap accepted records, and the particle's list is then
+// not kept (later iterations gather at R_i = H).  Whatever the capacity, margin or staging depth, a particle's sums visit the
 // same pairs in the same order with the same arithmetic.  A work group is
 // handled by one warp (sharing it between the warps of a block, as the force
 // loop does in sparse steps, was measured slower here: every warp pays the
@@ -418,6 +485,13 @@ __device__ void density_group(const View &v, int wg, int slice, int nslices, int
           if (writer) wc.gathers += nlive;
           if (gath) nl = min(acc - skipc, cap);
         }
+        if constexpr (G == 1) {
+          if (gath && acc > cap) {  // (the list filled up: one warp for this particle alone)
+            v.big[atomicAdd(&v.ds->n_big, 1)] = BigItem{lo, hi, h, i, it, wg};
+            wc.list_overflows++;
+            done = true;
+          }
+        }
         // the list this pass built (or, in the first pass, the one kept from
         // an earlier iteration), in order
         if (!done && (gath || first) && nl > 0) {
@@ -425,8 +499,9 @@ __device__ void density_group(const View &v, int wg, int slice, int nslices, int
           else dens_list<false>(s, lst, ls, nl, H2, Hinv);
           if (writer) wc.evals += (unsigned long long)nl;
         }
-        // a list that filled up: the next pass lists the records after it (for
-        // several lanes per particle, every lane of the particle goes on)
+        if constexpr (G == 1) break;
+        // a list that filled up: the next pass lists the records after it
+        // (every lane of the particle goes on)
         const unsigned ob = __ballot_sync(FULL, gath && acc > skipc + cap);
         const bool over = gath && (ob & gmask) != 0u;
         if (over) {
@@ -455,32 +530,8 @@ __device__ void density_group(const View &v, int wg, int slice, int nslices, int
       const double s2 = group_sum<G>((double)s.p2);
       const int cnt = group_sum_i<G>(s.cnt) - 1;  // (the particle itself is among its candidates)
       if (!done) {
-        // Halley step in FP64 (Newton where its denominator is not positive),
-        // kept inside the bracket [lo, hi] (F grows with h).  With
-        // g = S_w - C: a = h g' = 3 S_w - S_t, b = h^2 g'' = sum q^2 w'' - 2 a,
-        // dh / h = -2 g a / (2 a^2 - g b)
         const double hd = (double)h;
-        const double Fr = sn - Cw;              // g, the sign of F(h)
-        const double dFr = 3.0 * sn - stt;      // a
-        if (Fr < 0.0) lo = hd;
-        else hi = hd;
-        double hn;
-        if (Fr == 0.0) {
-          hn = hd;
-        } else if (dFr > 0.0) {
-          const double den = 2.0 * dFr * dFr - Fr * (s2 - 2.0 * dFr);
-          // (Halley, or Newton where its denominator is not positive: one division)
-          // (the quotient in FP32: the conversions and the 2-ulp division move
-          // the new h by about 4e-7 of the step, far inside the FP64
-          // convergence test's tolerance)
-          const bool hal = den > 0.0;
-          hn = hd - hd * (double)__fdividef((float)(hal ? 2.0 * Fr * dFr : Fr),
-                                            (float)(hal ? den : dFr));
-        } else {
-          hn = NAN;
-        }
-        if (!(hn >= lo && hn <= hi)) hn = isinf(hi) ? 2.0 * hd : 0.5 * (lo + hi);
-        hn = fmin(fmax(hn, 0.5 * hd), 2.0 * hd);
+        const double hn = next_h(hd, sn, stt, s2, Cw, lo, hi);
         const bool conv = fabs(hn - hd) <= v.h_tol * hd;
         const bool over = !conv && hn > (double)hcap;
         const bool last = it == v.h_max_iter - 1;
@@ -503,25 +554,7 @@ __device__ void density_group(const View &v, int wg, int slice, int nslices, int
             } else if (!conv) {
               wc.noconv++;
             }
-            // density, grad-h factor f = [1 + h/(3 rho) drho/dh]^-1, equation of state
-            const float Hinv3 = Hinv * Hinv * Hinv;
-            const float rho = KERNEL_NORM * sr * Hinv3;
-            const float f = 3.0f * sr / (3.0f * sr - srt);
-            const double dtp =
-                ((double)(ti - v.ti_begin[i]) - 0.5 * (double)(v.ti_end[i] - v.ti_begin[i])) *
-                v.dt_min;
-            float Ap = v.A[i] + v.Adot[i] * (float)dtp;
-            const float g = (float)v.gamma;
-            if (init_entropy) Ap = (g - 1.0f) * v.A[i] / powf(rho, g - 1.0f);  // A holds u
-            const float P = Ap * powf(rho, g);
-            const float c = sqrtf(g * P / rho);
-            v.h[i] = h;
-            v.rho[i] = rho;
-            v.f[i] = f;
-            v.P[i] = P;
-            v.c[i] = c;
-            v.rec_xH[i] = make_float4(xl.x, xl.y, xl.z, H);
-            v.rec_h[i] = make_float4(rho, f * P / (rho * rho), c, Hinv);
+            write_density(v, i, xl, h, H, Hinv, sr, srt, ti, init_entropy);
             if (v.ngb_density) v.ngb_density[i] = cnt;
           }
         } else {
@@ -534,6 +567,133 @@ __device__ void density_group(const View &v, int wg, int slice, int nslices, int
   __syncwarp();
   if (writer && nslices == 1) leaf_hmax_update(v, W.L0, W.L1);
   __syncwarp();
+}
+
+// A particle whose candidates did not fit its list (list_cap), by one warp:
+// the h iteration goes on from where density_group left it, each iteration
+// one pass over the candidates.  The lanes test and evaluate 32 records at a
+// time, then lane a adds up term a of the accepted ones in record order: the
+// particle's sums are those of dens_pair, term by term.  (Before, density_group
+// ran further passes over the group's records, list_cap of them listed in each,
+// with all 32 lanes waiting: time grows with the square of the candidates.  In
+// 302k clustered particles whose background meets clumps of 4,099, a first
+// density pass took 16.1 ms; 0.95 ms without those particles and 0.78 ms for
+// them here.  2.1M: 4.27 -> 4.18 + 0.13 ms.  Bound by the latency of its longest
+// iterations, one warp each.)
+template <bool UM>
+__device__ void density_big(const View &v, const BigItem &b, int flags, const CellFrame &F, float hcap,
+                            float exc, long long ti, StageD &st, WarpCounters &wc) {
+  const int lane = lane_id();
+  const int i = b.i;
+  const double Cw = v.eta * v.eta * v.eta * GAMMA_K_D * GAMMA_K_D * GAMMA_K_D / (double)KERNEL_NORM;
+  const float4 xl = v.rec_xm[i];
+  const float3 lo3 = leaf_offset(v, i, F);
+  const float4 xi = make_float4(xl.x + lo3.x, xl.y + lo3.y, xl.z + lo3.z, xl.w);
+  const float cx = xi.x + F.kx * F.wq, cy = xi.y + F.ky * F.wq, cz = xi.z + F.kz * F.wq;
+  const float ceps = 1e-5f * F.wf;
+  const float4 *srcs[1] = {v.rec_xm};
+  // per record of a block: w, 3 w + q w', q^2, w, 3 w + q w', w'', m (the search
+  // without spheres leaves their room free)
+  float *const term = reinterpret_cast<float *>(st.sph);
+  double lo = b.lo, hi = b.hi;
+  float h = b.h;
+  for (int it = b.it; it < v.h_max_iter; it++) {
+    const float H = GAMMA_K * h, H2 = H * H, Hinv = 1.0f / H;
+    float s_hi = 0.0f, s_lo = 0.0f, p2 = 0.0f;  // this lane's sum; lane 2: sum q^2 w''
+    int cnt = 0;
+    auto consume = [&](int base, int total) {
+      wc.cand += (unsigned long long)total;
+      for (int k0 = 0; k0 < total; k0 += 32) {
+        const float4 pj = st.rec[base + k0 + lane];  // (buffers hold whole blocks)
+        const float dx = xi.x - pj.x, dy = xi.y - pj.y, dz = xi.z - pj.z;
+        const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+        const bool acc = k0 + lane < total && r2 < H2;
+        const unsigned mask = __ballot_sync(FULL, acc);
+        if (mask == 0u) continue;
+        if (acc) {
+          const float rr = r2 * rsqrtf(fmaxf(r2, 1e-30f));
+          const float qq = rr * Hinv;
+          float wq, dwq;
+          kernel_wd(qq, wq, dwq);
+          const float tt = fmaf(qq, dwq, 3.0f * wq);
+          float4 *t = reinterpret_cast<float4 *>(term + __popc(mask & ((1u << lane) - 1u)) * 8);
+          t[0] = make_float4(wq, tt, qq * qq, wq);
+          t[1] = make_float4(tt, kernel_d2w(qq), pj.w, 0.0f);
+        }
+        const int m = __popc(mask);
+        // (rounds of 4, filled up with zeros, which change no sum)
+        if (lane < ((4 - (m & 3)) & 3) * 8) term[m * 8 + lane] = 0.0f;
+        __syncwarp();
+        cnt += m;
+        for (int k = 0; k < m; k += 4) {
+          float x[4], y[4], w[4];
+#pragma unroll
+          for (int q = 0; q < 4; q++) {
+            x[q] = term[(k + q) * 8 + (lane & 7)];
+            y[q] = term[(k + q) * 8 + 5];
+            if (!UM) w[q] = term[(k + q) * 8 + 6];
+          }
+#pragma unroll
+          for (int q = 0; q < 4; q++) {
+            p2 = fmaf(x[q], y[q], p2);
+            if (UM || lane < 2) fast2sum(s_hi, s_lo, x[q]);
+            else fast2sum_prod(s_hi, s_lo, x[q], w[q]);
+          }
+        }
+        __syncwarp();
+      }
+    };
+    const float R2 = H2 * 1.0002f, Rc = H + ceps;
+    auto leaf_ok = [&](int l, float sx, float sy, float sz, LeafBox &) {
+      return box_gap2(xi.x, xi.y, xi.z, xi.x, xi.y, xi.z, v.leaf_lo[l], v.leaf_hi[l], sx, sy, sz) < R2;
+    };
+    auto chunk_ok = [&](int g, float sx, float sy, float sz) {
+      return box_gap2(cx, cy, cz, cx, cy, cz, v.chunk_lo[g], v.chunk_hi[g], sx, sy, sz) < Rc * Rc;
+    };
+    const Reach reach = {cx, cy, cz, cx, cy, cz, Rc, exc, nullptr, 0};
+    int skip = 0;
+    bool more = false;
+    do {
+      const int nlist = search(v, F, reach, st, leaf_ok, chunk_ok, skip, more);
+      stage_list<false>(srcs, st, nlist, consume, wc);
+      skip += nlist;
+    } while (more && !st.failed);
+    if (st.failed) return;
+    wc.gathers++;
+    if (lane == 0) wc.evals += (unsigned long long)cnt;
+    const double part = (double)s_hi + (double)s_lo;
+    const double sn = __shfl_sync(FULL, part, 0), stt = __shfl_sync(FULL, part, 1);
+    const double s2 = (double)__shfl_sync(FULL, p2, 2);
+    const double hd = (double)h;
+    const double hn = next_h(hd, sn, stt, s2, Cw, lo, hi);
+    const bool conv = fabs(hn - hd) <= v.h_tol * hd;
+    const bool over = !conv && hn > (double)hcap;
+    if (conv || over || it == v.h_max_iter - 1) {
+      float sr, srt;
+      if constexpr (UM) {
+        const double mu = (double)v.ds->m_uniform;
+        sr = (float)(mu * sn);
+        srt = (float)(mu * stt);
+      } else {
+        sr = (float)__shfl_sync(FULL, part, 3);
+        srt = (float)__shfl_sync(FULL, part, 4);
+      }
+      if (lane == 0) {
+        wc.pairs += (unsigned long long)(cnt - 1);  // (the particle itself is among its candidates)
+        wc.iters += (unsigned long long)(it + 1);
+        if (over) {
+          wc.overflow++;
+          atomic_max_float_pos(&v.ds->want_h_bits, (float)hn);
+        } else if (!conv) {
+          wc.noconv++;
+        }
+        write_density(v, i, xl, h, H, Hinv, sr, srt, ti, (flags & SPH_DENSITY_INIT_ENTROPY) != 0);
+        if (v.ngb_density) v.ngb_density[i] = cnt - 1;
+      }
+      break;
+    }
+    h = (float)hn;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1088,6 +1248,34 @@ __global__ void __launch_bounds__(PT, 2) k_density(View v, int flags, int bin_fi
   flush_counters(ds, wc, true);
 }
 
+// The particles the step's density launches left to one warp each, pulled from
+// head_big (none in most steps: the blocks return at once).
+template <bool UM>
+__global__ void __launch_bounds__(PT, 2) k_density_big(View v, int flags) {
+  DevState *ds = v.ds;
+  const int lane = lane_id();
+  const int nb = ds->n_big;
+  // (a support that outgrew its cell halts the step, but its density launch
+  // updates every other particle all the same, and the redone step starts its
+  // iterations from their h)
+  if (nb == 0 || (ds->halt && ds->first_error != SPH_ERR_CELL_OVERFLOW)) return;
+  const float exc = __uint_as_float(ds->excursion_bits);
+  StageD st;
+  stage_init(st, max(v.stage_depth, 2), v.wait_limit);  // (one warp's work is a chain of latencies)
+  const float hcap = (float)((ds->w - 2.0 * (double)exc) / GAMMA_K_D * (1.0 - 1e-6));
+  WarpCounters wc = {0, 0, 0, 0, 0, 0};
+  for (;;) {
+    int item = 0;
+    if (lane == 0) item = atomicAdd(&ds->head_big, 1);
+    item = __shfl_sync(FULL, item, 0);
+    if (item >= nb || st.failed) break;
+    const BigItem b = v.big[item];
+    if (!SPH_IN(ds, b.wg, ds->n_groups, SPH_CHECK_GROUP)) break;
+    density_big<UM>(v, b, flags, frame_of(v, ds, b.wg), hcap, exc, ds->ti, st, wc);
+  }
+  flush_counters(ds, wc, true);
+}
+
 template <int G, bool VAR>
 __global__ void __launch_bounds__(PT, 2) k_force(View v, int bin_filter, int persistent) {
   DevState *ds = v.ds;
@@ -1157,16 +1345,17 @@ __global__ void __launch_bounds__(PT, 2) k_force(View v, int bin_filter, int per
   flush_counters(ds, wc, false);
 }
 
-// The largest support of the leaves of every work group that the last
-// whole-step density launch split (one warp per group; nothing when it split
-// none).
+// The largest support of the leaves of every work group that the whole-step
+// density launch split, or else of those with a particle left to k_density_big
+// (one warp per group).
 __global__ void __launch_bounds__(PT) k_leaf_hmax(View v) {
   DevState *ds = v.ds;
-  if (ds->halt || ds->dens_split <= 1) return;
-  const int nq = ds->n_active_groups + ds->n_heavy_groups;
+  const bool split = ds->dens_split > 1;
+  const int nq = split ? ds->n_active_groups + ds->n_heavy_groups : ds->n_big;
+  if (ds->halt) return;
   const int nw = (int)(gridDim.x * blockDim.x) >> 5;
   for (int k = (int)(blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < nq; k += nw) {
-    const int wg = active_group(v, ds, k);
+    const int wg = split ? active_group(v, ds, k) : v.big[k].wg;
     if (!SPH_IN(ds, wg, ds->n_groups, SPH_CHECK_GROUP)) break;
     const int L0 = v.group_leaf0[wg], L1 = v.group_leaf0[wg + 1];
     // (checks build: a leaf range out of bounds is skipped, as group_of does)
@@ -1290,14 +1479,7 @@ cudaError_t density_g(const View &v, int flags, int bin_filter, bool persistent,
   } else {
     k_density<G, false><<<grid, PT, DENS_SMEM, st>>>(v, flags, bin_filter, persistent ? 1 : 0);
   }
-  cudaError_t e = cudaGetLastError();
-  // after a whole-step launch: the leaves of the groups it split
-  if (e == cudaSuccess && G == 1 && bin_filter < 0 && persistent) {
-    note_launches(1);
-    k_leaf_hmax<<<v.grid_util / 2 > 0 ? v.grid_util / 2 : 1, PT, 0, st>>>(v);
-    e = cudaGetLastError();
-  }
-  return e;
+  return cudaGetLastError();
 }
 
 template <int G>
@@ -1319,8 +1501,14 @@ int blocks_per_sm_g(bool density) {
     return 0;
   }
   if (density && G == 1) {
-    // the equal-mass instance uses the same staging area
+    // the equal-mass instance and k_density_big use the same staging area
     if (cudaFuncSetAttribute((const void *)k_density<1, true>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+            cudaSuccess ||
+        cudaFuncSetAttribute((const void *)k_density_big<true>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+            cudaSuccess ||
+        cudaFuncSetAttribute((const void *)k_density_big<false>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
       cudaGetLastError();
       return 0;
@@ -1363,6 +1551,15 @@ cudaError_t launch_density(const View &v, int flags, int bin_filter, bool persis
     case 32: return density_g<32>(v, flags, bin_filter, persistent, grid, st);
     default: return cudaErrorInvalidValue;
   }
+}
+
+cudaError_t launch_density_rest(const View &v, int flags, int grid, cudaStream_t st) {
+  if (grid <= 0 || v.G != 1) return cudaSuccess;  // (several lanes per particle leave nothing)
+  note_launches(2);
+  if (v.uniform_mass) k_density_big<true><<<grid, PT, DENS_SMEM, st>>>(v, flags);
+  else k_density_big<false><<<grid, PT, DENS_SMEM, st>>>(v, flags);
+  k_leaf_hmax<<<v.grid_util / 2 > 0 ? v.grid_util / 2 : 1, PT, 0, st>>>(v);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_force(const View &v, int bin_filter, bool persistent, int grid,
