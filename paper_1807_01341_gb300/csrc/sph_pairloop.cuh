@@ -365,8 +365,13 @@ __device__ __forceinline__ float3 leaf_offset(const View &v, int i, const CellFr
 // ---------------------------------------------------------------------------
 constexpr int STAGE_DEPTH_MAX = 3;  // staging buffers per warp (copies in flight)
 
-template <int S, int NREC, int LC>
+// (TAGS: room for the staged records' particle and cell; SHARE, the forward
+// force loop's: room for a batch's accept masks, and the search's spheres and
+// chunk list lie in the room of the staged records, so that every search sets
+// its spheres and none runs while records are in use)
+template <int S, int NREC, int LC, bool TAGS = true, bool SHARE = false>
 struct Stage {
+  static constexpr int SLOTS = S;  // staged records
   static constexpr int LCAP = LC;  // accepted neighbour leaves listed per search pass
   static constexpr int CCAP = 128; // accepted chunks gathered per search segment
   float4 *rec;     // NREC arrays of S staged records, back to back (first: positions);
@@ -379,6 +384,7 @@ struct Stage {
   float4 *sph;     // the round's particles: position (group frame), search radius
   float4 *tst;     // the round's live particles: position (group frame), squared test radius
   int2 *chk;       // accepted chunks of a search segment: first leaf, count | cell << 16
+  unsigned *mask;  // (SHARE) accept masks of a batch: word q of lane l at 32 q + l
   uint64_t *bar;   // one mbarrier per staging buffer
   int *meta;       // per staging buffer: first listed leaf, leaves, records
   uint32_t phase;  // parity of the next phase of each buffer's barrier (bit b)
@@ -388,26 +394,31 @@ struct Stage {
   bool stall;      // testing: this staging issues no copy and never arrives
   bool failed;
   static constexpr size_t bytes() {
-    return sizeof(float4) * ((size_t)S * NREC + LC + 64) + sizeof(int2) * CCAP +
-           sizeof(int) * (LC + LEAF_MAX_LIMIT + S) + (size_t)S + 64;
+    return sizeof(float4) * ((size_t)S * NREC + LC + (SHARE ? 32 : 64)) +
+           (SHARE ? 0 : sizeof(int2) * CCAP) + sizeof(int) * (LC + LEAF_MAX_LIMIT) +
+           (TAGS ? (sizeof(int) + 1) * (size_t)S : 0) + (SHARE ? sizeof(unsigned) * S : 0) + 64;
   }
   // sph, tst and chk back to back: free between one round's last consume and
   // the next search, they serve a block's cross-warp reductions (the staged
-  // records and the leaf list stay in place)
-  static constexpr size_t red_offset() { return sizeof(float4) * ((size_t)S * NREC + LC); }
-  static constexpr size_t red_bytes() { return sizeof(float4) * 64 + sizeof(int2) * CCAP; }
+  // records and the leaf list stay in place); with SHARE the records' room does
+  static constexpr size_t red_offset() { return SHARE ? 0 : sizeof(float4) * ((size_t)S * NREC + LC); }
+  static constexpr size_t red_bytes() {
+    return SHARE ? sizeof(float4) * S * NREC : sizeof(float4) * 64 + sizeof(int2) * CCAP;
+  }
   __device__ void carve(char *base) {
     rec = reinterpret_cast<float4 *>(base);
     lshift = rec + (size_t)S * NREC;
-    sph = lshift + LC;
-    tst = sph + 32;
-    chk = reinterpret_cast<int2 *>(tst + 32);
-    lpack = reinterpret_cast<int *>(chk + CCAP);
+    sph = SHARE ? rec : lshift + LC;
+    tst = SHARE ? lshift + LC : sph + 32;
+    chk = reinterpret_cast<int2 *>(SHARE ? sph + 32 : tst + 32);
+    lpack = SHARE ? reinterpret_cast<int *>(tst + 32) : reinterpret_cast<int *>(chk + CCAP);
+    static_assert(!SHARE || S * NREC >= 32 + CCAP / 2, "the search's room fits the records'");
     act = lpack + LC;
     recj = act + LEAF_MAX_LIMIT;
-    recc = reinterpret_cast<uint8_t *>(recj + S);
-    bar = reinterpret_cast<uint64_t *>(recc + S);  // 8-byte aligned: every part above is
+    recc = reinterpret_cast<uint8_t *>(recj + (TAGS ? S : 0));
+    bar = reinterpret_cast<uint64_t *>(recc + (TAGS ? S : 0));  // 8-byte aligned: every part above is
     meta = reinterpret_cast<int *>(bar + STAGE_DEPTH_MAX);
+    mask = reinterpret_cast<unsigned *>(bar + 8);
   }
 };
 
@@ -633,14 +644,17 @@ __device__ __forceinline__ int search(const View &v, const CellFrame &F, const R
 // A barrier wait that gives up sets st.failed and counts a timeout; the warp
 // then waits (bounded again) for every copy it still has in flight before it
 // returns, so that no copy lands in shared memory the warp has left.
-template <bool TAG = true, int S, int NREC, int LC, class Consume>
-__device__ __forceinline__ void stage_list(const float4 *const *srcs, Stage<S, NREC, LC> &st,
-                                           int nlist, Consume consume, WarpCounters &wc) {
+template <bool TAG = true, int S, int NREC, int LC, bool TAGS, bool SHARE, class Consume>
+__device__ __forceinline__ void stage_list(const float4 *const *srcs,
+                                           Stage<S, NREC, LC, TAGS, SHARE> &st, int nlist,
+                                           Consume consume, WarpCounters &wc) {
+  static_assert(!TAG || TAGS, "no room for tags");
   const int lane = lane_id();
   const int depth = st.depth;
   // (a multiple of 32 records per buffer: the tests read whole blocks of 32)
   const int Sb = (S / depth) & ~31;
   int e_next = 0, issued = 0, done = 0;
+  if constexpr (SHARE) fence_proxy_async();  // the search's accesses before the first bulk writes
   // the next listed leaves that fit Sb records, into buffer b
   auto issue = [&](int b) {
     const int e = e_next;
@@ -738,6 +752,12 @@ __device__ __forceinline__ void stage_list(const float4 *const *srcs, Stage<S, N
 
 using StageD = Stage<S_DENS, 1, 320>;
 using StageF = Stage<S_FORCE, 3, 256>;
+// the forward force loop (S_PAIR staged candidates per warp): two blocks of 8
+// warps fill an SM's shared memory (14,464 bytes a warp); the variants' tags
+// cost room for 48 leaves
+constexpr int S_PAIR = 192;
+template <bool VAR>
+using StageP = Stage<S_PAIR, 3, VAR ? 128 : 176, VAR, true>;
 
 // depth: staging buffers (1..STAGE_DEPTH_MAX, and S / depth >= 32);
 // wait_limit: polls of each bounded barrier wait (<= 0: WAIT_LIMIT);

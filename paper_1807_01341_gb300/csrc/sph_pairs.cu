@@ -102,6 +102,14 @@ __device__ __forceinline__ void fast2sum_prod(float &hi, float &lo, float x, flo
   hi = t;
 }
 
+// two of them at once, packed
+__device__ __forceinline__ void fast2sum_prod2(float2 &hi, float2 &lo, float2 x, float2 y) {
+  const float2 t = __ffma2_rn(x, y, hi);
+  const float2 e = __fadd2_rn(t, make_float2(-hi.x, -hi.y));
+  lo = __fadd2_rn(lo, __ffma2_rn(x, y, make_float2(-e.x, -e.y)));
+  hi = t;
+}
+
 struct DSum {
   float n_hi, n_lo, t_hi, t_lo, r_hi, r_lo, rt_hi, rt_lo;
   float p2;
@@ -709,7 +717,7 @@ __device__ __forceinline__ void request_wake(const View &v, int j, int b) {
 // is compiled in; the base scheme runs the instance without it.
 template <int G, bool COOP, bool VAR>
 __device__ void force_group(const View &v, int wg, int slice, int nslices, int bin_filter, int m_act,
-                            const CellFrame &F, float Hmax, float exc, StageF &st,
+                            const CellFrame &F, float Hmax, float exc, StageP<VAR> &st,
                             WarpCounters &wc) {
   static_assert(!COOP || G == 1, "cooperative groups use one lane per particle");
   const int lane = lane_id();
@@ -737,7 +745,7 @@ __device__ void force_group(const View &v, int wg, int slice, int nslices, int b
   const float alpha = (float)v.alpha;
   const float g = (float)v.gamma;
   const float4 *srcs[3] = {v.rec_xH, v.rec_v, v.rec_h};
-  const float4 *sx_rec = st.rec, *sv_rec = st.rec + S_FORCE, *sh_rec = st.rec + 2 * S_FORCE;
+  const float4 *sx_rec = st.rec, *sv_rec = st.rec + S_PAIR, *sh_rec = st.rec + 2 * S_PAIR;
 
   for (int r = s0; r < s1 && !st.failed; r += P) {
     const int slot = r + grp;
@@ -753,8 +761,8 @@ __device__ void force_group(const View &v, int wg, int slice, int nslices, int b
     const float nHi4 = KERNEL_NORM * Hinv2 * Hinv2;
     const float Hs = warp_max(valid ? xi.w : 0.0f);
     const int nsph = compact_spheres(st.sph, sub == 0 && valid, make_float4(xi.x, xi.y, xi.z, xi.w));
-    float ax_hi = 0.f, ax_lo = 0.f, ay_hi = 0.f, ay_lo = 0.f, az_hi = 0.f, az_lo = 0.f;
-    float ad_hi = 0.f, ad_lo = 0.f;
+    // compensated sums of (a_x, a_y) and (a_z, dA/dt)
+    float2 xy_hi = {0.f, 0.f}, xy_lo = {0.f, 0.f}, zd_hi = {0.f, 0.f}, zd_lo = {0.f, 0.f};
     float vs = 2.0f * hi4.z;
     int cnt = 0;
     int bmin = 127;  // limiter: smallest bin among the neighbours
@@ -796,7 +804,7 @@ __device__ void force_group(const View &v, int wg, int slice, int nslices, int b
       // per-lane form for every count of live particles)
       if (G == 1) {
         const bool in = kb + lane < total;
-        const float4 pj = sx_rec[min(base + kb + lane, S_FORCE - 1)];
+        const float4 pj = sx_rec[min(base + kb + lane, S_PAIR - 1)];
         const float Hj2 = pj.w * pj.w;
         const float2 px = make_float2(pj.x, pj.x), py = make_float2(pj.y, pj.y),
                      pz = make_float2(pj.z, pj.z);
@@ -820,7 +828,7 @@ __device__ void force_group(const View &v, int wg, int slice, int nslices, int b
       } else {
 #pragma unroll
         for (int u = sub; u < 32; u += G) {
-          const float4 pj = sx_rec[min(base + kb + u, S_FORCE - 1)];
+          const float4 pj = sx_rec[min(base + kb + u, S_PAIR - 1)];
           const float dx = xi.x - pj.x, dy = xi.y - pj.y, dz = xi.z - pj.z;
           const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
           mask |= (kb + u < total && (r2 < Hi2 || r2 < pj.w * pj.w)) ? (1u << u) : 0u;
@@ -830,68 +838,83 @@ __device__ void force_group(const View &v, int wg, int slice, int nslices, int b
     };
     auto consume = [&](int base, int total) {
       wc.cand += (unsigned long long)total * nlive;
-      // two blocks of 32 records per evaluation round: the lanes' accepted
-      // counts even out over 64 records (records still in index order; the
-      // density loop, at its register limit, keeps rounds of 32)
-      for (int k0 = 0; k0 < total; k0 += 64) {
-        // (every lane calls the test, which votes; the second call's
-        // condition is the same in all lanes)
-        const unsigned m0 = test_block(base, total, k0);
-        const unsigned m1 = k0 + 32 < total ? test_block(base, total, k0 + 32) : 0u;
-        unsigned long long mask = valid ? ((unsigned long long)m1 << 32) | m0 : 0ull;
-        while (mask) {
-          // (the particle itself is accepted too: r = 0, it adds nothing but
-          // the signal velocity 2 c_i, the start value; one count subtracted below)
-          const int k = base + k0 + __ffsll(mask) - 1;
-          mask &= mask - 1;
-          const float4 pj = sx_rec[k];
-          const float4 vj = sv_rec[k];
-          const float4 hj = sh_rec[k];
-          const float dx = xi.x - pj.x, dy = xi.y - pj.y, dz = xi.z - pj.z;
-          const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-          cnt++;
-          if ((VAR && v.limiter)) {
+      // The whole batch's accept masks, then each lane through its particle's
+      // pairs in record order.  The batch lies on one side of the group, so
+      // some particles accept many of its records and others few, and the
+      // longest lane sets the time: the more records the lanes go through
+      // before they wait for one another, the more their counts even out.
+      // 16.8M particles, all active: 21.0 ms with rounds of 64 records, 19.5
+      // with 128, 18.4 with 192, all that fits beside the leaf list (the start,
+      // 64 and without the packed sums: 21.5); 2.1M clustered 4.21 -> 3.76 ms;
+      // with the variants 390 -> 270 us at 111k.  The pairs spread over all
+      // lanes, each owner adding its own up afterwards: 22.3 ms at 16.8M.
+      int left = 0;
+      const int wend = (total + 31) >> 5;
+#pragma unroll 1
+      for (int q = 0; q < wend; q++) {
+        unsigned m = test_block(base, total, 32 * q);
+        if (!valid) m = 0u;
+        st.mask[q * 32 + lane] = m;
+        left += __popc(m);
+      }
+      // (the particle itself is accepted too: r = 0, it adds nothing but the
+      // signal velocity 2 c_i, the start value; one count subtracted below)
+      cnt += left;
+      int kb = base - 1, q = 0;
+      unsigned cur = st.mask[lane];
+      for (; left > 0; left--) {
+        while (cur == 0u) {
+          q++;
+          kb += 32;
+          cur = st.mask[q * 32 + lane];
+        }
+        const int k = kb + __ffs(cur);
+        cur &= cur - 1;
+        const float4 pj = sx_rec[k];
+        const float4 vj = sv_rec[k];
+        const float4 hj = sh_rec[k];
+        const float dx = xi.x - pj.x, dy = xi.y - pj.y, dz = xi.z - pj.z;
+        const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+        if ((VAR && v.limiter)) {
+          const int j = st.recj[k];
+          if (j != i) {
+            const int bj = v.bin[j];
+            bmin = min(bmin, bj);
+            // waking: an inactive neighbour on a step more than 4x longer
+            if (bj > m_act && bj > bi + 2) request_wake(v, j, bi + 2);
+          }
+        }
+        if (r2 > 0.0f) {
+          const float rinv = rsqrtf(r2);
+          const float rr = r2 * rinv;
+          const float qi = rr * hi4.w, qj = rr * hj.w;
+          const float dwi = qi < 1.0f ? kernel_dw(qi) * nHi4 : 0.0f;
+          const float hj2 = hj.w * hj.w;
+          const float dwj = qj < 1.0f ? kernel_dw(qj) * (KERNEL_NORM * hj2 * hj2) : 0.0f;
+          const float dvdr = fmaf(vi.x - vj.x, dx, fmaf(vi.y - vj.y, dy, (vi.z - vj.z) * dz));
+          // Monaghan signal-velocity viscosity, beta = 3 (as in Eq. 1)
+          const float wij = fminf(0.0f, dvdr * rinv);
+          const float vsij = hi4.z + hj.z - 3.0f * wij;
+          // (fast division: 2 ulp, the pair term's only divide)
+          float Pi = __fdividef(-alpha * vsij * wij, hi4.x + hj.x);
+          if ((VAR && v.balsara)) {
+            // mean of the pair's Balsara factors (j's from its last density)
             const int j = st.recj[k];
-            if (j != i) {
-              const int bj = v.bin[j];
-              bmin = min(bmin, bj);
-              // waking: an inactive neighbour on a step more than 4x longer
-              if (bj > m_act && bj > bi + 2) request_wake(v, j, bi + 2);
-            }
+            const float dv = fabsf(v.div_v[j]);
+            const float Bj = dv / (dv + fabsf(v.curl_v[j]) + 1e-4f * hj.z * GAMMA_K * hj.w);
+            Pi *= 0.5f * (Bi + Bj);
           }
-          if (r2 > 0.0f) {
-            const float rinv = rsqrtf(r2);
-            const float rr = r2 * rinv;
-            const float qi = rr * hi4.w, qj = rr * hj.w;
-            const float dwi = qi < 1.0f ? kernel_dw(qi) * nHi4 : 0.0f;
-            const float hj2 = hj.w * hj.w;
-            const float dwj = qj < 1.0f ? kernel_dw(qj) * (KERNEL_NORM * hj2 * hj2) : 0.0f;
-            const float dvdr = fmaf(vi.x - vj.x, dx, fmaf(vi.y - vj.y, dy, (vi.z - vj.z) * dz));
-            // Monaghan signal-velocity viscosity, beta = 3 (as in Eq. 1)
-            const float wij = fminf(0.0f, dvdr * rinv);
-            const float vsij = hi4.z + hj.z - 3.0f * wij;
-            // (fast division: 2 ulp, the pair term's only divide)
-            float Pi = __fdividef(-alpha * vsij * wij, hi4.x + hj.x);
-            if ((VAR && v.balsara)) {
-              // mean of the pair's Balsara factors (j's from its last density)
-              const int j = st.recj[k];
-              const float dv = fabsf(v.div_v[j]);
-              const float Bj = dv / (dv + fabsf(v.curl_v[j]) + 1e-4f * hj.z * GAMMA_K * hj.w);
-              Pi *= 0.5f * (Bi + Bj);
-            }
-            const float dWb = 0.5f * (dwi + dwj);
-            const float sc = vj.w * fmaf(hi4.y, dwi, fmaf(hj.y, dwj, Pi * dWb)) * rinv;
-            // (the terms of a cancel in part, so a term can exceed the running
-            // sum; that addition then keeps an error of about one unit in the
-            // last place of the sum, as a plain FP32 partial sum would)
-            fast2sum(ax_hi, ax_lo, -sc * dx);
-            fast2sum(ay_hi, ay_lo, -sc * dy);
-            fast2sum(az_hi, az_lo, -sc * dz);
-            fast2sum(ad_hi, ad_lo, vj.w * Pi * dWb * (dvdr * rinv));
-            vs = fmaxf(vs, vsij);
-          } else {
-            vs = fmaxf(vs, hi4.z + hj.z);
-          }
+          const float dWb = 0.5f * (dwi + dwj);
+          const float sc = vj.w * fmaf(hi4.y, dwi, fmaf(hj.y, dwj, Pi * dWb)) * rinv;
+          // (the terms of a cancel in part, so a term can exceed the running
+          // sum; that addition then keeps an error of about one unit in the
+          // last place of the sum, as a plain FP32 partial sum would)
+          fast2sum_prod2(xy_hi, xy_lo, make_float2(-sc, -sc), make_float2(dx, dy));
+          fast2sum_prod2(zd_hi, zd_lo, make_float2(-sc, vj.w * Pi * dWb),
+                         make_float2(dz, dvdr * rinv));
+          vs = fmaxf(vs, vsij);
+        } else {
+          vs = fmaxf(vs, hi4.z + hj.z);
         }
       }
     };
@@ -902,6 +925,8 @@ __device__ void force_group(const View &v, int wg, int slice, int nslices, int b
     int skip = 0, nlist = 0;
     bool more = false;
     do {
+      // (the staging took the spheres' room)
+      if (more) compact_spheres(st.sph, sub == 0 && valid, make_float4(xi.x, xi.y, xi.z, xi.w));
       nlist = search(v, F, reach, st, leaf_ok, chunk_ok, skip, more, part);
       stage_list<VAR>(srcs, st, nlist, consume, wc);  // (particle tags for the variants only)
       skip += nlist;
@@ -910,11 +935,11 @@ __device__ void force_group(const View &v, int wg, int slice, int nslices, int b
     double sax, say, saz, sad;
     if constexpr (COOP) {
       // combine the 8 warps' partial sums, in warp order
-      float *mine = red_area<StageF>(warp);
-      mine[0 * 32 + lane] = ax_hi; mine[1 * 32 + lane] = ax_lo;
-      mine[2 * 32 + lane] = ay_hi; mine[3 * 32 + lane] = ay_lo;
-      mine[4 * 32 + lane] = az_hi; mine[5 * 32 + lane] = az_lo;
-      mine[6 * 32 + lane] = ad_hi; mine[7 * 32 + lane] = ad_lo;
+      float *mine = red_area<StageP<VAR>>(warp);
+      mine[0 * 32 + lane] = xy_hi.x; mine[1 * 32 + lane] = xy_lo.x;
+      mine[2 * 32 + lane] = xy_hi.y; mine[3 * 32 + lane] = xy_lo.y;
+      mine[4 * 32 + lane] = zd_hi.x; mine[5 * 32 + lane] = zd_lo.x;
+      mine[6 * 32 + lane] = zd_hi.y; mine[7 * 32 + lane] = zd_lo.y;
       mine[8 * 32 + lane] = vs;
       reinterpret_cast<int *>(mine)[9 * 32 + lane] = cnt;
       reinterpret_cast<int *>(mine)[10 * 32 + lane] = st.failed ? 1 : 0;
@@ -924,7 +949,7 @@ __device__ void force_group(const View &v, int wg, int slice, int nslices, int b
       float vm = 0.0f;
       int c = 0, fl = 0, bm = 127;
       for (int w = 0; w < WARPS_PER_BLOCK; w++) {
-        const float *rw = red_area<StageF>(w);
+        const float *rw = red_area<StageP<VAR>>(w);
         a0 += (double)rw[0 * 32 + lane] + (double)rw[1 * 32 + lane];
         a1 += (double)rw[2 * 32 + lane] + (double)rw[3 * 32 + lane];
         a2 += (double)rw[4 * 32 + lane] + (double)rw[5 * 32 + lane];
@@ -947,10 +972,10 @@ __device__ void force_group(const View &v, int wg, int slice, int nslices, int b
       cnt = c - 1;
       bmin = bm;
     } else {
-      sax = group_sum<G>((double)ax_hi + (double)ax_lo);
-      say = group_sum<G>((double)ay_hi + (double)ay_lo);
-      saz = group_sum<G>((double)az_hi + (double)az_lo);
-      sad = group_sum<G>((double)ad_hi + (double)ad_lo);
+      sax = group_sum<G>((double)xy_hi.x + (double)xy_lo.x);
+      say = group_sum<G>((double)xy_hi.y + (double)xy_lo.y);
+      saz = group_sum<G>((double)zd_hi.x + (double)zd_lo.x);
+      sad = group_sum<G>((double)zd_hi.y + (double)zd_lo.y);
       cnt = group_sum_i<G>(cnt) - 1;
       vs = group_max<G>(vs);
       if ((VAR && v.limiter)) {
@@ -1290,7 +1315,7 @@ __global__ void __launch_bounds__(PT, 2) k_force(View v, int bin_filter, int per
   }
   __syncthreads();
   if (!s_go) return;
-  StageF st;
+  StageP<VAR> st;
   stage_init(st, v.stage_depth, v.wait_limit);
   const int m_act = ds->m_act;
   const float Hmax = s_Hmax;
@@ -1467,6 +1492,9 @@ __global__ void k_entropy_from_u(View v) {
 
 constexpr size_t DENS_SMEM = StageD::bytes() * WARPS_PER_BLOCK;
 constexpr size_t FORCE_SMEM = StageF::bytes() * WARPS_PER_BLOCK;
+constexpr size_t PAIR_WARP =
+    StageP<true>::bytes() > StageP<false>::bytes() ? StageP<true>::bytes() : StageP<false>::bytes();
+constexpr size_t PAIR_SMEM = PAIR_WARP * WARPS_PER_BLOCK;
 
 template <int G>
 cudaError_t density_g(const View &v, int flags, int bin_filter, bool persistent, int grid,
@@ -1485,16 +1513,16 @@ cudaError_t density_g(const View &v, int flags, int bin_filter, bool persistent,
 template <int G>
 cudaError_t force_g(const View &v, int bin_filter, bool persistent, int grid, cudaStream_t st) {
   if (G == 1 && (v.balsara || v.limiter))
-    k_force<1, true><<<grid, PT, FORCE_SMEM, st>>>(v, bin_filter, persistent ? 1 : 0);
+    k_force<1, true><<<grid, PT, PAIR_SMEM, st>>>(v, bin_filter, persistent ? 1 : 0);
   else
-    k_force<G, false><<<grid, PT, FORCE_SMEM, st>>>(v, bin_filter, persistent ? 1 : 0);
+    k_force<G, false><<<grid, PT, PAIR_SMEM, st>>>(v, bin_filter, persistent ? 1 : 0);
   return cudaGetLastError();
 }
 
 template <int G>
 int blocks_per_sm_g(bool density) {
   const void *fn = density ? (const void *)k_density<G, false> : (const void *)k_force<G, false>;
-  const size_t smem = density ? DENS_SMEM : FORCE_SMEM;
+  const size_t smem = density ? DENS_SMEM : PAIR_SMEM;
   if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
       cudaSuccess) {
     cudaGetLastError();
@@ -1521,7 +1549,7 @@ int blocks_per_sm_g(bool density) {
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
             cudaSuccess ||
         cudaFuncSetAttribute((const void *)k_gradient, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem) != cudaSuccess) {
+                             (int)FORCE_SMEM) != cudaSuccess) {
       cudaGetLastError();
       return 0;
     }
