@@ -748,6 +748,49 @@ __device__ __forceinline__ double widen(float f) {
   return __hiloint2double((int)hi, (int)(b << 29));
 }
 
+// The kernel of one particle (c = m (8/pi) / H^3, hi = 1 / H) at a grid point:
+// offsets in units of H, q2 their square sum, f about the same in FP32.
+// Forward: adds m W to the point.  BWD: adds to acc the point's d loss / d x,
+// y, z and, unscaled, d h.
+template <bool BWD>
+struct GridKernel {
+  double c, T, c_in, c_out;  // dW/dr = T w'(q); scales of the two pieces
+  __device__ GridKernel(double c_, double hi)
+      : c(c_), T(c_ * hi), c_in(BWD ? T : -6.0 * c_), c_out(BWD ? -6.0 * T : 2.0 * c_) {}
+  __device__ __forceinline__ void point(double dx, double dy, double dz, double q2, float f,
+                                        long long gidx, double *rho_g, const double *rho_bar,
+                                        double (&acc)[4]) const {
+    const double y0 = f > 1e-30f ? widen(rsqrtf(f)) : 0.0;
+    const double t = q2 * y0;
+    const double e = fma(-t, y0, 1.0);
+    const double pe = fma(0.375, e, 0.5) * e;
+    const double q = fma(t, pe, t);
+    const double u = 1.0 - q;
+    const bool inner = __double2hiint(q) < 0x3fe00000;  // q < 1/2
+    const bool in = __double2hiint(u) >= 0;             // q <= 1
+    const double sq = inner ? q : u;
+    const double s2 = sq * sq;
+    if (!BWD) {
+      // 1 - 6 q^2 (1 - q), 2 (1 - q)^3
+      const double w = fma(s2 * u, inner ? c_in : c_out, inner ? c : 0.0);
+      if (in) atomicAdd(&rho_g[gidx], w);
+    } else {
+      const double gb = in ? rho_bar[gidx] : 0.0;
+      // w' / q: -12 + 18 q, -6 (1 - q)^2 / q
+      const double yq = fma(y0, pe, y0);
+      const double v = inner ? fma(18.0, q, -12.0) : s2 * yq;
+      const double g = (gb * (inner ? c_in : c_out)) * v;
+      acc[0] = fma(g, dx, acc[0]);
+      acc[1] = fma(g, dy, acc[1]);
+      acc[2] = fma(g, dz, acc[2]);
+      // 3 w + q w': 3 + q^2 (36 q - 30), (1 - q)^2 (6 - 12 q)
+      const double wh =
+          fma(s2, fma(inner ? 36.0 : -12.0, q, inner ? -30.0 : 6.0), inner ? 3.0 : 0.0);
+      acc[3] = fma(gb, wh, acc[3]);
+    }
+  }
+};
+
 // Adds m W(|x_g - x|, h) of every particle to the grid points within its
 // support (FP64 atomics); with BWD, reads d loss / d rho_g instead and
 // accumulates d loss / d x, d h (and d v through the drift to the tick).
@@ -766,10 +809,17 @@ __device__ __forceinline__ double widen(float f) {
 // selected coefficients, its scale folded into them.  One thread per particle
 // computed the offsets of each point anew, with FP64 square roots and
 // divisions, 45 and more FP64 instructions per point of the whole box.
-// 110,592 particles on a 64^3 grid (113 points in a support): 1885 -> 422 us,
-// backward 3385 -> 703 us; 32,768 on 32^3 301 -> 113 us and 394 -> 161 us; the
+// 110,592 particles on a 64^3 grid (113 points in a support): 1885 -> 463 us,
+// backward 3385 -> 787 us; 262,144 on 32^3 209 -> 182 us and 314 -> 220 us;
+// 2,744 on 128^3 (supports of 40,000 points) 153 -> 2.5 ms and 182 -> 4.3 ms; the
 // error against 64-bit sums in another order is 4e-16 to 6e-16 either way.
-constexpr int GD_WARPS = 4, GD_SIDE = 32;
+// Where at least GD_LANES of a warp's particles have boxes of at most GD_FEW
+// points, those are one lane's work each, all at once: a warp per particle costs
+// some 20 FP64 instructions before its first point (27,000 particles on a 16^3
+// grid: 114 us, at start 75 us; here 74 us).  With 2 or 3 such particles in a
+// warp, clumps on a fine grid, the lanes' own way costs more (111k on 64^3: 737
+// against 462 us).
+constexpr int GD_WARPS = 4, GD_SIDE = 32, GD_FEW = 27, GD_LANES = 16;
 struct GridWarp {
   double d[3][GD_SIDE];   // (x - x_g) / H along each axis
   double d2x[GD_SIDE];    // its square, first axis
@@ -779,7 +829,7 @@ struct GridWarp {
 };
 
 template <bool BWD>
-__global__ void __launch_bounds__(GD_WARPS * 32)
+__global__ void __launch_bounds__(GD_WARPS * 32, 6)
     k_grid_density(sph_particles p, int ng, long long ti, double dt_min, double box,
                    double *rho_g, const double *rho_bar, sph_adjoint adj, int per_warp) {
   __shared__ GridWarp s_w[GD_WARPS];
@@ -807,8 +857,33 @@ __global__ void __launch_bounds__(GD_WARPS * 32)
 #pragma unroll
       for (int k = 0; k < 3; k++) grid_range(X[k], H, s, ng, a0[k], na[k]);
     }
-    double o_x = 0.0, o_y = 0.0, o_z = 0.0, o_h = 0.0;  // BWD: this lane's particle
-    for (int k = 0; k < cnt; k++) {
+    double o[4] = {0.0, 0.0, 0.0, 0.0};  // BWD: this lane's particle
+    // boxes of a few points: one lane per particle, all at once
+    bool few = na[0] > 0 && na[1] > 0 && na[2] > 0 && na[0] <= GD_FEW && na[1] <= GD_FEW &&
+               na[2] <= GD_FEW && na[0] * na[1] * na[2] <= GD_FEW;
+    if (__popc(__ballot_sync(FULL, few)) < GD_LANES) few = false;
+    if (few) {
+      const GridKernel<BWD> K(C, Hinv);
+      for (int c = 0; c < na[2]; c++) {
+        const int iz = ((a0[2] + c) % ng + ng) % ng;
+        const double dz = min_img(X[2] - (iz + 0.5) * s, box) * Hinv;
+        for (int b = 0; b < na[1]; b++) {
+          const int iy = ((a0[1] + b) % ng + ng) % ng;
+          const double dy = min_img(X[1] - (iy + 0.5) * s, box) * Hinv;
+          for (int a = 0; a < na[0]; a++) {
+            const int ix = ((a0[0] + a) % ng + ng) % ng;
+            const double dx = min_img(X[0] - (ix + 0.5) * s, box) * Hinv;
+            const double q2 = fma(dz, dz, fma(dy, dy, dx * dx));
+            if (q2 < 1.0)
+              K.point(dx, dy, dz, q2, (float)q2, ix + (long long)ng * (iy + (long long)ng * iz), rho_g,
+                      rho_bar, o);
+          }
+        }
+      }
+    }
+    for (unsigned todo = __ballot_sync(FULL, !few && na[0] > 0 && na[1] > 0 && na[2] > 0); todo;
+         todo &= todo - 1u) {
+      const int k = __ffs(todo) - 1;
       const double hi = shfl_d(Hinv, k), c = shfl_d(C, k);
       const double xk[3] = {shfl_d(X[0], k), shfl_d(X[1], k), shfl_d(X[2], k)};
       int ak[3], nk[3];
@@ -817,45 +892,14 @@ __global__ void __launch_bounds__(GD_WARPS * 32)
         ak[q] = __shfl_sync(FULL, a0[q], k);
         nk[q] = __shfl_sync(FULL, na[q], k);
       }
-      if (nk[0] <= 0 || nk[1] <= 0 || nk[2] <= 0) continue;
-      // the kernel (or its derivatives) over the two pieces, scaled
-      const double T = c * hi;  // dW/dr = T w'(q)
-      const double c_in = BWD ? T : -6.0 * c, c_out = BWD ? -6.0 * T : 2.0 * c;
-      double gx = 0.0, gy = 0.0, gz = 0.0, gh = 0.0;
+      const GridKernel<BWD> K(c, hi);
+      double acc[4] = {0.0, 0.0, 0.0, 0.0};
       auto point = [&](unsigned int id) {
         const int ix = id & 31, iy = (id >> 5) & 31, iz = id >> 10;
-        const double dy = S.d[1][iy], dz = S.d[2][iz];
-        const double q2 = fma(dz, dz, fma(dy, dy, S.d2x[ix]));
-        const float f = S.f2[0][ix] + S.f2[1][iy] + S.f2[2][iz];
-        const double y0 = f > 1e-30f ? widen(rsqrtf(f)) : 0.0;
-        const double t = q2 * y0;
-        const double e = fma(-t, y0, 1.0);
-        const double pe = fma(0.375, e, 0.5) * e;
-        const double q = fma(t, pe, t);
-        const double u = 1.0 - q;
-        const bool inner = __double2hiint(q) < 0x3fe00000;  // q < 1/2
-        const bool in = __double2hiint(u) >= 0;             // q <= 1
-        const double sq = inner ? q : u;
-        const double s2 = sq * sq;
+        const double dx = BWD ? S.d[0][ix] : 0.0, dy = S.d[1][iy], dz = S.d[2][iz];
         const long long gidx = S.ix[0][ix] + (long long)ng * (S.ix[1][iy] + (long long)ng * S.ix[2][iz]);
-        if (!BWD) {
-          // 1 - 6 q^2 (1 - q), 2 (1 - q)^3
-          const double w = fma(s2 * u, inner ? c_in : c_out, inner ? c : 0.0);
-          if (in) atomicAdd(&rho_g[gidx], w);
-        } else {
-          const double gb = in ? rho_bar[gidx] : 0.0;
-          // w' / q: -12 + 18 q, -6 (1 - q)^2 / q
-          const double yq = fma(y0, pe, y0);
-          const double v = inner ? fma(18.0, q, -12.0) : s2 * yq;
-          const double g = (gb * (inner ? c_in : c_out)) * v;
-          gx = fma(g, S.d[0][ix], gx);
-          gy = fma(g, dy, gy);
-          gz = fma(g, dz, gz);
-          // 3 w + q w': 3 + q^2 (36 q - 30), (1 - q)^2 (6 - 12 q)
-          const double wh = fma(s2, fma(inner ? 36.0 : -12.0, q, inner ? -30.0 : 6.0),
-                                inner ? 3.0 : 0.0);
-          gh = fma(gb, wh, gh);
-        }
+        K.point(dx, dy, dz, fma(dz, dz, fma(dy, dy, S.d2x[ix])),
+                S.f2[0][ix] + S.f2[1][iy] + S.f2[2][iz], gidx, rho_g, rho_bar, acc);
       };
       for (int z0 = 0; z0 < nk[2]; z0 += GD_SIDE)
         for (int y0 = 0; y0 < nk[1]; y0 += GD_SIDE)
@@ -912,31 +956,31 @@ __global__ void __launch_bounds__(GD_WARPS * 32)
         // the four sums over the warp, half the values dropped at each of the
         // first two exchanges (6 additions instead of 20)
         const bool up = lane & 16, up2 = lane & 8;
-        double v0 = up ? gz : gx, v1 = up ? gh : gy;
-        v0 += __shfl_xor_sync(FULL, up ? gx : gz, 16);
-        v1 += __shfl_xor_sync(FULL, up ? gy : gh, 16);
+        double v0 = up ? acc[2] : acc[0], v1 = up ? acc[3] : acc[1];
+        v0 += __shfl_xor_sync(FULL, up ? acc[0] : acc[2], 16);
+        v1 += __shfl_xor_sync(FULL, up ? acc[1] : acc[3], 16);
         double r = up2 ? v1 : v0;
         r += __shfl_xor_sync(FULL, up2 ? v0 : v1, 8);
 #pragma unroll
         for (int o = 4; o; o >>= 1) r += __shfl_xor_sync(FULL, r, o);
         const double r0 = shfl_d(r, 0), r1 = shfl_d(r, 8), r2 = shfl_d(r, 16), r3 = shfl_d(r, 24);
         if (lane == k) {
-          o_x = r0;
-          o_y = r1;
-          o_z = r2;
-          // dW/dh = -GAMMA_K (8/pi) H^-4 (3 w + q w')
-          o_h = -GAMMA_K_D * T * r3;
+          o[0] = r0;
+          o[1] = r1;
+          o[2] = r2;
+          o[3] = r3;
         }
       }
     }
     if (BWD && lane < cnt) {
-      adj.x[j] += o_x;
-      adj.y[j] += o_y;
-      adj.z[j] += o_z;
-      adj.vx[j] += o_x * dtd;
-      adj.vy[j] += o_y * dtd;
-      adj.vz[j] += o_z * dtd;
-      adj.h[j] += o_h;
+      adj.x[j] += o[0];
+      adj.y[j] += o[1];
+      adj.z[j] += o[2];
+      adj.vx[j] += o[0] * dtd;
+      adj.vy[j] += o[1] * dtd;
+      adj.vz[j] += o[2] * dtd;
+      // dW/dh = -GAMMA_K (8/pi) H^-4 (3 w + q w')
+      adj.h[j] += -GAMMA_K_D * (C * Hinv) * o[3];
     }
   }
 }
@@ -1038,9 +1082,13 @@ cudaError_t launch_grid_density(const sph_particles &p, int n_grid, long long ti
   note_launches(1);
   // particles per warp: up to 32 share a set-up, fewer where there would be
   // less than 16 warps per SM (110,592 particles, where this gives 32 and 23
-  // warps per SM: 422 us; 22 particles per warp, 33 warps per SM: 477 us)
+  // warps per SM: 422 us; 22 particles per warp, 33 warps per SM: 477 us, both
+  // before the lanes' own way)
   const long long slots = 16ll * num_sms;
-  const int per_warp = (int)std::max<long long>(1, std::min<long long>(32, p.n / slots));
+  int per_warp = (int)std::max<long long>(1, std::min<long long>(32, p.n / slots));
+  // (few points per particle, 48 n_grid^3 / n on average: the lanes work on a
+  // particle each, and every lane should have one)
+  if (48.0 * n_grid * n_grid * n_grid <= 12.0 * (double)p.n) per_warp = 32;
   const long long warps = (p.n + per_warp - 1) / per_warp;
   const int grid = (int)std::min<long long>((warps + GD_WARPS - 1) / GD_WARPS, 64ll * num_sms);
   sph_adjoint none;

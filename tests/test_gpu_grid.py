@@ -42,7 +42,8 @@ def direct(x, m, h, bar, ng):
 
 
 @pytest.mark.parametrize("n,ng,h_lo,h_hi", [(1, 9, 0.1, 0.1), (33, 80, 0.1, 0.13), (40, 45, 1e-4, 0.25),
-                                            (2500, 16, 0.01, 0.06), (5003, 8, 1e-3, 0.05)])
+                                            (2500, 16, 0.01, 0.06), (5003, 8, 1e-3, 0.05),
+                                            (4099, 10, 0.02, 0.09)])
 def test_grid_density_and_adjoint(env, n, ng, h_lo, h_hi):
     torch, sim = env
     rng = np.random.default_rng(n + ng)
