@@ -381,7 +381,7 @@ int build_cells(sph_ctx *ctx, sph_particles *p, cudaStream_t st) {
   SPH_CUDA(launch_build(v, ba, nc, w, (int)n_cells, !ctx->built, st));
   SPH_CUDA(launch_refresh_all(v, st));
   // cost estimate of every work group (only heavy-group scheduling uses it)
-  if (ctx->prm.heavy_factor > 0.0) SPH_CUDA(launch_group_cost(v, ctx->grid_dens, st));
+  if (ctx->prm.heavy_factor > 0.0) SPH_CUDA(launch_group_cost(v, 2 * ctx->grid_util, st));
   // no wake request survives a reordering (a halted step may have left some)
   if (ctx->prm.limiter)
     SPH_CUDA(cudaMemsetAsync(b.wake_bin, 0x7f, sizeof(int32_t) * (size_t)ctx->n_max, st));

@@ -26,6 +26,67 @@ __device__ __forceinline__ int nwarps() { return (gridDim.x * blockDim.x) >> 5; 
 __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
 
 // ---------------------------------------------------------------------------
+// FP64 values by integer arithmetic
+// ---------------------------------------------------------------------------
+// An FP64 instruction, a conversion to or from FP64 among them, occupies an SM
+// for 16 cycles, 64 issue slots, and the passes over the particles were bound
+// by them (23 per particle in the drift, 20 in a step's close).  The
+// conversions and the scalings by powers of two below give the same bits from
+// integer instructions; what they do not cover takes the FP64 instruction.
+
+// (double)f
+__device__ __forceinline__ double widen(float f) {
+  const unsigned int b = __float_as_uint(f), a = b & 0x7fffffffu;
+  if (a - 0x00800000u >= 0x7f000000u && a != 0u) return (double)f;  // subnormal, infinite, NaN
+  const unsigned int hi = (b & 0x80000000u) | (a ? (a >> 3) + 0x38000000u : 0u);
+  return __hiloint2double((int)hi, (int)(b << 29));
+}
+
+// (double)k
+__device__ __forceinline__ double widen(long long k) {
+  return k > -(1ll << 24) && k < (1ll << 24) ? widen((float)(int)k) : (double)k;
+}
+
+// (float)d, rounded to nearest even
+__device__ __forceinline__ float narrow(double d) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(d);
+  const unsigned long long a = b & 0x7fffffffffffffffull;
+  if (a == 0ull) return __uint_as_float((unsigned int)(b >> 32));
+  const unsigned int e = (unsigned int)(a >> 52);
+  if (e - 898u >= 254u - 2u) return (float)d;  // outside the normal range of FP32, or near its ends
+  const unsigned long long r = a - (896ull << 52);
+  const unsigned int f = (unsigned int)((r + 0x0fffffffull + ((r >> 29) & 1ull)) >> 29);
+  return __uint_as_float((unsigned int)(b >> 63) << 31 | f);
+}
+
+// Half of a step of D ticks: 0.5 D dt_min in FP64 and rounded to FP32.  D is a
+// power of two (or 0, before a particle's first step) unless the limiter cut
+// the step.
+struct Half {
+  double d;
+  float f;
+};
+__device__ __forceinline__ Half half_step(long long D, double dt_min) {
+  if (D == 0) return {0.0, 0.0f};
+  const int k = 63 - __clzll(D);
+  const int hi = __double2hiint(dt_min), e = (hi >> 20) + k - 1;  // (dt_min > 0)
+  if (D > 0 && (D & (D - 1)) == 0 && (hi >> 20) > 0 && e < 2047) {
+    const double h = __hiloint2double(hi + ((k - 1) << 20), __double2loint(dt_min));
+    if (k > 0 || (hi >> 20) > 1) return {h, narrow(h)};
+  }
+  const double h = 0.5 * (double)D * dt_min;
+  return {h, (float)h};
+}
+
+// The half-kick of a particle: v += a h, A += Adot h.
+__device__ __forceinline__ void half_kick(const Half &h, const float4 &a, float4 &v) {
+  v.x += a.x * h.f;
+  v.y += a.y * h.f;
+  v.z += a.z * h.f;
+  v.w = narrow(fma(widen(a.w), h.d, widen(v.w)));
+}
+
+// ---------------------------------------------------------------------------
 // active set
 // ---------------------------------------------------------------------------
 
@@ -167,11 +228,11 @@ __device__ void relevant_part(View &v, int b0, int nb) {
 // x - g wq (g: a corner's index on the box-wide grid of step wq) rounded
 // once, then to FP32, as the periodic image nearest the corner
 __device__ __forceinline__ float leaf_rel(double x, int g, double wq, double box, float hbox) {
-  double d = fma(-(double)g, wq, x);
-  float f = (float)d;
+  double d = fma(-widen((long long)g), wq, x);
+  float f = narrow(d);
   if (fabsf(f) > hbox) {  // (only across the periodic boundary)
     d -= copysign(box, d);
-    f = (float)d;
+    f = narrow(d);
   }
   return f;
 }
@@ -231,10 +292,10 @@ __device__ void chunk_update(const View &v, int g, bool do_drift, bool do_bins) 
     if (do_drift) {
       const long long td = v.ti_drift[i];
       if (td != ti) {
-        const double dt = (double)(ti - td) * v.dt_min;
-        x = wrap_pos_fast(x + (double)v.vx[i] * dt, v.box);
-        y = wrap_pos_fast(y + (double)v.vy[i] * dt, v.box);
-        z = wrap_pos_fast(z + (double)v.vz[i] * dt, v.box);
+        const double dt = widen(ti - td) * v.dt_min;
+        x = wrap_pos_fast(fma(widen(v.vx[i]), dt, x), v.box);
+        y = wrap_pos_fast(fma(widen(v.vy[i]), dt, y), v.box);
+        z = wrap_pos_fast(fma(widen(v.vz[i]), dt, z), v.box);
         v.x[i] = x;
         v.y[i] = y;
         v.z[i] = z;
@@ -257,9 +318,10 @@ __device__ void chunk_update(const View &v, int g, bool do_drift, bool do_bins) 
     const int bi = v.bin[i] & (MAX_BINS - 1);
     // (the middle of the particle's step: its length is 2^bin, or shorter once
     // the limiter woke it)
-    const double dtp =
-        ((double)(ti - v.ti_begin[i]) - 0.5 * (double)(v.ti_end[i] - v.ti_begin[i])) * v.dt_min;
-    const float fdtp = (float)dtp;
+    // (ti - t_begin) - (t_end - t_begin) / 2, in half ticks
+    const long long tb = v.ti_begin[i];
+    const long long m2 = 2 * (ti - tb) - (v.ti_end[i] - tb);
+    const float fdtp = narrow(widen(m2) * (0.5 * v.dt_min));
     const float vpx = v.vx[i] + v.ax[i] * fdtp;
     const float vpy = v.vy[i] + v.ay[i] * fdtp;
     const float vpz = v.vz[i] + v.az[i] * fdtp;
@@ -268,7 +330,7 @@ __device__ void chunk_update(const View &v, int g, bool do_drift, bool do_bins) 
     if (v.predict) {
       // Gadget-2 prediction from the last density (at the start of the step):
       // rho exp(-div v dt), h exp(div v dt / 3)
-      const float x = v.div_v[i] * (float)((double)(ti - v.ti_begin[i]) * v.dt_min);
+      const float x = v.div_v[i] * (float)((double)(ti - tb) * v.dt_min);
       rho *= expf(-x);
       hh *= expf(x * (1.0f / 3.0f));
     }
@@ -543,8 +605,7 @@ __global__ void k_next_time(View v, long long *out, int count_step) {
   next_time(v, out, count_step);
 }
 
-// The end of a step in one launch: for every active particle (one warp per
-// active leaf) the closing half-kick of its old step, its new bin (as
+// The end of a step in one launch: for every active particle the closing half-kick of its old step, its new bin (as
 // k_bins), the opening half-kick of the new step -- the same arithmetic as
 // k_kick and k_bins in the same order -- then, in the last block to finish,
 // the next tick and the step's counters (as k_next_time).
@@ -562,24 +623,29 @@ __global__ void __launch_bounds__(UT) k_close_step(View v) {
   if (!s_go) return;  // the whole block (a halted step changes nothing)
   const int nq = ds->n_active_leaves, m_act = ds->m_act;
   const long long ti = ds->ti;
-  for (int k = gwarp(); k < nq; k += nwarps()) {
-    const int leaf = v.q_active[k];
-    if (!SPH_IN(ds, leaf, ds->n_leaves, SPH_CHECK_ACTIVE_LEAF)) continue;  // (warp-uniform)
-    const int a = v.leaf_start[leaf], b = v.leaf_start[leaf + 1];
-    int minb = 127;
-    unsigned long long mask = 0ull;
-    for (int base = a; base < b; base += 32) {  // (the same trip count in every lane)
-      const int i = base + lane_id();
-      const int old = i < b ? (int)v.bin[i] : 0;
+  // (several leaves per warp where there are more leaves than warps: a leaf of
+  // 11 particles alone leaves two thirds of the lanes idle)
+  __shared__ int s_min[UT / 32][LEAVES_PER_WARP];
+  __shared__ unsigned long long s_mask[UT / 32][LEAVES_PER_WARP];
+  const int lane = lane_id(), warp = threadIdx.x >> 5;
+  const int per = leaves_per_warp(nq);
+  for (int k0 = gwarp() * per; k0 < nq; k0 += nwarps() * per) {
+    const LeafRun L = leaf_run(v, k0, per, nq);
+    if (lane < per) {
+      s_min[warp][lane] = 127;
+      s_mask[warp][lane] = 0ull;
+    }
+    __syncwarp();
+    for (int r = 0; r < L.total; r += 32) {  // (the same trip count in every lane)
+      int q;
+      const int i = leaf_run_particle(L, r + lane, &q);
+      const int old = i >= 0 ? (int)v.bin[i] : 0;
       int nb = old;
-      if (i < b && old <= m_act) {
+      if (i >= 0 && old <= m_act) {
         // closing half-kick of the old step
-        double half = 0.5 * (double)(v.ti_end[i] - v.ti_begin[i]) * v.dt_min;
-        float hf = (float)half;
-        v.vx[i] += v.ax[i] * hf;
-        v.vy[i] += v.ay[i] * hf;
-        v.vz[i] += v.az[i] * hf;
-        v.A[i] = (float)((double)v.A[i] + (double)v.Adot[i] * half);
+        float4 vel = make_float4(v.vx[i], v.vy[i], v.vz[i], v.A[i]);
+        const float4 acc = make_float4(v.ax[i], v.ay[i], v.az[i], v.Adot[i]);
+        half_kick(half_step(v.ti_end[i] - v.ti_begin[i], v.dt_min), acc, vel);
         // Eq. 1 and Eq. 2, increases only on a multiple of the new step
         bool small;
         nb = bin_of(v, v.h[i], v.vsig[i], small);
@@ -591,27 +657,24 @@ __global__ void __launch_bounds__(UT) k_close_step(View v) {
         v.ti_begin[i] = ti;
         v.ti_end[i] = ti + (1ll << nb);
         // opening half-kick of the new step
-        half = 0.5 * (double)(v.ti_end[i] - v.ti_begin[i]) * v.dt_min;
-        hf = (float)half;
-        v.vx[i] += v.ax[i] * hf;
-        v.vy[i] += v.ay[i] * hf;
-        v.vz[i] += v.az[i] * hf;
-        v.A[i] = (float)((double)v.A[i] + (double)v.Adot[i] * half);
+        half_kick(half_step(1ll << nb, v.dt_min), acc, vel);
+        v.vx[i] = vel.x;
+        v.vy[i] = vel.y;
+        v.vz[i] = vel.z;
+        v.A[i] = vel.w;
       }
-      count_bin_change(delta, i < b && nb != old, old, nb);
-      if (i < b) {
-        minb = min(minb, nb);
-        mask |= 1ull << nb;
+      count_bin_change(delta, i >= 0 && nb != old, old, nb);
+      if (i >= 0) {
+        atomicMin(&s_min[warp][q], nb);
+        atomicOr(&s_mask[warp][q], 1ull << nb);
       }
     }
-    for (int o = 16; o; o >>= 1) {
-      minb = min(minb, __shfl_xor_sync(0xffffffffu, minb, o));
-      mask |= __shfl_xor_sync(0xffffffffu, mask, o);
+    __syncwarp();
+    if (lane < per && L.leaf >= 0) {
+      v.leaf_min_bin[L.leaf] = (uint8_t)s_min[warp][lane];
+      v.leaf_bin_mask[L.leaf] = s_mask[warp][lane];
     }
-    if (lane_id() == 0) {
-      v.leaf_min_bin[leaf] = (uint8_t)minb;
-      v.leaf_bin_mask[leaf] = mask;
-    }
+    __syncwarp();
   }
   __syncthreads();
   for (int t = threadIdx.x; t < MAX_BINS; t += blockDim.x)
@@ -776,7 +839,7 @@ __global__ void k_diag_final(const double *partials, int nblocks, double *out) {
 // ---------------------------------------------------------------------------
 cudaError_t launch_refresh_all(const View &v, cudaStream_t st) {
   note_launches(1);
-  k_refresh<<<2 * v.grid_util, UT, 0, st>>>(v);
+  k_refresh<<<4 * v.grid_util, 128, 0, st>>>(v);  // (as k_drift)
   return cudaGetLastError();
 }
 

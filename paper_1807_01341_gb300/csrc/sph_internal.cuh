@@ -261,6 +261,56 @@ __device__ __forceinline__ bool all_coop(const View &v, const DevState *ds) {
   return v.G == 1 && ds->n_active_groups + ds->n_heavy_groups <= v.coop_max_groups;
 }
 
+// Consecutive entries of the active-leaf queue taken by one warp, their
+// particles numbered through, so that the lanes stay full: lane q (< per)
+// holds entry q.
+constexpr int LEAVES_PER_WARP = 8;
+struct LeafRun {
+  int leaf, first, start;  // lane q: leaf (-1: none), its first particle, its first number
+  int total;               // particles (all lanes)
+};
+__device__ __forceinline__ int leaves_per_warp(int n_leaves) {
+  const int nw = (int)(gridDim.x * blockDim.x) >> 5;
+  return max(1, min(LEAVES_PER_WARP, n_leaves / nw));
+}
+__device__ __forceinline__ LeafRun leaf_run(const View &v, int k0, int per, int n_leaves) {
+  const int lane = threadIdx.x & 31;
+  LeafRun L = {-1, 0, 0, 0};
+  int cnt = 0;
+  if (lane < per && k0 + lane < n_leaves) {
+    L.leaf = v.q_active[k0 + lane];
+    if (SPH_IN(v.ds, L.leaf, v.ds->n_leaves, SPH_CHECK_ACTIVE_LEAF)) {
+      L.first = v.leaf_start[L.leaf];
+      cnt = v.leaf_start[L.leaf + 1] - L.first;
+    } else {
+      L.leaf = -1;
+    }
+  }
+  int incl = cnt;
+#pragma unroll
+  for (int o = 1; o < LEAVES_PER_WARP; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
+  L.start = incl - cnt;
+  L.total = __shfl_sync(0xffffffffu, incl, LEAVES_PER_WARP - 1);
+  if (lane >= LEAVES_PER_WARP) L.start = L.total;
+  return L;
+}
+// Particle with number t of the run and its entry q (-1 past the end; every
+// lane of the warp calls it).
+__device__ __forceinline__ int leaf_run_particle(const LeafRun &L, int t, int *q) {
+  int e = 0;
+#pragma unroll
+  for (int w = LEAVES_PER_WARP / 2; w; w >>= 1) {
+    const int s = __shfl_sync(0xffffffffu, L.start, e + w);
+    if (s <= t) e += w;
+  }
+  const int f = __shfl_sync(0xffffffffu, L.first, e), s = __shfl_sync(0xffffffffu, L.start, e);
+  *q = e;
+  return t < L.total ? f + (t - s) : -1;
+}
+
 // Number of integer bins active at tick ti: particles on bin b are active
 // when ti is a multiple of 2^b, i.e. b <= ctz(ti) (every bin at tick 0).
 __host__ __device__ __forceinline__ int max_active_bin(long long ti) {

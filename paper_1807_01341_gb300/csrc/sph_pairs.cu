@@ -1422,55 +1422,62 @@ __global__ void __launch_bounds__(PT, 2) k_gradient(View v) {
   if (lane == 0 && wc.timeout) record_error(ds, SPH_ERR_TIMEOUT, wc.timeout, true);
 }
 
-// Estimated cost of each work group: the particles in the leaves (in cells of
+// Estimated cost of each work group: the particles in the cells (in cells of
 // more than CHUNK leaves: in the leaf chunks) that a box around the group,
 // grown by the largest support among its particles, reaches.  One warp per
-// group; the search lists nothing, its tests only count.  The sum over all
-// groups goes to group_cost_sum (the mark kernel compares each group with the
-// mean).
-__global__ void __launch_bounds__(PT, 2) k_group_cost(View v) {
+// group, one neighbour cell per lane; the large cells' chunks go across the
+// lanes.  The sum over all groups goes to group_cost_sum (the mark kernel
+// compares each group with the mean).  Only the order in which groups start
+// depends on it, so whole cells do (with a search of the leaves, as the pair
+// loops run it: 2.07 ms at 16.8M particles, COST_NOTE).
+__global__ void __launch_bounds__(PT) k_group_cost(View v) {
   DevState *ds = v.ds;
   if (ds->build_bad | ds->build_fail) return;  // (a build that was stopped)
-  StageD st;
-  stage_init(st);
   const int lane = lane_id();
   const int ng = ds->n_groups;
+  const float exc = __uint_as_float(ds->excursion_bits);
   const int nwarps = gridDim.x * WARPS_PER_BLOCK;
+  unsigned long long sum = 0ull;
   for (int g = blockIdx.x * WARPS_PER_BLOCK + (threadIdx.x >> 5); g < ng; g += nwarps) {
     const CellFrame F = frame_of(v, ds, g);
     const Group W = group_of(v, g, F);
     const int i = W.a + lane;  // a work group holds at most 32 particles
-    const float Hl = i < W.b ? GAMMA_K * v.h[i] : 0.0f;
-    const float R = warp_max(Hl);
+    const float R = warp_max(i < W.b ? GAMMA_K * v.h[i] : 0.0f);
     const float qox = F.kx * F.wq, qoy = F.ky * F.wq, qoz = F.kz * F.wq;
     const float clx = W.lx + qox, cly = W.ly + qoy, clz = W.lz + qoz;
     const float chx = W.hx + qox, chy = W.hy + qoy, chz = W.hz + qoz;
     const float Rc = R + 1e-5f * F.wf;
-    long long count = 0;
-    auto leaf_ok = [&](int l, float sx, float sy, float sz, LeafBox &) {
-      if (box_gap2(W.lx, W.ly, W.lz, W.hx, W.hy, W.hz, v.leaf_lo[l], v.leaf_hi[l], sx, sy, sz) <
-          R * R * 1.0002f)
-        count += v.leaf_start[l + 1] - v.leaf_start[l];
-      return false;
-    };
-    auto chunk_ok = [&](int c, float sx, float sy, float sz) {
-      if (box_gap2(clx, cly, clz, chx, chy, chz, v.chunk_lo[c], v.chunk_hi[c], sx, sy, sz) < Rc * Rc) {
-        count += v.leaf_start[v.chunk_leaf_start[c + 1]] - v.leaf_start[v.chunk_leaf_start[c]];
+    int count = 0, g0 = 0, nch = 0;
+    if (lane < 27) {
+      const int dxc = lane / 9 - 1, dyc = (lane / 3) % 3 - 1, dzc = lane % 3 - 1;
+      const float gx = fmaxf(0.0f, fmaxf(dxc * F.wf - exc - chx, clx - ((dxc + 1) * F.wf + exc)));
+      const float gy = fmaxf(0.0f, fmaxf(dyc * F.wf - exc - chy, cly - ((dyc + 1) * F.wf + exc)));
+      const float gz = fmaxf(0.0f, fmaxf(dzc * F.wf - exc - chz, clz - ((dzc + 1) * F.wf + exc)));
+      if (gx * gx + gy * gy + gz * gz < Rc * Rc) {
+        const int cj = (wrap_cell(F.cx + dxc, F.nc) * F.nc + wrap_cell(F.cy + dyc, F.nc)) * F.nc +
+                       wrap_cell(F.cz + dzc, F.nc);
+        const int leaves = v.cell_leaf_start[cj + 1] - v.cell_leaf_start[cj];
+        if (leaves <= CHUNK) {
+          count = v.cell_start[cj + 1] - v.cell_start[cj];
+        } else {
+          g0 = v.cell_chunk_start[cj];
+          nch = v.cell_chunk_start[cj + 1] - g0;
+        }
       }
-      return false;
-    };
-    bool more = false;
-    const Reach reach = {clx, cly, clz, chx, chy, chz, Rc, __uint_as_float(ds->excursion_bits),
-                         nullptr, 0};
-    search(v, F, reach, st, leaf_ok, chunk_ok, 0, more);
-    for (int o = 16; o; o >>= 1) count += __shfl_xor_sync(FULL, count, o);
-    if (lane == 0) {
-      const int c = (int)min(count, (long long)0x7fffffff);
-      v.group_cost[g] = c;
-      atomicAdd(&ds->group_cost_sum, (unsigned long long)c);
     }
-    __syncwarp();
+    for (unsigned big = __ballot_sync(FULL, nch > 0); big; big &= big - 1u) {
+      const int q = __ffs(big) - 1;
+      const int c0 = __shfl_sync(FULL, g0, q), cn = __shfl_sync(FULL, nch, q);
+      const float sx = (q / 9 - 1) * F.wf, sy = ((q / 3) % 3 - 1) * F.wf, sz = (q % 3 - 1) * F.wf;
+      for (int c = c0 + lane; c < c0 + cn; c += 32)
+        if (box_gap2(clx, cly, clz, chx, chy, chz, v.chunk_lo[c], v.chunk_hi[c], sx, sy, sz) < Rc * Rc)
+          count += v.leaf_start[v.chunk_leaf_start[c + 1]] - v.leaf_start[v.chunk_leaf_start[c]];
+    }
+    const int c = __reduce_add_sync(FULL, count);  // (at most 2^24 particles)
+    if (lane == 0) v.group_cost[g] = c;
+    sum += (unsigned long long)c;
   }
+  if (lane == 0 && sum) atomicAdd(&ds->group_cost_sum, sum);
 }
 
 // Entropy from the initial internal energy (A holds u before the first
@@ -1480,13 +1487,14 @@ __global__ void k_entropy_from_u(View v) {
   if (ds->halt) return;
   const int nq = ds->n_active_leaves, m_act = ds->m_act;
   const float g = (float)v.gamma;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  for (int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < nq; k += nw) {
-    const int leaf = v.q_active[k];
-    if (!SPH_IN(ds, leaf, ds->n_leaves, SPH_CHECK_ACTIVE_LEAF)) continue;
-    const int a = v.leaf_start[leaf], b = v.leaf_start[leaf + 1];
-    for (int i = a + lane_id(); i < b; i += 32)
-      if ((int)v.bin[i] <= m_act) v.A[i] = (g - 1.0f) * v.A[i] / powf(v.rho[i], g - 1.0f);
+  const int nw = (gridDim.x * blockDim.x) >> 5, per = leaves_per_warp(nq);
+  for (int k = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per; k < nq; k += nw * per) {
+    const LeafRun L = leaf_run(v, k, per, nq);
+    for (int r = 0; r < L.total; r += 32) {
+      int q;
+      const int i = leaf_run_particle(L, r + lane_id(), &q);
+      if (i >= 0 && (int)v.bin[i] <= m_act) v.A[i] = (g - 1.0f) * v.A[i] / powf(v.rho[i], g - 1.0f);
+    }
   }
 }
 
@@ -1621,10 +1629,7 @@ int persistent_blocks_per_sm(int G, bool density) {
 
 cudaError_t launch_group_cost(const View &v, int grid, cudaStream_t st) {
   note_launches(1);
-  cudaError_t e = cudaFuncSetAttribute(k_group_cost, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)DENS_SMEM);
-  if (e != cudaSuccess) return e;
-  k_group_cost<<<grid, PT, DENS_SMEM, st>>>(v);
+  k_group_cost<<<grid, PT, 0, st>>>(v);
   return cudaGetLastError();
 }
 
