@@ -64,6 +64,7 @@ struct Buffers {
   // neighbour lists of the density loop: list_cap entries per lane of every
   // warp of a persistent density launch
   float2 *nbr = nullptr;
+  float *bal = nullptr;       // balsara: the particles' factors
   int8_t *ngb_bin = nullptr;  // limiter: smallest neighbour bin of each active particle
   int32_t *wake_bin = nullptr, *q_wake = nullptr;  // limiter: wake requests and their queue
   // state
@@ -279,6 +280,7 @@ View make_view(const sph_ctx *ctx, const sph_particles *p) {
   v.balsara = q.balsara;
   v.predict = q.predict_inactive;
   v.limiter = q.limiter;
+  v.bal = b.bal;
   v.ngb_bin = b.ngb_bin;
   v.wake_bin = b.wake_bin;
   v.q_wake = b.q_wake;
@@ -714,7 +716,7 @@ int sph_create(const sph_params *params, int64_t n_max, sph_ctx **out) {
     // that share a work group (those of a persistent launch; a per-bin launch
     // uses at most as many)
     ctx->list_blocks = ctx->grid_dens;
-    if ((r = dalloc(&b.ngb_bin, n)) || (r = dalloc(&b.wake_bin, n)) ||
+    if ((r = dalloc(&b.bal, params->balsara ? n : 1)) || (r = dalloc(&b.ngb_bin, n)) || (r = dalloc(&b.wake_bin, n)) ||
         (r = dalloc(&b.q_wake, n)) ||
         (r = dalloc(&b.nbr, (long long)ctx->list_blocks * WARPS_PER_BLOCK * 32 * params->list_cap)))
       break;
@@ -764,7 +766,7 @@ int sph_destroy(sph_ctx *ctx) {
   dfree(b.cell_start); dfree(b.cell_leaf_start); dfree(b.cell_stamp); dfree(b.cell_rel_stamp);
   dfree(b.cell_chunk_start); dfree(b.q_act_cells);
   dfree(b.ds); dfree(b.diag);
-  dfree(b.nbr); dfree(b.ngb_bin); dfree(b.wake_bin); dfree(b.q_wake);
+  dfree(b.nbr); dfree(b.bal); dfree(b.ngb_bin); dfree(b.wake_bin); dfree(b.q_wake);
   if (b.h_ds) cudaFreeHost(b.h_ds);
   delete ctx;
   return SPH_OK;

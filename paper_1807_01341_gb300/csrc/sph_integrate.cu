@@ -349,8 +349,9 @@ __device__ void chunk_update(const View &v, int g, bool do_drift, bool do_bins) 
       v.c[i] = c;
     }
     v.rec_h[i] = make_float4(rho, fP, c, 1.0f / H);
+    if (v.balsara) v.bal[i] = balsara_factor(v.div_v[i], v.curl_v[i], c, 1.0f / H);
   }
-  for (int o = 16; o; o >>= 1) exc = fmaxf(exc, __shfl_xor_sync(0xffffffffu, exc, o));
+  exc = warp_max_f(exc);
   if (lane == 0) s_exc[warp] = exc;
   __syncthreads();  // the chunk's records are in shared memory
   // phase 2: one leaf per warp, one particle per lane
@@ -372,18 +373,17 @@ __device__ void chunk_update(const View &v, int g, bool do_drift, bool do_bins) 
         mask = 1ull << minb;
       }
     }
-    for (int o = 16; o; o >>= 1) {
-      bx = fminf(bx, __shfl_xor_sync(0xffffffffu, bx, o));
-      by = fminf(by, __shfl_xor_sync(0xffffffffu, by, o));
-      bz = fminf(bz, __shfl_xor_sync(0xffffffffu, bz, o));
-      tx = fmaxf(tx, __shfl_xor_sync(0xffffffffu, tx, o));
-      ty = fmaxf(ty, __shfl_xor_sync(0xffffffffu, ty, o));
-      tz = fmaxf(tz, __shfl_xor_sync(0xffffffffu, tz, o));
-      Hm = fmaxf(Hm, __shfl_xor_sync(0xffffffffu, Hm, o));
-      if (do_bins) {
-        minb = min(minb, __shfl_xor_sync(0xffffffffu, minb, o));
-        mask |= __shfl_xor_sync(0xffffffffu, mask, o);
-      }
+    bx = warp_min_f(bx);
+    by = warp_min_f(by);
+    bz = warp_min_f(bz);
+    tx = warp_max_f(tx);
+    ty = warp_max_f(ty);
+    tz = warp_max_f(tz);
+    Hm = warp_max_f(Hm);
+    if (do_bins) {
+      minb = __reduce_min_sync(0xffffffffu, minb);
+      mask = (unsigned long long)__reduce_or_sync(0xffffffffu, (unsigned int)mask) |
+             (unsigned long long)__reduce_or_sync(0xffffffffu, (unsigned int)(mask >> 32)) << 32;
     }
     if (lane == 0) {
       v.leaf_lo[leaf] = make_float4(bx, by, bz, Hm);
@@ -409,15 +409,13 @@ __device__ void chunk_update(const View &v, int g, bool do_drift, bool do_bins) 
       lx = lo.x; ly = lo.y; lz = lo.z; Hm = lo.w;
       hx = hi.x; hy = hi.y; hz = hi.z;
     }
-    for (int o = 16; o; o >>= 1) {
-      lx = fminf(lx, __shfl_xor_sync(0xffffffffu, lx, o));
-      ly = fminf(ly, __shfl_xor_sync(0xffffffffu, ly, o));
-      lz = fminf(lz, __shfl_xor_sync(0xffffffffu, lz, o));
-      hx = fmaxf(hx, __shfl_xor_sync(0xffffffffu, hx, o));
-      hy = fmaxf(hy, __shfl_xor_sync(0xffffffffu, hy, o));
-      hz = fmaxf(hz, __shfl_xor_sync(0xffffffffu, hz, o));
-      Hm = fmaxf(Hm, __shfl_xor_sync(0xffffffffu, Hm, o));
-    }
+    lx = warp_min_f(lx);
+    ly = warp_min_f(ly);
+    lz = warp_min_f(lz);
+    hx = warp_max_f(hx);
+    hy = warp_max_f(hy);
+    hz = warp_max_f(hz);
+    Hm = warp_max_f(Hm);
     if (lane == 0) {
       v.chunk_lo[g] = make_float4(lx, ly, lz, Hm);
       v.chunk_hi[g] = make_float4(hx, hy, hz, 0.0f);

@@ -111,6 +111,7 @@ struct View {
   uint8_t *active;
   int32_t *ngb_density, *ngb_force;
   float *div_v, *curl_v;     // velocity divergence and |curl| (variants; may be null)
+  float *bal;                // balsara: each particle's factor, with the records (step scratch)
   int8_t *ngb_bin;           // limiter: smallest bin among the force neighbours (step scratch)
   int32_t *wake_bin;         // limiter: smallest bin an active neighbour asks an inactive
                              // particle down to (WAKE_NONE: none; reset once applied)
@@ -189,6 +190,18 @@ struct AdjWork {
   double *ka, *kb, *km;          // density-adjoint coefficients of the active particles
 };
 
+// smallest and largest value of a warp, one instruction (five exchanges otherwise)
+__device__ __forceinline__ float warp_min_f(float x) {
+  float r;
+  asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float warp_max_f(float x) {
+  float r;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+  return r;
+}
+
 // address of a DevState field on the device, computed on the host
 #define SPH_DS_FIELD(ds, field) \
   (reinterpret_cast<decltype(&((DevState *)nullptr)->field)>( \
@@ -246,6 +259,12 @@ __host__ __device__ __forceinline__ int leaf_kz(uint32_t k) { return (int)((k >>
 
 __device__ __forceinline__ int wrap_cell(int c, int nc) {
   return c < 0 ? c + nc : (c >= nc ? c - nc : c);
+}
+
+// Balsara factor |div v| / (|div v| + |curl v| + 1e-4 c / h), h = 1 / (GAMMA_K / H)
+__device__ __forceinline__ float balsara_factor(float div_v, float curl_v, float c, float Hinv) {
+  const float dv = fabsf(div_v);
+  return dv / (dv + fabsf(curl_v) + 1e-4f * c * GAMMA_K * Hinv);
 }
 
 // k-th entry of the active work-group queue: the heavy groups first (they

@@ -127,11 +127,7 @@ __device__ __forceinline__ float2 dist2_x2(float2 ax, float2 ay, float2 az, floa
   return __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
 }
 
-__device__ __forceinline__ float warp_max(float x) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) x = fmaxf(x, __shfl_xor_sync(FULL, x, o));
-  return x;
-}
+__device__ __forceinline__ float warp_max(float x) { return warp_max_f(x); }
 
 __device__ __forceinline__ int warp_incl_scan(int x) {
   const int lane = lane_id();
@@ -338,15 +334,12 @@ __device__ __forceinline__ Group group_of(const View &v, int g, const CellFrame 
     lx = lo.x + ox; ly = lo.y + oy; lz = lo.z + oz;
     hx = hi.x + ox; hy = hi.y + oy; hz = hi.z + oz;
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    lx = fminf(lx, __shfl_xor_sync(FULL, lx, o));
-    ly = fminf(ly, __shfl_xor_sync(FULL, ly, o));
-    lz = fminf(lz, __shfl_xor_sync(FULL, lz, o));
-    hx = fmaxf(hx, __shfl_xor_sync(FULL, hx, o));
-    hy = fmaxf(hy, __shfl_xor_sync(FULL, hy, o));
-    hz = fmaxf(hz, __shfl_xor_sync(FULL, hz, o));
-  }
+  lx = warp_min_f(lx);
+  ly = warp_min_f(ly);
+  lz = warp_min_f(lz);
+  hx = warp_max_f(hx);
+  hy = warp_max_f(hy);
+  hz = warp_max_f(hz);
   G.lx = lx; G.ly = ly; G.lz = lz; G.hx = hx; G.hy = hy; G.hz = hz;
   return G;
 }
@@ -366,7 +359,7 @@ __device__ __forceinline__ float3 leaf_offset(const View &v, int i, const CellFr
 constexpr int STAGE_DEPTH_MAX = 3;  // staging buffers per warp (copies in flight)
 
 // (TAGS: room for the staged records' particle and cell; SHARE, the forward
-// force loop's: room for a batch's accept masks, and the search's spheres and
+// force and gradient loops': room for a batch's accept masks, and the search's spheres and
 // chunk list lie in the room of the staged records, so that every search sets
 // its spheres and none runs while records are in use)
 template <int S, int NREC, int LC, bool TAGS = true, bool SHARE = false>
@@ -758,6 +751,10 @@ using StageF = Stage<S_FORCE, 3, 256>;
 constexpr int S_PAIR = 192;
 template <bool VAR>
 using StageP = Stage<S_PAIR, 3, VAR ? 128 : 176, VAR, true>;
+
+// the velocity-gradient loop: positions and velocities alone
+constexpr int S_GRAD = 224;
+using StageG = Stage<S_GRAD, 2, 208, true, true>;
 
 // depth: staging buffers (1..STAGE_DEPTH_MAX, and S / depth >= 32);
 // wait_limit: polls of each bounded barrier wait (<= 0: WAIT_LIMIT);

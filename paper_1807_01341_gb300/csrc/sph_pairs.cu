@@ -767,12 +767,7 @@ __device__ void force_group(const View &v, int wg, int slice, int nslices, int b
     int cnt = 0;
     int bmin = 127;  // limiter: smallest bin among the neighbours
     const int bi = ((VAR && v.limiter) && valid) ? (int)v.bin[i] : 0;  // limiter: i's bin
-    // Balsara factor of i: |div v| / (|div v| + |curl v| + 1e-4 c / h), h = 1 / (GAMMA_K / H)
-    float Bi = 1.0f;
-    if ((VAR && v.balsara) && valid) {
-      const float dv = fabsf(v.div_v[i]);
-      Bi = dv / (dv + fabsf(v.curl_v[i]) + 1e-4f * hi4.z * GAMMA_K * hi4.w);
-    }
+    const float Bi = VAR && v.balsara && valid ? v.bal[i] : 1.0f;
     auto leaf_ok = [&](int l, float sx, float sy, float sz, LeafBox &lb) {
       const float4 loj = v.leaf_lo[l], hij = v.leaf_hi[l];
       const float R = fmaxf(Hs, loj.w);
@@ -899,9 +894,7 @@ __device__ void force_group(const View &v, int wg, int slice, int nslices, int b
           float Pi = __fdividef(-alpha * vsij * wij, hi4.x + hj.x);
           if ((VAR && v.balsara)) {
             // mean of the pair's Balsara factors (j's from its last density)
-            const int j = st.recj[k];
-            const float dv = fabsf(v.div_v[j]);
-            const float Bj = dv / (dv + fabsf(v.curl_v[j]) + 1e-4f * hj.z * GAMMA_K * hj.w);
+            const float Bj = v.bal[st.recj[k]];
             Pi *= 0.5f * (Bi + Bj);
           }
           const float dWb = 0.5f * (dwi + dwj);
@@ -1006,7 +999,7 @@ __device__ void force_group(const View &v, int wg, int slice, int nslices, int b
 // at neighbour-cell boundaries in record order.
 // ---------------------------------------------------------------------------
 __device__ void gradient_group(const View &v, int wg, int m_act, const CellFrame &F, float exc,
-                               StageF &st, WarpCounters &wc) {
+                               StageG &st, WarpCounters &wc) {
   const int lane = lane_id();
   const Group W = group_of(v, wg, F);
   const int a = W.a, b = W.b;
@@ -1016,8 +1009,8 @@ __device__ void gradient_group(const View &v, int wg, int m_act, const CellFrame
   const float clx = W.lx + qox, cly = W.ly + qoy, clz = W.lz + qoz;
   const float chx = W.hx + qox, chy = W.hy + qoy, chz = W.hz + qoz;
   const float ceps = 1e-5f * F.wf;
-  const float4 *srcs[3] = {v.rec_xH, v.rec_v, v.rec_h};
-  const float4 *sx_rec = st.rec, *sv_rec = st.rec + S_FORCE;
+  const float4 *srcs[2] = {v.rec_xH, v.rec_v};
+  const float4 *sx_rec = st.rec, *sv_rec = st.rec + S_GRAD;
   const bool valid = lane < nact;  // (a group holds at most 32 particles)
   const int i = valid ? st.act[lane] : a;
   const float4 xl = v.rec_xH[i];
@@ -1028,46 +1021,69 @@ __device__ void gradient_group(const View &v, int wg, int m_act, const CellFrame
   const float nHi4 = KERNEL_NORM * Hinv * Hinv * Hinv * Hinv;
   const float Hs = warp_max(valid ? xi.w : 0.0f);
   const int nsph = compact_spheres(st.sph, valid, make_float4(xi.x, xi.y, xi.z, xi.w));
+  if (valid) st.tst[lane] = make_float4(xi.x, xi.y, xi.z, Hi2);
+  __syncwarp();
   float d_hi = 0.f, d_lo = 0.f, x_hi = 0.f, x_lo = 0.f, y_hi = 0.f, y_lo = 0.f, z_hi = 0.f,
         z_lo = 0.f;
   float pd = 0.f, px = 0.f, py = 0.f, pz = 0.f;
   int cur = -1;
   auto consume = [&](int base, int total) {
     wc.cand += (unsigned long long)total * (unsigned long long)nact;
-    for (int k0 = 0; k0 < total; k0 += 32) {
-      unsigned mask = 0u;
-      for (int u = 0; u < 32; u++) {
-        const float4 pj = sx_rec[min(base + k0 + u, S_FORCE - 1)];
-        const float dx = xi.x - pj.x, dy = xi.y - pj.y, dz = xi.z - pj.z;
-        const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-        mask |= (k0 + u < total && r2 < Hi2) ? (1u << u) : 0u;
+    // accept masks of the whole batch (as the force loop), the records across
+    // the lanes, two particles per packed test
+    int left = 0;
+    const int wend = (total + 31) >> 5;
+#pragma unroll 1
+    for (int w = 0; w < wend; w++) {
+      const bool in = 32 * w + lane < total;
+      const float4 pj = sx_rec[min(base + 32 * w + lane, S_GRAD - 1)];
+      const float2 qx = make_float2(pj.x, pj.x), qy = make_float2(pj.y, pj.y),
+                   qz = make_float2(pj.z, pj.z);
+      unsigned m = 0u;
+      for (int q = 0; q < nact; q += 2) {
+        const float4 t0 = st.tst[q], t1 = st.tst[min(q + 1, nact - 1)];
+        const float2 r2 = dist2_x2(make_float2(t0.x, t1.x), make_float2(t0.y, t1.y),
+                                   make_float2(t0.z, t1.z), qx, qy, qz);
+        const unsigned m0 = __ballot_sync(FULL, in && r2.x < t0.w);
+        const unsigned m1 = __ballot_sync(FULL, in && r2.y < t1.w);
+        if (q == lane) m = m0;
+        if (q + 1 == lane) m = m1;
       }
-      if (!valid) mask = 0u;
-      while (mask) {
-        const int k = base + k0 + __ffs(mask) - 1;
-        mask &= mask - 1;
-        const int ci = st.recc[k];
-        if (ci != cur) {
-          fold(d_hi, d_lo, pd);
-          fold(x_hi, x_lo, px);
-          fold(y_hi, y_lo, py);
-          fold(z_hi, z_lo, pz);
-          pd = px = py = pz = 0.f;
-          cur = ci;
-        }
-        const float4 pj = sx_rec[k];
-        const float4 vj = sv_rec[k];
-        const float dx = xi.x - pj.x, dy = xi.y - pj.y, dz = xi.z - pj.z;
-        const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-        if (r2 > 0.0f) {  // (the particle itself and coincident ones add nothing)
-          const float rinv = rsqrtf(r2);
-          const float g1 = vj.w * kernel_dw(r2 * rinv * Hinv) * nHi4 * rinv;
-          const float wx = vi.x - vj.x, wy = vi.y - vj.y, wz = vi.z - vj.z;
-          pd = fmaf(fmaf(wx, dx, fmaf(wy, dy, wz * dz)), g1, pd);
-          px = fmaf(fmaf(wy, dz, -wz * dy), g1, px);
-          py = fmaf(fmaf(wz, dx, -wx * dz), g1, py);
-          pz = fmaf(fmaf(wx, dy, -wy * dx), g1, pz);
-        }
+      if (!valid) m = 0u;
+      st.mask[w * 32 + lane] = m;
+      left += __popc(m);
+    }
+    int kb = base - 1, w = 0;
+    unsigned mask = st.mask[lane];
+    for (; left > 0; left--) {
+      while (mask == 0u) {
+        w++;
+        kb += 32;
+        mask = st.mask[w * 32 + lane];
+      }
+      const int k = kb + __ffs(mask);
+      mask &= mask - 1;
+      const int ci = st.recc[k];
+      if (ci != cur) {
+        fold(d_hi, d_lo, pd);
+        fold(x_hi, x_lo, px);
+        fold(y_hi, y_lo, py);
+        fold(z_hi, z_lo, pz);
+        pd = px = py = pz = 0.f;
+        cur = ci;
+      }
+      const float4 pj = sx_rec[k];
+      const float4 vj = sv_rec[k];
+      const float dx = xi.x - pj.x, dy = xi.y - pj.y, dz = xi.z - pj.z;
+      const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+      if (r2 > 0.0f) {  // (the particle itself and coincident ones add nothing)
+        const float rinv = rsqrtf(r2);
+        const float g1 = vj.w * kernel_dw(r2 * rinv * Hinv) * nHi4 * rinv;
+        const float wx = vi.x - vj.x, wy = vi.y - vj.y, wz = vi.z - vj.z;
+        pd = fmaf(fmaf(wx, dx, fmaf(wy, dy, wz * dz)), g1, pd);
+        px = fmaf(fmaf(wy, dz, -wz * dy), g1, px);
+        py = fmaf(fmaf(wz, dx, -wx * dz), g1, py);
+        pz = fmaf(fmaf(wx, dy, -wy * dx), g1, pz);
       }
     }
   };
@@ -1085,6 +1101,8 @@ __device__ void gradient_group(const View &v, int wg, int m_act, const CellFrame
   int skip = 0;
   bool more = false;
   do {
+    // (the staging took the spheres' room)
+    if (more) compact_spheres(st.sph, valid, make_float4(xi.x, xi.y, xi.z, xi.w));
     const int nlist = search(v, F, reach, st, leaf_ok, chunk_ok, skip, more);
     stage_list(srcs, st, nlist, consume, wc);
     skip += nlist;
@@ -1095,10 +1113,14 @@ __device__ void gradient_group(const View &v, int wg, int m_act, const CellFrame
   fold(y_hi, y_lo, py);
   fold(z_hi, z_lo, pz);
   if (valid) {
-    const float rho = v.rec_h[i].x;  // this step's density
+    const float4 hi4 = v.rec_h[i];
+    const float rho = hi4.x;  // this step's density
     const float cx = x_hi + x_lo, cy = y_hi + y_lo, cz = z_hi + z_lo;
-    v.div_v[i] = -(d_hi + d_lo) / rho;
-    v.curl_v[i] = sqrtf(fmaf(cx, cx, fmaf(cy, cy, cz * cz))) / rho;
+    const float div = -(d_hi + d_lo) / rho;
+    const float curl = sqrtf(fmaf(cx, cx, fmaf(cy, cy, cz * cz))) / rho;
+    v.div_v[i] = div;
+    v.curl_v[i] = curl;
+    if (v.balsara) v.bal[i] = balsara_factor(div, curl, hi4.z, hi4.w);
   }
 }
 
@@ -1404,7 +1426,7 @@ __global__ void __launch_bounds__(PT, 2) k_gradient(View v) {
   }
   __syncthreads();
   if (!s_go) return;
-  StageF st;
+  StageG st;
   stage_init(st, v.stage_depth, v.wait_limit);
   const int lane = lane_id();
   const int m_act = ds->m_act;
@@ -1429,7 +1451,7 @@ __global__ void __launch_bounds__(PT, 2) k_gradient(View v) {
 // lanes.  The sum over all groups goes to group_cost_sum (the mark kernel
 // compares each group with the mean).  Only the order in which groups start
 // depends on it, so whole cells do (with a search of the leaves, as the pair
-// loops run it: 2.07 ms at 16.8M particles, COST_NOTE).
+// loops run it: 2.07 ms at 16.8M particles, 223 us at 2.1M clustered; here 0.37 ms and 79 us).
 __global__ void __launch_bounds__(PT) k_group_cost(View v) {
   DevState *ds = v.ds;
   if (ds->build_bad | ds->build_fail) return;  // (a build that was stopped)
@@ -1499,7 +1521,7 @@ __global__ void k_entropy_from_u(View v) {
 }
 
 constexpr size_t DENS_SMEM = StageD::bytes() * WARPS_PER_BLOCK;
-constexpr size_t FORCE_SMEM = StageF::bytes() * WARPS_PER_BLOCK;
+constexpr size_t GRAD_SMEM = StageG::bytes() * WARPS_PER_BLOCK;
 constexpr size_t PAIR_WARP =
     StageP<true>::bytes() > StageP<false>::bytes() ? StageP<true>::bytes() : StageP<false>::bytes();
 constexpr size_t PAIR_SMEM = PAIR_WARP * WARPS_PER_BLOCK;
@@ -1557,7 +1579,7 @@ int blocks_per_sm_g(bool density) {
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
             cudaSuccess ||
         cudaFuncSetAttribute((const void *)k_gradient, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)FORCE_SMEM) != cudaSuccess) {
+                             (int)GRAD_SMEM) != cudaSuccess) {
       cudaGetLastError();
       return 0;
     }
@@ -1636,7 +1658,7 @@ cudaError_t launch_group_cost(const View &v, int grid, cudaStream_t st) {
 cudaError_t launch_gradient(const View &v, int grid, cudaStream_t st) {
   if (grid <= 0) return cudaSuccess;
   note_launches(1);
-  k_gradient<<<grid, PT, FORCE_SMEM, st>>>(v);
+  k_gradient<<<grid, PT, GRAD_SMEM, st>>>(v);
   return cudaGetLastError();
 }
 
