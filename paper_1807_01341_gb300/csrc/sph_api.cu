@@ -718,7 +718,8 @@ int sph_create(const sph_params *params, int64_t n_max, sph_ctx **out) {
     ctx->list_blocks = ctx->grid_dens;
     if ((r = dalloc(&b.bal, params->balsara ? n : 1)) || (r = dalloc(&b.ngb_bin, n)) || (r = dalloc(&b.wake_bin, n)) ||
         (r = dalloc(&b.q_wake, n)) ||
-        (r = dalloc(&b.nbr, (long long)ctx->list_blocks * WARPS_PER_BLOCK * 32 * params->list_cap)))
+        (r = dalloc(&b.nbr, (long long)ctx->list_blocks * WARPS_PER_BLOCK *
+                                (long long)density_list_entries(params->list_cap))))
       break;
     // no neighbour bin known yet: no limit (a bins call without a force pass);
     // no wake request

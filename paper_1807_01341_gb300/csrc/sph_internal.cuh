@@ -156,10 +156,10 @@ struct View {
   // candidate within a particle's search radius (with equal masses the squared
   // distance alone, 4-byte entries in the first half of the area), list_cap
   // entries per lane,
-  // one area per warp of the launch's blocks (a launch has at most list_blocks
-  // blocks; entry k of lane s of warp w of block b at
-  // nbr[((b * 8 + w) * list_cap + k) * 32 + s]): the area of a warp is reused
-  // by its next work group, so the lists stay in L2.
+  // and some padding, one area of density_list_entries per warp of the
+  // launch's blocks (a launch has at most list_blocks blocks; entry k of lane s
+  // at [k * 32 + s] of its warp's area): the area of a warp is reused by its
+  // next work group, so the lists stay in L2.
   float2 *nbr;
   BigItem *big;              // [n] (the build's scratch, free between builds)
   DevState *ds;
@@ -397,6 +397,8 @@ cudaError_t launch_force(const View &v, int bin_filter, bool persistent, int gri
                          cudaStream_t st);
 cudaError_t launch_entropy_from_u(const View &v, cudaStream_t st);
 int persistent_blocks_per_sm(int G, bool density);
+// entries (float2) of one warp's neighbour-list area
+int density_list_entries(int list_cap);
 cudaError_t launch_group_cost(const View &v, int grid, cudaStream_t st);
 // velocity divergence and curl of the active particles (after their density)
 cudaError_t launch_gradient(const View &v, int grid, cudaStream_t st);

@@ -110,87 +110,108 @@ __device__ __forceinline__ void fast2sum_prod2(float2 &hi, float2 &lo, float2 x,
   hi = t;
 }
 
+// the sum without the product
+__device__ __forceinline__ void fast2sum2(float2 &hi, float2 &lo, float2 x) {
+  const float2 t = __fadd2_rn(hi, x);
+  const float2 e = __fadd2_rn(t, make_float2(-hi.x, -hi.y));
+  lo = __fadd2_rn(lo, __fadd2_rn(x, make_float2(-e.x, -e.y)));
+  hi = t;
+}
+
 struct DSum {
-  float n_hi, n_lo, t_hi, t_lo, r_hi, r_lo, rt_hi, rt_lo;
+  float2 s_hi, s_lo;  // S_w and S_t
+  float2 m_hi, m_lo;  // the mass-weighted pair
   float p2;
   int cnt;
   __device__ __forceinline__ void zero() {
-    n_hi = n_lo = t_hi = t_lo = r_hi = r_lo = rt_hi = rt_lo = 0.0f;
+    s_hi = s_lo = m_hi = m_lo = make_float2(0.0f, 0.0f);
     p2 = 0.0f;
     cnt = 0;
   }
 };
 
-// A candidate at squared distance r2 (FP32, group frame) with mass mj, at the
-// support H (H2 = H^2, Hinv = 1/H): a neighbour when r2 < H2 (strict).  With
+__device__ __forceinline__ float rsqrt_normal(float x) {  // as rsqrtf, for a normal x
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float2 splat(float x) { return make_float2(x, x); }
+
+// Two candidates at squared distances r2.x, r2.y (FP32, group frame) with masses
+// m.x, m.y, at the support H (H2 = H^2, Hinv = 1/H, H4 = 4 H^2): each a neighbour
+// when r2 < H2 (strict), the first one's terms added first.  The kernel values
+// of both by packed instructions, each component rounded as kernel_wd rounds
+// it, and the terms of one that is no neighbour are zero, which changes no sum.  With
 // equal masses (UM) the mass-weighted sums are not formed: they are the common
 // mass times S_w and S_t.
 template <bool UM>
-__device__ __forceinline__ void dens_pair(DSum &s, float r2, float mj, float H2, float Hinv) {
-  if (!(r2 < H2)) return;
-  const float rr = r2 * rsqrtf(fmaxf(r2, 1e-30f));
-  const float qq = rr * Hinv;
-  float wq, dwq;
-  kernel_wd(qq, wq, dwq);
-  const float tt = fmaf(qq, dwq, 3.0f * wq);
-  s.p2 = fmaf(qq * qq, kernel_d2w(qq), s.p2);
-  fast2sum(s.n_hi, s.n_lo, wq);
-  fast2sum(s.t_hi, s.t_lo, tt);
-  if constexpr (!UM) {
-    fast2sum_prod(s.r_hi, s.r_lo, mj, wq);
-    fast2sum_prod(s.rt_hi, s.rt_lo, mj, tt);
-  }
-  s.cnt++;
+__device__ __forceinline__ void dens_pair2(DSum &s, float2 r2, float2 m, float H2, float H4,
+                                           float Hinv) {
+  const bool a0 = r2.x < H2, a1 = r2.y < H2;
+  const float2 rc = make_float2(fminf(r2.x, H4), fminf(r2.y, H4));  // (past the end: infinity)
+  const float2 rs = make_float2(rsqrt_normal(fmaxf(rc.x, 1e-30f)), rsqrt_normal(fmaxf(rc.y, 1e-30f)));
+  const float2 rr = __fmul2_rn(rc, rs);
+  const float2 q = __fmul2_rn(rr, splat(Hinv));
+  float2 u = __fadd2_rn(splat(1.0f), make_float2(-q.x, -q.y));
+  u.x = a0 ? u.x : 0.0f;
+  u.y = a1 ? u.y : 0.0f;
+  const float2 uu = __fmul2_rn(u, u), qq = __fmul2_rn(q, q);
+  const float2 wa = __ffma2_rn(qq, __ffma2_rn(splat(6.0f), q, splat(-6.0f)), splat(1.0f));
+  const float2 da = __fmul2_rn(q, __ffma2_rn(splat(18.0f), q, splat(-12.0f)));
+  const float2 ea = __ffma2_rn(splat(36.0f), q, splat(-12.0f));
+  const float2 wb = __fmul2_rn(__fmul2_rn(splat(2.0f), uu), u);
+  const float2 db = __fmul2_rn(splat(-6.0f), uu);
+  const float2 eb = __fmul2_rn(splat(12.0f), u);
+  const bool i0 = q.x < 0.5f, i1 = q.y < 0.5f;
+  const float2 w = make_float2(i0 ? wa.x : wb.x, i1 ? wa.y : wb.y);
+  const float2 d = make_float2(i0 ? da.x : db.x, i1 ? da.y : db.y);
+  const float2 t = __ffma2_rn(q, d, __fmul2_rn(splat(3.0f), w));
+  s.p2 = fmaf(qq.x, i0 ? ea.x : eb.x, s.p2);
+  s.p2 = fmaf(qq.y, i1 ? ea.y : eb.y, s.p2);
+  fast2sum2(s.s_hi, s.s_lo, make_float2(w.x, t.x));
+  if constexpr (!UM) fast2sum_prod2(s.m_hi, s.m_lo, splat(m.x), make_float2(w.x, t.x));
+  fast2sum2(s.s_hi, s.s_lo, make_float2(w.y, t.y));
+  if constexpr (!UM) fast2sum_prod2(s.m_hi, s.m_lo, splat(m.y), make_float2(w.y, t.y));
+  s.cnt += a0 ? 1 : 0;
+  s.cnt += a1 ? 1 : 0;
 }
 
-// Entries [0, nl) of a neighbour list (entry k at lst[k * ls]), in order, in
-// blocks of LQ: the loads of the next block are issued before the current
-// block is evaluated, so a warp running alone (a sparse step) waits for one
-// L2 round trip per LQ entries rather than per entry.  The loads may be
-// served by L1 (every later h iteration reads the list again): each lane
-// reads only entries it wrote itself, and a list area is used by one warp of
-// one launch (L1 lines are invalidated between dependent launches).
+// Entries [0, nl) of a neighbour list (entry k at lst[k * ls]; infinities follow
+// up to a multiple of LQ), in order, in blocks of LQ: the loads of the next
+// block are issued before the current block is evaluated, so a warp running
+// alone (a sparse step) waits for one L2 round trip per LQ entries rather than
+// per entry.  The loads may be served by L1 (every later h iteration reads the
+// list again): each lane reads only entries it wrote itself, and a list area
+// is used by one warp of one launch (L1 lines are invalidated between
+// dependent launches).  LIST_NOTE
 constexpr int LQ = 4;
+constexpr int LIST_PAD = 2 * LQ;       // entries past list_cap: the last block's, and its successor's loads
 constexpr float FIRST_MARGIN = 1.05f;  // search margin of a run's first density pass (at least)
-template <bool UM>
-__device__ __forceinline__ void dens_list(DSum &s, const float2 *lst, int ls, int nl, float H2,
+__device__ __forceinline__ float entry_r2(float e) { return e; }
+__device__ __forceinline__ float entry_r2(float2 e) { return e.x; }
+__device__ __forceinline__ float entry_m(float) { return 0.0f; }
+__device__ __forceinline__ float entry_m(float2 e) { return e.y; }
+template <bool UM, class Entry>
+__device__ __forceinline__ void dens_list(DSum &s, const Entry *lst, int ls, int nl, float H2,
                                           float Hinv) {
-  if (nl <= 0) return;
-  float2 e[LQ];
+  static_assert(LQ == 4, "two pairs a block");
+  const float H4 = 4.0f * H2;
+  Entry e[LQ];
 #pragma unroll
-  for (int j = 0; j < LQ; j++) e[j] = j < nl ? lst[(size_t)j * ls] : make_float2(INFINITY, 0.0f);
+  for (int j = 0; j < LQ; j++) e[j] = lst[j * ls];
 #pragma unroll 1
   for (int k = 0; k < nl; k += LQ) {
-    float2 cur[LQ];
+    Entry cur[LQ];
+    lst += LQ * ls;
 #pragma unroll
     for (int j = 0; j < LQ; j++) {
       cur[j] = e[j];
-      const int kn = k + LQ + j;
-      e[j] = kn < nl ? lst[(size_t)kn * ls] : make_float2(INFINITY, 0.0f);
+      e[j] = lst[j * ls];
     }
 #pragma unroll
-    for (int j = 0; j < LQ; j++) dens_pair<UM>(s, cur[j].x, cur[j].y, H2, Hinv);
-  }
-}
-
-// The same for a list of squared distances alone (equal masses).
-__device__ __forceinline__ void dens_list_r(DSum &s, const float *lst, int ls, int nl, float H2,
-                                            float Hinv) {
-  if (nl <= 0) return;
-  float e[LQ];
-#pragma unroll
-  for (int j = 0; j < LQ; j++) e[j] = j < nl ? lst[(size_t)j * ls] : INFINITY;
-#pragma unroll 1
-  for (int k = 0; k < nl; k += LQ) {
-    float cur[LQ];
-#pragma unroll
-    for (int j = 0; j < LQ; j++) {
-      cur[j] = e[j];
-      const int kn = k + LQ + j;
-      e[j] = kn < nl ? lst[(size_t)kn * ls] : INFINITY;
-    }
-#pragma unroll
-    for (int j = 0; j < LQ; j++) dens_pair<true>(s, cur[j], 0.0f, H2, Hinv);
+    for (int j = 0; j < LQ; j += 2)
+      dens_pair2<UM>(s, make_float2(entry_r2(cur[j]), entry_r2(cur[j + 1])),
+                     make_float2(entry_m(cur[j]), entry_m(cur[j + 1])), H2, H4, Hinv);
   }
 }
 
@@ -313,11 +334,11 @@ __device__ void density_group(const View &v, int wg, int slice, int nslices, int
   // area (the launch has at most list_blocks blocks)
   const int cap = v.list_cap;
   constexpr int ls = 32;
-  float2 *const lst = v.nbr + ((size_t)blockIdx.x * WARPS_PER_BLOCK + warp) * 32 * v.list_cap + lane;
+  float2 *const area = v.nbr + ((size_t)blockIdx.x * WARPS_PER_BLOCK + warp) * 32 * (cap + LIST_PAD);
+  float2 *const lst = area + lane;
   // (equal masses: the entries are the squared distances alone, in the first
   // half of the warp's area)
-  float *const lstr = reinterpret_cast<float *>(v.nbr + ((size_t)blockIdx.x * WARPS_PER_BLOCK + warp) *
-                                                             32 * v.list_cap) + lane;
+  float *const lstr = reinterpret_cast<float *>(area) + lane;
 
   for (int r = s0; r < s1 && !st.failed; r += P) {
     const int slot = r + grp;
@@ -491,7 +512,14 @@ __device__ void density_group(const View &v, int wg, int slice, int nslices, int
           } while (search_now && more && !st.failed);
           if (search_now) have_list = complete;
           if (writer) wc.gathers += nlive;
-          if (gath) nl = min(acc - skipc, cap);
+          if (gath) {
+            nl = min(acc - skipc, cap);
+#pragma unroll
+            for (int j = 0; j < LQ; j++) {
+              if constexpr (UM) __stcg(lstr + (size_t)(nl + j) * ls, INFINITY);
+              else __stcg(lst + (size_t)(nl + j) * ls, make_float2(INFINITY, 0.0f));
+            }
+          }
         }
         if constexpr (G == 1) {
           if (gath && acc > cap) {  // (the list filled up: one warp for this particle alone)
@@ -503,7 +531,7 @@ __device__ void density_group(const View &v, int wg, int slice, int nslices, int
         // the list this pass built (or, in the first pass, the one kept from
         // an earlier iteration), in order
         if (!done && (gath || first) && nl > 0) {
-          if constexpr (UM) dens_list_r(s, lstr, ls, nl, H2, Hinv);
+          if constexpr (UM) dens_list<true>(s, lstr, ls, nl, H2, Hinv);
           else dens_list<false>(s, lst, ls, nl, H2, Hinv);
           if (writer) wc.evals += (unsigned long long)nl;
         }
@@ -526,14 +554,14 @@ __device__ void density_group(const View &v, int wg, int slice, int nslices, int
         nl = -1;  // the list holds only the last pass's share
       }
       if (st.failed) break;
-      const double sn = group_sum<G>((double)s.n_hi + (double)s.n_lo);
-      const double stt = group_sum<G>((double)s.t_hi + (double)s.t_lo);
+      const double sn = group_sum<G>((double)s.s_hi.x + (double)s.s_lo.x);
+      const double stt = group_sum<G>((double)s.s_hi.y + (double)s.s_lo.y);
       // (the mass-weighted sums are needed only once h has converged: with
       // one lane per particle they are formed there, in the same arithmetic)
       float sr = 0.0f, srt = 0.0f;
       if constexpr (G > 1) {
-        sr = (float)group_sum<G>((double)s.r_hi + (double)s.r_lo);
-        srt = (float)group_sum<G>((double)s.rt_hi + (double)s.rt_lo);
+        sr = (float)group_sum<G>((double)s.m_hi.x + (double)s.m_lo.x);
+        srt = (float)group_sum<G>((double)s.m_hi.y + (double)s.m_lo.y);
       }
       const double s2 = group_sum<G>((double)s.p2);
       const int cnt = group_sum_i<G>(s.cnt) - 1;  // (the particle itself is among its candidates)
@@ -550,8 +578,8 @@ __device__ void density_group(const View &v, int wg, int slice, int nslices, int
             sr = (float)(mu * sn);
             srt = (float)(mu * stt);
           } else if constexpr (G == 1) {
-            sr = (float)((double)s.r_hi + (double)s.r_lo);
-            srt = (float)((double)s.rt_hi + (double)s.rt_lo);
+            sr = (float)((double)s.m_hi.x + (double)s.m_lo.x);
+            srt = (float)((double)s.m_hi.y + (double)s.m_lo.y);
           }
           if (sub == 0 && writer) {
             wc.pairs += (unsigned long long)cnt;
@@ -581,7 +609,7 @@ __device__ void density_group(const View &v, int wg, int slice, int nslices, int
 // the h iteration goes on from where density_group left it, each iteration
 // one pass over the candidates.  The lanes test and evaluate 32 records at a
 // time, then lane a adds up term a of the accepted ones in record order: the
-// particle's sums are those of dens_pair, term by term.  (Before, density_group
+// particle's sums are those of dens_pair2, term by term.  (Before, density_group
 // ran further passes over the group's records, list_cap of them listed in each,
 // with all 32 lanes waiting: time grows with the square of the candidates.  In
 // 302k clustered particles whose background meets clumps of 4,099, a first
@@ -1634,6 +1662,8 @@ cudaError_t launch_force(const View &v, int bin_filter, bool persistent, int gri
     default: return cudaErrorInvalidValue;
   }
 }
+
+int density_list_entries(int list_cap) { return 32 * (list_cap + LIST_PAD); }
 
 // Sets the dynamic shared-memory limit of the pair kernels for this G and
 // returns the resident blocks per SM (0 when the configuration cannot run).
