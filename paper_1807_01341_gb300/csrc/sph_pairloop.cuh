@@ -367,6 +367,7 @@ struct Stage {
   static constexpr int SLOTS = S;  // staged records
   static constexpr int LCAP = LC;  // accepted neighbour leaves listed per search pass
   static constexpr int CCAP = 128; // accepted chunks gathered per search segment
+  static constexpr int START_WORDS = S / 32;
   float4 *rec;     // NREC arrays of S staged records, back to back (first: positions);
                    // with depth d, buffer b holds slots [b S/d, (b+1) S/d) of each
   float4 *lshift;  // per listed leaf: offset of its corner (x, y, z), first particle (w bits)
@@ -380,16 +381,20 @@ struct Stage {
   unsigned *mask;  // (SHARE) accept masks of a batch: word q of lane l at 32 q + l
   uint64_t *bar;   // one mbarrier per staging buffer
   int *meta;       // per staging buffer: first listed leaf, leaves, records
+  unsigned *starts;  // per staging buffer: bit t set where a leaf's first record lies in slot t
   uint32_t phase;  // parity of the next phase of each buffer's barrier (bit b)
   int depth;       // staging buffers in use (1..STAGE_DEPTH_MAX)
   long long wait_limit;  // polls of a bounded barrier wait
   int *stall_ctr;  // testing: stalls still to make (a launch's first staging claims one)
   bool stall;      // testing: this staging issues no copy and never arrives
   bool failed;
+  // (a multiple of 16: the next warp's records, which bulk copies write, follow)
   static constexpr size_t bytes() {
-    return sizeof(float4) * ((size_t)S * NREC + LC + (SHARE ? 32 : 64)) +
-           (SHARE ? 0 : sizeof(int2) * CCAP) + sizeof(int) * (LC + LEAF_MAX_LIMIT) +
-           (TAGS ? (sizeof(int) + 1) * (size_t)S : 0) + (SHARE ? sizeof(unsigned) * S : 0) + 64;
+    return (sizeof(float4) * ((size_t)S * NREC + LC + (SHARE ? 32 : 64)) +
+            (SHARE ? 0 : sizeof(int2) * CCAP) + sizeof(int) * (LC + LEAF_MAX_LIMIT) +
+            (TAGS ? (sizeof(int) + 1) * (size_t)S : 0) + (SHARE ? sizeof(unsigned) * S : 0) + 64 +
+            sizeof(unsigned) * STAGE_DEPTH_MAX * START_WORDS + 15) /
+           16 * 16;
   }
   // sph, tst and chk back to back: free between one round's last consume and
   // the next search, they serve a block's cross-warp reductions (the staged
@@ -411,7 +416,8 @@ struct Stage {
     recc = reinterpret_cast<uint8_t *>(recj + (TAGS ? S : 0));
     bar = reinterpret_cast<uint64_t *>(recc + (TAGS ? S : 0));  // 8-byte aligned: every part above is
     meta = reinterpret_cast<int *>(bar + STAGE_DEPTH_MAX);
-    mask = reinterpret_cast<unsigned *>(bar + 8);
+    starts = reinterpret_cast<unsigned *>(bar + 8);
+    mask = starts + STAGE_DEPTH_MAX * START_WORDS;
   }
 };
 
@@ -630,8 +636,10 @@ __device__ __forceinline__ int search(const View &v, const CellFrame &F, const R
 // of the next depth - 1 batches are in flight while a batch is consumed.  A
 // batch is as many consecutive listed leaves as fit one buffer.  When a batch
 // has landed, each position record is moved into the work group's frame (its
-// leaf's corner offset added) and tagged with its particle index and
-// neighbour-cell index (TAG; a loop that reads only the positions skips the
+// leaf's corner offset added; its leaf found by counting the leaf starts up to
+// its slot, 32 records at a time: a loop over the leaves kept two lanes of three
+// idle, SHIFT_NOTE) and tagged with its particle index and neighbour-cell index
+// (TAG, which spends the leaf list's first-particle words; a loop that reads only the positions skips the
 // tags); then consume(base, total) sees records base .. base + total - 1.
 // Batches are consumed in list order whatever the depth.
 // A barrier wait that gives up sets st.failed and counts a timeout; the warp
@@ -675,13 +683,23 @@ __device__ __forceinline__ void stage_list(const float4 *const *srcs,
       st.meta[3 * b + 2] = total;
       if (!stall) mbar_expect_tx(&st.bar[b], (uint32_t)(total * NREC * (int)sizeof(float4)));
     }
+    // where each leaf starts in the buffer
+    const bool mine = (take >> lane) & 1u;
+    const int rel = incl - c;
+#pragma unroll 1
+    for (int w = 0; 32 * w < total; w++) {
+      const unsigned word =
+          __reduce_or_sync(FULL, mine && (rel >> 5) == w ? 1u << (rel & 31) : 0u);
+      if (lane == 0) st.starts[b * (S / 32) + w] = word;
+    }
     __syncwarp();
-    if (!stall && ((take >> lane) & 1u)) {
+    if (!stall && mine) {
       const int ja = __float_as_int(st.lshift[e + lane].w);
-      const int slot = b * Sb + incl - c;
+      const int slot = b * Sb + rel;
       for (int r = 0; r < NREC; r++)
         bulk_g2s(st.rec + (size_t)r * S + slot, srcs[r] + ja, (uint32_t)(c * sizeof(float4)),
                  &st.bar[b]);
+      if constexpr (TAG) st.lshift[e + lane].w = __int_as_float(ja - rel);
     }
     __syncwarp();
     if (lane == 0 && !stall) mbar_arrive(&st.bar[b]);
@@ -702,27 +720,30 @@ __device__ __forceinline__ void stage_list(const float4 *const *srcs,
       break;
     }
     st.phase ^= 1u << b;
-    const int e = st.meta[3 * b], k = st.meta[3 * b + 1], total = st.meta[3 * b + 2];
+    const int e = st.meta[3 * b], total = st.meta[3 * b + 2];
     const int base0 = b * Sb;
-    int base = base0;
-    for (int q = 0; q < k; q++) {
-      const float4 sh = st.lshift[e + q];
-      const int pk = st.lpack[e + q];
-      const int cq = pk & 0xffff;
-      const int ja = __float_as_int(sh.w);
-      (void)ja;
-      for (int t = lane; t < cq; t += 32) {
-        float4 rr = st.rec[base + t];
+    // each record into the group's frame, 32 at a time: its leaf is the number
+    // of leaf starts up to its slot
+    const unsigned upto = 0xffffffffu >> (31 - lane);
+    int leaf = e - 1;
+#pragma unroll 1
+    for (int t0 = 0; t0 < total; t0 += 32) {
+      const unsigned word = st.starts[b * (S / 32) + (t0 >> 5)];
+      const int t = t0 + lane;
+      if (t < total) {
+        const int l = leaf + __popc(word & upto);
+        const float4 sh = st.lshift[l];
+        float4 rr = st.rec[base0 + t];
         rr.x += sh.x;
         rr.y += sh.y;
         rr.z += sh.z;
-        st.rec[base + t] = rr;
+        st.rec[base0 + t] = rr;
         if constexpr (TAG) {
-          st.recj[base + t] = ja + t;
-          st.recc[base + t] = (uint8_t)(pk >> 16);
+          st.recj[base0 + t] = __float_as_int(sh.w) + t;
+          st.recc[base0 + t] = (uint8_t)(st.lpack[l] >> 16);
         }
       }
-      base += cq;
+      leaf += __popc(word);
     }
     __syncwarp();
     consume(base0, total);
@@ -764,6 +785,7 @@ template <class St>
 __device__ __forceinline__ void stage_init(St &st, int depth = 1, long long wait_limit = 0,
                                            int *stall_ctr = nullptr) {
   extern __shared__ __align__(16) char smem_dyn[];
+  static_assert(St::bytes() % 16 == 0, "every warp's area is aligned for bulk copies");
   const int warp = threadIdx.x >> 5;
   st.carve(smem_dyn + (size_t)warp * St::bytes());
   st.phase = 0u;
