@@ -188,6 +188,7 @@ __device__ __forceinline__ void dens_pair2(DSum &s, float2 r2, float2 m, float H
 // 3.90 ms, 262k 0.398 -> 0.368 ms.
 constexpr int LQ = 4;
 constexpr int LIST_PAD = 2 * LQ;       // entries past list_cap: the last block's, and its successor's loads
+constexpr int TRANSPOSE_MAX = 20;      // live particles up to which the records go across the lanes
 constexpr float FIRST_MARGIN = 1.05f;  // search margin of a run's first density pass (at least)
 __device__ __forceinline__ float entry_r2(float e) { return e; }
 __device__ __forceinline__ float entry_r2(float2 e) { return e.x; }
@@ -396,14 +397,8 @@ __device__ void density_group(const View &v, int wg, int slice, int nslices, int
                                    make_float4(xi.x, xi.y, xi.z, Ri));
           }
           const float T2 = Ri * Ri;
-          int ntst = 32 + 1, my_rank = 0;
-          if constexpr (G == 1) {
-            const unsigned vm = __ballot_sync(FULL, gath);
-            ntst = __popc(vm);
-            my_rank = __popc(vm & ((1u << lane) - 1u));
-            if (gath) st.tst[my_rank] = make_float4(xi.x, xi.y, xi.z, T2);
-            __syncwarp();
-          }
+          TestSet ts = {0, 0};
+          if constexpr (G == 1) ts = test_set(st.tst, gath, xi.x, xi.y, xi.z, T2);
           const unsigned nlive = __popc(__ballot_sync(FULL, gath && sub == 0));
           // accept mask of the staged records base+kb .. base+kb+31 for this lane
           // (a staging buffer holds a multiple of 32 records, so the block
@@ -411,28 +406,15 @@ __device__ void density_group(const View &v, int wg, int slice, int nslices, int
           auto test_block = [&](int base, int total, int kb) -> unsigned {
             unsigned mask = 0u;
             const unsigned bvalid = total - kb >= 32 ? FULL : (1u << (total - kb)) - 1u;
-            if (G == 1 && ntst <= TRANSPOSE_MAX) {
-              const float4 pj = st.rec[base + kb + lane];
-              const float2 px = make_float2(pj.x, pj.x), py = make_float2(pj.y, pj.y),
-                           pz = make_float2(pj.z, pj.z);
-              int q = 0;
-#pragma unroll 2
-              for (; q + 1 < ntst; q += 2) {  // two live particles per packed test
-                const float4 t0 = st.tst[q], t1 = st.tst[q + 1];
-                const float2 r2 = dist2_x2(make_float2(t0.x, t1.x), make_float2(t0.y, t1.y),
-                                           make_float2(t0.z, t1.z), px, py, pz);
-                const unsigned m0 = __ballot_sync(FULL, r2.x < t0.w);
-                const unsigned m1 = __ballot_sync(FULL, r2.y < t1.w);
-                if (q == my_rank) mask = m0;
-                if (q + 1 == my_rank) mask = m1;
-              }
-              if (q < ntst) {
-                const float4 t = st.tst[q];
-                const float dx = t.x - pj.x, dy = t.y - pj.y, dz = t.z - pj.z;
-                const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                const unsigned m = __ballot_sync(FULL, r2 < t.w);
-                if (q == my_rank) mask = m;
-              }
+            // (with more live particles each lane tests the 32 records itself: no
+            // votes; this loop is slower with either form alone, 18.7 ms at
+            // 16.8M particles with the vote form for every count)
+            if (G == 1 && ts.n <= TRANSPOSE_MAX) {
+              unsigned *const masks = reinterpret_cast<unsigned *>(st.recj);  // (no tags here)
+              test_masks<false>(st.tst, ts.n, st.rec[base + kb + lane], true, masks);
+              __syncwarp();
+              mask = masks[ts.rank];
+              __syncwarp();
             } else if (G == 1) {
               const float2 xx = make_float2(xi.x, xi.x), yy = make_float2(xi.y, xi.y),
                            zz = make_float2(xi.z, xi.z);
@@ -809,58 +791,9 @@ __device__ void force_group(const View &v, int wg, int slice, int nslices, int b
       const float R = fmaxf(Hs, loc.w) + ceps;
       return box_gap2(clx, cly, clz, chx, chy, chz, loc, v.chunk_hi[gg], sx, sy, sz) < R * R;
     };
-    // the valid particles of the round, for the transposed candidate test
-    int ntst = 32 + 1, my_rank = 0;
-    if constexpr (G == 1) {
-      const unsigned vm = __ballot_sync(FULL, valid);
-      ntst = __popc(vm);
-      my_rank = __popc(vm & ((1u << lane) - 1u));
-      if (valid) st.tst[my_rank] = make_float4(xi.x, xi.y, xi.z, Hi2);
-      __syncwarp();
-    }
+    TestSet ts = {0, 0};
+    if constexpr (G == 1) ts = test_set(st.tst, valid, xi.x, xi.y, xi.z, Hi2);
     const unsigned nlive = __popc(__ballot_sync(FULL, valid && sub == 0));
-    // accept mask of the staged records kb .. kb+31 for this lane's particle
-    // (each record tested against the batch's end: reading the block whole
-    // and masking the tail, as the density loop does, measured slower here)
-    auto test_block = [&](int base, int total, int kb) -> unsigned {
-      unsigned mask = 0u;
-      // (one lane per particle: always the transposed form here -- with its
-      // test on the record's support as well, it measured faster than the
-      // per-lane form for every count of live particles)
-      if (G == 1) {
-        const bool in = kb + lane < total;
-        const float4 pj = sx_rec[min(base + kb + lane, S_PAIR - 1)];
-        const float Hj2 = pj.w * pj.w;
-        const float2 px = make_float2(pj.x, pj.x), py = make_float2(pj.y, pj.y),
-                     pz = make_float2(pj.z, pj.z);
-        int q = 0;
-        for (; q + 1 < ntst; q += 2) {  // two valid particles per packed test
-          const float4 t0 = st.tst[q], t1 = st.tst[q + 1];
-          const float2 r2 = dist2_x2(make_float2(t0.x, t1.x), make_float2(t0.y, t1.y),
-                                     make_float2(t0.z, t1.z), px, py, pz);
-          const unsigned m0 = __ballot_sync(FULL, in && (r2.x < t0.w || r2.x < Hj2));
-          const unsigned m1 = __ballot_sync(FULL, in && (r2.y < t1.w || r2.y < Hj2));
-          if (q == my_rank) mask = m0;
-          if (q + 1 == my_rank) mask = m1;
-        }
-        if (q < ntst) {
-          const float4 t = st.tst[q];
-          const float dx = t.x - pj.x, dy = t.y - pj.y, dz = t.z - pj.z;
-          const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-          const unsigned m = __ballot_sync(FULL, in && (r2 < t.w || r2 < Hj2));
-          if (q == my_rank) mask = m;
-        }
-      } else {
-#pragma unroll
-        for (int u = sub; u < 32; u += G) {
-          const float4 pj = sx_rec[min(base + kb + u, S_PAIR - 1)];
-          const float dx = xi.x - pj.x, dy = xi.y - pj.y, dz = xi.z - pj.z;
-          const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-          mask |= (kb + u < total && (r2 < Hi2 || r2 < pj.w * pj.w)) ? (1u << u) : 0u;
-        }
-      }
-      return mask;
-    };
     auto consume = [&](int base, int total) {
       wc.cand += (unsigned long long)total * nlive;
       // The whole batch's accept masks, then each lane through its particle's
@@ -873,25 +806,39 @@ __device__ void force_group(const View &v, int wg, int slice, int nslices, int b
       // 64 and without the packed sums: 21.5); 2.1M clustered 4.21 -> 3.76 ms;
       // with the variants 390 -> 270 us at 111k.  The pairs spread over all
       // lanes, each owner adding its own up afterwards: 22.3 ms at 16.8M.
-      int left = 0;
       const int wend = (total + 31) >> 5;
 #pragma unroll 1
       for (int q = 0; q < wend; q++) {
-        unsigned m = test_block(base, total, 32 * q);
-        if (!valid) m = 0u;
-        st.mask[q * 32 + lane] = m;
-        left += __popc(m);
+        if constexpr (G == 1) {
+          const float4 pj = sx_rec[min(base + 32 * q + lane, S_PAIR - 1)];
+          test_masks<true>(st.tst, ts.n, pj, 32 * q + lane < total, st.mask + 32 * q);
+        } else {
+          unsigned m = 0u;
+#pragma unroll
+          for (int u = sub; u < 32; u += G) {
+            const float4 pj = sx_rec[min(base + 32 * q + u, S_PAIR - 1)];
+            const float dx = xi.x - pj.x, dy = xi.y - pj.y, dz = xi.z - pj.z;
+            const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+            m |= (32 * q + u < total && (r2 < Hi2 || r2 < pj.w * pj.w)) ? (1u << u) : 0u;
+          }
+          st.mask[32 * q + lane] = m;
+        }
       }
+      __syncwarp();
+      const unsigned *const mask = st.mask + (G == 1 ? ts.rank : lane);
+      int left = 0;
+      if (valid)
+        for (int q = 0; q < wend; q++) left += __popc(mask[32 * q]);
       // (the particle itself is accepted too: r = 0, it adds nothing but the
       // signal velocity 2 c_i, the start value; one count subtracted below)
       cnt += left;
       int kb = base - 1, q = 0;
-      unsigned cur = st.mask[lane];
+      unsigned cur = mask[0];
       for (; left > 0; left--) {
         while (cur == 0u) {
           q++;
           kb += 32;
-          cur = st.mask[q * 32 + lane];
+          cur = mask[32 * q];
         }
         const int k = kb + __ffs(cur);
         cur &= cur - 1;
@@ -1058,8 +1005,7 @@ __device__ void gradient_group(const View &v, int wg, int m_act, const CellFrame
   const float nHi4 = KERNEL_NORM * Hinv * Hinv * Hinv * Hinv;
   const float Hs = warp_max(valid ? xi.w : 0.0f);
   const int nsph = compact_spheres(st.sph, valid, make_float4(xi.x, xi.y, xi.z, xi.w));
-  if (valid) st.tst[lane] = make_float4(xi.x, xi.y, xi.z, Hi2);
-  __syncwarp();
+  const TestSet ts = test_set(st.tst, valid, xi.x, xi.y, xi.z, Hi2);
   float d_hi = 0.f, d_lo = 0.f, x_hi = 0.f, x_lo = 0.f, y_hi = 0.f, y_lo = 0.f, z_hi = 0.f,
         z_lo = 0.f;
   float pd = 0.f, px = 0.f, py = 0.f, pz = 0.f;
@@ -1068,35 +1014,21 @@ __device__ void gradient_group(const View &v, int wg, int m_act, const CellFrame
     wc.cand += (unsigned long long)total * (unsigned long long)nact;
     // accept masks of the whole batch (as the force loop), the records across
     // the lanes, two particles per packed test
-    int left = 0;
     const int wend = (total + 31) >> 5;
 #pragma unroll 1
-    for (int w = 0; w < wend; w++) {
-      const bool in = 32 * w + lane < total;
-      const float4 pj = sx_rec[min(base + 32 * w + lane, S_GRAD - 1)];
-      const float2 qx = make_float2(pj.x, pj.x), qy = make_float2(pj.y, pj.y),
-                   qz = make_float2(pj.z, pj.z);
-      unsigned m = 0u;
-      for (int q = 0; q < nact; q += 2) {
-        const float4 t0 = st.tst[q], t1 = st.tst[min(q + 1, nact - 1)];
-        const float2 r2 = dist2_x2(make_float2(t0.x, t1.x), make_float2(t0.y, t1.y),
-                                   make_float2(t0.z, t1.z), qx, qy, qz);
-        const unsigned m0 = __ballot_sync(FULL, in && r2.x < t0.w);
-        const unsigned m1 = __ballot_sync(FULL, in && r2.y < t1.w);
-        if (q == lane) m = m0;
-        if (q + 1 == lane) m = m1;
-      }
-      if (!valid) m = 0u;
-      st.mask[w * 32 + lane] = m;
-      left += __popc(m);
-    }
-    int kb = base - 1, w = 0;
-    unsigned mask = st.mask[lane];
+    for (int w = 0; w < wend; w++)
+      test_masks<false>(st.tst, ts.n, sx_rec[min(base + 32 * w + lane, S_GRAD - 1)],
+                        32 * w + lane < total, st.mask + 32 * w);
+    __syncwarp();
+    int left = 0, kb = base - 1, w = 0;
+    if (valid)
+      for (int q = 0; q < wend; q++) left += __popc(st.mask[32 * q + ts.rank]);
+    unsigned mask = st.mask[ts.rank];
     for (; left > 0; left--) {
       while (mask == 0u) {
         w++;
         kb += 32;
-        mask = st.mask[w * 32 + lane];
+        mask = st.mask[w * 32 + ts.rank];
       }
       const int k = kb + __ffs(mask);
       mask &= mask - 1;
