@@ -1054,16 +1054,7 @@ cudaError_t launch_adj_step(const View &v, const AdjWork &w, const sph_particles
                             const sph_particles &post, const sph_adjoint &adj, long long ti,
                             int first, int grid_pairs, cudaStream_t st) {
   if (v.n == 0) return cudaSuccess;
-  cudaError_t e;
-  if ((e = cudaFuncSetAttribute(k_adj_force, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)ADJ_FORCE_SMEM)) != cudaSuccess)
-    return e;
-  if ((e = cudaFuncSetAttribute(k_adj_density<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)ADJ_DENS_SMEM)) != cudaSuccess)
-    return e;
-  if ((e = cudaFuncSetAttribute(k_adj_density<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)ADJ_DENS_SMEM)) != cudaSuccess)
-    return e;
+  // (the pair kernels' shared memory is set by adj_blocks_per_sm)
   const int g = grid_for(v.n);
   note_launches(6);
   k_adj_gather<<<g, 256, 0, st>>>(v, w, adj, v.gamma);

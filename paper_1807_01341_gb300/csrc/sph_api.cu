@@ -109,6 +109,8 @@ struct sph_ctx {
   long long rebuilds = 0, redone = 0;
   long long steps_seen = 0;    // device step counter at the last sph_step_sync
   int pending = 0;             // steps enqueued since the last sph_step_sync
+  bool fresh = false;          // the host mirror of the device state is current (nothing that
+                               // changes it was enqueued since sph_step_sync read it)
   bool init_pending = false;   // the entropy-initialising step is enqueued, not yet confirmed
   // optional CUDA-event timing of the pair-loop launches (0 density, 1 force)
   bool prof_on = false;
@@ -357,6 +359,7 @@ void prof_collect(sph_ctx *ctx) {
 
 int build_cells(sph_ctx *ctx, sph_particles *p, cudaStream_t st) {
   if (!valid_particles(ctx, p)) return SPH_ERR_ARG;
+  ctx->fresh = false;
   Buffers &b = ctx->b;
   const long long n = p->n;
   if (n > BUILD_MAX) return SPH_ERR_CUDA;
@@ -402,6 +405,16 @@ int build_cells(sph_ctx *ctx, sph_particles *p, cudaStream_t st) {
   ctx->w = w;
   ctx->built = true;
   ctx->rebuilds++;
+  return SPH_OK;
+}
+
+// Sets the current and next tick (ti >= 0) and clears the status, one launch.
+int set_state(sph_ctx *ctx, long long ti, bool clear, cudaStream_t st) {
+  ctx->fresh = false;
+  SPH_CUDA(launch_set_state(ctx->b.ds, ti, clear, st));
+  // (a halted step may have left wake requests that its close never applied)
+  if (clear && ctx->prm.limiter && ctx->n_max > 0)
+    SPH_CUDA(cudaMemsetAsync(ctx->b.wake_bin, 0x7f, sizeof(int32_t) * (size_t)ctx->n_max, st));
   return SPH_OK;
 }
 
@@ -463,11 +476,11 @@ int plain_body(sph_ctx *ctx, const View &v, int flags, cudaStream_t st) {
   return SPH_OK;
 }
 
-// After a halted step: rebuild with wider cells when the cells overflowed.
+// After a halted step (its state just read): rebuild with wider cells when the
+// cells overflowed.
 int recover(sph_ctx *ctx, sph_particles *p, cudaStream_t st, bool *redo) {
   *redo = false;
-  SPH_TRY(read_state(ctx, st));
-  const DevState &h = *ctx->b.h_ds;
+  const DevState h = *ctx->b.h_ds;
   if (!h.halt) return SPH_OK;
   if (h.first_error != SPH_ERR_CELL_OVERFLOW) return h.first_error ? h.first_error : SPH_ERR_CUDA;
   // the cells are too small for the supports: rebuild.  When an h iteration
@@ -790,6 +803,7 @@ int sph_grid_info(const sph_ctx *ctx, int *nc, int *n_leaves) {
 
 int sph_mark_active(sph_ctx *ctx, sph_particles *p, int64_t ti_current, void *stream) {
   if (!ctx || !valid_particles(ctx, p)) return SPH_ERR_ARG;
+  ctx->fresh = false;
   if (!ctx->built) return SPH_ERR_NOT_BUILT;
   SPH_CUDA(launch_mark(make_view(ctx, p), ti_current < 0 ? -1 : ti_current, S(stream)));
   return SPH_OK;
@@ -797,6 +811,7 @@ int sph_mark_active(sph_ctx *ctx, sph_particles *p, int64_t ti_current, void *st
 
 int sph_kick_drift(sph_ctx *ctx, sph_particles *p, int phase, void *stream) {
   if (!ctx || !valid_particles(ctx, p)) return SPH_ERR_ARG;
+  ctx->fresh = false;
   if (!ctx->built) return SPH_ERR_NOT_BUILT;
   View v = make_view(ctx, p);
   switch (phase) {
@@ -810,6 +825,7 @@ int sph_kick_drift(sph_ctx *ctx, sph_particles *p, int phase, void *stream) {
 
 int sph_density_active(sph_ctx *ctx, sph_particles *p, int flags, void *stream) {
   if (!ctx || !valid_particles(ctx, p)) return SPH_ERR_ARG;
+  ctx->fresh = false;
   if (!ctx->built) return SPH_ERR_NOT_BUILT;
   View v = make_view(ctx, p);
   SPH_CUDA(launch_density(v, flags, -1, true, ctx->grid_dens, S(stream)));
@@ -821,6 +837,7 @@ int sph_density_active(sph_ctx *ctx, sph_particles *p, int flags, void *stream) 
 
 int sph_force_active(sph_ctx *ctx, sph_particles *p, void *stream) {
   if (!ctx || !valid_particles(ctx, p)) return SPH_ERR_ARG;
+  ctx->fresh = false;
   if (!ctx->built) return SPH_ERR_NOT_BUILT;
   SPH_CUDA(launch_force(make_view(ctx, p), -1, true, ctx->grid_force, S(stream)));
   return SPH_OK;
@@ -828,6 +845,7 @@ int sph_force_active(sph_ctx *ctx, sph_particles *p, void *stream) {
 
 int sph_timestep_bins(sph_ctx *ctx, sph_particles *p, int64_t *ti_next_dev, void *stream) {
   if (!ctx || !valid_particles(ctx, p)) return SPH_ERR_ARG;
+  ctx->fresh = false;
   if (!ctx->built) return SPH_ERR_NOT_BUILT;
   SPH_CUDA(launch_bins(make_view(ctx, p), reinterpret_cast<long long *>(ti_next_dev), 0, S(stream)));
   return SPH_OK;
@@ -835,13 +853,9 @@ int sph_timestep_bins(sph_ctx *ctx, sph_particles *p, int64_t *ti_next_dev, void
 
 int sph_begin_run(sph_ctx *ctx, void *stream) {
   if (!ctx) return SPH_ERR_ARG;
-  cudaStream_t st = S(stream);
-  long long zero = 0;
-  SPH_CUDA(cudaMemcpyAsync(SPH_DS_FIELD(ctx->b.ds, ti), &zero, sizeof(zero), cudaMemcpyHostToDevice, st));
-  SPH_CUDA(cudaMemcpyAsync(SPH_DS_FIELD(ctx->b.ds, ti_next), &zero, sizeof(zero), cudaMemcpyHostToDevice, st));
-  SPH_TRY(sph_clear_status(ctx, stream));
+  SPH_TRY(set_state(ctx, 0, true, S(stream)));
   SPH_TRY(sph_reset_counters(ctx, stream));
-  SPH_CUDA(cudaStreamSynchronize(st));
+  SPH_CUDA(cudaStreamSynchronize(S(stream)));
   ctx->entropy_ready = false;
   ctx->pending = 0;
   ctx->init_pending = false;
@@ -852,6 +866,7 @@ int sph_step_async(sph_ctx *ctx, sph_particles *p, int form, void *stream) {
   if (!ctx || !valid_particles(ctx, p) ||
       (form != SPH_FORM_PLAIN && form != SPH_FORM_BATCHED && form != SPH_FORM_BATCHED_NOGRAPH))
     return SPH_ERR_ARG;
+  ctx->fresh = false;
   cudaStream_t st = S(stream);
   if (!ctx->built) SPH_TRY(build_cells(ctx, p, st));
   View v = make_view(ctx, p);
@@ -894,6 +909,7 @@ int sph_step_sync(sph_ctx *ctx, sph_particles *p, int *completed, void *stream) 
   ctx->pending = 0;
   bool redo = false;
   SPH_TRY(recover(ctx, p, st, &redo));
+  ctx->fresh = !redo;
   return SPH_OK;
 }
 
@@ -922,7 +938,8 @@ int sph_step_graph(sph_ctx *ctx, sph_particles *p, int n_steps, void *stream) {
 
 int sph_get_time(sph_ctx *ctx, int64_t *ti_current, int64_t *ti_next) {
   if (!ctx) return SPH_ERR_ARG;
-  SPH_CUDA(cudaMemcpy(ctx->b.h_ds, ctx->b.ds, sizeof(DevState), cudaMemcpyDeviceToHost));
+  if (!ctx->fresh)
+    SPH_CUDA(cudaMemcpy(ctx->b.h_ds, ctx->b.ds, sizeof(DevState), cudaMemcpyDeviceToHost));
   if (ti_current) *ti_current = ctx->b.h_ds->ti;
   if (ti_next) *ti_next = ctx->b.h_ds->ti_next;
   return SPH_OK;
@@ -930,9 +947,7 @@ int sph_get_time(sph_ctx *ctx, int64_t *ti_current, int64_t *ti_next) {
 
 int sph_set_time(sph_ctx *ctx, int64_t ti_current, void *stream) {
   if (!ctx || ti_current < 0) return SPH_ERR_ARG;
-  long long t = ti_current;
-  SPH_CUDA(cudaMemcpyAsync(SPH_DS_FIELD(ctx->b.ds, ti), &t, sizeof(t), cudaMemcpyHostToDevice, S(stream)));
-  SPH_CUDA(cudaMemcpyAsync(SPH_DS_FIELD(ctx->b.ds, ti_next), &t, sizeof(t), cudaMemcpyHostToDevice, S(stream)));
+  SPH_TRY(set_state(ctx, ti_current, false, S(stream)));
   SPH_CUDA(cudaStreamSynchronize(S(stream)));
   return SPH_OK;
 }
@@ -968,15 +983,7 @@ int sph_get_check_report(sph_ctx *ctx, int *site, int64_t *index, int64_t *bound
 
 int sph_clear_status(sph_ctx *ctx, void *stream) {
   if (!ctx) return SPH_ERR_ARG;
-  cudaStream_t st = S(stream);
-  SPH_CUDA(cudaMemsetAsync(SPH_DS_FIELD(ctx->b.ds, halt), 0, sizeof(unsigned int), st));
-  SPH_CUDA(cudaMemsetAsync(SPH_DS_FIELD(ctx->b.ds, first_error), 0, sizeof(int), st));
-  SPH_CUDA(cudaMemsetAsync(SPH_DS_FIELD(ctx->b.ds, err_count), 0, sizeof(((DevState *)0)->err_count), st));
-  SPH_CUDA(cudaMemsetAsync(SPH_DS_FIELD(ctx->b.ds, check_site), 0, sizeof(int), st));
-  // (a halted step may have left wake requests that its close never applied)
-  if (ctx->n_max > 0)
-    SPH_CUDA(cudaMemsetAsync(ctx->b.wake_bin, 0x7f, sizeof(int32_t) * (size_t)ctx->n_max, st));
-  return SPH_OK;
+  return set_state(ctx, -1, true, S(stream));
 }
 
 int sph_get_counters(sph_ctx *ctx, sph_counters *out) {
@@ -1012,6 +1019,7 @@ int sph_get_bin_counts(sph_ctx *ctx, int64_t *counts, int n_bins, void *stream) 
 int sph_reset_counters(sph_ctx *ctx, void *stream) {
   if (!ctx) return SPH_ERR_ARG;
   cudaStream_t st = S(stream);
+  ctx->fresh = false;
   const size_t off = offsetof(DevState, s_pairs_density);
   const size_t len = offsetof(DevState, bin_count) - off;
   SPH_CUDA(cudaMemsetAsync(reinterpret_cast<char *>(ctx->b.ds) + off, 0, len, st));
@@ -1064,8 +1072,7 @@ int sph_state_copy(const sph_ctx *ctx, const sph_particles *src, sph_particles *
 
 int sph_resume(sph_ctx *ctx, sph_particles *p, int64_t ti_current, int first, void *stream) {
   if (!ctx || !valid_particles(ctx, p) || ti_current < 0) return SPH_ERR_ARG;
-  SPH_TRY(sph_set_time(ctx, ti_current, stream));
-  SPH_TRY(sph_clear_status(ctx, stream));
+  SPH_TRY(set_state(ctx, ti_current, true, S(stream)));
   SPH_CUDA(cudaStreamSynchronize(S(stream)));
   ctx->built = false;  // a new input order: the next step rebuilds, the permutation restarts
   ctx->entropy_ready = !first;

@@ -128,6 +128,16 @@ __global__ void k_begin_step(View v, long long ti_arg) {
   ds->s_gathers_density = ds->s_list_overflows = ds->s_evals_density = 0ull;
 }
 
+__global__ void k_set_state(DevState *ds, long long ti, int clear) {
+  if (ti >= 0) ds->ti = ds->ti_next = ti;
+  if (clear) {
+    ds->halt = 0u;
+    ds->first_error = 0;
+    for (int k = 0; k < 16; k++) ds->err_count[k] = 0ull;
+    ds->check_site = 0;
+  }
+}
+
 // One thread per leaf: a leaf holds active particles when its smallest bin is
 // active.  Queues the leaf, and the first leaf of each cell queues the cell.
 __global__ void k_mark_leaves(View v) {
@@ -838,6 +848,12 @@ __global__ void k_diag_final(const double *partials, int nblocks, double *out) {
 cudaError_t launch_refresh_all(const View &v, cudaStream_t st) {
   note_launches(1);
   k_refresh<<<4 * v.grid_util, 128, 0, st>>>(v);  // (as k_drift)
+  return cudaGetLastError();
+}
+
+cudaError_t launch_set_state(DevState *ds, long long ti, bool clear, cudaStream_t st) {
+  note_launches(1);
+  k_set_state<<<1, 1, 0, st>>>(ds, ti, clear ? 1 : 0);
   return cudaGetLastError();
 }
 

@@ -379,6 +379,8 @@ cudaError_t launch_build(const View &v, const BuildArrays &b, int nc, double w, 
                          bool first, cudaStream_t st);
 // sph_integrate.cu
 cudaError_t launch_refresh_all(const View &v, cudaStream_t st);
+// current and next tick (ti >= 0); clear: the status and the check report
+cudaError_t launch_set_state(DevState *ds, long long ti, bool clear, cudaStream_t st);
 cudaError_t launch_mark(const View &v, long long ti_or_neg, cudaStream_t st);
 cudaError_t launch_drift(const View &v, cudaStream_t st);
 cudaError_t launch_kick(const View &v, int phase, cudaStream_t st);
