@@ -1456,13 +1456,17 @@ __global__ void __launch_bounds__(PT) k_group_cost(View v) {
         }
       }
     }
-    for (unsigned big = __ballot_sync(FULL, nch > 0); big; big &= big - 1u) {
-      const int q = __ffs(big) - 1;
-      const int c0 = __shfl_sync(FULL, g0, q), cn = __shfl_sync(FULL, nch, q);
+    // the large cells' chunks, 32 at a time over all of them
+    const int cstart = warp_incl_scan(nch) - nch;
+    const int T = __shfl_sync(FULL, cstart + nch, 26);
+    for (int t0 = 0; t0 < T; t0 += 32) {
+      const int t = t0 + lane;
+      const int q = seg_of(cstart, 27, min(t, T - 1));
+      const int c = __shfl_sync(FULL, g0, q) + t - __shfl_sync(FULL, cstart, q);
       const float sx = (q / 9 - 1) * F.wf, sy = ((q / 3) % 3 - 1) * F.wf, sz = (q % 3 - 1) * F.wf;
-      for (int c = c0 + lane; c < c0 + cn; c += 32)
-        if (box_gap2(clx, cly, clz, chx, chy, chz, v.chunk_lo[c], v.chunk_hi[c], sx, sy, sz) < Rc * Rc)
-          count += v.leaf_start[v.chunk_leaf_start[c + 1]] - v.leaf_start[v.chunk_leaf_start[c]];
+      if (t < T &&
+          box_gap2(clx, cly, clz, chx, chy, chz, v.chunk_lo[c], v.chunk_hi[c], sx, sy, sz) < Rc * Rc)
+        count += v.leaf_start[v.chunk_leaf_start[c + 1]] - v.leaf_start[v.chunk_leaf_start[c]];
     }
     const int c = __reduce_add_sync(FULL, count);  // (at most 2^24 particles)
     if (lane == 0) v.group_cost[g] = c;
