@@ -165,11 +165,23 @@ __global__ void k_adj_gather(View v, AdjWork w, sph_adjoint adj, double gamma) {
 //    chunks with its index modulo 8) and combine the particle's own sums in
 //    warp order through the start of their staging buffers
 // ---------------------------------------------------------------------------
-template <class St = StageF>
+// The adjoint loops run the forward loops' scheme: a batch's accept masks
+// first, the records across the lanes, then each lane its own pairs; the FP32
+// values become FP64 by integer instructions (widen).  One step's gradient of
+// 32,768 particles has about as many groups as the chip has warps, so what
+// counts is the longest warp's chain of pairs and their 10 (density: 3) FP64
+// atomics each: 128 records' masks by every lane on its own and conversions at
+// the FP64 rate took 1304 us, now 998 (density passes 325 -> 194 and 507 ->
+// 359).  Two blocks an SM (128 registers) give 1183: their spread of the work
+// is no better and the loop body stalls on its spilled operands.
+constexpr int S_ADJ = 160, S_ADJ_DENS = 256;  // staged records of three arrays, of one
+using StageA = Stage<S_ADJ, 3, 208, true, true>;
+using StageB = Stage<S_ADJ_DENS, 1, 320, true, true>;
+
+template <class St = StageA>
 __device__ __forceinline__ double *adj_red_area(int warp) {
   extern __shared__ __align__(16) char smem_dyn[];
-  static_assert(StageF::bytes() % 16 == 0 && S_FORCE * 3 * 16 >= 11 * 32 * 8 &&
-                    StageD::bytes() % 16 == 0 && S_DENS * 16 >= 5 * 32 * 8,
+  static_assert(S_ADJ * 3 * 16 >= 11 * 32 * 8 && S_ADJ_DENS * 16 >= 5 * 32 * 8,
                 "the reduction areas fit the start of a staging buffer");
   return reinterpret_cast<double *>(smem_dyn + (size_t)warp * St::bytes());
 }
@@ -201,7 +213,7 @@ __device__ __forceinline__ void coop_reduce(double (&part)[N], bool &failed) {
 
 template <bool COOP>
 __device__ void force_adj_group(const View &v, const AdjWork &w, int wg, const CellFrame &F,
-                                StageF &st, WarpCounters &wc) {
+                                StageA &st, WarpCounters &wc) {
   const int lane = lane_id();
   const int warp = threadIdx.x >> 5;
   const Group Wg = group_of(v, wg, F);
@@ -214,7 +226,7 @@ __device__ void force_adj_group(const View &v, const AdjWork &w, int wg, const C
   const float ceps = 1e-5f * F.wf;
   const float alpha = (float)v.alpha;
   const float4 *srcs[3] = {v.rec_xH, v.rec_v, v.rec_h};
-  const float4 *sx_rec = st.rec, *sv_rec = st.rec + S_FORCE, *sh_rec = st.rec + 2 * S_FORCE;
+  const float4 *sx_rec = st.rec, *sv_rec = st.rec + S_ADJ, *sh_rec = st.rec + 2 * S_ADJ;
   // one round: a work group holds at most 32 particles
   const bool valid = lane < nact;
   const int i = valid ? st.act[lane] : a;
@@ -235,6 +247,7 @@ __device__ void force_adj_group(const View &v, const AdjWork &w, int wg, const C
                          : 0.0f;
   const bool live = valid && (abx != 0.0f || aby != 0.0f || abz != 0.0f || Bi != 0.0f);
   const int nsph = compact_spheres(st.sph, live, make_float4(xi.x, xi.y, xi.z, xi.w));
+  const TestSet ts = test_set(st.tst, live, xi.x, xi.y, xi.z, Hi2);
   // the particle's own adjoint sums: FP32 partial sums per neighbour cell,
   // folded into FP64 where the cell changes (FP64 arithmetic is scarce)
   double dxi = 0.0, dyi = 0.0, dzi = 0.0, dvxi = 0.0, dvyi = 0.0, dvzi = 0.0;
@@ -243,9 +256,9 @@ __device__ void force_adj_group(const View &v, const AdjWork &w, int wg, const C
   float pH = 0.f, pQ = 0.f, pc = 0.f, pr = 0.f;
   int cur = -1;
   auto fold_cell = [&]() {
-    dxi += (double)pdx; dyi += (double)pdy; dzi += (double)pdz;
-    dvxi += (double)pvx; dvyi += (double)pvy; dvzi += (double)pvz;
-    Hbi += (double)pH; Qbi += (double)pQ; cbi += (double)pc; rbi += (double)pr;
+    dxi += widen(pdx); dyi += widen(pdy); dzi += widen(pdz);
+    dvxi += widen(pvx); dvyi += widen(pvy); dvzi += widen(pvz);
+    Hbi += widen(pH); Qbi += widen(pQ); cbi += widen(pc); rbi += widen(pr);
     pdx = pdy = pdz = pvx = pvy = pvz = pH = pQ = pc = pr = 0.f;
   };
   auto leaf_ok = [&](int l, float sx, float sy, float sz, LeafBox &lb) {
@@ -261,93 +274,97 @@ __device__ void force_adj_group(const View &v, const AdjWork &w, int wg, const C
     return box_gap2(clx, cly, clz, chx, chy, chz, loc, v.chunk_hi[gg], sx, sy, sz) < R * R;
   };
   auto consume = [&](int base, int total) {
-    const int end = base + total;
-    for (int k0 = base; k0 < end; k0 += 32) {
-      unsigned mask = 0u;
-#pragma unroll
-      for (int u = 0; u < 32; u++) {
-        const float4 pj = sx_rec[min(k0 + u, S_FORCE - 1)];
-        const float dx = xi.x - pj.x, dy = xi.y - pj.y, dz = xi.z - pj.z;
-        const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-        mask |= (k0 + u < end && (r2 < Hi2 || r2 < pj.w * pj.w)) ? (1u << u) : 0u;
+    // accept masks of the whole batch (as the forward force loop)
+    const int wend = (total + 31) >> 5;
+#pragma unroll 1
+    for (int q = 0; q < wend; q++)
+      test_masks<true>(st.tst, ts.n, sx_rec[min(base + 32 * q + lane, S_ADJ - 1)],
+                       32 * q + lane < total, st.mask + 32 * q);
+    __syncwarp();
+    int left = 0, k0 = base - 1, word = 0;
+    if (live)
+      for (int q = 0; q < wend; q++) left += __popc(st.mask[32 * q + ts.rank]);
+    unsigned mask = st.mask[ts.rank];
+    for (; left > 0; left--) {
+      while (mask == 0u) {
+        word++;
+        k0 += 32;
+        mask = st.mask[32 * word + ts.rank];
       }
-      if (!live) mask = 0u;
-      while (mask) {
-        const int k = k0 + __ffs(mask) - 1;
-        mask &= mask - 1;
-        const int j = st.recj[k];
-        if (j == i) continue;
-        const int ci = st.recc[k];
-        if (ci != cur) {
-          fold_cell();
-          cur = ci;
-        }
-        const float4 pj = sx_rec[k];
-        const float4 vj = sv_rec[k];
-        const float4 hj = sh_rec[k];
-        const float dx = xi.x - pj.x, dy = xi.y - pj.y, dz = xi.z - pj.z;
-        const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-        if (!(r2 > 0.0f)) continue;  // coincident: no direction, no gradient
-        const float rinv = rsqrtf(r2);
-        const float r = r2 * rinv;
-        const float qi = r * hi4.w, qj = r * hj.w;
-        const float hj2 = hj.w * hj.w;
-        const float nHj4 = KERNEL_NORM * hj2 * hj2;
-        const float wpi = qi < 1.0f ? kernel_dw(qi) : 0.0f;
-        const float wpj = qj < 1.0f ? kernel_dw(qj) : 0.0f;
-        const float wppi = qi < 1.0f ? kernel_d2w(qi) : 0.0f;
-        const float wppj = qj < 1.0f ? kernel_d2w(qj) : 0.0f;
-        const float dWi = wpi * nHi4, dWj = wpj * nHj4;
-        const float dvx = vi.x - vj.x, dvy = vi.y - vj.y, dvz = vi.z - vj.z;
-        const float dvdr = fmaf(dvx, dx, fmaf(dvy, dy, dvz * dz));
-        const float uu = dvdr * rinv;
-        const float wij = fminf(0.0f, uu);
-        const float vsij = hi4.z + hj.z - 3.0f * wij;
-        const float rs = hi4.x + hj.x;
-        const float Pi = -alpha * vsij * wij / rs;
-        const float Wb = 0.5f * (dWi + dWj);
-        const float K = fmaf(hi4.y, dWi, fmaf(hj.y, dWj, Pi * Wb));
-        const float mj = vj.w;
-        const float gdot = fmaf(abx, dx, fmaf(aby, dy, abz * dz));
-        // the pair's share of the loss: -m_j K / r (abar . d) + B m_j Pi Wb u
-        const float Kb = -mj * rinv * gdot;
-        const float Pib = fmaf(Kb, Wb, Bi * mj * Wb * uu);
-        const float Wbb = fmaf(Kb, Pi, Bi * mj * Pi * uu);
-        float ub = Bi * mj * Pi * Wb;
-        const float dWib = fmaf(Kb, hi4.y, 0.5f * Wbb);
-        const float dWjb = fmaf(Kb, hj.y, 0.5f * Wbb);
-        const float cpart = Pib * (-alpha * wij / rs);
-        const float rpart = Pib * (-Pi / rs);
-        if (uu < 0.0f) ub = fmaf(Pib, -alpha * (vsij - 3.0f * wij) / rs, ub);
-        const float rinvb = fmaf(-mj * K, gdot, ub * dvdr);
-        // dW/dr and dW/dH of each smoothing length (q w'' + 4 w' over H^5)
-        const float rb = fmaf(dWib, wppi * nHi4 * hi4.w,
-                              fmaf(dWjb, wppj * nHj4 * hj.w, -rinvb * rinv * rinv));
-        const float Hib = -dWib * fmaf(qi, wppi, 4.0f * wpi) * nHi4 * hi4.w;
-        const float Hjb = -dWjb * fmaf(qj, wppj, 4.0f * wpj) * nHj4 * hj.w;
-        const float gK = -mj * K * rinv;
-        const float ex = dx * rinv, ey = dy * rinv, ez = dz * rinv;
-        const float bx = fmaf(gK, abx, fmaf(ub * rinv, dvx, rb * ex));
-        const float by = fmaf(gK, aby, fmaf(ub * rinv, dvy, rb * ey));
-        const float bz = fmaf(gK, abz, fmaf(ub * rinv, dvz, rb * ez));
-        const float vbx = ub * ex, vby = ub * ey, vbz = ub * ez;
-        pdx += bx; pdy += by; pdz += bz;
-        pvx += vbx; pvy += vby; pvz += vbz;
-        pH += Hib;
-        pQ += Kb * dWi;
-        pc += cpart;
-        pr += rpart;
-        atomicAdd(&w.xb[j], -(double)bx);
-        atomicAdd(&w.yb[j], -(double)by);
-        atomicAdd(&w.zb[j], -(double)bz);
-        atomicAdd(&w.vpxb[j], -(double)vbx);
-        atomicAdd(&w.vpyb[j], -(double)vby);
-        atomicAdd(&w.vpzb[j], -(double)vbz);
-        atomicAdd(&w.hb[j], (double)GAMMA_K * (double)Hjb);
-        atomicAdd(&w.Qb[j], (double)(Kb * dWj));
-        atomicAdd(&w.cb[j], (double)cpart);
-        atomicAdd(&w.rhob[j], (double)rpart);
+      const int k = k0 + __ffs(mask);
+      mask &= mask - 1;
+      const int j = st.recj[k];
+      if (j == i) continue;
+      const int ci = st.recc[k];
+      if (ci != cur) {
+        fold_cell();
+        cur = ci;
       }
+      const float4 pj = sx_rec[k];
+      const float4 vj = sv_rec[k];
+      const float4 hj = sh_rec[k];
+      const float dx = xi.x - pj.x, dy = xi.y - pj.y, dz = xi.z - pj.z;
+      const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+      if (!(r2 > 0.0f)) continue;  // coincident: no direction, no gradient
+      const float rinv = rsqrtf(r2);
+      const float r = r2 * rinv;
+      const float qi = r * hi4.w, qj = r * hj.w;
+      const float hj2 = hj.w * hj.w;
+      const float nHj4 = KERNEL_NORM * hj2 * hj2;
+      const float wpi = qi < 1.0f ? kernel_dw(qi) : 0.0f;
+      const float wpj = qj < 1.0f ? kernel_dw(qj) : 0.0f;
+      const float wppi = qi < 1.0f ? kernel_d2w(qi) : 0.0f;
+      const float wppj = qj < 1.0f ? kernel_d2w(qj) : 0.0f;
+      const float dWi = wpi * nHi4, dWj = wpj * nHj4;
+      const float dvx = vi.x - vj.x, dvy = vi.y - vj.y, dvz = vi.z - vj.z;
+      const float dvdr = fmaf(dvx, dx, fmaf(dvy, dy, dvz * dz));
+      const float uu = dvdr * rinv;
+      const float wij = fminf(0.0f, uu);
+      const float vsij = hi4.z + hj.z - 3.0f * wij;
+      const float rs = hi4.x + hj.x;
+      const float Pi = -alpha * vsij * wij / rs;
+      const float Wb = 0.5f * (dWi + dWj);
+      const float K = fmaf(hi4.y, dWi, fmaf(hj.y, dWj, Pi * Wb));
+      const float mj = vj.w;
+      const float gdot = fmaf(abx, dx, fmaf(aby, dy, abz * dz));
+      // the pair's share of the loss: -m_j K / r (abar . d) + B m_j Pi Wb u
+      const float Kb = -mj * rinv * gdot;
+      const float Pib = fmaf(Kb, Wb, Bi * mj * Wb * uu);
+      const float Wbb = fmaf(Kb, Pi, Bi * mj * Pi * uu);
+      float ub = Bi * mj * Pi * Wb;
+      const float dWib = fmaf(Kb, hi4.y, 0.5f * Wbb);
+      const float dWjb = fmaf(Kb, hj.y, 0.5f * Wbb);
+      const float cpart = Pib * (-alpha * wij / rs);
+      const float rpart = Pib * (-Pi / rs);
+      if (uu < 0.0f) ub = fmaf(Pib, -alpha * (vsij - 3.0f * wij) / rs, ub);
+      const float rinvb = fmaf(-mj * K, gdot, ub * dvdr);
+      // dW/dr and dW/dH of each smoothing length (q w'' + 4 w' over H^5)
+      const float rb = fmaf(dWib, wppi * nHi4 * hi4.w,
+                            fmaf(dWjb, wppj * nHj4 * hj.w, -rinvb * rinv * rinv));
+      const float Hib = -dWib * fmaf(qi, wppi, 4.0f * wpi) * nHi4 * hi4.w;
+      const float Hjb = -dWjb * fmaf(qj, wppj, 4.0f * wpj) * nHj4 * hj.w;
+      const float gK = -mj * K * rinv;
+      const float ex = dx * rinv, ey = dy * rinv, ez = dz * rinv;
+      const float bx = fmaf(gK, abx, fmaf(ub * rinv, dvx, rb * ex));
+      const float by = fmaf(gK, aby, fmaf(ub * rinv, dvy, rb * ey));
+      const float bz = fmaf(gK, abz, fmaf(ub * rinv, dvz, rb * ez));
+      const float vbx = ub * ex, vby = ub * ey, vbz = ub * ez;
+      pdx += bx; pdy += by; pdz += bz;
+      pvx += vbx; pvy += vby; pvz += vbz;
+      pH += Hib;
+      pQ += Kb * dWi;
+      pc += cpart;
+      pr += rpart;
+      atomicAdd(&w.xb[j], -widen(bx));
+      atomicAdd(&w.yb[j], -widen(by));
+      atomicAdd(&w.zb[j], -widen(bz));
+      atomicAdd(&w.vpxb[j], -widen(vbx));
+      atomicAdd(&w.vpyb[j], -widen(vby));
+      atomicAdd(&w.vpzb[j], -widen(vbz));
+      atomicAdd(&w.hb[j], (double)GAMMA_K * widen(Hjb));
+      atomicAdd(&w.Qb[j], widen(Kb * dWj));
+      atomicAdd(&w.cb[j], widen(cpart));
+      atomicAdd(&w.rhob[j], widen(rpart));
     }
   };
   const Reach reach = {clx, cly, clz, chx, chy, chz,
@@ -356,6 +373,7 @@ __device__ void force_adj_group(const View &v, const AdjWork &w, int wg, const C
   int skip = 0, nlist = 0;
   bool more = false;
   do {
+    if (more) compact_spheres(st.sph, live, make_float4(xi.x, xi.y, xi.z, xi.w));  // (the staging took their room)
     nlist = search(v, F, reach, st, leaf_ok, chunk_ok, skip, more, COOP ? warp : -1);
     stage_list(srcs, st, nlist, consume, wc);
     skip += nlist;
@@ -364,7 +382,7 @@ __device__ void force_adj_group(const View &v, const AdjWork &w, int wg, const C
   if constexpr (COOP) {
     double sum[10] = {dxi, dyi, dzi, dvxi, dvyi, dvzi, Hbi, Qbi, cbi, rbi};
     bool failed = st.failed;
-    coop_reduce<StageF, 10>(sum, failed);
+    coop_reduce<StageA, 10>(sum, failed);
     st.failed = failed;  // the same in every warp
     dxi = sum[0]; dyi = sum[1]; dzi = sum[2];
     dvxi = sum[3]; dvyi = sum[4]; dvzi = sum[5];
@@ -396,7 +414,7 @@ __global__ void __launch_bounds__(PT, 1) k_adj_force(View v, AdjWork w) {
   }
   __syncthreads();
   if (!s_go) return;  // the whole block
-  StageF st;
+  StageA st;
   stage_init(st);
   const int lane = lane_id();
   const int nq = s_nq;
@@ -481,7 +499,7 @@ __global__ void k_adj_eos(View v, AdjWork w, sph_adjoint adj, int first) {
 // Pass 2: every pair's r-derivative r_bar = (ka m_j w' + kb m_j (4 w' + q w'') + km w') / H.
 template <int PASS, bool COOP>
 __device__ void density_adj_group(const View &v, const AdjWork &w, int wg, const CellFrame &F,
-                                  StageD &st, WarpCounters &wc) {
+                                  StageB &st, WarpCounters &wc) {
   const int lane = lane_id();
   const int warp = threadIdx.x >> 5;
   const Group Wg = group_of(v, wg, F);
@@ -515,6 +533,7 @@ __device__ void density_adj_group(const View &v, const AdjWork &w, int wg, const
   }
   const float Hs = warp_max(live ? H : 0.0f);
   const int nsph = compact_spheres(st.sph, live, make_float4(xi.x, xi.y, xi.z, H));
+  const TestSet ts = test_set(st.tst, live, xi.x, xi.y, xi.z, H2);
   // FP32 partial sums per neighbour cell, folded into FP64 where the cell changes
   double sr = 0.0, srt = 0.0, s1 = 0.0, s2 = 0.0;
   double dxi = 0.0, dyi = 0.0, dzi = 0.0;
@@ -522,9 +541,9 @@ __device__ void density_adj_group(const View &v, const AdjWork &w, int wg, const
   int cur = -1;
   auto fold_cell = [&]() {
     if (PASS == 1) {
-      sr += (double)p0; srt += (double)p1; s1 += (double)p2; s2 += (double)p3;
+      sr += widen(p0); srt += widen(p1); s1 += widen(p2); s2 += widen(p3);
     } else {
-      dxi += (double)p0; dyi += (double)p1; dzi += (double)p2;
+      dxi += widen(p0); dyi += widen(p1); dzi += widen(p2);
     }
     p0 = p1 = p2 = p3 = 0.f;
   };
@@ -539,49 +558,53 @@ __device__ void density_adj_group(const View &v, const AdjWork &w, int wg, const
            Rc * Rc;
   };
   auto consume = [&](int base, int total) {
-    const int end = base + total;
-    for (int k0 = base; k0 < end; k0 += 32) {
-      unsigned mask = 0u;
-#pragma unroll
-      for (int u = 0; u < 32; u++) {
-        const float4 pj = st.rec[min(k0 + u, S_DENS - 1)];
-        const float dx = xi.x - pj.x, dy = xi.y - pj.y, dz = xi.z - pj.z;
-        const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-        mask |= (k0 + u < end && r2 < H2) ? (1u << u) : 0u;
+    // accept masks of the whole batch (as the forward force loop)
+    const int wend = (total + 31) >> 5;
+#pragma unroll 1
+    for (int q = 0; q < wend; q++)
+      test_masks<false>(st.tst, ts.n, st.rec[min(base + 32 * q + lane, S_ADJ_DENS - 1)],
+                       32 * q + lane < total, st.mask + 32 * q);
+    __syncwarp();
+    int left = 0, k0 = base - 1, word = 0;
+    if (live)
+      for (int q = 0; q < wend; q++) left += __popc(st.mask[32 * q + ts.rank]);
+    unsigned mask = st.mask[ts.rank];
+    for (; left > 0; left--) {
+      while (mask == 0u) {
+        word++;
+        k0 += 32;
+        mask = st.mask[32 * word + ts.rank];
       }
-      if (!live) mask = 0u;
-      while (mask) {
-        const int k = k0 + __ffs(mask) - 1;
-        mask &= mask - 1;
-        const int j = st.recj[k];
-        const int ci = st.recc[k];
-        if (ci != cur) {
-          fold_cell();
-          cur = ci;
-        }
-        const float4 pj = st.rec[k];
-        const float dx = xi.x - pj.x, dy = xi.y - pj.y, dz = xi.z - pj.z;
-        const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-        const float rr = r2 * rsqrtf(fmaxf(r2, 1e-30f));
-        const float q = rr * Hinv;
-        float wq, dwq;
-        kernel_wd(q, wq, dwq);
-        const float d2 = kernel_d2w(q);
-        if (PASS == 1) {
-          p0 += pj.w * wq;
-          p1 += pj.w * fmaf(q, dwq, 3.0f * wq);
-          p2 += q * dwq;
-          p3 += pj.w * q * fmaf(q, d2, 4.0f * dwq);
-        } else {
-          if (j == i || !(r2 > 0.0f)) continue;
-          const float rbar = (ka * pj.w * dwq + kb * pj.w * fmaf(q, d2, 4.0f * dwq) + km * dwq) * Hinv;
-          const float rinv = rsqrtf(r2);
-          const float bx = rbar * dx * rinv, by = rbar * dy * rinv, bz = rbar * dz * rinv;
-          p0 += bx; p1 += by; p2 += bz;
-          atomicAdd(&w.xb[j], -(double)bx);
-          atomicAdd(&w.yb[j], -(double)by);
-          atomicAdd(&w.zb[j], -(double)bz);
-        }
+      const int k = k0 + __ffs(mask);
+      mask &= mask - 1;
+      const int j = st.recj[k];
+      const int ci = st.recc[k];
+      if (ci != cur) {
+        fold_cell();
+        cur = ci;
+      }
+      const float4 pj = st.rec[k];
+      const float dx = xi.x - pj.x, dy = xi.y - pj.y, dz = xi.z - pj.z;
+      const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+      const float rr = r2 * rsqrtf(fmaxf(r2, 1e-30f));
+      const float q = rr * Hinv;
+      float wq, dwq;
+      kernel_wd(q, wq, dwq);
+      const float d2 = kernel_d2w(q);
+      if (PASS == 1) {
+        p0 += pj.w * wq;
+        p1 += pj.w * fmaf(q, dwq, 3.0f * wq);
+        p2 += q * dwq;
+        p3 += pj.w * q * fmaf(q, d2, 4.0f * dwq);
+      } else {
+        if (j == i || !(r2 > 0.0f)) continue;
+        const float rbar = (ka * pj.w * dwq + kb * pj.w * fmaf(q, d2, 4.0f * dwq) + km * dwq) * Hinv;
+        const float rinv = rsqrtf(r2);
+        const float bx = rbar * dx * rinv, by = rbar * dy * rinv, bz = rbar * dz * rinv;
+        p0 += bx; p1 += by; p2 += bz;
+        atomicAdd(&w.xb[j], -widen(bx));
+        atomicAdd(&w.yb[j], -widen(by));
+        atomicAdd(&w.zb[j], -widen(bz));
       }
     }
   };
@@ -591,6 +614,7 @@ __device__ void density_adj_group(const View &v, const AdjWork &w, int wg, const
                        st.sph, nsph};
   if (Hs > 0.0f) {
     do {
+      if (more) compact_spheres(st.sph, live, make_float4(xi.x, xi.y, xi.z, H));  // (the staging took their room)
       nlist = search(v, F, reach, st, leaf_ok, chunk_ok, skip, more, COOP ? warp : -1);
       stage_list(srcs, st, nlist, consume, wc);
       skip += nlist;
@@ -600,7 +624,7 @@ __device__ void density_adj_group(const View &v, const AdjWork &w, int wg, const
   if constexpr (COOP) {
     double sum[4] = {PASS == 1 ? sr : dxi, PASS == 1 ? srt : dyi, PASS == 1 ? s1 : dzi, s2};
     bool failed = st.failed;
-    coop_reduce<StageD, 4>(sum, failed);
+    coop_reduce<StageB, 4>(sum, failed);
     st.failed = failed;  // the same in every warp
     if (PASS == 1) {
       sr = sum[0]; srt = sum[1]; s1 = sum[2]; s2 = sum[3];
@@ -655,7 +679,7 @@ __global__ void __launch_bounds__(PT, 1) k_adj_density(View v, AdjWork w) {
   }
   __syncthreads();
   if (!s_go) return;  // the whole block
-  StageD st;
+  StageB st;
   stage_init(st);
   const int lane = lane_id();
   const int nq = s_nq;
@@ -739,15 +763,6 @@ __device__ __forceinline__ double shfl_d(double x, int src) {
   return __shfl_sync(FULL, x, src);
 }
 
-// a float as a double, by its bits (normal numbers and 0: the conversion
-// instruction runs at the FP64 rate)
-__device__ __forceinline__ double widen(float f) {
-  const unsigned int b = __float_as_uint(f);
-  if ((b & 0x7f800000u) == 0u) return 0.0;
-  const unsigned int hi = (b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u);
-  return __hiloint2double((int)hi, (int)(b << 29));
-}
-
 // The kernel of one particle (c = m (8/pi) / H^3, hi = 1 / H) at a grid point:
 // offsets in units of H, q2 their square sum, f about the same in FP32.
 // Forward: adds m W to the point.  BWD: adds to acc the point's d loss / d x,
@@ -816,7 +831,7 @@ struct GridKernel {
 // Where at least GD_LANES of a warp's particles have boxes of at most GD_FEW
 // points, those are one lane's work each, all at once: a warp per particle costs
 // some 20 FP64 instructions before its first point (27,000 particles on a 16^3
-// grid: 114 us, at start 75 us; here 74 us).  With 2 or 3 such particles in a
+// grid: 114 us, a lane per particle 75 us; here 74 us).  With 2 or 3 such particles in a
 // warp, clumps on a fine grid, the lanes' own way costs more (111k on 64^3: 737
 // against 462 us).
 constexpr int GD_WARPS = 4, GD_SIDE = 32, GD_FEW = 27, GD_LANES = 16;
@@ -1025,8 +1040,8 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-constexpr size_t ADJ_DENS_SMEM = StageD::bytes() * WARPS_PER_BLOCK;
-constexpr size_t ADJ_FORCE_SMEM = StageF::bytes() * WARPS_PER_BLOCK;
+constexpr size_t ADJ_DENS_SMEM = StageB::bytes() * WARPS_PER_BLOCK;
+constexpr size_t ADJ_FORCE_SMEM = StageA::bytes() * WARPS_PER_BLOCK;
 
 int grid_for(long long n) {
   long long g = (n + 255) / 256;

@@ -34,19 +34,6 @@ __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
 // conversions and the scalings by powers of two below give the same bits from
 // integer instructions; what they do not cover takes the FP64 instruction.
 
-// (double)f
-__device__ __forceinline__ double widen(float f) {
-  const unsigned int b = __float_as_uint(f), a = b & 0x7fffffffu;
-  if (a - 0x00800000u >= 0x7f000000u && a != 0u) return (double)f;  // subnormal, infinite, NaN
-  const unsigned int hi = (b & 0x80000000u) | (a ? (a >> 3) + 0x38000000u : 0u);
-  return __hiloint2double((int)hi, (int)(b << 29));
-}
-
-// (double)k
-__device__ __forceinline__ double widen(long long k) {
-  return k > -(1ll << 24) && k < (1ll << 24) ? widen((float)(int)k) : (double)k;
-}
-
 // (float)d, rounded to nearest even
 __device__ __forceinline__ float narrow(double d) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(d);

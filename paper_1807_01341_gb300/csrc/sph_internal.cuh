@@ -190,6 +190,20 @@ struct AdjWork {
   double *ka, *kb, *km;          // density-adjoint coefficients of the active particles
 };
 
+// (double)f by integer instructions: an FP64 instruction, a conversion among
+// them, holds an SM for 16 cycles (64 issue slots)
+__device__ __forceinline__ double widen(float f) {
+  const unsigned int b = __float_as_uint(f), a = b & 0x7fffffffu;
+  if (a - 0x00800000u >= 0x7f000000u && a != 0u) return (double)f;  // subnormal, infinite, NaN
+  const unsigned int hi = (b & 0x80000000u) | (a ? (a >> 3) + 0x38000000u : 0u);
+  return __hiloint2double((int)hi, (int)(b << 29));
+}
+
+// (double)k
+__device__ __forceinline__ double widen(long long k) {
+  return k > -(1ll << 24) && k < (1ll << 24) ? widen((float)(int)k) : (double)k;
+}
+
 // smallest and largest value of a warp, one instruction (five exchanges otherwise)
 __device__ __forceinline__ float warp_min_f(float x) {
   float r;

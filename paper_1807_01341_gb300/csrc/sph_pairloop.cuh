@@ -15,7 +15,6 @@ namespace {
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int PT = WARPS_PER_BLOCK * 32;
 constexpr int S_DENS = 256;   // staged candidate records per warp, density loop
-constexpr int S_FORCE = 128;  // staged candidates per warp, force loop (3 records each)
 constexpr long long WAIT_LIMIT = 1ll << 22;  // bounded mbarrier wait (iterations)
 
 __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
@@ -810,7 +809,6 @@ __device__ __forceinline__ void stage_list(const float4 *const *srcs,
 }
 
 using StageD = Stage<S_DENS, 1, 320>;
-using StageF = Stage<S_FORCE, 3, 256>;
 // the forward force loop (S_PAIR staged candidates per warp): two blocks of 8
 // warps fill an SM's shared memory (14,464 bytes a warp); the variants' tags
 // cost room for 48 leaves
