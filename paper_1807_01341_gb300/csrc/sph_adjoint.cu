@@ -826,8 +826,9 @@ struct GridKernel {
 // divisions, 45 and more FP64 instructions per point of the whole box.
 // 110,592 particles on a 64^3 grid (113 points in a support): 1885 -> 463 us,
 // backward 3385 -> 787 us; 262,144 on 32^3 209 -> 182 us and 314 -> 220 us;
-// 2,744 on 128^3 (supports of 40,000 points) 153 -> 2.5 ms and 182 -> 4.3 ms; the
-// error against 64-bit sums in another order is 4e-16 to 6e-16 either way.
+// 2,744 on 128^3 (supports of 40,000 points) 153 -> 2.5 ms and 182 -> 4.3 ms.
+// Against extended precision a point's W is off by 4.0e-17 rms (before 4.5e-17),
+// its d/dh by 1.1e-16 (1.5e-16).
 // Where at least GD_LANES of a warp's particles have boxes of at most GD_FEW
 // points, those are one lane's work each, all at once: a warp per particle costs
 // some 20 FP64 instructions before its first point (27,000 particles on a 16^3

@@ -11,9 +11,11 @@
 //
 // A build is a fixed chain of launches whose sizes live on the device (no
 // host read between the keys and the finished structure): keys, one launch
-// per 8-bit digit, one gather of every particle array into scratch and one
+// per 8-bit digit (up to 65,536 particles one for all of them), one gather of every particle array into scratch and one
 // copy back, one pass that splits every octree node and one compaction, for
 // the particles (leaves) and again for the leaves (chunks and work groups).
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cstddef>
 #include <utility>
@@ -408,6 +410,125 @@ __global__ void __launch_bounds__(RS_THREADS, 2)
   for (int r = 0; r < ITEMS; r++) {
     const int p = r * THREADS + tid;
     if (p < count && SPH_IN(ds, pos[r], n, SPH_CHECK_SCATTER)) ovals[pos[r]] = s_vals[p];
+  }
+}
+
+// The same sort of up to 65,536 pairs in one launch: the 8 or 16 blocks of a
+// cluster hold them all in shared memory, a pair in one word (key << 16 |
+// index, so keys of up to 48 bits), every pass within the cluster.  Block c
+// holds the places [c T, (c + 1) T), T = 1024 ITEMS, past the end filled with
+// the largest word, which every digit leaves at the end.  A pass ranks the words as k_rs_pass
+// does, gives its digit counts to every block, orders its words by digit and
+// writes them in runs to their places, the other blocks' shared memory among
+// them; a cluster barrier before the counts are read and one before the words
+// are.  (Keys and indices are read before the first barrier and written after
+// the last: in place.)
+//
+// A small sort is latency: a launch per digit took 7 to 8 us and a gap of 2 us
+// with one to 16 blocks at work, a pass in here takes what its barriers and the
+// votes of its ranking do.  Keys counted to records packed, 5 passes: 4,096
+// pairs 48 -> 24 us, 16,384 52 -> 26, 32,768 53 -> 32, 40,000 52 -> 36, 65,536 (6
+// passes) 65 -> 49.  With 8 blocks for all sizes 40,000 took 56 us and 32,768 37;
+// 16 blocks for 4,096 take 27.  The line is the 16-bit index: keys of more than
+// 48 bits (64 cells an axis) and more pairs take a launch per digit.
+constexpr int RC_THREADS = 1024, RC_INDEX_BITS = 16;
+constexpr int RC_MAX = 16 * RC_THREADS * 4;  // of the largest instance below
+static_assert(RC_MAX <= 1 << RC_INDEX_BITS, "an index has 16 bits");
+template <int BLOCKS, int ITEMS>
+__global__ void __cluster_dims__(BLOCKS, 1, 1) __launch_bounds__(RC_THREADS, 1)
+    k_rs_cluster(unsigned long long *keys, unsigned int *vals, int n, int passes,
+                 const unsigned int *bad, DevState *ds) {
+  namespace cg = cooperative_groups;
+  constexpr int T = RC_THREADS * ITEMS, WARPS = RC_THREADS / 32;
+  extern __shared__ unsigned long long s_words[];  // in order, then by digit of the block
+  unsigned long long *const s_order = s_words, *const s_stage = s_words + T;
+  __shared__ unsigned short s_wcnt[WARPS][RS_DIGITS];
+  __shared__ unsigned int s_all[BLOCKS][RS_DIGITS];  // every block's digit counts
+  __shared__ unsigned int s_lofs[RS_DIGITS], s_gofs[RS_DIGITS], s_sums[33];
+  if (bad && *bad != 0u) return;  // (the whole cluster: an earlier launch wrote it)
+  cg::cluster_group cluster = cg::this_cluster();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int self = (int)cluster.block_rank();
+  unsigned long long word[ITEMS];
+#pragma unroll
+  for (int r = 0; r < ITEMS; r++) {
+    const int o = self * T + warp * (32 * ITEMS) + r * 32 + lane;
+    word[r] = o < n ? keys[o] << RC_INDEX_BITS | (unsigned int)o : ~0ull;
+  }
+  cluster.sync();  // every block runs before its shared memory is written
+  for (int p = 0; p < passes; p++) {
+    const int shift = RC_INDEX_BITS + 8 * p;
+    auto digit = [&](unsigned long long w) { return (unsigned int)(w >> shift) & 255u; };
+    for (int k = lane; k < RS_DIGITS; k += 32) s_wcnt[warp][k] = 0;
+    __syncwarp();
+    unsigned int rank[ITEMS];
+#pragma unroll
+    for (int r = 0; r < ITEMS; r++) {
+      const unsigned int d = digit(word[r]);
+      const unsigned peers = equal_lanes<8>(d);
+      const int leader = __ffs(peers) - 1;
+      unsigned int old = 0u;
+      if (lane == leader) {
+        old = s_wcnt[warp][d];
+        s_wcnt[warp][d] = (unsigned short)(old + __popc(peers));
+      }
+      rank[r] = __shfl_sync(FULL, old, leader) + __popc(peers & ((1u << lane) - 1u));
+      __syncwarp();
+    }
+    __syncthreads();
+    unsigned int mine = 0u;
+    if (tid < RS_DIGITS) {
+#pragma unroll
+      for (int q = 0; q < WARPS; q++) {
+        const unsigned int c = s_wcnt[q][tid];
+        s_wcnt[q][tid] = (unsigned short)mine;
+        mine += c;
+      }
+#pragma unroll
+      for (int b = 0; b < BLOCKS; b++) *cluster.map_shared_rank(&s_all[self][tid], b) = mine;
+    }
+    const unsigned int lofs = block_exclusive<unsigned int>(mine, s_sums, nullptr);
+    cluster.sync();
+    unsigned int tot = 0u, prev = 0u;
+    if (tid < RS_DIGITS) {
+#pragma unroll
+      for (int b = 0; b < BLOCKS; b++) {
+        const unsigned int c = s_all[b][tid];
+        prev += b < self ? c : 0u;
+        tot += c;
+      }
+    }
+    const unsigned int gofs = block_exclusive<unsigned int>(tot, s_sums, nullptr);
+    if (tid < RS_DIGITS) {
+      s_lofs[tid] = lofs;
+      s_gofs[tid] = gofs + prev - lofs;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < ITEMS; r++) {
+      const unsigned int d = digit(word[r]);
+      s_stage[s_lofs[d] + s_wcnt[warp][d] + rank[r]] = word[r];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < ITEMS; r++) {
+      const int k = r * RC_THREADS + tid;
+      const unsigned long long w = s_stage[k];
+      const unsigned int to = s_gofs[digit(w)] + (unsigned int)k;
+      if (SPH_IN(ds, to, BLOCKS * T, SPH_CHECK_SCATTER))
+        *cluster.map_shared_rank(&s_order[to % T], to / T) = w;
+    }
+    cluster.sync();
+#pragma unroll
+    for (int r = 0; r < ITEMS; r++) word[r] = s_order[warp * (32 * ITEMS) + r * 32 + lane];
+  }
+#pragma unroll
+  for (int r = 0; r < ITEMS; r++) {
+    const int o = self * T + warp * (32 * ITEMS) + r * 32 + lane;
+    if (o < n) {
+      keys[o] = word[r] >> RC_INDEX_BITS;
+      vals[o] = (unsigned int)word[r] & ((1u << RC_INDEX_BITS) - 1u);
+    }
   }
 }
 
@@ -952,11 +1073,38 @@ SortWork sort_work(unsigned int *w, int n_tiles) {
   return s;
 }
 
-// every pass; the keys' digits have been counted.  A pass clears the status
-// row that the next one chains on.
+// whether one cluster sorts them (k_rs_cluster)
+inline bool cluster_sorts(int n, int nbits) { return n <= RC_MAX && nbits + RC_INDEX_BITS <= 64; }
+
+template <int BLOCKS, int ITEMS>
+cudaError_t launch_cluster_sort(unsigned long long *keys, unsigned int *vals, int n, int nbits,
+                                const unsigned int *bad, DevState *ds, cudaStream_t st) {
+  const auto kernel = k_rs_cluster<BLOCKS, ITEMS>;
+  constexpr int smem = 2 * RC_THREADS * ITEMS * (int)sizeof(unsigned long long);
+  cudaError_t e =
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e == cudaSuccess && BLOCKS > 8)
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
+  note_launches(1);
+  kernel<<<BLOCKS, RC_THREADS, smem, st>>>(keys, vals, n, passes_of(nbits), bad, ds);
+  return cudaGetLastError();
+}
+
+// Every pass.  Of more pairs than one cluster sorts, the keys' digits have been
+// counted; a pass clears the status row that the next one chains on.
 cudaError_t sort_passes(unsigned long long *const keys[2], unsigned int *const vals[2], int n,
                         int nbits, const SortWork &s, bool *result_in_alt, unsigned int *fail,
                         const unsigned int *bad, DevState *ds, cudaStream_t st) {
+  if (cluster_sorts(n, nbits)) {
+    *result_in_alt = false;
+    const auto sort = n <= 8 * RC_THREADS    ? launch_cluster_sort<8, 1>
+                      : n <= 16 * RC_THREADS ? launch_cluster_sort<16, 1>
+                      : n <= 32 * RC_THREADS ? launch_cluster_sort<16, 2>
+                      : n <= 48 * RC_THREADS ? launch_cluster_sort<16, 3>
+                                             : launch_cluster_sort<16, 4>;
+    return sort(keys[0], vals[0], n, nbits, bad, ds, st);
+  }
   const int passes = passes_of(nbits);
   note_launches(passes);
   for (int p = 0; p < passes; p++) {
@@ -994,8 +1142,10 @@ cudaError_t radix_sort_indices(unsigned long long *keys, unsigned int *vals,
   const SortWork s = sort_work(work, tiles_of(n));
   cudaError_t e = cudaMemsetAsync(s.ticket, 0, s.zero_words * sizeof(unsigned int), st);
   if (e != cudaSuccess) return e;
-  note_launches(1);
-  k_rs_count<<<std::min(blocks_for(n, 256), 1024), 256, 0, st>>>(keys, n, s.totals, passes_of(nbits));
+  if (!cluster_sorts(n, nbits)) {
+    note_launches(1);
+    k_rs_count<<<std::min(blocks_for(n, 256), 1024), 256, 0, st>>>(keys, n, s.totals, passes_of(nbits));
+  }
   unsigned long long *const ks[2] = {keys, keys_alt};
   unsigned int *const vs[2] = {vals, vals_alt};
   return sort_passes(ks, vs, n, nbits, s, result_in_alt, s.fail, nullptr, nullptr, st);
@@ -1035,7 +1185,8 @@ cudaError_t launch_build(const View &v, const BuildArrays &b, int nc, double w, 
   // (1024 / w = 1024 nc / box, rounded once more than a division by w would be:
   // inside the margin of axis_code)
   k_cell_keys<<<std::min(blocks_for(n, 256), v.grid_util), 256, 0, st>>>(
-      v, nc, w, (double)(1 << MORTON_BITS) / w, b.keys[0], s.totals, passes_of(nbits));
+      v, nc, w, (double)(1 << MORTON_BITS) / w, b.keys[0], s.totals,
+      cluster_sorts(n, nbits) ? 0 : passes_of(nbits));
   bool alt = false;
   unsigned int *const vals[2] = {b.vals[0], b.vals[1]};
   unsigned long long *const ks[2] = {b.keys[0], b.keys[1]};

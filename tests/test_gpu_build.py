@@ -107,3 +107,27 @@ def test_order_and_leaves(env, n, nc, leaf_max, kind):
     ctx.build_cells(p)
     again = perm[np.argsort(keys_of(x[perm], nc)[1], kind="stable")]
     assert np.array_equal(ctx.perm_tensor(n).cpu().numpy(), again)
+
+
+@pytest.mark.parametrize("n,nc", [(8191, 8), (8193, 64), (16384, 20), (16384, 65), (16385, 11),
+                                  (32768, 64), (32769, 30), (49152, 40), (49153, 40), (65535, 64),
+                                  (65536, 16), (65536, 65)])
+def test_order_of_one_cluster(env, n, nc):
+    """The sizes up to 65,536 and keys up to 48 bits (64 cells per axis) that
+    one cluster sorts: the edges of its instances, and both ends of the rule."""
+    torch, sim = env
+    rng = np.random.default_rng(n * 100 + nc)
+    pos = positions("uniform" if n % 2 else "clumps", n, nc, rng)
+    pos[rng.integers(0, n, size=n // 16)] = np.nextafter(1.0, 0.0)  # the largest key, many times
+    ctx = sim.Context(sim.Params(n_cells_override=nc, leaf_max=16), n)
+    p = sim.Particles(n)
+    p.m.fill_(1.0)
+    p.h.fill_(0.01)
+    for k, name in enumerate("xyz"):
+        getattr(p, name).copy_(torch.as_tensor(pos[:, k].copy()))
+    for _ in range(2):  # the second one starts from the sorted order
+        ctx.build_cells(p)
+        key = keys_of(pos, nc)[1]
+        perm = ctx.perm_tensor(n).cpu().numpy()
+        assert np.array_equal(perm, np.argsort(key, kind="stable"))
+        assert ctx.grid_info() == (nc, count_leaves(key[perm], 16))
