@@ -33,6 +33,8 @@ __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
 // by them (23 per particle in the drift, 20 in a step's close).  The
 // conversions and the scalings by powers of two below give the same bits from
 // integer instructions; what they do not cover takes the FP64 instruction.
+// 16.8M particles: step close 1.70 -> 0.60 ms, record refresh 1.63 -> 1.0, A
+// from u 0.52 -> 0.15.
 
 // (float)d, rounded to nearest even
 __device__ __forceinline__ float narrow(double d) {
@@ -600,10 +602,11 @@ __global__ void k_next_time(View v, long long *out, int count_step) {
   next_time(v, out, count_step);
 }
 
-// The end of a step in one launch: for every active particle the closing half-kick of its old step, its new bin (as
-// k_bins), the opening half-kick of the new step -- the same arithmetic as
-// k_kick and k_bins in the same order -- then, in the last block to finish,
-// the next tick and the step's counters (as k_next_time).
+// The end of a step in one launch: for every active particle the closing
+// half-kick of its old step, its new bin (as k_bins), the opening half-kick of
+// the new step -- the same arithmetic as k_kick and k_bins in the same order --
+// then, in the last block to finish, the next tick and the step's counters (as
+// k_next_time).
 __global__ void __launch_bounds__(UT) k_close_step(View v) {
   DevState *ds = v.ds;
   __shared__ int delta[MAX_BINS];

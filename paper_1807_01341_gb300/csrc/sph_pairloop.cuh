@@ -401,10 +401,10 @@ __device__ __forceinline__ float3 leaf_offset(const View &v, int i, const CellFr
 // ---------------------------------------------------------------------------
 constexpr int STAGE_DEPTH_MAX = 3;  // staging buffers per warp (copies in flight)
 
-// (TAGS: room for the staged records' particle and cell; SHARE, the forward
-// force and gradient loops': room for a batch's accept masks, and the search's spheres and
-// chunk list lie in the room of the staged records, so that every search sets
-// its spheres and none runs while records are in use)
+// (TAGS: room for the staged records' particle and cell; SHARE, of every loop
+// but the forward density's: room for a batch's accept masks, and the search's
+// spheres and chunk list lie in the room of the staged records, so that every
+// search sets its spheres and none runs while records are in use)
 template <int S, int NREC, int LC, bool TAGS = true, bool SHARE = false>
 struct Stage {
   static constexpr int SLOTS = S;  // staged records
@@ -675,15 +675,16 @@ __device__ __forceinline__ int search(const View &v, const CellFrame &F, const R
 
 // Stages the records of listed leaves [0, nlist) into shared memory by bulk
 // copies (TMA), through `depth` buffers of S / depth records (rounded down to
-// a multiple of 32) each: the copies
-// of the next depth - 1 batches are in flight while a batch is consumed.  A
-// batch is as many consecutive listed leaves as fit one buffer.  When a batch
-// has landed, each position record is moved into the work group's frame (its
-// leaf's corner offset added; its leaf found by counting the leaf starts up to
-// its slot, 32 records at a time: a loop over the leaves kept two lanes of three
-// idle: density at 16.8M particles 19.0 -> 18.2 ms, force 17.5 -> 17.3) and tagged with its particle index and neighbour-cell index
-// (TAG, which spends the leaf list's first-particle words; a loop that reads only the positions skips the
-// tags); then consume(base, total) sees records base .. base + total - 1.
+// a multiple of 32) each: the copies of the next depth - 1 batches are in
+// flight while a batch is consumed.  A batch is as many consecutive listed
+// leaves as fit one buffer.  When a batch has landed, each position record is
+// moved into the work group's frame (its leaf's corner offset added; its leaf
+// found by counting the leaf starts up to its slot, 32 records at a time: a
+// loop over the leaves kept two lanes of three idle: density at 16.8M particles
+// 19.0 -> 18.2 ms, force 17.5 -> 17.3) and tagged with its particle index and
+// neighbour-cell index (TAG, which spends the leaf list's first-particle words;
+// a loop that reads only the positions skips the tags); then consume(base,
+// total) sees records base .. base + total - 1.
 // Batches are consumed in list order whatever the depth.
 // A barrier wait that gives up sets st.failed and counts a timeout; the warp
 // then waits (bounded again) for every copy it still has in flight before it

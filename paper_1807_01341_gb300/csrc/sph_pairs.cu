@@ -185,7 +185,8 @@ __device__ __forceinline__ void dens_pair2(DSum &s, float2 r2, float2 m, float H
 // is used by one warp of one launch (L1 lines are invalidated between
 // dependent launches).  Two entries at a time against one by one with guarded
 // loads: density at 16.8M particles 20.2 -> 19.0 ms, 2.1M clustered 4.13 ->
-// 3.90 ms, 262k 0.398 -> 0.368 ms.
+// 3.90 ms, 262k 0.398 -> 0.368 ms (now, the staging faster too: 18.2, 3.80 and
+// 0.354 ms).
 constexpr int LQ = 4;
 constexpr int LIST_PAD = 2 * LQ;       // entries past list_cap: the last block's, and its successor's loads
 constexpr int TRANSPOSE_MAX = 20;      // live particles up to which the records go across the lanes
@@ -802,10 +803,12 @@ __device__ void force_group(const View &v, int wg, int slice, int nslices, int b
       // longest lane sets the time: the more records the lanes go through
       // before they wait for one another, the more their counts even out.
       // 16.8M particles, all active: 21.0 ms with rounds of 64 records, 19.5
-      // with 128, 18.4 with 192, all that fits beside the leaf list (the start,
-      // 64 and without the packed sums: 21.5); 2.1M clustered 4.21 -> 3.76 ms;
+      // with 128, 18.4 with 192, all that fits beside the leaf list (before, 64
+      // and without the packed sums: 21.5); 2.1M clustered 4.21 -> 3.76 ms;
       // with the variants 390 -> 270 us at 111k.  The pairs spread over all
       // lanes, each owner adding its own up afterwards: 22.3 ms at 16.8M.
+      // (With the packed kernels, the staging's bit masks and the paired tests
+      // since: 16.7 ms, 3.45 ms and 233 us.)
       const int wend = (total + 31) >> 5;
 #pragma unroll 1
       for (int q = 0; q < wend; q++) {
