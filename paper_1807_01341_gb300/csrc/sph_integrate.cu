@@ -287,14 +287,31 @@ __device__ void chunk_update(const View &v, int g, bool do_drift, bool do_bins) 
   float exc = 0.0f;
   // phase 1: particles, coalesced
   for (int i = pa + (int)threadIdx.x; i < pb; i += (int)blockDim.x) {
+    // (every load before the first store: the compiler keeps a load behind a
+    // store that might write what it reads, and a round of the block waited for
+    // four groups of them one after the other.  Drift of all 16.8M particles
+    // 1.55 -> 1.25 ms, sparse steps of 302k clustered 13 -> 10 us, of 2.1M 19 ->
+    // 15.  That takes 60 registers, 8 blocks an SM: 111k particles in leaves of
+    // 8, two waves of chunks then, 17 -> 19 us; 48 registers 15 us there, but
+    // 1.44 ms and 11 and 16 us.)
     double x = v.x[i], y = v.y[i], z = v.z[i];
+    const long long td = do_drift ? v.ti_drift[i] : ti;
+    const int pl = v.pleaf[i];
+    const float vx = v.vx[i], vy = v.vy[i], vz = v.vz[i];
+    const int bi = v.bin[i] & (MAX_BINS - 1);
+    const long long tb = v.ti_begin[i], te = v.ti_end[i];
+    const float ax = v.ax[i], ay = v.ay[i], az = v.az[i];
+    const float A = v.A[i], Adot = v.Adot[i], m = v.m[i], f = v.f[i];
+    float hh = v.h[i], rho = v.rho[i];
+    const float dv = v.predict || v.balsara ? v.div_v[i] : 0.0f;
+    const float cv = v.balsara ? v.curl_v[i] : 0.0f;
+    const uint32_t lk = v.leaf_k[pl];
     if (do_drift) {
-      const long long td = v.ti_drift[i];
       if (td != ti) {
         const double dt = widen(ti - td) * v.dt_min;
-        x = wrap_pos_fast(fma(widen(v.vx[i]), dt, x), v.box);
-        y = wrap_pos_fast(fma(widen(v.vy[i]), dt, y), v.box);
-        z = wrap_pos_fast(fma(widen(v.vz[i]), dt, z), v.box);
+        x = wrap_pos_fast(fma(widen(vx), dt, x), v.box);
+        y = wrap_pos_fast(fma(widen(vy), dt, y), v.box);
+        z = wrap_pos_fast(fma(widen(vz), dt, z), v.box);
         v.x[i] = x;
         v.y[i] = y;
         v.z[i] = z;
@@ -305,7 +322,6 @@ __device__ void chunk_update(const View &v, int g, bool do_drift, bool do_bins) 
     // FP64 runs at 1/64 of the FP32 rate on this GPU and bounds this pass,
     // so the only FP64 step is one fused multiply-add from the corner's
     // index on the box-wide Morton grid (one rounding).
-    const uint32_t lk = v.leaf_k[v.pleaf[i]];
     const int kx = leaf_kx(lk), ky = leaf_ky(lk), kz = leaf_kz(lk);
     const float fx = leaf_rel(x, gcx + kx, wq, v.box, hbox);
     const float fy = leaf_rel(y, gcy + ky, wq, v.box, hbox);
@@ -314,26 +330,23 @@ __device__ void chunk_update(const View &v, int g, bool do_drift, bool do_bins) 
     // (the bound is padded by 1e-6 of the cell width below)
     const float ex = fx + (float)kx * wqf, ey = fy + (float)ky * wqf, ez = fz + (float)kz * wqf;
     exc = fmaxf(exc, fmaxf(fmaxf(fmaxf(-ex, ex - wf), fmaxf(-ey, ey - wf)), fmaxf(-ez, ez - wf)));
-    const int bi = v.bin[i] & (MAX_BINS - 1);
     // (the middle of the particle's step: its length is 2^bin, or shorter once
     // the limiter woke it)
     // (ti - t_begin) - (t_end - t_begin) / 2, in half ticks
-    const long long tb = v.ti_begin[i];
-    const long long m2 = 2 * (ti - tb) - (v.ti_end[i] - tb);
+    const long long m2 = 2 * (ti - tb) - (te - tb);
     const float fdtp = narrow(widen(m2) * (0.5 * v.dt_min));
-    const float vpx = v.vx[i] + v.ax[i] * fdtp;
-    const float vpy = v.vy[i] + v.ay[i] * fdtp;
-    const float vpz = v.vz[i] + v.az[i] * fdtp;
-    const float Ap = v.A[i] + v.Adot[i] * fdtp;  // (as the density loop predicts it)
-    float hh = v.h[i], rho = v.rho[i];
+    const float vpx = vx + ax * fdtp;
+    const float vpy = vy + ay * fdtp;
+    const float vpz = vz + az * fdtp;
+    const float Ap = A + Adot * fdtp;  // (as the density loop predicts it)
     if (v.predict) {
       // Gadget-2 prediction from the last density (at the start of the step):
       // rho exp(-div v dt), h exp(div v dt / 3)
-      const float x = v.div_v[i] * (float)((double)(ti - tb) * v.dt_min);
+      const float x = dv * (float)((double)(ti - tb) * v.dt_min);
       rho *= expf(-x);
       hh *= expf(x * (1.0f / 3.0f));
     }
-    const float H = GAMMA_K * hh, m = v.m[i];
+    const float H = GAMMA_K * hh;
     v.rec_xm[i] = make_float4(fx, fy, fz, m);
     v.rec_xH[i] = make_float4(fx, fy, fz, H);
     v.rec_v[i] = make_float4(vpx, vpy, vpz, m);
@@ -343,12 +356,12 @@ __device__ void chunk_update(const View &v, int g, bool do_drift, bool do_bins) 
     if (rho > 0.0f) {
       const float P = Ap * powf(rho, g_);
       c = sqrtf(g_ * P / rho);
-      fP = v.f[i] * P / (rho * rho);
+      fP = f * P / (rho * rho);
       v.P[i] = P;
       v.c[i] = c;
     }
     v.rec_h[i] = make_float4(rho, fP, c, 1.0f / H);
-    if (v.balsara) v.bal[i] = balsara_factor(v.div_v[i], v.curl_v[i], c, 1.0f / H);
+    if (v.balsara) v.bal[i] = balsara_factor(dv, cv, c, 1.0f / H);
   }
   exc = warp_max_f(exc);
   if (lane == 0) s_exc[warp] = exc;
