@@ -61,36 +61,48 @@ __global__ void k_adj_prepare(sph_particles pre, sph_particles post, sph_particl
   const long long n = pre.n;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
-    const bool act = pre.ti_end[i] == ti;
+    // (here and in the gather and the scatter every load stands before the first
+    // store: the compiler keeps a load behind a store that might write what it
+    // reads.  32,768 particles: 7.5 -> 5.1 us, the scatter 9.4 -> 5.4.)
+    const long long te = pre.ti_end[i], tb = pre.ti_begin[i];
+    const bool act = te == ti;
+    const sph_particles &now = act ? post : pre;
+    const float h = now.h[i], rho = now.rho[i], f = now.f[i];
+    const float Adot_now = act ? post.Adot[i] : 0.0f;
+    const long long ptb = act ? post.ti_begin[i] : 0, pte = act ? post.ti_end[i] : 0;
+    const double avx = act ? adj.vx[i] : 0.0, avy = act ? adj.vy[i] : 0.0,
+                 avz = act ? adj.vz[i] : 0.0, aA = act ? adj.A[i] : 0.0;
+    const double aax = act ? adj.ax[i] : 0.0, aay = act ? adj.ay[i] : 0.0,
+                 aaz = act ? adj.az[i] : 0.0, aAdot = act ? adj.Adot[i] : 0.0;
+    const float vx = pre.vx[i], vy = pre.vy[i], vz = pre.vz[i];
+    const float ax = pre.ax[i], ay = pre.ay[i], az = pre.az[i];
+    const float A = pre.A[i], Adot = pre.Adot[i], m = pre.m[i];
+    const int bi = pre.bin[i] & (MAX_BINS - 1);
     // positions at the step's tick (the forward drift, applied to every particle)
     const double dtd = (double)(ti - pre.ti_drift[i]) * dt_min;
     double x = pre.x[i], y = pre.y[i], z = pre.z[i];
     if (dtd != 0.0) {
-      x = wrap_box(x + (double)pre.vx[i] * dtd, box);
-      y = wrap_box(y + (double)pre.vy[i] * dtd, box);
-      z = wrap_box(z + (double)pre.vz[i] * dtd, box);
+      x = wrap_box(x + (double)vx * dtd, box);
+      y = wrap_box(y + (double)vy * dtd, box);
+      z = wrap_box(z + (double)vz * dtd, box);
     }
     W.x[i] = x;
     W.y[i] = y;
     W.z[i] = z;
     // prediction at the tick
-    const int bi = pre.bin[i] & (MAX_BINS - 1);
-    const double dtp = ((double)(ti - pre.ti_begin[i]) - 0.5 * (double)(1ll << bi)) * dt_min;
+    const double dtp = ((double)(ti - tb) - 0.5 * (double)(1ll << bi)) * dt_min;
     const float fdtp = (float)dtp;
-    W.vx[i] = pre.vx[i] + pre.ax[i] * fdtp;
-    W.vy[i] = pre.vy[i] + pre.ay[i] * fdtp;
-    W.vz[i] = pre.vz[i] + pre.az[i] * fdtp;
-    const float h = act ? post.h[i] : pre.h[i];
-    const float rho = act ? post.rho[i] : pre.rho[i];
-    const float f = act ? post.f[i] : pre.f[i];
+    W.vx[i] = vx + ax * fdtp;
+    W.vy[i] = vy + ay * fdtp;
+    W.vz[i] = vz + az * fdtp;
     float Ap;
-    if (first) Ap = (float)(gamma - 1.0) * pre.A[i] / powf(rho, (float)gamma - 1.0f);  // A holds u
-    else Ap = (float)((double)pre.A[i] + (double)pre.Adot[i] * dtp);
+    if (first) Ap = (float)(gamma - 1.0) * A / powf(rho, (float)gamma - 1.0f);  // A holds u
+    else Ap = (float)((double)A + (double)Adot * dtp);
     W.A[i] = Ap;
     W.h[i] = h;
     W.rho[i] = rho;
     W.f[i] = f;
-    W.m[i] = pre.m[i];
+    W.m[i] = m;
     // the cell build's refresh predicts with a and Adot: zero, so the records
     // carry exactly v_pred and A_pred; vsig carries the forward Adot of the
     // active particles (the force adjoint needs it)
@@ -98,7 +110,7 @@ __global__ void k_adj_prepare(sph_particles pre, sph_particles post, sph_particl
     W.ay[i] = 0.0f;
     W.az[i] = 0.0f;
     W.Adot[i] = 0.0f;
-    W.vsig[i] = act ? post.Adot[i] : 0.0f;
+    W.vsig[i] = Adot_now;
     W.P[i] = 0.0f;
     W.c[i] = 0.0f;
     W.bin[i] = act ? 0 : 1;  // the backward marks bin 0 active
@@ -109,12 +121,11 @@ __global__ void k_adj_prepare(sph_particles pre, sph_particles post, sph_particl
     // adjoint of the two half-kicks of an active particle:
     // v += a dt_old / 2 and v += a dt_new / 2 (likewise A with Adot)
     if (act) {
-      const double half = 0.5 * (double)(pre.ti_end[i] - pre.ti_begin[i]) * dt_min +
-                          0.5 * (double)(post.ti_end[i] - post.ti_begin[i]) * dt_min;
-      adj.ax[i] += adj.vx[i] * half;
-      adj.ay[i] += adj.vy[i] * half;
-      adj.az[i] += adj.vz[i] * half;
-      adj.Adot[i] += adj.A[i] * half;
+      const double half = 0.5 * (double)(te - tb) * dt_min + 0.5 * (double)(pte - ptb) * dt_min;
+      adj.ax[i] = aax + avx * half;
+      adj.ay[i] = aay + avy * half;
+      adj.az[i] = aaz + avz * half;
+      adj.Adot[i] = aAdot + aA * half;
     }
   }
 }
@@ -127,33 +138,38 @@ __global__ void k_adj_gather(View v, AdjWork w, sph_adjoint adj, double gamma) {
   for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
        k += (long long)gridDim.x * blockDim.x) {
     const int o = w.perm[k];
-    w.xb[k] = adj.x[o];
-    w.yb[k] = adj.y[o];
-    w.zb[k] = adj.z[o];
-    w.hb[k] = adj.h[o];
-    w.rhob[k] = adj.rho[o];
-    w.fb[k] = adj.f[o];
+    const bool act = v.bin[k] == 0;
+    const double xb = adj.x[o], yb = adj.y[o], zb = adj.z[o], hb = adj.h[o], rb = adj.rho[o],
+                 fb = adj.f[o];
+    const double axb = act ? adj.ax[o] : 0.0, ayb = act ? adj.ay[o] : 0.0,
+                 azb = act ? adj.az[o] : 0.0, Adb = act ? adj.Adot[o] : 0.0;
+    const float sum = act ? v.vsig[k] : 0.0f, rho = act ? v.rho[k] : 1.0f;
+    w.xb[k] = xb;
+    w.yb[k] = yb;
+    w.zb[k] = zb;
+    w.hb[k] = hb;
+    w.fb[k] = fb;
     w.vpxb[k] = 0.0;
     w.vpyb[k] = 0.0;
     w.vpzb[k] = 0.0;
     w.Qb[k] = 0.0;
     w.cb[k] = 0.0;
-    if (v.bin[k] == 0) {
+    if (act) {
       // this step computed a and Adot of the active particles: their adjoints
       // are consumed here (what remains for the old values comes from the
       // prediction, added in the scatter)
-      w.axb[k] = adj.ax[o];
-      w.ayb[k] = adj.ay[o];
-      w.azb[k] = adj.az[o];
-      const double Adb = adj.Adot[o];
+      w.axb[k] = axb;
+      w.ayb[k] = ayb;
+      w.azb[k] = azb;
       w.Adotb[k] = Adb;
       adj.ax[o] = 0.0;
       adj.ay[o] = 0.0;
       adj.az[o] = 0.0;
       adj.Adot[o] = 0.0;
       // Adot = (gamma - 1)/2 rho^(1 - gamma) sum(...): its rho-dependence
-      w.rhob[k] += Adb * (double)v.vsig[k] * (1.0 - gamma) / (double)v.rho[k];
+      w.rhob[k] = rb + Adb * (double)sum * (1.0 - gamma) / (double)rho;
     } else {
+      w.rhob[k] = rb;
       w.axb[k] = w.ayb[k] = w.azb[k] = w.Adotb[k] = 0.0;
     }
   }
@@ -461,8 +477,16 @@ __global__ void k_adj_eos(View v, AdjWork w, sph_adjoint adj, int first) {
       w.cb[k] = 0.0;
       continue;
     }
-    const double f = v.f[k], P = v.P[k], c = v.c[k], Ap = v.A[k];
     const double Qb = w.Qb[k], cbar = w.cb[k];
+    // nothing came back to this particle's pressure and sound speed: every term
+    // below is a zero (in a sparse step nearly everywhere; the power and the
+    // divisions run at the FP64 rate: 32,768 particles, 18.7 -> 4 us in such a step)
+    if (!first && Qb == 0.0 && cbar == 0.0 && (v.f[k] + v.P[k] + v.c[k]) * 0.0f == 0.0f) {
+      w.cb[k] = 0.0;
+      w.Qb[k] = 0.0;
+      continue;
+    }
+    const double f = v.f[k], P = v.P[k], c = v.c[k], Ap = v.A[k];
     double rb = w.rhob[k];
     w.fb[k] += Qb * P / (rho * rho);
     double Pb = Qb * f / (rho * rho);
@@ -720,9 +744,10 @@ __global__ void k_adj_scatter(View v, AdjWork w, sph_particles pre, sph_particle
        k += (long long)gridDim.x * blockDim.x) {
     const int o = w.perm[k];
     const double xb = w.xb[k], yb = w.yb[k], zb = w.zb[k];
-    adj.x[o] = xb;
-    adj.y[o] = yb;
-    adj.z[o] = zb;
+    const double avx = adj.vx[o], avy = adj.vy[o], avz = adj.vz[o];
+    const double aax = adj.ax[o], aay = adj.ay[o], aaz = adj.az[o];
+    const double aA = adj.A[o], aAdot = adj.Adot[o];
+    const double cb = w.cb[k], Qb = w.Qb[k], hb = w.hb[k], rb = w.rhob[k], fb = w.fb[k];
     // drift of this step: x(ti) = x + v (ti - ti_drift) dt_min, for the
     // particles the forward drifted (those whose ti_drift moved)
     const double dtd = (double)(post.ti_drift[o] - pre.ti_drift[o]) * dt_min;
@@ -730,21 +755,24 @@ __global__ void k_adj_scatter(View v, AdjWork w, sph_particles pre, sph_particle
     const int bi = pre.bin[o] & (MAX_BINS - 1);
     const double dtp = ((double)(ti - pre.ti_begin[o]) - 0.5 * (double)(1ll << bi)) * dt_min;
     const double vpx = w.vpxb[k], vpy = w.vpyb[k], vpz = w.vpzb[k];
-    adj.vx[o] += vpx + xb * dtd;
-    adj.vy[o] += vpy + yb * dtd;
-    adj.vz[o] += vpz + zb * dtd;
-    adj.ax[o] += vpx * dtp;
-    adj.ay[o] += vpy * dtp;
-    adj.az[o] += vpz * dtp;
+    adj.x[o] = xb;
+    adj.y[o] = yb;
+    adj.z[o] = zb;
+    adj.vx[o] = avx + (vpx + xb * dtd);
+    adj.vy[o] = avy + (vpy + yb * dtd);
+    adj.vz[o] = avz + (vpz + zb * dtd);
+    adj.ax[o] = aax + vpx * dtp;
+    adj.ay[o] = aay + vpy * dtp;
+    adj.az[o] = aaz + vpz * dtp;
     if (first) {
-      adj.A[o] = w.cb[k];  // A held u before the first step
+      adj.A[o] = cb;  // A held u before the first step
     } else {
-      adj.A[o] += w.Qb[k];
-      adj.Adot[o] += w.Qb[k] * dtp;
+      adj.A[o] = aA + Qb;
+      adj.Adot[o] = aAdot + Qb * dtp;
     }
-    adj.h[o] = w.hb[k];
-    adj.rho[o] = w.rhob[k];
-    adj.f[o] = w.fb[k];
+    adj.h[o] = hb;
+    adj.rho[o] = rb;
+    adj.f[o] = fb;
   }
 }
 
