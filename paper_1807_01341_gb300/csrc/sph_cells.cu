@@ -567,6 +567,16 @@ __device__ __forceinline__ bool build_stopped(const DevState *ds) {
   return ds->build_bad != 0u || ds->build_fail != 0u;
 }
 
+// No work queue survives a build: their entries are indices into the structure
+// before it, and the density loop's lie in the build's scratch.
+__device__ __forceinline__ void clear_queues(DevState *ds) {
+  ds->n_active_leaves = ds->n_active_groups = ds->n_heavy_groups = 0;
+  ds->n_active_cells = ds->n_drift_chunks = 0;
+  ds->n_bin_groups = ds->n_bin_coop = 0;
+  ds->n_wake = 0;
+  ds->n_big = ds->head_big = ds->dens_split = 0;
+}
+
 // Words 0-11 the 8-byte arrays, 12-30 the 4-byte ones (the mass first), 31 the
 // particle's index in the first build's order (below 2^24) with its bin above.
 // (old: the composed permutation so far, or null for the first build.)  Also
@@ -621,8 +631,7 @@ __global__ void __launch_bounds__(256)
     ds->nc = nc;
     ds->n_cells = nc * nc * nc;
     ds->w = w;
-    ds->n_active_leaves = 0;
-    ds->n_active_groups = 0;
+    clear_queues(ds);
     ds->excursion_bits = ds->Hmax_bits = ds->want_h_bits = 0u;
     ds->group_cost_sum = 0ull;
     // equal masses: the density loop sums the kernel alone (rho = m sum w)
@@ -1045,7 +1054,7 @@ __global__ void k_build_empty(DevState *ds, int32_t *leaf_start, int32_t *chunk_
   ds->n_cells = nc * nc * nc;
   ds->w = w;
   ds->n_leaves = ds->n_chunks = ds->n_groups = 0;
-  ds->n_active_leaves = ds->n_active_groups = 0;
+  clear_queues(ds);
   ds->excursion_bits = ds->Hmax_bits = ds->want_h_bits = 0u;
   ds->group_cost_sum = 0ull;
   ds->m_uniform = 0.0f;

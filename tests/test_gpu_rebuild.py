@@ -1,0 +1,59 @@
+"""What a cell build leaves behind it: the work queues of the structure before
+it, the composed permutation, and a build that is refused or gives up."""
+import numpy as np
+import pytest
+
+import sph_ics
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1807_01341_gb300 import build
+    build.build()
+    from paper_1807_01341_gb300 import sim
+    return torch, sim
+
+
+def host(p):
+    return {k: t.cpu().numpy().copy() for k, t in p.arrays().items()}
+
+
+@pytest.mark.parametrize("list_cap", [32, 512])
+def test_no_queue_survives_a_build(env, list_cap):
+    """Active set, density (with particles over their list, and heavy groups),
+    then a build: the passes find no active particle until the next marking."""
+    torch, sim = env
+    ic = sph_ics.clumpy_lattice(17, 3, 500, seed=7)
+    n = ic["pos"].shape[0]
+    ctx = sim.Context(sim.Params(list_cap=list_cap, leaf_max=16,
+                                 heavy_factor=0.5), n)
+    p = sim.Particles.from_ics(ic)
+    ctx.resume(p, 0, True)
+    ctx.build_cells(p)
+    ctx.mark_active(p, 0)
+    ctx.density_active(p, 1)
+    assert ctx.status()[0] == 0
+    if list_cap == 32:
+        assert ctx.counters()["list_overflows"] > 0
+    p.h.mul_(0.9)  # another grid, fewer groups and chunks than indices in the old queues
+    ctx.build_cells(p)
+    before = host(p)
+    ctx.kick_drift(p, 0)
+    ctx.density_active(p, 0)
+    ctx.force_active(p)
+    ctx.kick_drift(p, 1)
+    ctx.timestep_bins(p)
+    ctx.kick_drift(p, 2)
+    after = host(p)
+    for k in before:
+        assert np.array_equal(before[k], after[k], equal_nan=True), k
+    assert ctx.status()[0] == 0
+    ctx.mark_active(p, 0)  # and the next marking starts from a clean slate
+    ctx.density_active(p, 0)
+    assert p.active.all()
+    assert np.array_equal(p.rho.cpu().numpy() > 0, np.ones(n, bool))
