@@ -236,7 +236,9 @@ int sph_build_cells(sph_ctx *ctx, sph_particles *p, void *stream);
 
 /* After sph_build_cells: permutation (device, int32, length n) with
  * perm[k] = index, in the order of the first sph_build_cells call, of the
- * particle now at position k.  Valid until the next sph_build_cells. */
+ * particle now at position k.  Valid until the next sph_build_cells.  Later builds
+ * compose it; particles past those of the build before (a larger n) enter it at
+ * their own position. */
 const int32_t *sph_perm(const sph_ctx *ctx);
 /* Number of top-level cells per axis and number of leaves of the last build. */
 int sph_grid_info(const sph_ctx *ctx, int *n_cells_per_axis, int *n_leaves);

@@ -100,6 +100,7 @@ struct sph_ctx {
   int list_blocks = 0;  // blocks a density launch may have (each warp has a list area)
   Buffers b;
   bool built = false;
+  long long n_perm = 0;        // particles that the composed permutation covers (0: none yet)
   bool entropy_ready = false;  // the first density pass has converted u to A
   int nc = 0;
   double w = 0.0;
@@ -383,7 +384,7 @@ int build_cells(sph_ctx *ctx, sph_particles *p, cudaStream_t st) {
   const double w = ctx->prm.box / (double)nc;
   const BuildArrays ba = {{b.keys[0], b.keys[1]}, {b.vals[0], b.vals[1]}, b.build_work, b.scratch,
                           b.marks, b.perm, mark_stride(ctx->n_max)};
-  SPH_CUDA(launch_build(v, ba, nc, w, (int)n_cells, !ctx->built, st));
+  SPH_CUDA(launch_build(v, ba, nc, w, (int)n_cells, ctx->n_perm, st));
   SPH_CUDA(launch_refresh_all(v, st));
   // cost estimate of every work group (only heavy-group scheduling uses it)
   if (ctx->prm.heavy_factor > 0.0) SPH_CUDA(launch_group_cost(v, 2 * ctx->grid_util, st));
@@ -396,6 +397,7 @@ int build_cells(sph_ctx *ctx, sph_particles *p, cudaStream_t st) {
   if (h.build_bad) return SPH_ERR_ARG;
   if (h.build_fail) {
     ctx->built = false;
+    ctx->n_perm = 0;
     return (int)h.build_fail;
   }
   ctx->n_leaves = h.n_leaves;
@@ -404,6 +406,7 @@ int build_cells(sph_ctx *ctx, sph_particles *p, cudaStream_t st) {
   ctx->nc = nc;
   ctx->w = w;
   ctx->built = true;
+  ctx->n_perm = n;
   ctx->rebuilds++;
   return SPH_OK;
 }
@@ -1075,6 +1078,7 @@ int sph_resume(sph_ctx *ctx, sph_particles *p, int64_t ti_current, int first, vo
   SPH_TRY(set_state(ctx, ti_current, true, S(stream)));
   SPH_CUDA(cudaStreamSynchronize(S(stream)));
   ctx->built = false;  // a new input order: the next step rebuilds, the permutation restarts
+  ctx->n_perm = 0;
   ctx->entropy_ready = !first;
   ctx->pending = 0;
   ctx->init_pending = false;
@@ -1134,7 +1138,8 @@ int sph_step_bwd(sph_ctx *ctx, const sph_particles *pre, const sph_particles *po
   SPH_CUDA(launch_adj_prepare(*pre, *post, W, *adj, ti, first, ctx->prm.dt_min, ctx->prm.box,
                               ctx->prm.gamma, st));
   sph_ctx *sub = a.sub;
-  sub->built = false;  // the permutation of this build starts from the caller's order
+  sub->built = false;
+  sub->n_perm = 0;  // the permutation of this build starts from the caller's order
   SPH_TRY(build_cells(sub, &W, st));
   View v = make_view(sub, &W);
   SPH_CUDA(launch_mark(v, 1, st));  // bin 0 (the step's active particles) is active at tick 1

@@ -579,13 +579,13 @@ __device__ __forceinline__ void clear_queues(DevState *ds) {
 
 // Words 0-11 the 8-byte arrays, 12-30 the 4-byte ones (the mass first), 31 the
 // particle's index in the first build's order (below 2^24) with its bin above.
-// (old: the composed permutation so far, or null for the first build.)  Also
-// the masses' range, as float bits: masses are positive, and any other value
+// (old: the composed permutation of the first n_old particles; the others are
+// new to it and start at their own place.)  Also the masses' range, as float bits: masses are positive, and any other value
 // only makes the two ends differ, which selects the general density loop.
 static_assert(2 * PF8 + PF4 + 1 == 32 && BUILD_SCRATCH == 128 && BUILD_MAX <= 1ll << 24,
               "a particle's arrays fill one record");
 __global__ void __launch_bounds__(256)
-    k_pack(View v, Fields f, const int32_t *__restrict__ old) {
+    k_pack(View v, Fields f, const int32_t *__restrict__ old, long long n_old) {
   DevState *ds = v.ds;
   unsigned int nlo = 0u, hi = 0u;
   for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < v.n;
@@ -599,7 +599,7 @@ __global__ void __launch_bounds__(256)
     }
 #pragma unroll
     for (int q = 0; q < PF4; q++) w[2 * PF8 + q] = f.p4[q] ? f.p4[q][k] : 0u;
-    w[31] = (unsigned int)(old ? old[k] : (int32_t)k) | ((unsigned int)f.bin[k] << 24);
+    w[31] = (unsigned int)(k < n_old ? old[k] : (int32_t)k) | ((unsigned int)f.bin[k] << 24);
     char *r = f.records + k * BUILD_SCRATCH;
 #pragma unroll
     for (int q = 0; q < 4; q++) st_32b(r + 32 * q, w + 8 * q);
@@ -1166,7 +1166,7 @@ size_t build_work_words(long long n) {
 }
 
 cudaError_t launch_build(const View &v, const BuildArrays &b, int nc, double w, int n_cells,
-                         bool first, cudaStream_t st) {
+                         long long n_perm, cudaStream_t st) {
   const int n = (int)v.n;
   cudaError_t e = cudaMemsetAsync(SPH_DS_FIELD(v.ds, build_bad), 0, 4 * sizeof(unsigned int), st);
   if (e != cudaSuccess) return e;
@@ -1217,7 +1217,7 @@ cudaError_t launch_build(const View &v, const BuildArrays &b, int nc, double w, 
   f.records = b.scratch;
   // marks: of the particles, then of the leaves for the chunks and the groups
   uint8_t *lead = b.marks, *chunk_lead = b.marks + b.n_max, *group_lead = chunk_lead + b.n_max;
-  k_pack<<<std::min(blocks_for(n, 256), wide), 256, 0, st>>>(v, f, first ? nullptr : b.perm);
+  k_pack<<<std::min(blocks_for(n, 256), wide), 256, 0, st>>>(v, f, b.perm, n_perm);
   k_unpack<<<std::min(blocks_for(n, 256), wide), 256, 0, st>>>(v, f, b.vals[alt ? 1 : 0], b.perm,
                                                                lead, nc, w);
   k_leaf_nodes<<<std::min(blocks_for(n, 256), wide), 256, 0, st>>>(skeys, n, n_cells, v.leaf_max,

@@ -388,9 +388,9 @@ struct BuildArrays {
 // Everything of a cell build after its grid is chosen: keys, sort, permutation of the
 // particle arrays, leaves, chunks, work groups, the device state of the structure.  Invalid
 // input (ds->build_bad) or a failed wait (ds->build_fail) stops the remaining
-// kernels.  first: the composed permutation starts here.
+// kernels.  n_perm: particles in the composed permutation so far (0: it starts here).
 cudaError_t launch_build(const View &v, const BuildArrays &b, int nc, double w, int n_cells,
-                         bool first, cudaStream_t st);
+                         long long n_perm, cudaStream_t st);
 // sph_integrate.cu
 cudaError_t launch_refresh_all(const View &v, cudaStream_t st);
 // current and next tick (ti >= 0); clear: the status and the check report

@@ -57,3 +57,37 @@ def test_no_queue_survives_a_build(env, list_cap):
     ctx.density_active(p, 0)
     assert p.active.all()
     assert np.array_equal(p.rho.cpu().numpy() > 0, np.ones(n, bool))
+
+
+@pytest.mark.parametrize("sizes", [(0, 3000), (1000, 3000), (3000, 1000, 2500)])
+def test_builds_of_growing_sets(env, sizes):
+    """Particles that an earlier build of the context did not hold start the
+    composed permutation at their own place, and every array keeps its bytes."""
+    torch, sim = env
+    rng = np.random.default_rng(11)
+    big = max(sizes)
+    # (memory that was used before: a new allocation is not zero)
+    junk = torch.full((1 << 28,), -1, dtype=torch.int8, device="cuda")
+    del junk
+    torch.cuda.empty_cache()
+    ctx = sim.Context(sim.Params(n_cells_override=7), big)
+    perm = np.arange(0)
+    for n in sizes:
+        p = sim.Particles(n)
+        for name in "xyz":
+            getattr(p, name).copy_(torch.as_tensor(rng.uniform(size=n)))
+        p.m.fill_(1.0)
+        p.h.copy_(torch.as_tensor(rng.uniform(0.01, 0.02, size=n), dtype=torch.float32))
+        p.bin.copy_(torch.as_tensor(rng.integers(0, 50, size=n), dtype=torch.int8))
+        before = host(p)
+        ctx.build_cells(p)
+        if n == 0:
+            continue
+        now = host(p)
+        at = np.argsort(before["x"])[np.argsort(np.argsort(now["x"]))]  # who stands where
+        for name in ("x", "h", "bin"):
+            assert np.array_equal(now[name], before[name][at]), name
+        assert ctx.bin_counts() == np.bincount(before["bin"], minlength=64).tolist()
+        old = np.r_[perm[:n], np.arange(min(perm.size, n), n)]
+        perm = old[at]
+        assert np.array_equal(ctx.perm_tensor(n).cpu().numpy(), perm)
