@@ -128,7 +128,9 @@ typedef struct {
                            are in flight while a batch is evaluated.  Results do not
                            depend on it. */
   int wait_limit;       /* polls of every bounded device wait (0: 2^22, about half a
-                           second); a wait that gives up records SPH_ERR_TIMEOUT */
+                           second; those of a cell build poll at least 4,096 times, some
+                           milliseconds); a wait that gives up records SPH_ERR_TIMEOUT
+                           (in a build: the call returns it) */
   int test_stall;       /* testing only, 0 in normal use: the first test_stall density
                            launches make one warp wait on a staging barrier that no copy
                            completes, so that the wait gives up after wait_limit polls and
@@ -156,6 +158,11 @@ typedef struct {
                            after the current tick, its bin becomes bin_i + 2 and its
                            opening half-kick is cut to the shorter step (as Durier & Dalla
                            Vecchia 2012 describe it; sph_counters.wakes counts them) */
+  int test_build_stall; /* testing only, ignored by a library built without SPH_CHECKS: in the
+                           next cell build of more than 4,096 particles the first tile of a
+                           sort by digit passes (1), of the leaves' compaction (2) or of the
+                           chunks' (3) keeps its counts to itself, once, so that the waits of
+                           the tiles after it give up (SPH_ERR_TIMEOUT) */
 } sph_params;
 
 /* Particle state, structure of arrays, all device pointers of length n.
@@ -231,7 +238,8 @@ int sph_destroy(sph_ctx *ctx);
  * as they are until the next build).  Synchronises `stream` (to size the
  * grid and to check the input).  Errors: SPH_ERR_ARG (also when a position is not finite or an h
  * is not a positive finite number; nothing is reordered then),
- * SPH_ERR_CUDA. */
+ * SPH_ERR_TIMEOUT (a bounded wait gave up: there are no cells until a build
+ * succeeds), SPH_ERR_CUDA. */
 int sph_build_cells(sph_ctx *ctx, sph_particles *p, void *stream);
 
 /* After sph_build_cells: permutation (device, int32, length n) with

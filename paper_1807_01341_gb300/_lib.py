@@ -48,7 +48,7 @@ class sph_params(ctypes.Structure):
                 ("heavy_factor", _d), ("coop_max_groups", _i), ("list_cap", _i),
                 ("search_margin", _d), ("staging_depth", _i), ("wait_limit", _i),
                 ("test_stall", _i), ("test_bad_group", _i), ("balsara", _i),
-                ("predict_inactive", _i), ("limiter", _i)]
+                ("predict_inactive", _i), ("limiter", _i), ("test_build_stall", _i)]
 
 
 PARTICLE_FIELDS = [("x", "f8"), ("y", "f8"), ("z", "f8"), ("vx", "f4"), ("vy", "f4"),

@@ -181,6 +181,8 @@ bool valid_params(const sph_params *p) {
   if (p->wait_limit < 0 || p->test_stall < 0 || p->test_bad_group < 0) return false;
 #ifndef SPH_CHECKS
   if (p->test_bad_group != 0) return false;  // only a checks build may plant a bad index
+#else
+  if (p->test_build_stall < 0 || p->test_build_stall > 3) return false;
 #endif
   const int vars[3] = {p->balsara, p->predict_inactive, p->limiter};
   for (int f : vars)
@@ -657,6 +659,7 @@ void sph_default_params(sph_params *p) {
   p->balsara = 0;
   p->predict_inactive = 0;
   p->limiter = 0;
+  p->test_build_stall = 0;
 }
 
 const char *sph_strerror(int code) {
@@ -724,7 +727,12 @@ int sph_create(const sph_params *params, int64_t n_max, sph_ctx **out) {
         cudaMemcpy(SPH_DS_FIELD(b.ds, test_stall), &params->test_stall, sizeof(int),
                    cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(SPH_DS_FIELD(b.ds, test_bad_group), &params->test_bad_group, sizeof(int),
-                   cudaMemcpyHostToDevice) != cudaSuccess) {
+                   cudaMemcpyHostToDevice) != cudaSuccess
+#ifdef SPH_CHECKS
+        || cudaMemcpy(SPH_DS_FIELD(b.ds, test_build_stall), &params->test_build_stall, sizeof(int),
+                      cudaMemcpyHostToDevice) != cudaSuccess
+#endif
+    ) {
       r = SPH_ERR_CUDA;
       break;
     }

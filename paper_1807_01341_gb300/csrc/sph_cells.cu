@@ -30,7 +30,10 @@ constexpr unsigned FULL = 0xffffffffu;
 constexpr int TILE = 4096;                 // items of a sort or compaction tile
 constexpr int RS_DIGITS = 256;
 constexpr int RS_PASSES_MAX = 7;           // 30 Morton + at most 24 cell bits
-constexpr int POLL_LIMIT = 1 << 22;        // polls of a look-back before it gives up
+// Polls of a look-back before it gives up: wait_limit, where it is given, but
+// enough for the tiles before to run (a poll is one load; a staging wait's
+// suspends the warp).
+constexpr int POLL_LIMIT = 1 << 22, POLL_MIN = 4096;
 
 // ---------------------------------------------------------------------------
 // maximum smoothing length
@@ -208,29 +211,44 @@ __device__ __forceinline__ void st_relaxed(T *p, T x) {
 // so every tile before a running one is running or done and a wait ends; a
 // wait that exceeds its limit all the same (or meets another block's failure)
 // sets *fail and the build's later kernels return without writing.
-__device__ __forceinline__ bool poll_failed(int polls, unsigned int *fail) {
-  if (polls >= POLL_LIMIT) {
+__device__ __forceinline__ bool poll_failed(int polls, int limit, unsigned int *fail) {
+  if (polls >= limit) {
     atomicCAS(fail, 0u, (unsigned int)SPH_ERR_TIMEOUT);
     return true;
   }
   return (polls & 1023) == 1023 && ld_relaxed(fail) != 0u;
 }
 
+// Testing (a library built with SPH_CHECKS; sph_params.test_build_stall):
+// whether this tile keeps its status to itself (one thread of the tile asks).
+enum { STALL_SORT = 1, STALL_LEAVES = 2, STALL_CHUNKS = 3 };
+#ifdef SPH_CHECKS
+constexpr bool PLANTS = true;
+#else
+constexpr bool PLANTS = false;
+#endif
+__device__ __forceinline__ bool planted_stall(DevState *ds, int stage, int tile) {
+  return PLANTS && ds && tile == 0 && gridDim.x > 1 &&
+         atomicCAS(&ds->test_build_stall, stage, 0) == stage;
+}
+
 // Chain of one 64-bit word per tile (two counts of 31 bits; bits 62-63: the
 // state), looked back 32 tiles at a time by one warp.
 constexpr unsigned long long CH_AGG = 1ull << 62, CH_INC = 2ull << 62, CH_VAL = (1ull << 62) - 1ull;
 __device__ bool chain_prefix(unsigned long long *status, int tile, unsigned long long mine,
-                             unsigned long long *prefix, unsigned int *fail) {
+                             unsigned long long *prefix, DevState *ds, int stage, int limit) {
   const int lane = threadIdx.x & 31;
+  unsigned int *const fail = &ds->build_fail;
   unsigned long long pre = 0ull;
-  if (lane == 0) st_relaxed(&status[tile], (tile == 0 ? CH_INC : CH_AGG) | mine);
+  if (lane == 0 && !planted_stall(ds, stage, tile))
+    st_relaxed(&status[tile], (tile == 0 ? CH_INC : CH_AGG) | mine);
   for (int p = tile - 1; p >= 0; p -= 32) {
     const int t = p - lane;
     unsigned long long s = CH_INC;
     for (int polls = 0;; polls++) {
       s = t >= 0 ? ld_relaxed(&status[t]) : CH_INC;
       if (!__any_sync(FULL, (s & ~CH_VAL) == 0ull)) break;
-      if (__any_sync(FULL, poll_failed(polls, fail))) return false;
+      if (__any_sync(FULL, poll_failed(polls, limit, fail))) return false;
     }
     const unsigned inc = __ballot_sync(FULL, (s & CH_INC) != 0ull);
     const int last = inc ? __ffs(inc) - 1 : 31;
@@ -283,18 +301,19 @@ __global__ void __launch_bounds__(RS_THREADS, 2)
               unsigned long long *__restrict__ okeys, unsigned int *__restrict__ ovals, int n,
               int shift, unsigned int *cur, unsigned int *clear,
               const unsigned int *__restrict__ totals, unsigned int *ticket, unsigned int *fail,
-              const unsigned int *bad, DevState *ds) {
+              const unsigned int *bad, DevState *ds, int limit) {
   constexpr int THREADS = RS_THREADS, ITEMS = TILE / THREADS, WARPS = THREADS / 32;
   constexpr unsigned AGG = 1u << 30, INC = 2u << 30, VAL = AGG - 1u;
   __shared__ unsigned long long s_keys[TILE];
   __shared__ unsigned int s_lofs[RS_DIGITS], s_gofs[RS_DIGITS], s_sums[33];
-  __shared__ int s_tile, s_fail;
+  __shared__ int s_tile, s_fail, s_hold;
   unsigned int *const wcnt = reinterpret_cast<unsigned int *>(s_keys);  // [WARPS][256], until the scatter
   static_assert(WARPS * RS_DIGITS * 4 <= TILE * 8, "the warps' counters fit the staging area");
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid == 0) {
     s_tile = (int)atomicAdd(ticket, 1u);
     s_fail = ld_relaxed(fail) != 0u || (bad && *bad != 0u);
+    if (PLANTS) s_hold = planted_stall(ds, STALL_SORT, s_tile) ? 1 : 0;
   }
   for (int k = lane; k < RS_DIGITS; k += 32) wcnt[warp * RS_DIGITS + k] = 0u;
   __syncthreads();
@@ -333,7 +352,8 @@ __global__ void __launch_bounds__(RS_THREADS, 2)
       mine += c;
     }
     // (the padding of the last tile counts there, where nothing follows)
-    st_relaxed(&cur[tile * RS_DIGITS + tid], (tile == 0 ? INC : AGG) | mine);
+    if (!PLANTS || !s_hold)
+      st_relaxed(&cur[tile * RS_DIGITS + tid], (tile == 0 ? INC : AGG) | mine);
     tot = totals[tid];
   }
   const unsigned int lofs = block_exclusive<unsigned int>(mine, s_sums, nullptr);
@@ -359,7 +379,7 @@ __global__ void __launch_bounds__(RS_THREADS, 2)
           if (w[q] & INC) open = false;
         }
         if (ready) break;
-        if (poll_failed(polls, fail)) {
+        if (poll_failed(polls, limit, fail)) {
           ok = false;
           break;
         }
@@ -819,7 +839,8 @@ __global__ void __launch_bounds__(CT)
                 int32_t *__restrict__ leaf_start, int32_t *__restrict__ leaf_cell,
                 uint32_t *__restrict__ leaf_k, int32_t *__restrict__ cell_leaf_start,
                 int32_t *__restrict__ pleaf, unsigned long long *__restrict__ leaf_keys,
-                uint8_t *__restrict__ chunk_lead, uint8_t *__restrict__ group_lead, DevState *ds) {
+                uint8_t *__restrict__ chunk_lead, uint8_t *__restrict__ group_lead, DevState *ds,
+                int limit) {
   __shared__ unsigned int s_sums[33];
   __shared__ unsigned long long s_pre;
   __shared__ int s_tile, s_stop;
@@ -850,7 +871,7 @@ __global__ void __launch_bounds__(CT)
   unsigned int off = block_exclusive<unsigned int>(s, s_sums, &tot);
   if (threadIdx.x < 32) {
     unsigned long long pre = 0ull;
-    const bool ok = chain_prefix(status, tile, tot, &pre, &ds->build_fail);
+    const bool ok = chain_prefix(status, tile, tot, &pre, ds, STALL_LEAVES, limit);
     if (threadIdx.x == 0) {
       s_pre = pre;
       s_stop = ok ? 0 : 1;
@@ -981,7 +1002,7 @@ __global__ void __launch_bounds__(CT)
                  unsigned int *ticket, int32_t *__restrict__ chunk_leaf_start,
                  int32_t *__restrict__ chunk_cell, int32_t *__restrict__ cell_chunk_start,
                  int32_t *__restrict__ leaf_chunk, int32_t *__restrict__ group_leaf0,
-                 int32_t *__restrict__ group_cell, DevState *ds) {
+                 int32_t *__restrict__ group_cell, DevState *ds, int limit) {
   __shared__ unsigned long long s_sums[33];
   __shared__ unsigned long long s_pre;
   __shared__ int s_tile, s_stop;
@@ -1007,7 +1028,7 @@ __global__ void __launch_bounds__(CT)
   unsigned long long off = block_exclusive<unsigned long long>(mine, s_sums, &tot);
   if (threadIdx.x < 32) {
     unsigned long long pre = 0ull;
-    const bool ok = chain_prefix(status, tile, tot, &pre, &ds->build_fail);
+    const bool ok = chain_prefix(status, tile, tot, &pre, ds, STALL_CHUNKS, limit);
     if (threadIdx.x == 0) {
       s_pre = pre;
       s_stop = ok ? 0 : 1;
@@ -1104,7 +1125,7 @@ cudaError_t launch_cluster_sort(unsigned long long *keys, unsigned int *vals, in
 // counted; a pass clears the status row that the next one chains on.
 cudaError_t sort_passes(unsigned long long *const keys[2], unsigned int *const vals[2], int n,
                         int nbits, const SortWork &s, bool *result_in_alt, unsigned int *fail,
-                        const unsigned int *bad, DevState *ds, cudaStream_t st) {
+                        const unsigned int *bad, DevState *ds, int limit, cudaStream_t st) {
   if (cluster_sorts(n, nbits)) {
     *result_in_alt = false;
     const auto sort = n <= 8 * RC_THREADS    ? launch_cluster_sort<8, 1>
@@ -1120,7 +1141,7 @@ cudaError_t sort_passes(unsigned long long *const keys[2], unsigned int *const v
     const int a = p & 1, b = a ^ 1;
     k_rs_pass<<<tiles_of(n), RS_THREADS, 0, st>>>(
         keys[a], p == 0 ? nullptr : vals[a], keys[b], vals[b], n, 8 * p, s.row[a], s.row[b],
-        s.totals + p * RS_DIGITS, s.ticket + p, fail, bad, ds);
+        s.totals + p * RS_DIGITS, s.ticket + p, fail, bad, ds, limit);
   }
   *result_in_alt = (passes & 1) != 0;
   return cudaGetLastError();
@@ -1157,7 +1178,8 @@ cudaError_t radix_sort_indices(unsigned long long *keys, unsigned int *vals,
   }
   unsigned long long *const ks[2] = {keys, keys_alt};
   unsigned int *const vs[2] = {vals, vals_alt};
-  return sort_passes(ks, vs, n, nbits, s, result_in_alt, s.fail, nullptr, nullptr, st);
+  return sort_passes(ks, vs, n, nbits, s, result_in_alt, s.fail, nullptr, nullptr, POLL_LIMIT,
+                     st);
 }
 
 size_t build_work_words(long long n) {
@@ -1189,6 +1211,7 @@ cudaError_t launch_build(const View &v, const BuildArrays &b, int nc, double w, 
   int cell_bits = 1;
   while ((1LL << cell_bits) < n_cells) cell_bits++;
   const int nbits = KEY_MORTON_BITS + cell_bits;
+  const int limit = v.wait_limit > 0 ? (int)std::max<long long>(v.wait_limit, POLL_MIN) : POLL_LIMIT;
   const int wide = 2 * v.grid_util;  // 8 blocks of 256 threads per SM
   note_launches(7);
   // (1024 / w = 1024 nc / box, rounded once more than a division by w would be:
@@ -1200,7 +1223,7 @@ cudaError_t launch_build(const View &v, const BuildArrays &b, int nc, double w, 
   unsigned int *const vals[2] = {b.vals[0], b.vals[1]};
   unsigned long long *const ks[2] = {b.keys[0], b.keys[1]};
   e = sort_passes(ks, vals, n, nbits, s, &alt, SPH_DS_FIELD(v.ds, build_fail),
-                  SPH_DS_FIELD(v.ds, build_bad), v.ds, st);
+                  SPH_DS_FIELD(v.ds, build_bad), v.ds, limit, st);
   if (e != cudaSuccess) return e;
   const unsigned long long *skeys = b.keys[alt ? 1 : 0];
   unsigned long long *leaf_keys = b.keys[alt ? 0 : 1];
@@ -1224,7 +1247,7 @@ cudaError_t launch_build(const View &v, const BuildArrays &b, int nc, double w, 
                                                                    lead, v.cell_start, v.ds);
   k_leaf_emit<<<n_tiles, CT, 0, st>>>(skeys, lead, n, n_cells, leaf_chain, ticket, v.leaf_start,
                                       v.leaf_cell, v.leaf_k, v.cell_leaf_start, v.pleaf, leaf_keys,
-                                      chunk_lead, group_lead, v.ds);
+                                      chunk_lead, group_lead, v.ds, limit);
   // (one half of the blocks splits the leaves' octrees, the other marks groups)
   const int gb = std::min(blocks_for(n_cells, 8), v.grid_util);
   k_chunk_nodes<<<gb + std::min(blocks_for(n, 256), v.grid_util), 256, 0, st>>>(
@@ -1232,7 +1255,7 @@ cudaError_t launch_build(const View &v, const BuildArrays &b, int nc, double w, 
   k_chunk_emit<<<n_tiles, CT, 0, st>>>(v.leaf_cell, chunk_lead, group_lead, n_cells, group_chain,
                                        ticket + 1, v.chunk_leaf_start, v.chunk_cell,
                                        v.cell_chunk_start, v.leaf_chunk, v.group_leaf0,
-                                       v.group_cell, v.ds);
+                                       v.group_cell, v.ds, limit);
   return cudaGetLastError();
 }
 

@@ -42,6 +42,7 @@ struct DevState {
   int n_heavy_groups;    // active work groups whose estimated cost is well above the mean
   int test_stall;        // testing: density launches whose first warp still has to stall
   int test_bad_group;    // testing (checks build): density launches still to plant a bad group
+  int test_build_stall;  // testing (checks build): stage of a cell build that still has to stall
   unsigned long long group_cost_sum;  // sum over work groups of group_cost (written at build)
   double w;              // cell width
   // queues (written by mark)

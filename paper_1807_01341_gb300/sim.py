@@ -50,6 +50,7 @@ class Params:
     balsara: int = 0
     predict_inactive: int = 0
     limiter: int = 0
+    test_build_stall: int = 0
 
     def to_c(self) -> _lib.sph_params:
         p = _lib.sph_params()
