@@ -239,7 +239,7 @@ int sph_destroy(sph_ctx *ctx);
  * grid and to check the input).  Errors: SPH_ERR_ARG (also when a position is not finite or an h
  * is not a positive finite number; nothing is reordered then),
  * SPH_ERR_TIMEOUT (a bounded wait gave up: there are no cells until a build
- * succeeds), SPH_ERR_CUDA. */
+ * succeeds; sph_perm and copies to the input order still hold), SPH_ERR_CUDA. */
 int sph_build_cells(sph_ctx *ctx, sph_particles *p, void *stream);
 
 /* After sph_build_cells: permutation (device, int32, length n) with

@@ -398,8 +398,10 @@ int build_cells(sph_ctx *ctx, sph_particles *p, cudaStream_t st) {
   // non-finite positions or h: rejected before anything was reordered
   if (h.build_bad) return SPH_ERR_ARG;
   if (h.build_fail) {
+    // no cells, but the arrays are in the order that the permutation says: the
+    // new one if the build got as far, else still the old one
     ctx->built = false;
-    ctx->n_perm = 0;
+    if (h.build_moved) ctx->n_perm = n;
     return (int)h.build_fail;
   }
   ctx->n_leaves = h.n_leaves;
@@ -802,7 +804,9 @@ int sph_build_cells(sph_ctx *ctx, sph_particles *p, void *stream) {
   return build_cells(ctx, p, S(stream));
 }
 
-const int32_t *sph_perm(const sph_ctx *ctx) { return ctx && ctx->built ? ctx->b.perm : nullptr; }
+const int32_t *sph_perm(const sph_ctx *ctx) {
+  return ctx && (ctx->built || ctx->n_perm > 0) ? ctx->b.perm : nullptr;
+}
 
 int sph_grid_info(const sph_ctx *ctx, int *nc, int *n_leaves) {
   if (!ctx) return SPH_ERR_ARG;
@@ -1076,7 +1080,7 @@ int sph_state_copy(const sph_ctx *ctx, const sph_particles *src, sph_particles *
                    int to_input_order, void *stream) {
   if (!ctx || !valid_particles(ctx, src) || !valid_particles(ctx, dst) || src->n != dst->n)
     return SPH_ERR_ARG;
-  const int32_t *perm = (to_input_order && ctx->built) ? ctx->b.perm : nullptr;
+  const int32_t *perm = (to_input_order && ctx->n_perm > 0) ? ctx->b.perm : nullptr;
   SPH_CUDA(launch_state_copy(*src, *dst, perm, S(stream)));
   return SPH_OK;
 }

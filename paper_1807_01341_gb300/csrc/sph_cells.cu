@@ -651,6 +651,7 @@ __global__ void __launch_bounds__(256)
     ds->nc = nc;
     ds->n_cells = nc * nc * nc;
     ds->w = w;
+    ds->build_moved = 1u;
     clear_queues(ds);
     ds->excursion_bits = ds->Hmax_bits = ds->want_h_bits = 0u;
     ds->group_cost_sum = 0ull;
@@ -1190,7 +1191,7 @@ size_t build_work_words(long long n) {
 cudaError_t launch_build(const View &v, const BuildArrays &b, int nc, double w, int n_cells,
                          long long n_perm, cudaStream_t st) {
   const int n = (int)v.n;
-  cudaError_t e = cudaMemsetAsync(SPH_DS_FIELD(v.ds, build_bad), 0, 4 * sizeof(unsigned int), st);
+  cudaError_t e = cudaMemsetAsync(SPH_DS_FIELD(v.ds, build_bad), 0, BUILD_WORDS * sizeof(unsigned int), st);
   if (e != cudaSuccess) return e;
   if (n == 0) {
     for (int32_t *p : {v.cell_start, v.cell_leaf_start, v.cell_chunk_start})

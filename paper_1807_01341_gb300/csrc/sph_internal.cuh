@@ -87,11 +87,14 @@ struct DevState {
   // time-bin occupancy
   int bin_count[MAX_BINS];
   // the cell build in progress: invalid particles, the SPH_ERR_* that stopped
-  // it, the particles' mass range (largest inverted and plain float bits) --
-  // these four are cleared together -- and the largest smoothing length
-  unsigned int build_bad, build_fail, m_nlo_bits, m_hi_bits;
+  // it, the particles' mass range (largest inverted and plain float bits),
+  // whether it has put the particles into the new order -- BUILD_WORDS words
+  // cleared together -- and the largest smoothing length
+  unsigned int build_bad, build_fail, m_nlo_bits, m_hi_bits, build_moved;
   unsigned int build_hmax_bits;
 };
+
+constexpr int BUILD_WORDS = 5;
 
 // A particle that the density loop leaves to k_density_big: the state of its
 // h iteration and its work group.

@@ -47,6 +47,9 @@ def _run(stage, wait_limit):
         out["mark"] = 0
     except _lib.SphError as e:
         out["mark"] = e.code
+    saved = sim.Particles(N)
+    ctx.state_copy(p, saved, True)
+    out["who_copied"] = saved.m.cpu().numpy()
     ctx.build_cells(p)
     out["who"], out["x"], out["perm"] = p.m.cpu().numpy(), p.x.cpu().numpy(), ctx.perm_tensor(N).cpu().numpy()
     out["info"] = ctx.grid_info()
@@ -84,6 +87,10 @@ def test_build_gives_up_and_recovers(plain, tmp_path, stage, wait_limit):
     # nothing lost and nobody changed places without its arrays
     assert np.array_equal(np.sort(got["who_failed"]), np.arange(N) + 1.0)
     assert np.array_equal(got["x_failed"], x[got["who_failed"].astype(np.int64) - 1])
+    # copies to the input order, and the next build's permutation, are still
+    # relative to the order before the first build
+    assert np.array_equal(got["who_copied"], np.arange(N) + 1.0)
+    assert np.array_equal(got["perm"], got["who"].astype(np.int64) - 1)
     # the next build: the same order and cells
     assert np.array_equal(got["who"], p.m.cpu().numpy())
     assert np.array_equal(got["x"], p.x.cpu().numpy())
