@@ -154,16 +154,6 @@ __global__ void __launch_bounds__(256)
   digits_end(passes, s_hist, totals);
 }
 
-__global__ void __launch_bounds__(256)
-    k_rs_count(const unsigned long long *__restrict__ keys, int n, unsigned int *totals, int passes) {
-  __shared__ unsigned int s_hist[RS_PASSES_MAX * RS_DIGITS];
-  digits_begin(passes, s_hist);
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x)
-    digits_add(passes, s_hist, keys[i]);
-  digits_end(passes, s_hist, totals);
-}
-
 // ---------------------------------------------------------------------------
 // scans and look-back
 // ---------------------------------------------------------------------------
@@ -295,7 +285,13 @@ __device__ __forceinline__ unsigned equal_lanes(unsigned int x) {
 // 197 us at 2.1M.  Counting the next digit by destination tile during the
 // scatter needs no look-back but was slower at every size it could serve:
 // 47 against 37 us at one tile, 68 against 58 us at 64.)
+//
+// The look-back is that of Merrill and Garland's single-pass scan (2016) over
+// one status word per tile and digit.  Without CHAIN the tiles' digit counts
+// are there already (k_rs_tile_counts, `cur`; none for a single tile) and
+// nothing waits: for callers that have no way to hear of a wait that gave up.
 constexpr int RS_THREADS = 512;
+template <bool CHAIN>
 __global__ void __launch_bounds__(RS_THREADS, 2)
     k_rs_pass(const unsigned long long *__restrict__ keys, const unsigned int *__restrict__ vals,
               unsigned long long *__restrict__ okeys, unsigned int *__restrict__ ovals, int n,
@@ -310,17 +306,17 @@ __global__ void __launch_bounds__(RS_THREADS, 2)
   unsigned int *const wcnt = reinterpret_cast<unsigned int *>(s_keys);  // [WARPS][256], until the scatter
   static_assert(WARPS * RS_DIGITS * 4 <= TILE * 8, "the warps' counters fit the staging area");
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) {
+  if (CHAIN && tid == 0) {
     s_tile = (int)atomicAdd(ticket, 1u);
     s_fail = ld_relaxed(fail) != 0u || (bad && *bad != 0u);
     if (PLANTS) s_hold = planted_stall(ds, STALL_SORT, s_tile) ? 1 : 0;
   }
   for (int k = lane; k < RS_DIGITS; k += 32) wcnt[warp * RS_DIGITS + k] = 0u;
   __syncthreads();
-  if (s_fail) return;
-  const int tile = s_tile;
+  if (CHAIN && s_fail) return;
+  const int tile = CHAIN ? s_tile : (int)blockIdx.x;
   const int base = tile * TILE, count = min(TILE, n - base);
-  if (tid < RS_DIGITS) clear[tile * RS_DIGITS + tid] = 0u;
+  if (CHAIN && tid < RS_DIGITS) clear[tile * RS_DIGITS + tid] = 0u;
   unsigned long long key[ITEMS];
   unsigned int rank[ITEMS];
 #pragma unroll
@@ -352,13 +348,26 @@ __global__ void __launch_bounds__(RS_THREADS, 2)
       mine += c;
     }
     // (the padding of the last tile counts there, where nothing follows)
-    if (!PLANTS || !s_hold)
-      st_relaxed(&cur[tile * RS_DIGITS + tid], (tile == 0 ? INC : AGG) | mine);
-    tot = totals[tid];
+    if (CHAIN) {
+      if (!PLANTS || !s_hold)
+        st_relaxed(&cur[tile * RS_DIGITS + tid], (tile == 0 ? INC : AGG) | mine);
+      tot = totals[tid];
+    } else {
+      const int tiles = (int)gridDim.x;
+      tot = mine;
+      if (tiles > 1) {
+        tot = 0u;
+        for (int t = 0; t < tiles; t++) {
+          const unsigned int c = cur[t * RS_DIGITS + tid];
+          prev += t < tile ? c : 0u;
+          tot += c;
+        }
+      }
+    }
   }
   const unsigned int lofs = block_exclusive<unsigned int>(mine, s_sums, nullptr);
   const unsigned int gofs = block_exclusive<unsigned int>(tot, s_sums, nullptr);
-  if (tid < RS_DIGITS && tile > 0) {
+  if (CHAIN && tid < RS_DIGITS && tile > 0) {
     // LB tiles a round, their words loaded together: blocks that start
     // together walk back over one another, one word at a time half as many
     // rounds as there are tiles in flight
@@ -398,7 +407,7 @@ __global__ void __launch_bounds__(RS_THREADS, 2)
     s_gofs[tid] = gofs + prev - lofs;
   }
   __syncthreads();
-  if (s_fail) return;
+  if (CHAIN && s_fail) return;
 #pragma unroll
   for (int r = 0; r < ITEMS; r++) {
     const unsigned int d = (unsigned int)(key[r] >> shift) & 255u;
@@ -431,6 +440,21 @@ __global__ void __launch_bounds__(RS_THREADS, 2)
     const int p = r * THREADS + tid;
     if (p < count && SPH_IN(ds, pos[r], n, SPH_CHECK_SCATTER)) ovals[pos[r]] = s_vals[p];
   }
+}
+
+// digit counts of every tile
+__global__ void __launch_bounds__(RS_THREADS)
+    k_rs_tile_counts(const unsigned long long *__restrict__ keys, int n, int shift,
+                     unsigned int *__restrict__ counts) {
+  __shared__ unsigned int s_hist[RS_DIGITS];
+  if (threadIdx.x < RS_DIGITS) s_hist[threadIdx.x] = 0u;
+  __syncthreads();
+  const int end = min(n, ((int)blockIdx.x + 1) * TILE);
+#pragma unroll 8
+  for (int i = (int)blockIdx.x * TILE + (int)threadIdx.x; i < end; i += RS_THREADS)
+    atomicAdd(&s_hist[(keys[i] >> shift) & 255u], 1u);
+  __syncthreads();
+  if (threadIdx.x < RS_DIGITS) counts[blockIdx.x * RS_DIGITS + threadIdx.x] = s_hist[threadIdx.x];
 }
 
 // The same sort of up to 65,536 pairs in one launch: the 8 or 16 blocks of a
@@ -1087,17 +1111,16 @@ inline int blocks_for(long long n, int t) { return (int)((n + t - 1) / t); }
 inline int tiles_of(long long n) { return (int)((n + TILE - 1) / TILE); }
 inline int passes_of(int nbits) { return (nbits + 7) / 8; }
 
-// The sort's scratch: [tickets 7, failed wait][totals 7 x 256][status rows 2 x tiles x 256]
+// The sort's scratch: [tickets 7][totals 7 x 256][status rows 2 x tiles x 256]
 struct SortWork {
-  unsigned int *ticket, *fail, *totals, *row[2];
+  unsigned int *ticket, *totals, *row[2];
   size_t zero_words;  // from `ticket` on, zero before the keys are counted
 };
 SortWork sort_work(unsigned int *w, int n_tiles) {
   SortWork s;
   const size_t row = (size_t)n_tiles * RS_DIGITS;
   s.ticket = w;
-  s.fail = w + RS_PASSES_MAX;
-  s.totals = w + RS_PASSES_MAX + 1;
+  s.totals = w + RS_PASSES_MAX;
   s.row[0] = s.totals + RS_PASSES_MAX * RS_DIGITS;
   s.row[1] = s.row[0] + row;
   s.zero_words = (size_t)(s.row[1] - w);
@@ -1122,25 +1145,29 @@ cudaError_t launch_cluster_sort(unsigned long long *keys, unsigned int *vals, in
   return cudaGetLastError();
 }
 
+cudaError_t cluster_sort(unsigned long long *keys, unsigned int *vals, int n, int nbits,
+                         const unsigned int *bad, DevState *ds, bool *result_in_alt,
+                         cudaStream_t st) {
+  *result_in_alt = false;
+  const auto sort = n <= 8 * RC_THREADS    ? launch_cluster_sort<8, 1>
+                    : n <= 16 * RC_THREADS ? launch_cluster_sort<16, 1>
+                    : n <= 32 * RC_THREADS ? launch_cluster_sort<16, 2>
+                    : n <= 48 * RC_THREADS ? launch_cluster_sort<16, 3>
+                                           : launch_cluster_sort<16, 4>;
+  return sort(keys, vals, n, nbits, bad, ds, st);
+}
+
 // Every pass.  Of more pairs than one cluster sorts, the keys' digits have been
 // counted; a pass clears the status row that the next one chains on.
 cudaError_t sort_passes(unsigned long long *const keys[2], unsigned int *const vals[2], int n,
                         int nbits, const SortWork &s, bool *result_in_alt, unsigned int *fail,
                         const unsigned int *bad, DevState *ds, int limit, cudaStream_t st) {
-  if (cluster_sorts(n, nbits)) {
-    *result_in_alt = false;
-    const auto sort = n <= 8 * RC_THREADS    ? launch_cluster_sort<8, 1>
-                      : n <= 16 * RC_THREADS ? launch_cluster_sort<16, 1>
-                      : n <= 32 * RC_THREADS ? launch_cluster_sort<16, 2>
-                      : n <= 48 * RC_THREADS ? launch_cluster_sort<16, 3>
-                                             : launch_cluster_sort<16, 4>;
-    return sort(keys[0], vals[0], n, nbits, bad, ds, st);
-  }
+  if (cluster_sorts(n, nbits)) return cluster_sort(keys[0], vals[0], n, nbits, bad, ds, result_in_alt, st);
   const int passes = passes_of(nbits);
   note_launches(passes);
   for (int p = 0; p < passes; p++) {
     const int a = p & 1, b = a ^ 1;
-    k_rs_pass<<<tiles_of(n), RS_THREADS, 0, st>>>(
+    k_rs_pass<true><<<tiles_of(n), RS_THREADS, 0, st>>>(
         keys[a], p == 0 ? nullptr : vals[a], keys[b], vals[b], n, 8 * p, s.row[a], s.row[b],
         s.totals + p * RS_DIGITS, s.ticket + p, fail, bad, ds, limit);
   }
@@ -1162,30 +1189,34 @@ cudaError_t launch_reduce_hmax(const View &v, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-size_t sort_work_words(long long n) {
-  return (size_t)(RS_PASSES_MAX + 1 + RS_PASSES_MAX * RS_DIGITS) +
-         2 * (size_t)tiles_of(std::max<long long>(n, 1)) * RS_DIGITS;
+size_t order_work_words(long long n) {
+  return (size_t)tiles_of(std::max<long long>(n, 1)) * RS_DIGITS;
 }
 
 cudaError_t radix_sort_indices(unsigned long long *keys, unsigned int *vals,
                                unsigned long long *keys_alt, unsigned int *vals_alt, int n,
                                int nbits, unsigned int *work, bool *result_in_alt, cudaStream_t st) {
-  const SortWork s = sort_work(work, tiles_of(n));
-  cudaError_t e = cudaMemsetAsync(s.ticket, 0, s.zero_words * sizeof(unsigned int), st);
-  if (e != cudaSuccess) return e;
-  if (!cluster_sorts(n, nbits)) {
-    note_launches(1);
-    k_rs_count<<<std::min(blocks_for(n, 256), 1024), 256, 0, st>>>(keys, n, s.totals, passes_of(nbits));
-  }
   unsigned long long *const ks[2] = {keys, keys_alt};
   unsigned int *const vs[2] = {vals, vals_alt};
-  return sort_passes(ks, vs, n, nbits, s, result_in_alt, s.fail, nullptr, nullptr, POLL_LIMIT,
-                     st);
+  if (cluster_sorts(n, nbits)) return cluster_sort(ks[0], vs[0], n, nbits, nullptr, nullptr, result_in_alt, st);
+  // (7 passes: 4,096 keys 78 us, with the look-back 86; 20,000 107 and 98; 65,536 119 and 108)
+  const int passes = passes_of(nbits), tiles = tiles_of(n);
+  note_launches(tiles > 1 ? 2 * passes : passes);
+  for (int p = 0; p < passes; p++) {
+    const int a = p & 1, b = a ^ 1;
+    if (tiles > 1) k_rs_tile_counts<<<tiles, RS_THREADS, 0, st>>>(ks[a], n, 8 * p, work);
+    k_rs_pass<false><<<tiles, RS_THREADS, 0, st>>>(ks[a], p == 0 ? nullptr : vs[a], ks[b], vs[b], n,
+                                                   8 * p, work, nullptr, nullptr, nullptr, nullptr,
+                                                   nullptr, nullptr, 0);
+  }
+  *result_in_alt = (passes & 1) != 0;
+  return cudaGetLastError();
 }
 
 size_t build_work_words(long long n) {
   const long long t = tiles_of(std::max<long long>(n, 1));
-  return 4 + 4 * (size_t)t + sort_work_words(n);
+  return 4 + 4 * (size_t)t + RS_PASSES_MAX * (1 + RS_DIGITS) +
+         2 * (size_t)t * RS_DIGITS;
 }
 
 cudaError_t launch_build(const View &v, const BuildArrays &b, int nc, double w, int n_cells,

@@ -370,10 +370,10 @@ void note_launches(int n);
 // Largest h of the particles into ds->build_hmax_bits.
 cudaError_t launch_reduce_hmax(const View &v, cudaStream_t st);
 // Scratch words of radix_sort_indices and of a build over n items.
-size_t sort_work_words(long long n);
+size_t order_work_words(long long n);
 size_t build_work_words(long long n);
 // Sorts keys stably by their low nbits (at most 56), vals = the keys' indices in that order;
-// the result is in (keys, vals) or the alternates.
+// the result is in (keys, vals) or the alternates.  No kernel of it waits for another block.
 cudaError_t radix_sort_indices(unsigned long long *keys, unsigned int *vals,
                                unsigned long long *keys_alt, unsigned int *vals_alt, int n,
                                int nbits, unsigned int *work, bool *result_in_alt, cudaStream_t st);

@@ -21,7 +21,7 @@ constexpr size_t OFF_KEYS1 = OFF_KEYS0 + sizeof(unsigned long long) * NOALLOC_MA
 constexpr size_t OFF_VALS0 = OFF_KEYS1 + sizeof(unsigned long long) * NOALLOC_MAX;
 constexpr size_t OFF_VALS1 = OFF_VALS0 + sizeof(unsigned int) * NOALLOC_MAX;
 constexpr size_t OFF_WORK = OFF_VALS1 + sizeof(unsigned int) * NOALLOC_MAX;
-constexpr size_t WORK_WORDS = 10240;                        // sort_work_words(NOALLOC_MAX)
+constexpr size_t WORK_WORDS = 4096;                         // order_work_words(NOALLOC_MAX)
 constexpr size_t SCRATCH_BYTES = OFF_WORK + sizeof(unsigned int) * WORK_WORDS;  // 1.6 MB
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[SCRATCH_BYTES];
@@ -112,7 +112,7 @@ extern "C" int sph_cell_order_noalloc(const double *x, const double *y, const do
   auto *vals0 = reinterpret_cast<unsigned int *>(s + OFF_VALS0);
   auto *vals1 = reinterpret_cast<unsigned int *>(s + OFF_VALS1);
   auto *work = reinterpret_cast<unsigned int *>(s + OFF_WORK);
-  if (sort_work_words(n) > WORK_WORDS) return SPH_ERR_CUDA;
+  if (order_work_words(n) > WORK_WORDS) return SPH_ERR_CUDA;
   const int nc = n_cells_per_axis;
   const double w = box / (double)nc;
   const long long n_cells = (long long)nc * nc * nc;
