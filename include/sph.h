@@ -162,7 +162,8 @@ typedef struct {
                            next cell build of more than 4,096 particles the first tile of a
                            sort by digit passes (1), of the leaves' compaction (2) or of the
                            chunks' (3) keeps its counts to itself, once, so that the waits of
-                           the tiles after it give up (SPH_ERR_TIMEOUT) */
+                           the tiles after it give up (SPH_ERR_TIMEOUT); 4: every build sorts
+                           as where no thread-block cluster can be placed */
 } sph_params;
 
 /* Particle state, structure of arrays, all device pointers of length n.

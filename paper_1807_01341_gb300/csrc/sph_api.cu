@@ -100,6 +100,7 @@ struct sph_ctx {
   int list_blocks = 0;  // blocks a density launch may have (each warp has a list area)
   Buffers b;
   bool built = false;
+  int cluster_most = 0;        // most particles that one cluster sorts (cluster_sort_max)
   long long n_perm = 0;        // particles that the composed permutation covers (0: none yet)
   bool entropy_ready = false;  // the first density pass has converted u to A
   int nc = 0;
@@ -182,7 +183,7 @@ bool valid_params(const sph_params *p) {
 #ifndef SPH_CHECKS
   if (p->test_bad_group != 0) return false;  // only a checks build may plant a bad index
 #else
-  if (p->test_build_stall < 0 || p->test_build_stall > 3) return false;
+  if (p->test_build_stall < 0 || p->test_build_stall > 4) return false;
 #endif
   const int vars[3] = {p->balsara, p->predict_inactive, p->limiter};
   for (int f : vars)
@@ -385,7 +386,7 @@ int build_cells(sph_ctx *ctx, sph_particles *p, cudaStream_t st) {
   v = make_view(ctx, p);
   const double w = ctx->prm.box / (double)nc;
   const BuildArrays ba = {{b.keys[0], b.keys[1]}, {b.vals[0], b.vals[1]}, b.build_work, b.scratch,
-                          b.marks, b.perm, mark_stride(ctx->n_max)};
+                          b.marks, b.perm, mark_stride(ctx->n_max), ctx->cluster_most};
   SPH_CUDA(launch_build(v, ba, nc, w, (int)n_cells, ctx->n_perm, st));
   SPH_CUDA(launch_refresh_all(v, st));
   // cost estimate of every work group (only heavy-group scheduling uses it)
@@ -696,6 +697,10 @@ int sph_create(const sph_params *params, int64_t n_max, sph_ctx **out) {
       break;
     }
     ctx->grid_util = ctx->num_sms * 4;
+    ctx->cluster_most = cluster_sort_max();
+#ifdef SPH_CHECKS
+    if (params->test_build_stall == 4) ctx->cluster_most = 0;
+#endif
     const int G = params->threads_per_particle;
     ctx->grid_dens = ctx->num_sms * persistent_blocks_per_sm(G, true);
     ctx->grid_force = ctx->num_sms * persistent_blocks_per_sm(G, false);

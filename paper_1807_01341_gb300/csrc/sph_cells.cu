@@ -474,7 +474,9 @@ __global__ void __launch_bounds__(RS_THREADS)
 // pairs 48 -> 24 us, 16,384 52 -> 26, 32,768 53 -> 32, 40,000 52 -> 36, 65,536 (6
 // passes) 65 -> 49.  With 8 blocks for all sizes 40,000 took 56 us and 32,768 37;
 // 16 blocks for 4,096 take 27.  The line is the 16-bit index: keys of more than
-// 48 bits (64 cells an axis) and more pairs take a launch per digit.
+// 48 bits (64 cells an axis) and more pairs take a launch per digit, and so does
+// what the device cannot place (cluster_sort_max: a partition of a GPU may have
+// no 16, or no 8, SMs that form a cluster).
 constexpr int RC_THREADS = 1024, RC_INDEX_BITS = 16;
 constexpr int RC_MAX = 16 * RC_THREADS * 4;  // of the largest instance below
 static_assert(RC_MAX <= 1 << RC_INDEX_BITS, "an index has 16 bits");
@@ -1127,42 +1129,73 @@ SortWork sort_work(unsigned int *w, int n_tiles) {
   return s;
 }
 
-// whether one cluster sorts them (k_rs_cluster)
-inline bool cluster_sorts(int n, int nbits) { return n <= RC_MAX && nbits + RC_INDEX_BITS <= 64; }
+// Whether one cluster sorts them (k_rs_cluster); most: what this device's
+// clusters hold (cluster_sort_max).
+inline bool cluster_sorts(int n, int nbits, int most) {
+  return n <= most && nbits + RC_INDEX_BITS <= 64;
+}
 
 template <int BLOCKS, int ITEMS>
-cudaError_t launch_cluster_sort(unsigned long long *keys, unsigned int *vals, int n, int nbits,
-                                const unsigned int *bad, DevState *ds, cudaStream_t st) {
-  const auto kernel = k_rs_cluster<BLOCKS, ITEMS>;
-  constexpr int smem = 2 * RC_THREADS * ITEMS * (int)sizeof(unsigned long long);
-  cudaError_t e =
-      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e == cudaSuccess && BLOCKS > 8)
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e != cudaSuccess) return e;
-  note_launches(1);
-  kernel<<<BLOCKS, RC_THREADS, smem, st>>>(keys, vals, n, passes_of(nbits), bad, ds);
-  return cudaGetLastError();
+struct ClusterSort {
+  static constexpr int HOLDS = BLOCKS * RC_THREADS * ITEMS;
+  static constexpr int SMEM = 2 * RC_THREADS * ITEMS * (int)sizeof(unsigned long long);
+  static_assert(HOLDS <= RC_MAX, "an index has 16 bits");
+  // sets the kernel's attributes; whether the device can place such a cluster
+  static bool prepare() {
+    const auto kernel = k_rs_cluster<BLOCKS, ITEMS>;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = BLOCKS;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(BLOCKS);
+    c.blockDim = dim3(RC_THREADS);
+    c.dynamicSmemBytes = SMEM;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    int clusters = 0;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM) == cudaSuccess &&
+        (BLOCKS <= 8 ||
+         cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) &&
+        cudaOccupancyMaxActiveClusters(&clusters, kernel, &c) == cudaSuccess)
+      return clusters > 0;
+    cudaGetLastError();
+    return false;
+  }
+  static cudaError_t launch(unsigned long long *keys, unsigned int *vals, int n, int nbits,
+                            const unsigned int *bad, DevState *ds, cudaStream_t st) {
+    note_launches(1);
+    k_rs_cluster<BLOCKS, ITEMS>
+        <<<BLOCKS, RC_THREADS, SMEM, st>>>(keys, vals, n, passes_of(nbits), bad, ds);
+    return cudaGetLastError();
+  }
+};
+
+// the smallest instance that holds n (rising order)
+template <class F>
+auto with_cluster_sort(int n, F f) {
+  return n <= ClusterSort<8, 1>::HOLDS    ? f(ClusterSort<8, 1>())
+         : n <= ClusterSort<16, 1>::HOLDS ? f(ClusterSort<16, 1>())
+         : n <= ClusterSort<16, 2>::HOLDS ? f(ClusterSort<16, 2>())
+         : n <= ClusterSort<16, 3>::HOLDS ? f(ClusterSort<16, 3>())
+                                          : f(ClusterSort<16, 4>());
 }
 
 cudaError_t cluster_sort(unsigned long long *keys, unsigned int *vals, int n, int nbits,
                          const unsigned int *bad, DevState *ds, bool *result_in_alt,
                          cudaStream_t st) {
   *result_in_alt = false;
-  const auto sort = n <= 8 * RC_THREADS    ? launch_cluster_sort<8, 1>
-                    : n <= 16 * RC_THREADS ? launch_cluster_sort<16, 1>
-                    : n <= 32 * RC_THREADS ? launch_cluster_sort<16, 2>
-                    : n <= 48 * RC_THREADS ? launch_cluster_sort<16, 3>
-                                           : launch_cluster_sort<16, 4>;
-  return sort(keys, vals, n, nbits, bad, ds, st);
+  return with_cluster_sort(n, [&](auto s) { return s.launch(keys, vals, n, nbits, bad, ds, st); });
 }
 
 // Every pass.  Of more pairs than one cluster sorts, the keys' digits have been
 // counted; a pass clears the status row that the next one chains on.
 cudaError_t sort_passes(unsigned long long *const keys[2], unsigned int *const vals[2], int n,
                         int nbits, const SortWork &s, bool *result_in_alt, unsigned int *fail,
-                        const unsigned int *bad, DevState *ds, int limit, cudaStream_t st) {
-  if (cluster_sorts(n, nbits)) return cluster_sort(keys[0], vals[0], n, nbits, bad, ds, result_in_alt, st);
+                        const unsigned int *bad, DevState *ds, int limit, int cluster_most,
+                        cudaStream_t st) {
+  if (cluster_sorts(n, nbits, cluster_most))
+    return cluster_sort(keys[0], vals[0], n, nbits, bad, ds, result_in_alt, st);
   const int passes = passes_of(nbits);
   note_launches(passes);
   for (int p = 0; p < passes; p++) {
@@ -1189,16 +1222,29 @@ cudaError_t launch_reduce_hmax(const View &v, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+int cluster_sort_max() {
+  int most = 0;
+  while (most < RC_MAX) {
+    // (the next instance up)
+    const int holds = with_cluster_sort(most + 1, [](auto s) { return s.prepare() ? s.HOLDS : 0; });
+    if (holds == 0) break;
+    most = holds;
+  }
+  return most;
+}
+
 size_t order_work_words(long long n) {
   return (size_t)tiles_of(std::max<long long>(n, 1)) * RS_DIGITS;
 }
 
 cudaError_t radix_sort_indices(unsigned long long *keys, unsigned int *vals,
                                unsigned long long *keys_alt, unsigned int *vals_alt, int n,
-                               int nbits, unsigned int *work, bool *result_in_alt, cudaStream_t st) {
+                               int nbits, int cluster_most, unsigned int *work, bool *result_in_alt,
+                               cudaStream_t st) {
   unsigned long long *const ks[2] = {keys, keys_alt};
   unsigned int *const vs[2] = {vals, vals_alt};
-  if (cluster_sorts(n, nbits)) return cluster_sort(ks[0], vs[0], n, nbits, nullptr, nullptr, result_in_alt, st);
+  if (cluster_sorts(n, nbits, cluster_most))
+    return cluster_sort(ks[0], vs[0], n, nbits, nullptr, nullptr, result_in_alt, st);
   // (7 passes: 4,096 keys 78 us, with the look-back 86; 20,000 107 and 98; 65,536 119 and 108)
   const int passes = passes_of(nbits), tiles = tiles_of(n);
   note_launches(tiles > 1 ? 2 * passes : passes);
@@ -1250,12 +1296,12 @@ cudaError_t launch_build(const View &v, const BuildArrays &b, int nc, double w, 
   // inside the margin of axis_code)
   k_cell_keys<<<std::min(blocks_for(n, 256), v.grid_util), 256, 0, st>>>(
       v, nc, w, (double)(1 << MORTON_BITS) / w, b.keys[0], s.totals,
-      cluster_sorts(n, nbits) ? 0 : passes_of(nbits));
+      cluster_sorts(n, nbits, b.cluster_most) ? 0 : passes_of(nbits));
   bool alt = false;
   unsigned int *const vals[2] = {b.vals[0], b.vals[1]};
   unsigned long long *const ks[2] = {b.keys[0], b.keys[1]};
   e = sort_passes(ks, vals, n, nbits, s, &alt, SPH_DS_FIELD(v.ds, build_fail),
-                  SPH_DS_FIELD(v.ds, build_bad), v.ds, limit, st);
+                  SPH_DS_FIELD(v.ds, build_bad), v.ds, limit, b.cluster_most, st);
   if (e != cudaSuccess) return e;
   const unsigned long long *skeys = b.keys[alt ? 1 : 0];
   unsigned long long *leaf_keys = b.keys[alt ? 0 : 1];

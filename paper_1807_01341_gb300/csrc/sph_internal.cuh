@@ -372,11 +372,15 @@ cudaError_t launch_reduce_hmax(const View &v, cudaStream_t st);
 // Scratch words of radix_sort_indices and of a build over n items.
 size_t order_work_words(long long n);
 size_t build_work_words(long long n);
+// Most items that one cluster of blocks sorts on the current device (0: no cluster can be
+// placed); sets the attributes of those kernels there, so it is called before the first sort.
+int cluster_sort_max();
 // Sorts keys stably by their low nbits (at most 56), vals = the keys' indices in that order;
 // the result is in (keys, vals) or the alternates.  No kernel of it waits for another block.
 cudaError_t radix_sort_indices(unsigned long long *keys, unsigned int *vals,
                                unsigned long long *keys_alt, unsigned int *vals_alt, int n,
-                               int nbits, unsigned int *work, bool *result_in_alt, cudaStream_t st);
+                               int nbits, int cluster_most, unsigned int *work, bool *result_in_alt,
+                               cudaStream_t st);
 // The buffers of a cell build (one context's, sized for n_max particles).
 constexpr long long BUILD_MAX = 1ll << 24;  // most particles of a build
 constexpr size_t BUILD_SCRATCH = 128;       // scratch bytes per particle (its permuted arrays)
@@ -388,6 +392,7 @@ struct BuildArrays {
   uint8_t *marks;               // 3 * n_max, n_max a multiple of 8
   int32_t *perm;
   long long n_max;
+  int cluster_most;             // cluster_sort_max of the device
 };
 // Everything of a cell build after its grid is chosen: keys, sort, permutation of the
 // particle arrays, leaves, chunks, work groups, the device state of the structure.  Invalid

@@ -26,14 +26,15 @@ constexpr size_t SCRATCH_BYTES = OFF_WORK + sizeof(unsigned int) * WORK_WORDS;  
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[SCRATCH_BYTES];
 
-// Device address of the scratch array for each device, looked up once per
-// device (with that device current) on its first call and kept for the life
-// of the process (a cudaDeviceReset on that device invalidates it; the header
-// asks callers not to call again after one).
+// Device address of the scratch array for each device, and what a cluster
+// sorts there, looked up once per device (with that device current) on its
+// first call and kept for the life of the process (a cudaDeviceReset on that
+// device invalidates them; the header asks callers not to call again after one).
 std::mutex g_mu;
 void *g_addr[64] = {};
+int g_cluster_most[64] = {};
 
-cudaError_t scratch_address(void **out) {
+cudaError_t scratch_address(void **out, int *cluster_most) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -43,9 +44,11 @@ cudaError_t scratch_address(void **out) {
     void *p = nullptr;
     e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
     if (e != cudaSuccess) return e;
+    g_cluster_most[dev] = cluster_sort_max();
     g_addr[dev] = p;
   }
   *out = g_addr[dev];
+  *cluster_most = g_cluster_most[dev];
   return cudaSuccess;
 }
 
@@ -103,7 +106,8 @@ extern "C" int sph_cell_order_noalloc(const double *x, const double *y, const do
     return SPH_ERR_ARG;
   if (n > 0 && (!x || !y || !z || !perm)) return SPH_ERR_ARG;
   void *base = nullptr;
-  if (scratch_address(&base) != cudaSuccess) return SPH_ERR_CUDA;
+  int cluster_most = 0;
+  if (scratch_address(&base, &cluster_most) != cudaSuccess) return SPH_ERR_CUDA;
   if (n == 0) return SPH_OK;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   unsigned char *s = static_cast<unsigned char *>(base);
@@ -123,8 +127,8 @@ extern "C" int sph_cell_order_noalloc(const double *x, const double *y, const do
   while ((1LL << cell_bits) < n_cells) cell_bits++;
   // (each call clears or writes every part of the array it reads)
   bool alt = false;
-  if (radix_sort_indices(keys0, vals0, keys1, vals1, (int)n, KEY_MORTON_BITS + cell_bits, work, &alt,
-                         st) != cudaSuccess)
+  if (radix_sort_indices(keys0, vals0, keys1, vals1, (int)n, KEY_MORTON_BITS + cell_bits,
+                         cluster_most, work, &alt, st) != cudaSuccess)
     return SPH_ERR_CUDA;
   if (cudaMemcpyAsync(perm, alt ? vals1 : vals0, sizeof(int32_t) * (size_t)n,
                       cudaMemcpyDeviceToDevice, st) != cudaSuccess)

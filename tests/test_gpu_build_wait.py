@@ -1,8 +1,8 @@
 """A cell build whose bounded waits give up (the checks build's planted stall:
 one tile keeps its counts to itself): the call returns SPH_ERR_TIMEOUT, the
 particles are still the same set, there are no cells, and the next build is the
-one that an undisturbed context makes.  Run in a child process that loads the
-checks build."""
+one that an undisturbed context makes.  And builds where no thread-block cluster
+can be placed.  Both in a child process that loads the checks build."""
 import os
 import subprocess
 import sys
@@ -58,6 +58,32 @@ def _run(stage, wait_limit):
     return out
 
 
+def _run_without_clusters():
+    """Builds of sizes that a cluster sorts, with and without one."""
+    import torch
+    from paper_1807_01341_gb300 import sim
+    out = []
+    for n in (1, 4097, 16385, 40000, 65536):
+        rng = np.random.default_rng(n)
+        pos = rng.uniform(size=(n, 3))
+        perms, launches, infos = [], [], []
+        for stall in (0, 4):
+            ctx = sim.Context(sim.Params(n_cells_override=20, test_build_stall=stall), n)
+            p = sim.Particles(n)
+            for k, name in enumerate("xyz"):
+                getattr(p, name).copy_(torch.as_tensor(pos[:, k].copy()))
+            p.m.fill_(1.0)
+            p.h.fill_(0.01)
+            before = ctx.counters()["kernel_launches"]
+            ctx.build_cells(p)
+            launches.append(ctx.counters()["kernel_launches"] - before)
+            perms.append(ctx.perm_tensor(n).cpu().numpy())
+            infos.append(ctx.grid_info())
+            ctx.close()
+        out.append(dict(pos=pos, perms=perms, launches=launches, infos=infos))
+    return out
+
+
 @pytest.fixture(scope="module")
 def plain():
     torch = pytest.importorskip("torch")
@@ -99,6 +125,22 @@ def test_build_gives_up_and_recovers(plain, tmp_path, stage, wait_limit):
     ctx.close()
 
 
+def test_build_without_clusters(plain, tmp_path):
+    from test_gpu_build import keys_of
+    path = str(tmp_path / "out.npy")
+    env = dict(os.environ, SPH_GB300_CHECKS="1", PYTHONPATH=ROOT)
+    r = subprocess.run([sys.executable, os.path.abspath(__file__), "4", "0", path], env=env,
+                       capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout + r.stderr
+    for got in np.load(path, allow_pickle=True):
+        want = np.argsort(keys_of(got["pos"], 20)[1], kind="stable")
+        for perm in got["perms"]:
+            assert np.array_equal(perm, want)
+        assert got["infos"][0] == got["infos"][1]
+        # (43 bits of key: one launch where a cluster sorts, else six)
+        assert got["launches"][1] - got["launches"][0] == 5
+
+
 def test_short_wait_limit_leaves_builds_alone(plain):
     """wait_limit = 1: the waits of an undisturbed build are longer than that."""
     torch, _lib, sim = plain
@@ -117,4 +159,6 @@ def test_short_wait_limit_leaves_builds_alone(plain):
 
 if __name__ == "__main__":
     sys.path.insert(0, ROOT)
-    np.save(sys.argv[3], _run(int(sys.argv[1]), int(sys.argv[2])), allow_pickle=True)
+    stage = int(sys.argv[1])
+    res = _run_without_clusters() if stage == 4 else _run(stage, int(sys.argv[2]))
+    np.save(sys.argv[3], res, allow_pickle=True)
