@@ -1023,8 +1023,9 @@ __global__ void __launch_bounds__(GD_WARPS * 32, 6)
       adj.vx[j] += o[0] * dtd;
       adj.vy[j] += o[1] * dtd;
       adj.vz[j] += o[2] * dtd;
-      // dW/dh = -GAMMA_K (8/pi) H^-4 (3 w + q w')
-      adj.h[j] += -GAMMA_K_D * (C * Hinv) * o[3];
+      // dW/dh = -GAMMA_K (8/pi) H^-4 (3 w + q w'); a support without a point
+      // (of h = 0, whose 1 / H is infinite, among them) adds nothing
+      if (o[3] != 0.0) adj.h[j] += -GAMMA_K_D * (C * Hinv) * o[3];
     }
   }
 }

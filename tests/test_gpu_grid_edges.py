@@ -1,0 +1,57 @@
+"""Grid density and its adjoint where a support holds no point or is no number."""
+import numpy as np
+import pytest
+
+from test_gpu_grid import direct
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1807_01341_gb300 import build
+    build.build()
+    from paper_1807_01341_gb300 import sim
+    return torch, sim
+
+
+def state(sim, torch, pos, m, h):
+    p = sim.Particles(len(m))
+    for k, name in enumerate("xyz"):
+        getattr(p, name).copy_(torch.as_tensor(pos[:, k].copy()))
+    p.m.copy_(torch.as_tensor(m))
+    p.h.copy_(torch.as_tensor(h))
+    return p
+
+
+@pytest.mark.parametrize("n,ng", [(40, 9), (3000, 8)])
+@pytest.mark.parametrize("odd", [0.0, -0.01, np.nan, 1e-30])
+def test_supports_without_a_point(env, n, ng, odd):
+    """Particles whose h is zero (one of them on a grid point), negative, not a
+    number or tiny leave the grid and every adjoint as they are."""
+    torch, sim = env
+    rng = np.random.default_rng(n)
+    pos = rng.uniform(size=(n, 3))
+    m = rng.uniform(0.5, 1.5, size=n).astype(np.float32)
+    h = rng.uniform(0.02, 0.09, size=n).astype(np.float32)
+    off = np.arange(n) % 3 == 0
+    h[off] = odd
+    if odd <= 0.0:
+        pos[0] = 0.5 / ng
+    bar = rng.normal(size=ng ** 3)
+    p = state(sim, torch, pos, m, h)
+    ctx = sim.Context(sim.Params(), n)
+    adj = sim.Adjoint(n)
+    for k, name in enumerate(("x", "y", "z", "h")):
+        getattr(adj, name).fill_(k + 1.0)
+    rho = ctx.grid_density(p, ng, 0).cpu().numpy()
+    ctx.grid_density_bwd(p, ng, 0, torch.as_tensor(bar, device="cuda"), adj)
+    want, grad = direct(pos[~off], m[~off].astype(float), h[~off].astype(float), bar, ng)
+    assert np.allclose(rho, want, rtol=1e-12, atol=1e-12 * want.max())
+    for k, name in enumerate(("x", "y", "z", "h")):
+        got = getattr(adj, name).cpu().numpy()
+        assert np.array_equal(got[off], np.full(off.sum(), k + 1.0)), name
+        assert np.allclose(got[~off] - (k + 1.0), grad[k], rtol=1e-9, atol=1e-9 * np.abs(grad[k]).max())
