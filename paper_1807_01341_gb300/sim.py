@@ -91,19 +91,22 @@ class Particles:
             offs[name] = total
             total += (self.n * _ITEMSIZE[dt] + self.ALIGN - 1) // self.ALIGN * self.ALIGN
         self.storage = torch.zeros(max(total, self.ALIGN), dtype=torch.uint8, device=self.device)
+        # the arrays' buffer for good: `storage` may be given another tensor
+        self._buffer = self.storage
         self._offs = offs
         self._struct = None
 
     def __getattr__(self, name):
-        # an array's view is made when first asked for: a differentiable run
-        # takes a snapshot per step, whose 25 views cost the host 0.26 ms where
-        # the step's kernels took 0.3 ms
+        # an array's view is made when first asked for (that use pays for it): a
+        # differentiable run takes a snapshot per step of which it asks for no
+        # array, and the 25 views cost the host 0.2 ms where the step's kernels
+        # took 0.3 ms
         offs = self.__dict__.get("_offs")
         if offs is None or name not in offs:
             raise AttributeError(name)
         dt = _FIELD_TYPE[name]
         nbytes = self._count * _ITEMSIZE[dt]
-        view = self.storage[offs[name]:offs[name] + nbytes].view(_TORCH[dt])
+        view = self._buffer[offs[name]:offs[name] + nbytes].view(_TORCH[dt])
         self.__dict__[name] = view
         return view
 
@@ -137,7 +140,7 @@ class Particles:
         if s is None:
             s = _lib.sph_particles()
             s.n = self.n
-            base, d = self.storage.data_ptr(), self.__dict__
+            base, d = self._buffer.data_ptr(), self.__dict__
             for name, _ in _lib.PARTICLE_FIELDS:
                 if name in d:  # a view, a replaced array or an absent one
                     setattr(s, name, None if d[name] is None else d[name].data_ptr())
