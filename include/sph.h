@@ -238,7 +238,8 @@ int sph_destroy(sph_ctx *ctx);
  * loop then sums the kernel alone: rho = m sum w; masses are taken to stay
  * as they are until the next build).  Synchronises `stream` (to size the
  * grid and to check the input).  Errors: SPH_ERR_ARG (also when a position is not finite or an h
- * is not a positive finite number; nothing is reordered then),
+ * is not a positive finite number; nothing is reordered then, and the cells stay
+ * those of the build before unless the new grid has more of them),
  * SPH_ERR_TIMEOUT (a bounded wait gave up: there are no cells until a build
  * succeeds; sph_perm and copies to the input order still hold), SPH_ERR_CUDA. */
 int sph_build_cells(sph_ctx *ctx, sph_particles *p, void *stream);

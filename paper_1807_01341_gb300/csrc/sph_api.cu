@@ -382,6 +382,9 @@ int build_cells(sph_ctx *ctx, sph_particles *p, cudaStream_t st) {
     nc = (int)std::max(3.0, std::min((double)NC_MAX, ncd));
   }
   const long long n_cells = (long long)nc * nc * nc;
+  // (new cell arrays hold nothing of the structure before: if this build is
+  // refused there are no cells until one succeeds)
+  if (n_cells > ctx->b.cell_cap) ctx->built = false;
   SPH_TRY(ensure_cells(ctx, n_cells));
   v = make_view(ctx, p);
   const double w = ctx->prm.box / (double)nc;

@@ -91,3 +91,49 @@ def test_builds_of_growing_sets(env, sizes):
         old = np.r_[perm[:n], np.arange(min(perm.size, n), n)]
         perm = old[at]
         assert np.array_equal(ctx.perm_tensor(n).cpu().numpy(), perm)
+
+
+@pytest.mark.parametrize("finer", [True, False])
+def test_refused_build(env, finer):
+    """A build refused for a position that is no number: the cells before it
+    stay in use, or, where the new grid needed larger arrays, there are none
+    until a build succeeds; the particles and their permutation stay."""
+    torch, sim = env
+    from paper_1807_01341_gb300 import _lib
+    n = 4000
+    rng = np.random.default_rng(2)
+    ctx = sim.Context(sim.Params(), n)
+    p = sim.Particles(n)
+    for name in "xyz":
+        getattr(p, name).copy_(torch.as_tensor(rng.uniform(size=n)))
+    p.m.copy_(torch.arange(n) + 1.0)
+    p.h.fill_(0.06)
+    p.A.fill_(1.0)
+    ctx.build_cells(p)
+    info, perm = ctx.grid_info(), ctx.perm_tensor(n).cpu().numpy()
+    x0 = float(p.x[0])
+    p.x[0] = float("nan")
+    p.h.fill_(0.004 if finer else 0.09)
+    who = p.m.cpu().numpy()
+    with pytest.raises(_lib.SphError) as e:
+        ctx.build_cells(p)
+    assert e.value.code == _lib.SPH_ERR_ARG
+    assert np.array_equal(p.m.cpu().numpy(), who)
+    assert np.array_equal(ctx.perm_tensor(n).cpu().numpy(), perm)
+    p.x[0] = x0
+    p.h.fill_(0.06)
+    if finer:
+        with pytest.raises(_lib.SphError) as e:
+            ctx.mark_active(p, 0)
+        assert e.value.code == _lib.SPH_ERR_NOT_BUILT
+    else:
+        assert ctx.grid_info() == info
+        ctx.mark_active(p, 0)
+        ctx.density_active(p, 1)
+        assert ctx.status()[0] == 0 and p.active.all()
+    saved = sim.Particles(n)
+    ctx.state_copy(p, saved, True)
+    assert np.array_equal(saved.m.cpu().numpy(), np.arange(n) + 1.0)
+    ctx.resume(p, 0, True)
+    ctx.step(p, 1)
+    assert ctx.counters()["steps"] == 1
