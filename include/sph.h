@@ -112,8 +112,8 @@ typedef struct {
                            (squared distance and mass of every candidate within
                            search_margin x its support, kept across the h iterations;
                            a particle that has more is evaluated without a list, by a
-                           warp of its own, or, with several lanes per particle, in
-                           passes of list_cap); 32..4096.
+                           warp of its own or, where there are many, a lane; with several
+                           lanes per particle in passes of list_cap); 32..4096.
                            The library holds 8 x list_cap bytes per lane of every warp
                            of the persistent density grid for them (2 blocks of 8 warps
                            per SM: 319 MB at 512 on 152 SMs), whatever the particle count.

@@ -71,7 +71,7 @@ struct DevState {
   unsigned int Hmax_bits;       // max kernel support H (float bits) over all particles
   unsigned int want_h_bits;     // largest h an iteration wanted beyond the cell limit
   int dens_split;               // parts per work group of the last whole-step density launch
-  int n_big;              // density loop: particles left to one warp each (View::big)
+  int n_big, n_big_runs;  // density loop: particles whose list filled up (View::big), and their runs
   int head_big;           // work head of those
   // counters of the step in progress (reset when a step starts, added to the
   // totals when it completes, so a halted attempt leaves no trace)
@@ -97,7 +97,7 @@ struct DevState {
 constexpr int BUILD_WORDS = 5;
 
 // A particle that the density loop leaves to k_density_big: the state of its
-// h iteration and its work group.
+// h iteration and its work group (the same in a run).
 struct BigItem {
   double lo, hi;  // bracket
   float h;
@@ -166,6 +166,7 @@ struct View {
   // next work group, so the lists stay in L2.
   float2 *nbr;
   BigItem *big;              // [n] (the build's scratch, free between builds)
+  int *big_run;              // [n] runs of `big` left by one warp together: first | count - 1 << 24
   DevState *ds;
   // parameters
   double box, eta, gamma, alpha, cfl, h_tol, dt_min;
@@ -414,8 +415,8 @@ cudaError_t launch_close_step(const View &v, cudaStream_t st);
 // sph_pairs.cu
 cudaError_t launch_density(const View &v, int flags, int bin_filter, bool persistent,
                            int grid, cudaStream_t st);
-// The particles that the density launches since the step began left to one
-// warp each, then the supports of the leaves whose groups were split or had
+// The particles whose lists filled up in the density launches since the step
+// began, then the supports of the leaves whose groups were split or had
 // such particles.
 cudaError_t launch_density_rest(const View &v, int flags, int grid, cudaStream_t st);
 cudaError_t launch_force(const View &v, int bin_filter, bool persistent, int grid,

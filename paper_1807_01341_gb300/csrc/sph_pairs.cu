@@ -286,23 +286,24 @@ __device__ __forceinline__ void write_density(const View &v, int i, const float4
 // "gather": the search lists the leaves that the particle's sphere of radius
 // R_i = search_margin x H reaches, their records are staged, and every record
 // with r^2 < R_i^2 goes into the particle's neighbour list (squared distance
-// and mass).  Each h iteration evaluates its sums at its H from the list
-// alone, in record order, as long as H <= R_i; a particle whose h outgrows
-// R_i gathers again.  A list holds list_cap entries per lane.  A particle whose
-// gather accepts more is left to k_density_big; with several lanes per particle
-// the gather runs in passes over the same leaves, each pass listing (and
-// summing) the next list_cap accepted records, and the particle's list is then
-// not kept (later iterations gather at R_i = H).  Whatever the capacity, margin or staging depth, a particle's sums visit the
-// same pairs in the same order with the same arithmetic.  A work group is
-// handled by one warp (sharing it between the warps of a block, as the force
-// loop does in sparse steps, was measured slower here: every warp pays the
-// search's latency, then waits at the barriers of each h iteration), or, in
-// steps with few active groups, split by its active particles into `nslices`
-// consecutive slices, each a warp's own work item (slice `slice`): no warp
-// waits for another, and a slice's sums are those the whole group would give
-// (a particle's candidates and their order do not depend on the particles it
-// shares a warp with).  A split group's leaves get their largest support from
-// k_leaf_hmax, after every slice is done.
+// and mass).  Each h iteration evaluates its sums at its H from the list alone,
+// in record order, as long as H <= R_i; a particle whose h outgrows R_i gathers
+// again.  A list holds list_cap entries per lane.  A particle whose gather
+// accepts more is left to k_density_big, which keeps no list; with several
+// lanes per particle the gather runs in passes over the same leaves, each pass
+// listing (and summing) the next list_cap accepted records, and the particle's
+// list is then not kept (later iterations gather at R_i = H).  Whatever the
+// capacity, margin or staging depth, a particle's sums visit the same pairs in
+// the same order with the same arithmetic.  A work group is handled by one warp
+// (sharing it between the warps of a block, as the force loop does in sparse
+// steps, was measured slower here: every warp pays the search's latency, then
+// waits at the barriers of each h iteration), or, in steps with few active
+// groups, split by its active particles into `nslices` consecutive slices, each
+// a warp's own work item (slice `slice`): no warp waits for another, and a
+// slice's sums are those the whole group would give (a particle's candidates
+// and their order do not depend on the particles it shares a warp with).  A
+// split group's leaves get their largest support from k_leaf_hmax, after every
+// slice is done.
 template <int G, bool UM>
 __device__ void density_group(const View &v, int wg, int slice, int nslices, int flags,
                               int bin_filter, int m_act, const CellFrame &F, float hcap, float exc,
@@ -507,10 +508,21 @@ __device__ void density_group(const View &v, int wg, int slice, int nslices, int
           }
         }
         if constexpr (G == 1) {
-          if (gath && acc > cap) {  // (the list filled up: one warp for this particle alone)
-            v.big[atomicAdd(&v.ds->n_big, 1)] = BigItem{lo, hi, h, i, it, wg};
-            wc.list_overflows++;
-            done = true;
+          const bool full = gath && acc > cap;  // (the list filled up: left to k_density_big)
+          const unsigned fm = __ballot_sync(FULL, full);
+          if (fm) {
+            const int k = __popc(fm);
+            int at = 0;
+            if (lane == 0) {
+              at = atomicAdd(&v.ds->n_big, k);
+              v.big_run[atomicAdd(&v.ds->n_big_runs, 1)] = at | (k - 1) << 24;
+            }
+            at = __shfl_sync(FULL, at, 0) + __popc(fm & ((1u << lane) - 1u));
+            if (full) {
+              v.big[at] = BigItem{lo, hi, h, i, it, wg};
+              wc.list_overflows++;
+              done = true;
+            }
           }
         }
         // the list this pass built (or, in the first pass, the one kept from
@@ -588,6 +600,39 @@ __device__ void density_group(const View &v, int wg, int slice, int nslices, int
   __syncwarp();
   if (writer && nslices == 1) leaf_hmax_update(v, W.L0, W.L1);
   __syncwarp();
+}
+
+// One iteration's end for a particle that k_density_big evaluates at h: the sums
+// give the next h, or, true, the results (written and counted if `write`).
+template <bool UM>
+__device__ bool settle(const View &v, int i, const float4 &xl, double sn, double stt, double s2,
+                       double sm, double smt, int ngb, int it, double Cw, float hcap, long long ti,
+                       bool init_entropy, bool write, float &h, double &lo, double &hi,
+                       WarpCounters &wc) {
+  const double hd = (double)h;
+  const double hn = next_h(hd, sn, stt, s2, Cw, lo, hi);
+  const bool conv = fabs(hn - hd) <= v.h_tol * hd;
+  const bool over = !conv && hn > (double)hcap;
+  if (!(conv || over || it == v.h_max_iter - 1)) {
+    h = (float)hn;
+    return false;
+  }
+  const double mu = UM ? (double)v.ds->m_uniform : 0.0;
+  const float sr = (float)(UM ? mu * sn : sm), srt = (float)(UM ? mu * stt : smt);
+  if (write) {
+    wc.pairs += (unsigned long long)ngb;
+    wc.iters += (unsigned long long)(it + 1);
+    if (over) {
+      wc.overflow++;
+      atomic_max_float_pos(&v.ds->want_h_bits, (float)hn);
+    } else if (!conv) {
+      wc.noconv++;
+    }
+    const float H = GAMMA_K * h;
+    write_density(v, i, xl, h, H, 1.0f / H, sr, srt, ti, init_entropy);
+    if (v.ngb_density) v.ngb_density[i] = ngb;
+  }
+  return true;
 }
 
 // A particle whose candidates did not fit its list (list_cap), by one warp:
@@ -685,35 +730,105 @@ __device__ void density_big(const View &v, const BigItem &b, int flags, const Ce
     const double part = (double)s_hi + (double)s_lo;
     const double sn = __shfl_sync(FULL, part, 0), stt = __shfl_sync(FULL, part, 1);
     const double s2 = (double)__shfl_sync(FULL, p2, 2);
-    const double hd = (double)h;
-    const double hn = next_h(hd, sn, stt, s2, Cw, lo, hi);
-    const bool conv = fabs(hn - hd) <= v.h_tol * hd;
-    const bool over = !conv && hn > (double)hcap;
-    if (conv || over || it == v.h_max_iter - 1) {
-      float sr, srt;
-      if constexpr (UM) {
-        const double mu = (double)v.ds->m_uniform;
-        sr = (float)(mu * sn);
-        srt = (float)(mu * stt);
-      } else {
-        sr = (float)__shfl_sync(FULL, part, 3);
-        srt = (float)__shfl_sync(FULL, part, 4);
-      }
-      if (lane == 0) {
-        wc.pairs += (unsigned long long)(cnt - 1);  // (the particle itself is among its candidates)
-        wc.iters += (unsigned long long)(it + 1);
-        if (over) {
-          wc.overflow++;
-          atomic_max_float_pos(&v.ds->want_h_bits, (float)hn);
-        } else if (!conv) {
-          wc.noconv++;
+    if (settle<UM>(v, i, xl, sn, stt, s2, __shfl_sync(FULL, part, 3), __shfl_sync(FULL, part, 4),
+                   cnt - 1, it, Cw, hcap, ti, (flags & SPH_DENSITY_INIT_ENTROPY) != 0, lane == 0, h, lo,
+                   hi, wc))
+      break;  // (the particle itself is among its candidates)
+  }
+}
+
+// A run of particles of one work group whose lists filled up, one per lane: each
+// iteration one pass over the group's candidates, every lane adding its own
+// neighbours up in record order as they are staged, without a list.
+template <bool UM>
+__device__ void density_wide(const View &v, int first, int count, int flags, float hcap, float exc,
+                             long long ti, StageD &st, WarpCounters &wc) {
+  const int lane = lane_id();
+  const BigItem b = v.big[first + (lane < count ? lane : 0)];
+  const CellFrame F = frame_of(v, v.ds, b.wg);
+  const Group W = group_of(v, b.wg, F);
+  const int i = b.i;
+  const double Cw = v.eta * v.eta * v.eta * GAMMA_K_D * GAMMA_K_D * GAMMA_K_D / (double)KERNEL_NORM;
+  const float qox = F.kx * F.wq, qoy = F.ky * F.wq, qoz = F.kz * F.wq;
+  const float clx = W.lx + qox, cly = W.ly + qoy, clz = W.lz + qoz;
+  const float chx = W.hx + qox, chy = W.hy + qoy, chz = W.hz + qoz;
+  const float4 xl = v.rec_xm[i];
+  const float3 lo3 = leaf_offset(v, i, F);
+  const float4 xi = make_float4(xl.x + lo3.x, xl.y + lo3.y, xl.z + lo3.z, xl.w);
+  const float4 *srcs[1] = {v.rec_xm};
+  unsigned *const masks = reinterpret_cast<unsigned *>(st.recj);  // (no tags here)
+  double lo = b.lo, hi = b.hi;
+  float h = b.h;
+  bool done = lane >= count;
+  for (int it = b.it; it < v.h_max_iter; it++) {
+    const float H = GAMMA_K * h, H2 = H * H, H4 = 4.0f * H2, Hinv = 1.0f / H;
+    const float R = warp_max(done ? 0.0f : H);
+    if (R == 0.0f) break;
+    DSum s;
+    s.zero();
+    const int nsph = compact_spheres(st.sph, !done, make_float4(xi.x, xi.y, xi.z, H));
+    const TestSet ts = test_set(st.tst, !done, xi.x, xi.y, xi.z, H2);
+    auto consume = [&](int base, int total) {
+      wc.cand += (unsigned long long)total * (unsigned long long)ts.n;
+      const int wend = (total + 31) >> 5;
+#pragma unroll 1
+      for (int q = 0; q < wend; q++)
+        test_masks<false>(st.tst, ts.n, st.rec[base + 32 * q + lane], 32 * q + lane < total,
+                          masks + 32 * q);
+      __syncwarp();
+      int left = 0, q = 0, kb = base - 1;
+      if (!done)
+        for (int w = 0; w < wend; w++) left += __popc(masks[32 * w + ts.rank]);
+      wc.evals += (unsigned long long)left;
+      unsigned cur = masks[ts.rank];
+      auto next = [&]() {
+        while (cur == 0u) {
+          q++;
+          kb += 32;
+          cur = masks[32 * q + ts.rank];
         }
-        write_density(v, i, xl, h, H, Hinv, sr, srt, ti, (flags & SPH_DENSITY_INIT_ENTROPY) != 0);
-        if (v.ngb_density) v.ngb_density[i] = cnt - 1;
+        const int k = kb + __ffs(cur);
+        cur &= cur - 1;
+        return st.rec[k];
+      };
+      for (; left > 0; left -= 2) {
+        const float4 pa = next();
+        float2 r2 = make_float2(0.0f, INFINITY), m = make_float2(pa.w, 0.0f);
+        float dx = xi.x - pa.x, dy = xi.y - pa.y, dz = xi.z - pa.z;
+        r2.x = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+        if (left > 1) {
+          const float4 pb = next();
+          dx = xi.x - pb.x, dy = xi.y - pb.y, dz = xi.z - pb.z;
+          r2.y = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+          m.y = pb.w;
+        }
+        dens_pair2<UM>(s, r2, m, H2, H4, Hinv);
       }
-      break;
-    }
-    h = (float)hn;
+    };
+    const float R2 = R * R * 1.0002f, Rc = R + 1e-5f * F.wf;
+    auto leaf_ok = [&](int l, float sx, float sy, float sz, LeafBox &lb) {
+      const float4 lo4 = v.leaf_lo[l], hi4 = v.leaf_hi[l];
+      lb = leaf_box(lo4, hi4, sx, sy, sz, 0.0f);
+      return box_gap2(W.lx, W.ly, W.lz, W.hx, W.hy, W.hz, lo4, hi4, sx, sy, sz) < R2;
+    };
+    auto chunk_ok = [&](int g, float sx, float sy, float sz) {
+      return box_gap2(clx, cly, clz, chx, chy, chz, v.chunk_lo[g], v.chunk_hi[g], sx, sy, sz) < Rc * Rc;
+    };
+    const Reach reach = {clx, cly, clz, chx, chy, chz, Rc, exc, st.sph, nsph, true};
+    int skip = 0;
+    bool more = false;
+    do {
+      const int nlist = search(v, F, reach, st, leaf_ok, chunk_ok, skip, more);
+      stage_list<false>(srcs, st, nlist, consume, wc);
+      skip += nlist;
+    } while (more && !st.failed);
+    if (st.failed) return;
+    wc.gathers += (unsigned)ts.n;
+    if (!done)
+      done = settle<UM>(v, i, xl, (double)s.s_hi.x + (double)s.s_lo.x, (double)s.s_hi.y + (double)s.s_lo.y,
+                        (double)s.p2, (double)s.m_hi.x + (double)s.m_lo.x,
+                        (double)s.m_hi.y + (double)s.m_lo.y, s.cnt - 1, it, Cw, hcap, ti,
+                        (flags & SPH_DENSITY_INIT_ENTROPY) != 0, true, h, lo, hi, wc);
   }
 }
 
@@ -1267,8 +1382,19 @@ __global__ void __launch_bounds__(PT, 2) k_density(View v, int flags, int bin_fi
   flush_counters(ds, wc, true);
 }
 
-// The particles the step's density launches left to one warp each, pulled from
-// head_big (none in most steps: the blocks return at once).
+// The particles whose lists filled up in the step's density launches, pulled
+// from head_big (none in most steps: the blocks return at once).  Few of them,
+// in clumps' surroundings, take a warp each: their time is that of the longest
+// iterations.  With at least BIG_MANY per warp of the grid -- a first guess of h
+// several times too large -- what counts is the work, and a run of at least
+// WIDE_LANES that filled up together takes one warp, a particle per lane.  A
+// warp each against a lane each (first step, jittered lattice, h guessed 2.5
+// times too large): 5.7 particles per warp of the grid 1.01 and 1.13 ms, 9.0 1.50 and
+// 1.38, 45 5.4 and 3.0, 108 12.1 and 5.8 ms (in passes of list_cap records, as
+// several lanes per particle take them, 2.6 and 5.1; guessed 4 times too large
+// 14 and 28, here 5.2 and 10); 302k clustered with the background's h for all, 33 and 11.7.  Runs of 8
+// to 15 as runs: 9.0 particles per warp 1.38 ms, particle by particle 1.98.
+constexpr int BIG_MANY = 8, WIDE_LANES = 8;
 template <bool UM>
 __global__ void __launch_bounds__(PT, 2) k_density_big(View v, int flags) {
   DevState *ds = v.ds;
@@ -1282,15 +1408,24 @@ __global__ void __launch_bounds__(PT, 2) k_density_big(View v, int flags) {
   StageD st;
   stage_init(st, max(v.stage_depth, 2), v.wait_limit);  // (one warp's work is a chain of latencies)
   const float hcap = (float)((ds->w - 2.0 * (double)exc) / GAMMA_K_D * (1.0 - 1e-6));
+  const bool many = nb / BIG_MANY >= (int)gridDim.x * WARPS_PER_BLOCK;
+  const int items = many ? ds->n_big_runs : nb;
   WarpCounters wc = {0, 0, 0, 0, 0, 0};
   for (;;) {
     int item = 0;
     if (lane == 0) item = atomicAdd(&ds->head_big, 1);
     item = __shfl_sync(FULL, item, 0);
-    if (item >= nb || st.failed) break;
-    const BigItem b = v.big[item];
-    if (!SPH_IN(ds, b.wg, ds->n_groups, SPH_CHECK_GROUP)) break;
-    density_big<UM>(v, b, flags, frame_of(v, ds, b.wg), hcap, exc, ds->ti, st, wc);
+    if (item >= items || st.failed) break;
+    const int run = many ? v.big_run[item] : item;
+    const int first = run & 0xffffff, count = (run >> 24) + 1;
+    const int wg = v.big[first].wg;
+    if (!SPH_IN(ds, wg, ds->n_groups, SPH_CHECK_GROUP)) break;
+    if (count >= WIDE_LANES) {
+      density_wide<UM>(v, first, count, flags, hcap, exc, ds->ti, st, wc);
+    } else {
+      for (int k = 0; k < count && !st.failed; k++)
+        density_big<UM>(v, v.big[first + k], flags, frame_of(v, ds, wg), hcap, exc, ds->ti, st, wc);
+    }
   }
   flush_counters(ds, wc, true);
 }
@@ -1370,11 +1505,11 @@ __global__ void __launch_bounds__(PT, 2) k_force(View v, int bin_filter, int per
 __global__ void __launch_bounds__(PT) k_leaf_hmax(View v) {
   DevState *ds = v.ds;
   const bool split = ds->dens_split > 1;
-  const int nq = split ? ds->n_active_groups + ds->n_heavy_groups : ds->n_big;
+  const int nq = split ? ds->n_active_groups + ds->n_heavy_groups : ds->n_big_runs;
   if (ds->halt) return;
   const int nw = (int)(gridDim.x * blockDim.x) >> 5;
   for (int k = (int)(blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < nq; k += nw) {
-    const int wg = split ? active_group(v, ds, k) : v.big[k].wg;
+    const int wg = split ? active_group(v, ds, k) : v.big[v.big_run[k] & 0xffffff].wg;
     if (!SPH_IN(ds, wg, ds->n_groups, SPH_CHECK_GROUP)) break;
     const int L0 = v.group_leaf0[wg], L1 = v.group_leaf0[wg + 1];
     // (checks build: a leaf range out of bounds is skipped, as group_of does)
