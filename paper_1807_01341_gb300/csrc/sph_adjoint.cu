@@ -860,9 +860,12 @@ struct GridKernel {
 // Where at least GD_LANES of a warp's particles have boxes of at most GD_FEW
 // points, those are one lane's work each, all at once: a warp per particle costs
 // some 20 FP64 instructions before its first point (27,000 particles on a 16^3
-// grid: 114 us, a lane per particle 75 us; here 74 us).  With 2 or 3 such particles in a
-// warp, clumps on a fine grid, the lanes' own way costs more (111k on 64^3: 737
-// against 462 us).
+// grid: 114 us, a lane per particle 75 us; here 74 us).  With fewer such particles
+// a point of a lane's own costs about as much as a particle of the warp's, and
+// the longest lane counts: lanes only for twice as many particles as points (a
+// support that misses most points, 1,000,000 particles on 16^3: 553 -> 285 us,
+// backward 836 -> 323; with as many lanes as points clumps on a fine grid, 111k on
+// 64^3, take 702 against 495 us).
 constexpr int GD_WARPS = 4, GD_SIDE = 32, GD_FEW = 27, GD_LANES = 16;
 struct GridWarp {
   double d[3][GD_SIDE];   // (x - x_g) / H along each axis
@@ -903,9 +906,13 @@ __global__ void __launch_bounds__(GD_WARPS * 32, 6)
     }
     double o[4] = {0.0, 0.0, 0.0, 0.0};  // BWD: this lane's particle
     // boxes of a few points: one lane per particle, all at once
-    bool few = na[0] > 0 && na[1] > 0 && na[2] > 0 && na[0] <= GD_FEW && na[1] <= GD_FEW &&
-               na[2] <= GD_FEW && na[0] * na[1] * na[2] <= GD_FEW;
-    if (__popc(__ballot_sync(FULL, few)) < GD_LANES) few = false;
+    const int box3 = na[0] > 0 && na[1] > 0 && na[2] > 0 && na[0] <= GD_FEW && na[1] <= GD_FEW &&
+                             na[2] <= GD_FEW
+                         ? na[0] * na[1] * na[2]
+                         : 0;
+    bool few = box3 > 0 && box3 <= GD_FEW;
+    const int lanes = __popc(__ballot_sync(FULL, few));
+    if (lanes < GD_LANES && 2 * __reduce_max_sync(FULL, few ? box3 : 0) > lanes) few = false;
     if (few) {
       const GridKernel<BWD> K(C, Hinv);
       for (int c = 0; c < na[2]; c++) {

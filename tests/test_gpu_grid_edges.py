@@ -55,3 +55,29 @@ def test_supports_without_a_point(env, n, ng, odd):
         got = getattr(adj, name).cpu().numpy()
         assert np.array_equal(got[off], np.full(off.sum(), k + 1.0)), name
         assert np.allclose(got[~off] - (k + 1.0), grad[k], rtol=1e-9, atol=1e-9 * np.abs(grad[k]).max())
+
+
+@pytest.mark.parametrize("n,ng,h_lo,h_hi", [(4099, 8, 0.01, 0.03), (2048, 5, 0.02, 0.05),
+                                            (3001, 16, 0.005, 0.02)])
+def test_boxes_of_a_point_or_none(env, n, ng, h_lo, h_hi):
+    """Supports narrower than the grid's spacing, most of which miss every
+    point: a few lanes of a warp with a point each."""
+    torch, sim = env
+    rng = np.random.default_rng(ng)
+    pos = rng.uniform(size=(n, 3))
+    pos[::500] = 0.5 / ng + rng.integers(0, ng, size=(len(pos[::500]), 3)) / ng
+    m = rng.uniform(0.5, 1.5, size=n).astype(np.float32)
+    h = rng.uniform(h_lo, h_hi, size=n).astype(np.float32)
+    bar = rng.normal(size=ng ** 3)
+    p = state(sim, torch, pos, m, h)
+    ctx = sim.Context(sim.Params(), n)
+    adj = sim.Adjoint(n)
+    rho = ctx.grid_density(p, ng, 0).cpu().numpy()
+    ctx.grid_density_bwd(p, ng, 0, torch.as_tensor(bar, device="cuda"), adj)
+    want, grad = direct(pos, m.astype(float), h.astype(float), bar, ng)
+    # sums of at most n positive terms; an offset's error, 2^-52 of the box, grows
+    # by 1 / H where the kernel falls off
+    tol = 4 * 2.0 ** -52 * (n + 30 / (1.825742 * h_lo))
+    assert np.abs(rho - want).max() <= tol * want.max()
+    for name, g in zip(("x", "y", "z", "h"), grad):
+        assert np.abs(getattr(adj, name).cpu().numpy() - g).max() <= tol * np.abs(g).max(), name
