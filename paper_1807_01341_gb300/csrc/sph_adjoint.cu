@@ -1043,7 +1043,10 @@ __global__ void __launch_bounds__(GD_WARPS * 32, 6)
 // Every load of a particle's ~25 arrays is issued before the first store (src
 // and dst could overlap as far as the compiler knows, and one array after the
 // other kept one load in flight per thread: 2.1M particles 130 -> 67 us,
-// 6.9 TB/s).  With a permutation the scattered stores bound it.
+// 6.9 TB/s).  With a permutation the scattered stores bound it, and of states far
+// larger than L2 they are slower out of one batch per thread: one array after the
+// other then (2.1M particles 1628 -> 1504 us, 1575 array by array in the
+// structure's order; at 600,000 the batch is ahead, 91 against 104 us).
 struct CopyFields {
   const unsigned long long *s8[6];
   unsigned long long *d8[6];
@@ -1053,27 +1056,38 @@ struct CopyFields {
   uint8_t *d1[2];
 };
 
+template <bool BATCH>
 __global__ void __launch_bounds__(256)
     k_state_copy(CopyFields f, long long n, const int32_t *__restrict__ perm) {
   for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
        k += (long long)gridDim.x * blockDim.x) {
     const long long d = perm ? (long long)perm[k] : k;
-    unsigned long long a[6];
-    unsigned int b[19];
-    uint8_t c[2];
+    if constexpr (BATCH) {
+      unsigned long long a[6];
+      unsigned int b[19];
+      uint8_t c[2];
 #pragma unroll
-    for (int q = 0; q < 6; q++) a[q] = f.s8[q][k];
+      for (int q = 0; q < 6; q++) a[q] = f.s8[q][k];
 #pragma unroll
-    for (int q = 0; q < 19; q++) b[q] = f.d4[q] ? f.s4[q][k] : 0u;
+      for (int q = 0; q < 19; q++) b[q] = f.d4[q] ? f.s4[q][k] : 0u;
 #pragma unroll
-    for (int q = 0; q < 2; q++) c[q] = f.s1[q][k];
+      for (int q = 0; q < 2; q++) c[q] = f.s1[q][k];
 #pragma unroll
-    for (int q = 0; q < 6; q++) f.d8[q][d] = a[q];
+      for (int q = 0; q < 6; q++) f.d8[q][d] = a[q];
 #pragma unroll
-    for (int q = 0; q < 19; q++)
-      if (f.d4[q]) f.d4[q][d] = b[q];
+      for (int q = 0; q < 19; q++)
+        if (f.d4[q]) f.d4[q][d] = b[q];
 #pragma unroll
-    for (int q = 0; q < 2; q++) f.d1[q][d] = c[q];
+      for (int q = 0; q < 2; q++) f.d1[q][d] = c[q];
+    } else {
+#pragma unroll
+      for (int q = 0; q < 6; q++) f.d8[q][d] = f.s8[q][k];
+#pragma unroll
+      for (int q = 0; q < 19; q++)
+        if (f.d4[q]) f.d4[q][d] = f.s4[q][k];
+#pragma unroll
+      for (int q = 0; q < 2; q++) f.d1[q][d] = f.s1[q][k];
+    }
   }
 }
 
@@ -1196,7 +1210,12 @@ cudaError_t launch_state_copy(const sph_particles &src, const sph_particles &dst
   f.s1[1] = src.active;
   f.d1[0] = (uint8_t *)dst.bin;
   f.d1[1] = dst.active;
-  k_state_copy<<<grid_for(src.n), 256, 0, st>>>(f, src.n, perm);
+  // (126 bytes a particle and state: one of 2^20 fills the 129 MB of L2; 1,000,003
+  // particles 407 us in batches, 391 array by array, without the optional arrays 254, 261)
+  if (perm && src.n > 1ll << 20)
+    k_state_copy<false><<<grid_for(src.n), 256, 0, st>>>(f, src.n, perm);
+  else
+    k_state_copy<true><<<grid_for(src.n), 256, 0, st>>>(f, src.n, perm);
   return cudaGetLastError();
 }
 

@@ -137,3 +137,33 @@ def test_refused_build(env, finer):
     ctx.resume(p, 0, True)
     ctx.step(p, 1)
     assert ctx.counters()["steps"] == 1
+
+
+@pytest.mark.parametrize("n", [1, 4097, 1 << 20, (1 << 20) + 5])
+@pytest.mark.parametrize("optional", [True, False])
+def test_copy_to_the_input_order(env, n, optional):
+    """Every array back in the order before the build, byte for byte."""
+    torch, sim = env
+    ctx = sim.Context(sim.Params(n_cells_override=30), n)
+    p = sim.Particles(n, with_counts=optional, with_gradients=optional)
+    g = torch.Generator(device="cuda").manual_seed(n)
+    p.storage.copy_(torch.randint(0, 256, p.storage.shape, generator=g, device="cuda",
+                                  dtype=torch.uint8))
+    for name in "xyz":
+        getattr(p, name).copy_(torch.rand(n, generator=g, device="cuda", dtype=torch.float64))
+    p.h.fill_(0.01)
+    p.m.fill_(1.0)
+    p.bin.remainder_(60)
+    p.rho.fill_(-1.0)  # (the build's refresh computes P and c where rho > 0)
+    before = host(p)
+    ctx.build_cells(p)
+    out = sim.Particles(n, with_counts=optional)
+    out.storage.fill_(7)
+    ctx.state_copy(p, out, True)
+    after = host(out)
+    for name, a in before.items():
+        if name != "active":
+            assert np.array_equal(a.view(np.uint8), after[name].view(np.uint8)), name
+    assert not after["active"].any()
+    if not optional:
+        assert (after["curl_v"].view(np.uint8) == 7).all()  # absent in one of the two: left alone
