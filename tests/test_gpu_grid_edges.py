@@ -81,3 +81,61 @@ def test_boxes_of_a_point_or_none(env, n, ng, h_lo, h_hi):
     assert np.abs(rho - want).max() <= tol * want.max()
     for name, g in zip(("x", "y", "z", "h"), grad):
         assert np.abs(getattr(adj, name).cpu().numpy() - g).max() <= tol * np.abs(g).max(), name
+
+
+def bounds(x, m, h, bar, ng):
+    """Direct sums as in `direct`, each with the sum of what its terms may be off:
+    a relative error of 16 roundings and one for each term added, and the
+    offsets' absolute error of 2^-52 of the box through the kernel's slope."""
+    eps = 2.0 ** -52
+    n = len(m)
+    rho, drho, grad, dgrad = np.zeros(ng ** 3), np.zeros(ng ** 3), np.zeros((4, n)), np.zeros((4, n))
+    c = (np.arange(ng) + 0.5) / ng
+    for j in range(n):
+        H = 1.825742 * h[j]
+        d = [v - np.round(v) for v in (x[j, a] - c for a in range(3))]
+        r2 = d[2][:, None, None] ** 2 + d[1][None, :, None] ** 2 + d[0][None, None, :] ** 2
+        k = np.nonzero(r2 < H * H * (1 + 1e-12))
+        r = np.sqrt(r2[k])
+        q = np.minimum(r / H, 1.0)
+        w = np.where(q < 0.5, 1 - 6 * q ** 2 + 6 * q ** 3, 2 * (1 - q) ** 3)
+        wq = np.where(q < 0.5, -12 + 18 * q, -6 * (1 - q) ** 2 / np.maximum(q, 0.5))  # w' / q
+        w2 = np.where(q < 0.5, np.abs(-12 + 36 * q), 12 * (1 - q))
+        at = k[2] + ng * (k[1] + ng * k[0])
+        C = m[j] * 2.5464790894703255 / H ** 3
+        off = 4 * eps / H  # of q
+        rho[at] += C * w
+        drho[at] += C * (eps * (16 + n) * w + off * np.abs(wq * q) + off ** 2 * 12)
+        t = bar[at] * C / H
+        big = np.abs(t) * (eps * (16 + len(q)) * np.abs(wq) * q + off * (np.abs(wq) + w2 + 12 * off))
+        for a, i in ((0, 2), (1, 1), (2, 0)):
+            grad[a, j] = (t * wq * d[a][k[i]] / H).sum()
+            dgrad[a, j] = big.sum()
+        t = bar[at] * C * 1.825742 / H
+        wh = 3 * w + q * q * wq
+        grad[3, j] = -(t * wh).sum()
+        dgrad[3, j] = (np.abs(t) * (eps * (16 + len(q)) * (3 * w + q * q * np.abs(wq)) +
+                                    off * (4 * np.abs(wq * q) + q * w2 + 48 * off))).sum()
+    return rho, drho, grad, dgrad
+
+
+@pytest.mark.parametrize("n,ng,h_lo,h_hi", [(33, 80, 0.1, 0.13), (40, 45, 1e-4, 0.25),
+                                            (700, 24, 1e-3, 0.2)])
+def test_each_point_and_particle(env, n, ng, h_lo, h_hi):
+    """Every grid point and every particle against the bound of its own terms,
+    narrow supports beside wide ones of many tiles."""
+    torch, sim = env
+    rng = np.random.default_rng(n * ng)
+    pos = rng.uniform(size=(n, 3))
+    h = np.exp(rng.uniform(np.log(h_lo), np.log(h_hi), size=n)).astype(np.float32)
+    m = rng.uniform(0.5, 1.5, size=n).astype(np.float32)
+    bar = rng.normal(size=ng ** 3)
+    p = state(sim, torch, pos, m, h)
+    ctx = sim.Context(sim.Params(), n)
+    adj = sim.Adjoint(n)
+    rho = ctx.grid_density(p, ng, 0).cpu().numpy()
+    ctx.grid_density_bwd(p, ng, 0, torch.as_tensor(bar, device="cuda"), adj)
+    want, drho, grad, dgrad = bounds(pos, m.astype(float), h.astype(float), bar, ng)
+    assert (np.abs(rho - want) <= drho).all()
+    for name, g, dg in zip(("x", "y", "z", "h"), grad, dgrad):
+        assert (np.abs(getattr(adj, name).cpu().numpy() - g) <= dg).all(), name
