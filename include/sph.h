@@ -439,7 +439,8 @@ typedef struct {
  * to_input_order = 0: plain copy.  to_input_order = 1: src is the state ctx
  * works on (sorted by its cell builds) and dst receives it in the order of
  * the first sph_build_cells call (dst[sph_perm[k]] = src[k]); src and dst must
- * not overlap.  NULL optional arrays (ngb_*) are skipped.  Used for checkpoints. */
+ * not overlap, and hold as many particles as the permutation (SPH_ERR_ARG
+ * otherwise).  NULL optional arrays (ngb_*) are skipped.  Used for checkpoints. */
 int sph_state_copy(const sph_ctx *ctx, const sph_particles *src, sph_particles *dst,
                    int to_input_order, void *stream);
 

@@ -102,6 +102,7 @@ struct sph_ctx {
   bool built = false;
   int cluster_most = 0;        // most particles that one cluster sorts (cluster_sort_max)
   long long n_perm = 0;        // particles that the composed permutation covers (0: none yet)
+  long long perm_span = 0;     // and one past its largest index (more, after a build of fewer)
   bool entropy_ready = false;  // the first density pass has converted u to A
   int nc = 0;
   double w = 0.0;
@@ -362,6 +363,12 @@ void prof_collect(sph_ctx *ctx) {
   }
 }
 
+// The arrays are in the order of a build of n particles.
+void set_perm(sph_ctx *ctx, long long n) {
+  ctx->perm_span = ctx->n_perm > 0 ? std::max(ctx->perm_span, n) : n;
+  ctx->n_perm = n;
+}
+
 int build_cells(sph_ctx *ctx, sph_particles *p, cudaStream_t st) {
   if (!valid_particles(ctx, p)) return SPH_ERR_ARG;
   ctx->fresh = false;
@@ -406,7 +413,7 @@ int build_cells(sph_ctx *ctx, sph_particles *p, cudaStream_t st) {
     // no cells, but the arrays are in the order that the permutation says: the
     // new one if the build got as far, else still the old one
     ctx->built = false;
-    if (h.build_moved) ctx->n_perm = n;
+    if (h.build_moved) set_perm(ctx, n);
     return (int)h.build_fail;
   }
   ctx->n_leaves = h.n_leaves;
@@ -415,7 +422,7 @@ int build_cells(sph_ctx *ctx, sph_particles *p, cudaStream_t st) {
   ctx->nc = nc;
   ctx->w = w;
   ctx->built = true;
-  ctx->n_perm = n;
+  set_perm(ctx, n);
   ctx->rebuilds++;
   return SPH_OK;
 }
@@ -1090,6 +1097,8 @@ int sph_state_copy(const sph_ctx *ctx, const sph_particles *src, sph_particles *
   if (!ctx || !valid_particles(ctx, src) || !valid_particles(ctx, dst) || src->n != dst->n)
     return SPH_ERR_ARG;
   const int32_t *perm = (to_input_order && ctx->n_perm > 0) ? ctx->b.perm : nullptr;
+  // (of another number of particles the permutation has entries missing or past the end)
+  if (perm && (src->n > ctx->n_perm || dst->n < ctx->perm_span)) return SPH_ERR_ARG;
   SPH_CUDA(launch_state_copy(*src, *dst, perm, S(stream)));
   return SPH_OK;
 }

@@ -167,3 +167,32 @@ def test_copy_to_the_input_order(env, n, optional):
     assert not after["active"].any()
     if not optional:
         assert (after["curl_v"].view(np.uint8) == 7).all()  # absent in one of the two: left alone
+
+
+def test_copy_of_another_number_of_particles(env):
+    """After builds of 3000 and then 1000 particles the permutation's indices
+    reach 2999: a copy into 1000 places is refused, and so is one of more
+    particles than it covers; a restart makes it fit again."""
+    torch, sim = env
+    from paper_1807_01341_gb300 import _lib
+    ctx = sim.Context(sim.Params(n_cells_override=5), 3000)
+    states = {}
+    for n in (3000, 1000):
+        p = states[n] = sim.Particles(n)
+        for name in "xyz":
+            getattr(p, name).uniform_()
+        p.m.copy_(torch.arange(n) + 1.0)
+        p.h.fill_(0.01)
+        ctx.build_cells(p)
+    for n in (1000, 3000):
+        out = sim.Particles(n)
+        with pytest.raises(_lib.SphError) as e:
+            ctx.state_copy(states[n], out, True)
+        assert e.value.code == _lib.SPH_ERR_ARG
+        assert not out.storage.any()
+    p = states[1000]
+    who = p.m.cpu().numpy()
+    ctx.resume(p, 0, True)
+    ctx.build_cells(p)
+    ctx.state_copy(p, out := sim.Particles(1000), True)
+    assert np.array_equal(out.m.cpu().numpy(), who)
