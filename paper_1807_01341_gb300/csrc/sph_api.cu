@@ -277,9 +277,8 @@ View make_view(const sph_ctx *ctx, const sph_particles *p) {
   v.uniform_mass = ctx->uniform_mass ? 1 : 0;
   v.grid_util = ctx->grid_util;
   v.nbr = b.nbr;
-  static_assert(sizeof(BigItem) + sizeof(int) <= BUILD_SCRATCH, "the items fit the build's scratch");
+  static_assert(sizeof(BigItem) <= BUILD_SCRATCH, "the items fit the build's scratch");
   v.big = reinterpret_cast<BigItem *>(b.scratch);
-  v.big_run = reinterpret_cast<int *>(v.big + ctx->n_max);
   v.list_cap = q.list_cap;
   v.list_blocks = ctx->list_blocks;
   v.search_margin = (float)q.search_margin;

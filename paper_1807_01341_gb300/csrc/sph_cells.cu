@@ -620,7 +620,7 @@ __device__ __forceinline__ void clear_queues(DevState *ds) {
   ds->n_active_cells = ds->n_drift_chunks = 0;
   ds->n_bin_groups = ds->n_bin_coop = 0;
   ds->n_wake = 0;
-  ds->n_big = ds->n_big_runs = ds->head_big = ds->dens_split = 0;
+  ds->n_big = ds->head_big = ds->dens_split = 0;
 }
 
 // Words 0-11 the 8-byte arrays, 12-30 the 4-byte ones (the mass first), 31 the

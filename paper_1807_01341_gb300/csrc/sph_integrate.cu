@@ -109,7 +109,7 @@ __global__ void k_begin_step(View v, long long ti_arg) {
   ds->head_density = ds->head_force = ds->head_drift = ds->head_kick = 0;
   ds->head_open = ds->head_bins = ds->head_misc = 0;
   ds->head_coop_force = ds->head_grad = 0;
-  ds->n_big = ds->n_big_runs = ds->head_big = ds->dens_split = 0;
+  ds->n_big = ds->head_big = ds->dens_split = 0;
   ds->n_wake = 0;
   ds->s_pairs_density = ds->s_pairs_force = 0ull;
   ds->s_cand_density = ds->s_cand_force = 0ull;

@@ -71,7 +71,7 @@ struct DevState {
   unsigned int Hmax_bits;       // max kernel support H (float bits) over all particles
   unsigned int want_h_bits;     // largest h an iteration wanted beyond the cell limit
   int dens_split;               // parts per work group of the last whole-step density launch
-  int n_big, n_big_runs;  // density loop: particles whose list filled up (View::big), and their runs
+  int n_big;              // density loop: particles whose list filled up (View::big)
   int head_big;           // work head of those
   // counters of the step in progress (reset when a step starts, added to the
   // totals when it completes, so a halted attempt leaves no trace)
@@ -97,7 +97,7 @@ struct DevState {
 constexpr int BUILD_WORDS = 5;
 
 // A particle that the density loop leaves to k_density_big: the state of its
-// h iteration and its work group (the same in a run).
+// h iteration and its work group.
 struct BigItem {
   double lo, hi;  // bracket
   float h;
@@ -166,7 +166,6 @@ struct View {
   // next work group, so the lists stay in L2.
   float2 *nbr;
   BigItem *big;              // [n] (the build's scratch, free between builds)
-  int *big_run;              // [n] runs of `big` left by one warp together: first | count - 1 << 24
   DevState *ds;
   // parameters
   double box, eta, gamma, alpha, cfl, h_tol, dt_min;

@@ -508,21 +508,10 @@ __device__ void density_group(const View &v, int wg, int slice, int nslices, int
           }
         }
         if constexpr (G == 1) {
-          const bool full = gath && acc > cap;  // (the list filled up: left to k_density_big)
-          const unsigned fm = __ballot_sync(FULL, full);
-          if (fm) {
-            const int k = __popc(fm);
-            int at = 0;
-            if (lane == 0) {
-              at = atomicAdd(&v.ds->n_big, k);
-              v.big_run[atomicAdd(&v.ds->n_big_runs, 1)] = at | (k - 1) << 24;
-            }
-            at = __shfl_sync(FULL, at, 0) + __popc(fm & ((1u << lane) - 1u));
-            if (full) {
-              v.big[at] = BigItem{lo, hi, h, i, it, wg};
-              wc.list_overflows++;
-              done = true;
-            }
+          if (gath && acc > cap) {  // (the list filled up: left to k_density_big)
+            v.big[atomicAdd(&v.ds->n_big, 1)] = BigItem{lo, hi, h, i, it, wg};
+            wc.list_overflows++;
+            done = true;
           }
         }
         // the list this pass built (or, in the first pass, the one kept from
@@ -737,9 +726,9 @@ __device__ void density_big(const View &v, const BigItem &b, int flags, const Ce
   }
 }
 
-// A run of particles of one work group whose lists filled up, one per lane: each
-// iteration one pass over the group's candidates, every lane adding its own
-// neighbours up in record order as they are staged, without a list.
+// A run of particles of one work group (at most 32) whose lists filled up, one per
+// lane: each iteration one pass over the group's candidates, every lane adding its
+// own neighbours up in record order as they are staged, without a list.
 template <bool UM>
 __device__ void density_wide(const View &v, int first, int count, int flags, float hcap, float exc,
                              long long ti, StageD &st, WarpCounters &wc) {
@@ -759,8 +748,8 @@ __device__ void density_wide(const View &v, int first, int count, int flags, flo
   unsigned *const masks = reinterpret_cast<unsigned *>(st.recj);  // (no tags here)
   double lo = b.lo, hi = b.hi;
   float h = b.h;
-  bool done = lane >= count;
-  for (int it = b.it; it < v.h_max_iter; it++) {
+  bool done = lane >= count || b.it >= v.h_max_iter;
+  for (int it = b.it;; it++) {  // (a lane's own count: a group's slices need not agree)
     const float H = GAMMA_K * h, H2 = H * H, H4 = 4.0f * H2, Hinv = 1.0f / H;
     const float R = warp_max(done ? 0.0f : H);
     if (R == 0.0f) break;
@@ -1387,14 +1376,21 @@ __global__ void __launch_bounds__(PT, 2) k_density(View v, int flags, int bin_fi
 // in clumps' surroundings, take a warp each: their time is that of the longest
 // iterations.  With at least BIG_MANY per warp of the grid -- a first guess of h
 // several times too large -- what counts is the work, and a run of at least
-// WIDE_LANES that filled up together takes one warp, a particle per lane.  A
-// warp each against a lane each (first step, jittered lattice, h guessed 2.5
-// times too large): 5.7 particles per warp of the grid 1.01 and 1.13 ms, 9.0 1.50 and
-// 1.38, 45 5.4 and 3.0, 108 12.1 and 5.8 ms (in passes of list_cap records, as
-// several lanes per particle take them, 2.6 and 5.1; guessed 4 times too large
-// 14 and 28, here 5.2 and 10); 302k clustered with the background's h for all, 33 and 11.7.  Runs of 8
-// to 15 as runs: 9.0 particles per warp 1.38 ms, particle by particle 1.98.
-constexpr int BIG_MANY = 8, WIDE_LANES = 8;
+// WIDE_LANES entries of one work group (the lanes of a warp enter their
+// particles side by side) takes one warp, a particle per lane.  A warp each
+// against a lane each (first step of a jittered lattice, h guessed 2.5 times too
+// large): 5.7 particles per warp of the grid 1.01 and 1.13 ms, 9.0 1.50 and
+// 1.33, 45 5.4 and 3.0, 108 12.1 and 5.8 ms (in passes of list_cap records, as
+// several lanes per particle take them, the last two 2.6 and 5.1; with h 4 times
+// too large 14 and 28, here 5.2 and 10); 302k clustered particles with the
+// background's h for all, 33 and 11.6.  Runs of 8 to 15 as runs: 9.0 particles
+// per warp 1.38 ms, particle by particle 1.98.
+//
+// A warp claims RUN_STEP entries and takes the runs that start among them: with
+// 32, three runs of 10 one after the other, 9.0 particles per warp took 2.5 ms,
+// with 8 1.53, with 4 1.33.  (Runs marked by the density loop as it enters the
+// particles give the same times here, but its all-active launches 0.5 % more.)
+constexpr int BIG_MANY = 8, WIDE_LANES = 8, RUN_STEP = 4;
 template <bool UM>
 __global__ void __launch_bounds__(PT, 2) k_density_big(View v, int flags) {
   DevState *ds = v.ds;
@@ -1409,22 +1405,45 @@ __global__ void __launch_bounds__(PT, 2) k_density_big(View v, int flags) {
   stage_init(st, max(v.stage_depth, 2), v.wait_limit);  // (one warp's work is a chain of latencies)
   const float hcap = (float)((ds->w - 2.0 * (double)exc) / GAMMA_K_D * (1.0 - 1e-6));
   const bool many = nb / BIG_MANY >= (int)gridDim.x * WARPS_PER_BLOCK;
-  const int items = many ? ds->n_big_runs : nb;
+  const int items = many ? (nb + RUN_STEP - 1) / RUN_STEP : nb;
   WarpCounters wc = {0, 0, 0, 0, 0, 0};
   for (;;) {
     int item = 0;
     if (lane == 0) item = atomicAdd(&ds->head_big, 1);
     item = __shfl_sync(FULL, item, 0);
     if (item >= items || st.failed) break;
-    const int run = many ? v.big_run[item] : item;
-    const int first = run & 0xffffff, count = (run >> 24) + 1;
-    const int wg = v.big[first].wg;
-    if (!SPH_IN(ds, wg, ds->n_groups, SPH_CHECK_GROUP)) break;
-    if (count >= WIDE_LANES) {
-      density_wide<UM>(v, first, count, flags, hcap, exc, ds->ti, st, wc);
-    } else {
-      for (int k = 0; k < count && !st.failed; k++)
-        density_big<UM>(v, v.big[first + k], flags, frame_of(v, ds, wg), hcap, exc, ds->ti, st, wc);
+    if (!many) {
+      const BigItem b = v.big[item];
+      if (!SPH_IN(ds, b.wg, ds->n_groups, SPH_CHECK_GROUP)) break;
+      density_big<UM>(v, b, flags, frame_of(v, ds, b.wg), hcap, exc, ds->ti, st, wc);
+      continue;
+    }
+    // the runs of equal work groups that start among RUN_STEP entries (a group holds
+    // at most 32 particles, each entered once a step)
+    const int base = item * RUN_STEP, k0 = base + lane;
+    const int wg = k0 < nb ? v.big[k0].wg : -1, wg1 = k0 + 32 < nb ? v.big[k0 + 32].wg : -1;
+    int prev = __shfl_up_sync(FULL, wg, 1), prev1 = __shfl_up_sync(FULL, wg1, 1);
+    const int last = __shfl_sync(FULL, wg, 31);
+    if (lane == 0) {
+      prev = item > 0 ? v.big[k0 - 1].wg : -1;
+      prev1 = last;
+    }
+    unsigned starts = __ballot_sync(FULL, lane < RUN_STEP && wg >= 0 && wg != prev);
+    const unsigned ends = __ballot_sync(FULL, wg != prev), ends1 = __ballot_sync(FULL, wg1 != prev1);
+    for (; starts && !st.failed; starts &= starts - 1u) {
+      const int s = __ffs(starts) - 1;
+      const unsigned rest = s < 31 ? ends >> (s + 1) : 0u;
+      const int e = rest ? s + __ffs(rest) : 32 + (ends1 ? __ffs(ends1) - 1 : 32);
+      const int first = base + s, count = min(e, nb - base) - s;
+      if (!SPH_IN(ds, __shfl_sync(FULL, wg, s), ds->n_groups, SPH_CHECK_GROUP)) continue;
+      if (count >= WIDE_LANES) {
+        density_wide<UM>(v, first, count, flags, hcap, exc, ds->ti, st, wc);
+      } else {
+        for (int k = 0; k < count && !st.failed; k++) {
+          const BigItem b = v.big[first + k];
+          density_big<UM>(v, b, flags, frame_of(v, ds, b.wg), hcap, exc, ds->ti, st, wc);
+        }
+      }
     }
   }
   flush_counters(ds, wc, true);
@@ -1505,11 +1524,12 @@ __global__ void __launch_bounds__(PT, 2) k_force(View v, int bin_filter, int per
 __global__ void __launch_bounds__(PT) k_leaf_hmax(View v) {
   DevState *ds = v.ds;
   const bool split = ds->dens_split > 1;
-  const int nq = split ? ds->n_active_groups + ds->n_heavy_groups : ds->n_big_runs;
+  const int nq = split ? ds->n_active_groups + ds->n_heavy_groups : ds->n_big;
   if (ds->halt) return;
   const int nw = (int)(gridDim.x * blockDim.x) >> 5;
   for (int k = (int)(blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < nq; k += nw) {
-    const int wg = split ? active_group(v, ds, k) : v.big[v.big_run[k] & 0xffffff].wg;
+    const int wg = split ? active_group(v, ds, k) : v.big[k].wg;
+    if (!split && k > 0 && v.big[k - 1].wg == wg) continue;  // (its neighbour in the queue did it)
     if (!SPH_IN(ds, wg, ds->n_groups, SPH_CHECK_GROUP)) break;
     const int L0 = v.group_leaf0[wg], L1 = v.group_leaf0[wg + 1];
     // (checks build: a leaf range out of bounds is skipped, as group_of does)
