@@ -1113,7 +1113,8 @@ inline int blocks_for(long long n, int t) { return (int)((n + t - 1) / t); }
 inline int tiles_of(long long n) { return (int)((n + TILE - 1) / TILE); }
 inline int passes_of(int nbits) { return (nbits + 7) / 8; }
 
-// The sort's scratch: [tickets 7][totals 7 x 256][status rows 2 x tiles x 256]
+// The sort's scratch: [tickets 7, one unused][totals 7 x 256][status rows 2 x tiles x 256]
+// (a row's sectors whole: shifted by a word the passes of 913k pairs take 93 us, not 88)
 struct SortWork {
   unsigned int *ticket, *totals, *row[2];
   size_t zero_words;  // from `ticket` on, zero before the keys are counted
@@ -1122,7 +1123,7 @@ SortWork sort_work(unsigned int *w, int n_tiles) {
   SortWork s;
   const size_t row = (size_t)n_tiles * RS_DIGITS;
   s.ticket = w;
-  s.totals = w + RS_PASSES_MAX;
+  s.totals = w + RS_PASSES_MAX + 1;
   s.row[0] = s.totals + RS_PASSES_MAX * RS_DIGITS;
   s.row[1] = s.row[0] + row;
   s.zero_words = (size_t)(s.row[1] - w);
@@ -1261,7 +1262,7 @@ cudaError_t radix_sort_indices(unsigned long long *keys, unsigned int *vals,
 
 size_t build_work_words(long long n) {
   const long long t = tiles_of(std::max<long long>(n, 1));
-  return 4 + 4 * (size_t)t + RS_PASSES_MAX * (1 + RS_DIGITS) +
+  return 4 + 4 * (size_t)t + (RS_PASSES_MAX + 1 + RS_PASSES_MAX * RS_DIGITS) +
          2 * (size_t)t * RS_DIGITS;
 }
 
