@@ -856,7 +856,9 @@ struct GridKernel {
 // backward 3385 -> 787 us; 262,144 on 32^3 209 -> 182 us and 314 -> 220 us;
 // 2,744 on 128^3 (supports of 40,000 points) 153 -> 2.5 ms and 182 -> 4.3 ms.
 // Against extended precision a point's W is off by 4.0e-17 rms (before 4.5e-17),
-// its d/dh by 1.1e-16 (1.5e-16).
+// its d/dh by 1.1e-16 (1.5e-16).  Against 64-bit sums of the textbook form
+// (r / H, then the two cubics), whose roundings the form before shared, the
+// distance grew: densities and adjoints of a clumpy set 2.9e-16 -> 5.3e-16.
 // Where at least GD_LANES of a warp's particles have boxes of at most GD_FEW
 // points, those are one lane's work each, all at once: a warp per particle costs
 // some 20 FP64 instructions before its first point (27,000 particles on a 16^3

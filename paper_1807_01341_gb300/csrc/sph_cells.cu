@@ -11,9 +11,10 @@
 //
 // A build is a fixed chain of launches whose sizes live on the device (no
 // host read between the keys and the finished structure): keys, one launch
-// per 8-bit digit (up to 65,536 particles one for all of them), one gather of every particle array into scratch and one
-// copy back, one pass that splits every octree node and one compaction, for
-// the particles (leaves) and again for the leaves (chunks and work groups).
+// per 8-bit digit (up to 65,536 particles one for all of them), every particle
+// packed into a record and the records unpacked in the new order, one pass that
+// splits every octree node and one compaction, for the particles (leaves) and
+// again for the leaves (chunks and work groups).
 #include <cooperative_groups.h>
 
 #include <algorithm>

@@ -35,7 +35,7 @@ struct DevState {
   int nc;                // cells per axis
   int n_cells;           // nc^3
   int n_leaves;
-  int n_chunks;          // octree nodes of up to CHUNK leaves of one cell (see launch_chunks)
+  int n_chunks;          // octree nodes of up to CHUNK leaves of one cell
   int n_groups;          // work groups: runs of consecutive leaves of one cell, <= WG_MAX particles
   int n_active_groups;   // work groups holding active particles (light ones from the front of
                          // q_group, heavy ones from its back; see n_heavy_groups)
@@ -142,7 +142,7 @@ struct View {
   int32_t *pleaf;            // [n] leaf of each particle
   int32_t *group_leaf0;      // [n_groups + 1] first leaf of each work group
   int32_t *group_cell;       // [n_groups] cell of each work group
-  int32_t *group_cost;       // [n_groups] estimated neighbour records of one search (at build)
+  int32_t *group_cost;       // [n_groups] particles of the cells and chunks one search reaches (at build)
   // FP32 records read by the pair loops (cell-relative positions)
   float4 *rec_xm;  // x, y, z, m
   float4 *rec_xH;  // x, y, z, H

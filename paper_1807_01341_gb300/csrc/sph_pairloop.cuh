@@ -811,7 +811,7 @@ __device__ __forceinline__ void stage_list(const float4 *const *srcs,
 
 using StageD = Stage<S_DENS, 1, 320>;
 // the forward force loop (S_PAIR staged candidates per warp): two blocks of 8
-// warps fill an SM's shared memory (14,464 bytes a warp); the variants' tags
+// warps fill an SM's shared memory (14,416 bytes a warp); the variants' tags
 // cost room for 48 leaves
 constexpr int S_PAIR = 192;
 template <bool VAR>
