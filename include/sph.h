@@ -344,6 +344,10 @@ int sph_diagnostics(sph_ctx *ctx, const sph_particles *p, int64_t ti, double *ou
 
 /* Current and next tick of the device-resident timeline (synchronising). */
 int sph_get_time(sph_ctx *ctx, int64_t *ti_current, int64_t *ti_next);
+/* The same two ticks as the last sph_step_sync, sph_step or sph_step_graph of
+ * this context read them when its steps had ended, without a read of the device: what
+ * was enqueued since (a caller's own graph among it) does not show. */
+int sph_synced_time(const sph_ctx *ctx, int64_t *ti_current, int64_t *ti_next);
 /* Set the device-resident current tick (asynchronous). */
 int sph_set_time(sph_ctx *ctx, int64_t ti_current, void *stream);
 

@@ -118,6 +118,7 @@ def load(path: str = None):
     L.sph_step.argtypes = [_vp, P(sph_particles), _i, _vp]
     L.sph_step_graph.argtypes = [_vp, P(sph_particles), _i, _vp]
     L.sph_get_time.argtypes = [_vp, P(_i64), P(_i64)]
+    L.sph_synced_time.argtypes = [_vp, P(_i64), P(_i64)]
     L.sph_set_time.argtypes = [_vp, _i64, _vp]
     L.sph_get_status.argtypes = [_vp, P(_i), P(_i64)]
     L.sph_clear_status.argtypes = [_vp, _vp]
@@ -143,7 +144,7 @@ def load(path: str = None):
     for name in ("sph_create", "sph_destroy", "sph_build_cells", "sph_grid_info",
                  "sph_mark_active", "sph_kick_drift", "sph_density_active", "sph_force_active",
                  "sph_timestep_bins", "sph_begin_run", "sph_step_async", "sph_step_sync",
-                 "sph_step", "sph_step_graph", "sph_get_time",
+                 "sph_step", "sph_step_graph", "sph_get_time", "sph_synced_time",
                  "sph_set_time", "sph_get_status", "sph_clear_status", "sph_get_counters",
                  "sph_reset_counters", "sph_set_profiling", "sph_get_kernel_times",
                  "sph_reset_kernel_times", "sph_state_copy", "sph_resume", "sph_grid_density",
@@ -160,7 +161,7 @@ def exported_symbols():
             "sph_grid_info", "sph_mark_active", "sph_kick_drift", "sph_density_active",
             "sph_force_active", "sph_timestep_bins", "sph_begin_run", "sph_step_async",
             "sph_step_sync", "sph_step", "sph_step_graph",
-            "sph_get_time", "sph_set_time", "sph_get_status", "sph_clear_status",
+            "sph_get_time", "sph_synced_time", "sph_set_time", "sph_get_status", "sph_clear_status",
             "sph_get_counters", "sph_reset_counters", "sph_set_profiling",
             "sph_get_kernel_times", "sph_reset_kernel_times", "sph_cell_order_noalloc",
             "sph_state_copy", "sph_resume", "sph_grid_density", "sph_grid_density_bwd",

@@ -70,7 +70,7 @@ class Run:
         return s
 
     def _next_tick(self) -> int:
-        return self.ctx.get_time()[1]
+        return self.ctx.synced_time()[1]  # (of the step just taken)
 
     # -- forward -----------------------------------------------------------
     def forward(self, pos0: torch.Tensor, vel0: torch.Tensor, u0: torch.Tensor) -> torch.Tensor:

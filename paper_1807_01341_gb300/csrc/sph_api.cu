@@ -112,8 +112,7 @@ struct sph_ctx {
   long long rebuilds = 0, redone = 0;
   long long steps_seen = 0;    // device step counter at the last sph_step_sync
   int pending = 0;             // steps enqueued since the last sph_step_sync
-  bool fresh = false;          // the host mirror of the device state is current (nothing that
-                               // changes it was enqueued since sph_step_sync read it)
+  long long synced_ti[2] = {0, 0};  // current and next tick as the last sph_step_sync read them
   bool init_pending = false;   // the entropy-initialising step is enqueued, not yet confirmed
   // optional CUDA-event timing of the pair-loop launches (0 density, 1 force)
   bool prof_on = false;
@@ -370,7 +369,6 @@ void set_perm(sph_ctx *ctx, long long n) {
 
 int build_cells(sph_ctx *ctx, sph_particles *p, cudaStream_t st) {
   if (!valid_particles(ctx, p)) return SPH_ERR_ARG;
-  ctx->fresh = false;
   Buffers &b = ctx->b;
   const long long n = p->n;
   if (n > BUILD_MAX) return SPH_ERR_CUDA;
@@ -428,7 +426,6 @@ int build_cells(sph_ctx *ctx, sph_particles *p, cudaStream_t st) {
 
 // Sets the current and next tick (ti >= 0) and clears the status, one launch.
 int set_state(sph_ctx *ctx, long long ti, bool clear, cudaStream_t st) {
-  ctx->fresh = false;
   SPH_CUDA(launch_set_state(ctx->b.ds, ti, clear, st));
   // (a halted step may have left wake requests that its close never applied)
   if (clear && ctx->prm.limiter && ctx->n_max > 0)
@@ -833,7 +830,6 @@ int sph_grid_info(const sph_ctx *ctx, int *nc, int *n_leaves) {
 
 int sph_mark_active(sph_ctx *ctx, sph_particles *p, int64_t ti_current, void *stream) {
   if (!ctx || !valid_particles(ctx, p)) return SPH_ERR_ARG;
-  ctx->fresh = false;
   if (!ctx->built) return SPH_ERR_NOT_BUILT;
   SPH_CUDA(launch_mark(make_view(ctx, p), ti_current < 0 ? -1 : ti_current, S(stream)));
   return SPH_OK;
@@ -841,7 +837,6 @@ int sph_mark_active(sph_ctx *ctx, sph_particles *p, int64_t ti_current, void *st
 
 int sph_kick_drift(sph_ctx *ctx, sph_particles *p, int phase, void *stream) {
   if (!ctx || !valid_particles(ctx, p)) return SPH_ERR_ARG;
-  ctx->fresh = false;
   if (!ctx->built) return SPH_ERR_NOT_BUILT;
   View v = make_view(ctx, p);
   switch (phase) {
@@ -855,7 +850,6 @@ int sph_kick_drift(sph_ctx *ctx, sph_particles *p, int phase, void *stream) {
 
 int sph_density_active(sph_ctx *ctx, sph_particles *p, int flags, void *stream) {
   if (!ctx || !valid_particles(ctx, p)) return SPH_ERR_ARG;
-  ctx->fresh = false;
   if (!ctx->built) return SPH_ERR_NOT_BUILT;
   View v = make_view(ctx, p);
   SPH_CUDA(launch_density(v, flags, -1, true, ctx->grid_dens, S(stream)));
@@ -867,7 +861,6 @@ int sph_density_active(sph_ctx *ctx, sph_particles *p, int flags, void *stream) 
 
 int sph_force_active(sph_ctx *ctx, sph_particles *p, void *stream) {
   if (!ctx || !valid_particles(ctx, p)) return SPH_ERR_ARG;
-  ctx->fresh = false;
   if (!ctx->built) return SPH_ERR_NOT_BUILT;
   SPH_CUDA(launch_force(make_view(ctx, p), -1, true, ctx->grid_force, S(stream)));
   return SPH_OK;
@@ -875,7 +868,6 @@ int sph_force_active(sph_ctx *ctx, sph_particles *p, void *stream) {
 
 int sph_timestep_bins(sph_ctx *ctx, sph_particles *p, int64_t *ti_next_dev, void *stream) {
   if (!ctx || !valid_particles(ctx, p)) return SPH_ERR_ARG;
-  ctx->fresh = false;
   if (!ctx->built) return SPH_ERR_NOT_BUILT;
   SPH_CUDA(launch_bins(make_view(ctx, p), reinterpret_cast<long long *>(ti_next_dev), 0, S(stream)));
   return SPH_OK;
@@ -896,7 +888,6 @@ int sph_step_async(sph_ctx *ctx, sph_particles *p, int form, void *stream) {
   if (!ctx || !valid_particles(ctx, p) ||
       (form != SPH_FORM_PLAIN && form != SPH_FORM_BATCHED && form != SPH_FORM_BATCHED_NOGRAPH))
     return SPH_ERR_ARG;
-  ctx->fresh = false;
   cudaStream_t st = S(stream);
   if (!ctx->built) SPH_TRY(build_cells(ctx, p, st));
   View v = make_view(ctx, p);
@@ -937,9 +928,10 @@ int sph_step_sync(sph_ctx *ctx, sph_particles *p, int *completed, void *stream) 
   if (ctx->init_pending && done == 0) ctx->entropy_ready = false;  // the first step must rerun
   if (done > 0) ctx->init_pending = false;
   ctx->pending = 0;
+  ctx->synced_ti[0] = ctx->b.h_ds->ti;
+  ctx->synced_ti[1] = ctx->b.h_ds->ti_next;
   bool redo = false;
   SPH_TRY(recover(ctx, p, st, &redo));
-  ctx->fresh = !redo;
   return SPH_OK;
 }
 
@@ -968,10 +960,16 @@ int sph_step_graph(sph_ctx *ctx, sph_particles *p, int n_steps, void *stream) {
 
 int sph_get_time(sph_ctx *ctx, int64_t *ti_current, int64_t *ti_next) {
   if (!ctx) return SPH_ERR_ARG;
-  if (!ctx->fresh)
-    SPH_CUDA(cudaMemcpy(ctx->b.h_ds, ctx->b.ds, sizeof(DevState), cudaMemcpyDeviceToHost));
+  SPH_CUDA(cudaMemcpy(ctx->b.h_ds, ctx->b.ds, sizeof(DevState), cudaMemcpyDeviceToHost));
   if (ti_current) *ti_current = ctx->b.h_ds->ti;
   if (ti_next) *ti_next = ctx->b.h_ds->ti_next;
+  return SPH_OK;
+}
+
+int sph_synced_time(const sph_ctx *ctx, int64_t *ti_current, int64_t *ti_next) {
+  if (!ctx) return SPH_ERR_ARG;
+  if (ti_current) *ti_current = ctx->synced_ti[0];
+  if (ti_next) *ti_next = ctx->synced_ti[1];
   return SPH_OK;
 }
 
@@ -1049,7 +1047,6 @@ int sph_get_bin_counts(sph_ctx *ctx, int64_t *counts, int n_bins, void *stream) 
 int sph_reset_counters(sph_ctx *ctx, void *stream) {
   if (!ctx) return SPH_ERR_ARG;
   cudaStream_t st = S(stream);
-  ctx->fresh = false;
   const size_t off = offsetof(DevState, s_pairs_density);
   const size_t len = offsetof(DevState, bin_count) - off;
   SPH_CUDA(cudaMemsetAsync(reinterpret_cast<char *>(ctx->b.ds) + off, 0, len, st));

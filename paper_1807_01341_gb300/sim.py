@@ -283,6 +283,13 @@ class Context:
         check(self.L.sph_get_time(self.h, ctypes.byref(a), ctypes.byref(b)), "sph_get_time")
         return a.value, b.value
 
+    def synced_time(self):
+        """get_time as of the last synchronising step call, without a read of
+        the device."""
+        a, b = ctypes.c_int64(), ctypes.c_int64()
+        check(self.L.sph_synced_time(self.h, ctypes.byref(a), ctypes.byref(b)), "sph_synced_time")
+        return a.value, b.value
+
     def set_time(self, ti: int, stream=None):
         check(self.L.sph_set_time(self.h, int(ti), _stream_ptr(stream)), "sph_set_time")
 
