@@ -104,6 +104,9 @@ class Particles:
         offs = self.__dict__.get("_offs")
         if offs is None or name not in offs:
             raise AttributeError(name)
+        if torch.is_inference_mode_enabled():  # (the state outlives the mode of its first use)
+            with torch.inference_mode(False):
+                return self.__getattr__(name)
         dt = _FIELD_TYPE[name]
         nbytes = self._count * _ITEMSIZE[dt]
         view = self._buffer[offs[name]:offs[name] + nbytes].view(_TORCH[dt])

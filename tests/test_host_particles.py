@@ -33,3 +33,19 @@ def test_absent_arrays_and_copies():
     assert p.struct().ngb_force is None
     q.h.fill_(3.0)
     assert float(p.h.sum()) == 0.0 and float(q.h.sum()) == 15.0
+
+
+@pytest.mark.parametrize("mode", [torch.inference_mode, torch.no_grad])
+def test_first_use_inside_a_mode(mode):
+    """An array first asked for inside inference mode is an ordinary tensor."""
+    from paper_1807_01341_gb300 import sim
+    p = sim.Particles(6, device="cpu")
+    with mode():
+        assert float(p.h.sum()) == 0.0
+        p.x.fill_(2.0)
+    assert not p.h.is_inference()
+    p.h.copy_(torch.ones(6))
+    p.x[0] = 5.0
+    w = torch.ones(6, requires_grad=True)
+    (p.h * w).sum().backward()
+    assert torch.equal(w.grad, p.h) and float(p.x.sum()) == 15.0
