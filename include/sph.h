@@ -222,7 +222,10 @@ typedef struct {
 void sph_default_params(sph_params *p);
 
 /* Create a context for up to n_max particles on the current CUDA device.
- * Allocates the library's scratch.  Errors: SPH_ERR_ARG, SPH_ERR_NOMEM. */
+ * Allocates the library's scratch: 361 bytes per particle of n_max (131 of them
+ * the cell build's, 4 more with balsara), the density loop's lists (list_cap)
+ * and, grown at builds, 24 bytes per cell.  The first sph_step_bwd allocates as
+ * much again and 254 bytes per particle.  Errors: SPH_ERR_ARG, SPH_ERR_NOMEM. */
 int sph_create(const sph_params *params, int64_t n_max, sph_ctx **ctx);
 int sph_destroy(sph_ctx *ctx);
 
