@@ -499,7 +499,8 @@ __device__ void density_group(const View &v, int wg, int slice, int nslices, int
           if (search_now) have_list = complete;
           if (writer) wc.gathers += nlive;
           if (gath) {
-            nl = min(acc - skipc, cap);
+            // (none where only other lanes of the particle go on)
+            nl = max(0, min(acc - skipc, cap));
 #pragma unroll
             for (int j = 0; j < LQ; j++) {
               if constexpr (UM) __stcg(lstr + (size_t)(nl + j) * ls, INFINITY);
