@@ -497,7 +497,8 @@ int recover(sph_ctx *ctx, sph_particles *p, cudaStream_t st, bool *redo) {
   *redo = false;
   const DevState h = *ctx->b.h_ds;
   if (!h.halt) return SPH_OK;
-  if (h.first_error != SPH_ERR_CELL_OVERFLOW) return h.first_error ? h.first_error : SPH_ERR_CUDA;
+  // (first_error may be one that does not halt: an h that did not converge)
+  if (h.halt != (unsigned int)SPH_ERR_CELL_OVERFLOW) return (int)h.halt;
   // the cells are too small for the supports: rebuild.  When an h iteration
   // wanted to grow past the cell, size the new cells for the h it wanted.
   float want_h, Hmax;
@@ -1174,7 +1175,7 @@ int sph_step_bwd(sph_ctx *ctx, const sph_particles *pre, const sph_particles *po
   SPH_TRY(read_state(sub, st));
   const DevState &h = *sub->b.h_ds;
   if (h.halt || h.first_error) {
-    const int e = h.first_error ? h.first_error : SPH_ERR_CUDA;
+    const int e = h.halt ? (int)h.halt : h.first_error;
     SPH_TRY(sph_clear_status(sub, stream));
     return e;
   }

@@ -59,7 +59,7 @@ struct DevState {
   int head_grad;              // gradient loop (velocity divergence and curl)
   unsigned int blocks_done;   // blocks of the closing kernel of a step that have finished
   // errors
-  unsigned int halt;      // a step-invalidating error happened: kernels return
+  unsigned int halt;      // first SPH_ERR_* that invalidates the step (0: none): kernels return
   int first_error;        // first SPH_ERR_* code recorded
   unsigned long long err_count[16];
   // first failed bounds check (a library built with SPH_CHECKS)
@@ -232,7 +232,7 @@ __device__ __forceinline__ void record_error(DevState *ds, int code, unsigned lo
                                              bool halt) {
   atomicCAS(&ds->first_error, 0, code);
   atomicAdd(&ds->err_count[code & 15], count);
-  if (halt) atomicExch(&ds->halt, 1u);
+  if (halt) atomicCAS(&ds->halt, 0u, (unsigned int)code);
 }
 
 // No wake request (the limiter's waking of inactive neighbours): the byte

@@ -1400,7 +1400,8 @@ __global__ void __launch_bounds__(PT, 2) k_density_big(View v, int flags) {
   // (a support that outgrew its cell halts the step, but its density launch
   // updates every other particle all the same, and the redone step starts its
   // iterations from their h)
-  if (nb == 0 || (ds->halt && ds->first_error != SPH_ERR_CELL_OVERFLOW)) return;
+  const unsigned int halt = ds->halt;
+  if (nb == 0 || (halt && halt != (unsigned int)SPH_ERR_CELL_OVERFLOW)) return;
   const float exc = __uint_as_float(ds->excursion_bits);
   StageD st;
   stage_init(st, max(v.stage_depth, 2), v.wait_limit);  // (one warp's work is a chain of latencies)
