@@ -239,7 +239,8 @@ int sph_destroy(sph_ctx *ctx);
  * leaf_max particles.  Refreshes the FP32 cell-relative records every pair
  * loop reads, and finds whether every particle has the same mass (the density
  * loop then sums the kernel alone: rho = m sum w; masses are taken to stay
- * as they are until the next build).  Synchronises `stream` (to size the
+ * as they are until the next build).  No particle is active until the next
+ * sph_mark_active (a step marks by itself).  Synchronises `stream` (to size the
  * grid and to check the input).  Errors: SPH_ERR_ARG (also when a position is not finite or an h
  * is not a positive finite number; nothing is reordered then, and the cells stay
  * those of the build before unless the new grid has more of them),
