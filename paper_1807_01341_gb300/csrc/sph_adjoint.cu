@@ -853,7 +853,7 @@ struct GridKernel {
 // computed the offsets of each point anew, with FP64 square roots and
 // divisions, 45 and more FP64 instructions per point of the whole box.
 // 110,592 particles on a 64^3 grid (113 points in a support): 1885 -> 463 us,
-// backward 3385 -> 787 us; 262,144 on 32^3 209 -> 182 us and 314 -> 220 us;
+// backward 3385 -> 787 us; 262,144 on 32^3 514 -> 421 us and 894 -> 530 us;
 // 2,744 on 128^3 (supports of 40,000 points) 153 -> 2.5 ms and 182 -> 4.3 ms.
 // Against extended precision a point's W is off by 4.0e-17 rms (before 4.5e-17),
 // its d/dh by 1.1e-16 (1.5e-16).  Against 64-bit sums of the textbook form
@@ -862,12 +862,14 @@ struct GridKernel {
 // Where at least GD_LANES of a warp's particles have boxes of at most GD_FEW
 // points, those are one lane's work each, all at once: a warp per particle costs
 // some 20 FP64 instructions before its first point (27,000 particles on a 16^3
-// grid: 114 us, a lane per particle 75 us; here 74 us).  With fewer such particles
+// grid: 114 us, a lane per particle 75 us; here 72 us).  With fewer such particles
 // a point of a lane's own costs about as much as a particle of the warp's, and
 // the longest lane counts: lanes only for twice as many particles as points (a
 // support that misses most points, 1,000,000 particles on 16^3: 553 -> 285 us,
-// backward 836 -> 323; with as many lanes as points clumps on a fine grid, 111k on
-// 64^3, take 702 against 495 us).
+// backward 836 -> 323).  They come after the warp's own particles: first, every
+// warp sends them at once, and the points of a clump, or of a coarse grid, take
+// many additions each (a clumpy 111k on 64^3 460 -> 538 us where one clump meets a
+// point; 262,144 on 32^3 521 us first, 421 last).
 constexpr int GD_WARPS = 4, GD_SIDE = 32, GD_FEW = 27, GD_LANES = 16;
 struct GridWarp {
   double d[3][GD_SIDE];   // (x - x_g) / H along each axis
@@ -907,7 +909,7 @@ __global__ void __launch_bounds__(GD_WARPS * 32, 6)
       for (int k = 0; k < 3; k++) grid_range(X[k], H, s, ng, a0[k], na[k]);
     }
     double o[4] = {0.0, 0.0, 0.0, 0.0};  // BWD: this lane's particle
-    // boxes of a few points: one lane per particle, all at once
+    // boxes of a few points: one lane per particle, all at once (below)
     const int box3 = na[0] > 0 && na[1] > 0 && na[2] > 0 && na[0] <= GD_FEW && na[1] <= GD_FEW &&
                              na[2] <= GD_FEW
                          ? na[0] * na[1] * na[2]
@@ -915,25 +917,6 @@ __global__ void __launch_bounds__(GD_WARPS * 32, 6)
     bool few = box3 > 0 && box3 <= GD_FEW;
     const int lanes = __popc(__ballot_sync(FULL, few));
     if (lanes < GD_LANES && 2 * __reduce_max_sync(FULL, few ? box3 : 0) > lanes) few = false;
-    if (few) {
-      const GridKernel<BWD> K(C, Hinv);
-      for (int c = 0; c < na[2]; c++) {
-        const int iz = ((a0[2] + c) % ng + ng) % ng;
-        const double dz = min_img(X[2] - (iz + 0.5) * s, box) * Hinv;
-        for (int b = 0; b < na[1]; b++) {
-          const int iy = ((a0[1] + b) % ng + ng) % ng;
-          const double dy = min_img(X[1] - (iy + 0.5) * s, box) * Hinv;
-          for (int a = 0; a < na[0]; a++) {
-            const int ix = ((a0[0] + a) % ng + ng) % ng;
-            const double dx = min_img(X[0] - (ix + 0.5) * s, box) * Hinv;
-            const double q2 = fma(dz, dz, fma(dy, dy, dx * dx));
-            if (q2 < 1.0)
-              K.point(dx, dy, dz, q2, (float)q2, ix + (long long)ng * (iy + (long long)ng * iz), rho_g,
-                      rho_bar, o);
-          }
-        }
-      }
-    }
     for (unsigned todo = __ballot_sync(FULL, !few && na[0] > 0 && na[1] > 0 && na[2] > 0); todo;
          todo &= todo - 1u) {
       const int k = __ffs(todo) - 1;
@@ -1022,6 +1005,25 @@ __global__ void __launch_bounds__(GD_WARPS * 32, 6)
           o[1] = r1;
           o[2] = r2;
           o[3] = r3;
+        }
+      }
+    }
+    if (few) {
+      const GridKernel<BWD> K(C, Hinv);
+      for (int c = 0; c < na[2]; c++) {
+        const int iz = ((a0[2] + c) % ng + ng) % ng;
+        const double dz = min_img(X[2] - (iz + 0.5) * s, box) * Hinv;
+        for (int b = 0; b < na[1]; b++) {
+          const int iy = ((a0[1] + b) % ng + ng) % ng;
+          const double dy = min_img(X[1] - (iy + 0.5) * s, box) * Hinv;
+          for (int a = 0; a < na[0]; a++) {
+            const int ix = ((a0[0] + a) % ng + ng) % ng;
+            const double dx = min_img(X[0] - (ix + 0.5) * s, box) * Hinv;
+            const double q2 = fma(dz, dz, fma(dy, dy, dx * dx));
+            if (q2 < 1.0)
+              K.point(dx, dy, dz, q2, (float)q2, ix + (long long)ng * (iy + (long long)ng * iz), rho_g,
+                      rho_bar, o);
+          }
         }
       }
     }
